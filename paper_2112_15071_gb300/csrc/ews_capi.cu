@@ -65,6 +65,11 @@ constexpr double kC2 = -1.0 / 24.0;
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+// Steps of one resident launch without receivers, and the bytes of staged tap
+// values one may fill with them (a launch costs about two steps).
+constexpr int kResidentSteps = 4096;
+constexpr size_t kResidentStage = 4u << 20;
+
 // ---- tile shapes of the forward passes ----
 // Plain forward steps (no free surface, no coarse medium grid, no history
 // capture) may run the passes of another tile shape; the others use 32 x 8.
@@ -583,6 +588,61 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
     return EWS_OK;
 }
 
+// Steps n0 .. n0 + nsteps - 1 of a small grid with the fields resident in
+// shared memory, one launch per res_chunk steps.  Accounted like the passes
+// it runs: per step one velocity pass, one stress pass and the point terms.
+bool resident_eligible(const ews_sim* s) {
+    return s->res && s->tile_req == EWS_TILE_AUTO && !s->profiling;
+}
+ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
+                          float* dseis, int ld, float* vcap) {
+    const DevSource S = source_taps(s, src, dt);
+    const bool rec = s->nrec > 0 && dseis;
+    ResidentRun r{};
+    r.plan = s->res;
+    r.g = s->g;
+    r.F = s->F();
+    r.M = s->M();
+    r.B = s->B;
+    r.S = &S;
+    r.wavelet = s->wavelet;
+    r.dt = (float)dt;
+    r.inbox = s->res_inbox;
+    r.err = s->err;
+    r.nrec = rec ? s->nrec : 0;
+    r.taps = s->rtaps;
+    r.tlist = s->res_list;
+    r.tstart = s->res_start;
+    r.stage = s->res_stage;
+    r.seis = rec ? dseis : nullptr;
+    r.ld = ld;
+    r.fstride = (long long)s->fstride;
+    s->fresh = false;
+    const int chunk = rec ? s->res_chunk : kResidentSteps;
+    for (int m = 0; m < nsteps; m += chunk) {
+        r.n0 = n0 + m;
+        r.nsteps = std::min(chunk, nsteps - m);
+        if (s->res_epoch > 0xF0000000u) {              // before the tags wrap around
+            CK(cudaMemsetAsync(s->res_inbox, 0, resident_inbox_bytes(*s->res), s->stream));
+            s->res_epoch = 0;
+        }
+        r.epoch = s->res_epoch;
+        s->res_epoch += (unsigned)r.nsteps;
+        // v^{n+1/2} of step n0 + m goes to slot m + 1 of the history
+        r.vcap = vcap ? vcap + (size_t)(m + 1) * 3 * s->fstride : nullptr;
+        CK(launch_resident(r, s->stream));
+    }
+    s->launches[EWS_KERNEL_VELOCITY] += nsteps;
+    s->launches[EWS_KERNEL_STRESS] += nsteps;
+    if (S.kind == EWS_SOURCE_MOMENT && rec) {
+        s->launches[EWS_KERNEL_POINTS] += nsteps;
+    } else {
+        if (S.kind >= 0) s->launches[EWS_KERNEL_INJECT] += nsteps;
+        if (rec) s->launches[EWS_KERNEL_RECORD] += nsteps;
+    }
+    return EWS_OK;
+}
+
 // The time loop of steps_direct, captured once into a CUDA graph per
 // (state generation, step range, dt, output buffers) and replayed: one
 // graph launch per call instead of 4-5 kernel launches per step.  With
@@ -590,6 +650,8 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
 // them).
 ews_status steps(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
                  float* dseis, int ld, float* vcap = nullptr) {
+    if (resident_eligible(s) && nsteps > 0)
+        return steps_resident(s, src, n0, nsteps, dt, dseis, ld, vcap);
     if (s->profiling || nsteps <= 0) return steps_direct(s, src, n0, nsteps, dt, dseis, ld, vcap);
     GraphEntry* hit = nullptr;
     for (GraphEntry& ge : s->graphs)
@@ -1225,6 +1287,22 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
     e = stencil_plan_create(s->g, s->F(), s->M(), s->B, o.storage, &s->plan);
     if (e != cudaSuccess)
         return cleanup(fail(EWS_ECUDA, "stencil plan (TMA descriptors): %s", cudaGetErrorString(e)));
+    int sms = 0, coop = 0;
+    ResidentPlan rp;
+    if (s->wide() && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+        resident_plan(s->g, o.boundary, sms, &rp)) {
+        e = resident_prepare(rp, o.boundary);
+        if (e != cudaSuccess)
+            return cleanup(fail(EWS_ECUDA, "resident time loop: %s", cudaGetErrorString(e)));
+        e = dev_malloc((void**)&s->res_inbox, resident_inbox_bytes(rp));
+        if (e != cudaSuccess) return cleanup(fail(EWS_ENOMEM, "halo inboxes: %s", cudaGetErrorString(e)));
+        e = cudaMemset(s->res_inbox, 0, resident_inbox_bytes(rp));
+        if (e == cudaSuccess) e = cudaDeviceSynchronize();
+        if (e != cudaSuccess) return cleanup(fail(EWS_ECUDA, "halo inboxes: %s", cudaGetErrorString(e)));
+        s->res = new (std::nothrow) ResidentPlan(rp);
+        if (!s->res) return cleanup(fail(EWS_ENOMEM, "host allocation failed"));
+    }
     *out = s;
     return EWS_OK;
 }
@@ -1245,6 +1323,11 @@ void ews_destroy(ews_sim* s) {
     dev_free(s->psi);
     dev_free(s->wavelet);
     dev_free(s->rtaps);
+    delete s->res;
+    dev_free(s->res_inbox);
+    dev_free(s->res_list);
+    dev_free(s->res_start);
+    dev_free(s->res_stage);
     dev_free(s->seis_buf);
     dev_free(s->adj);
     dev_free(s->acc64);
@@ -1421,10 +1504,30 @@ ews_status ews_set_receivers(ews_sim* s, int nrec, const double* pos) {
     dev_free(s->rtaps);
     s->rtaps = nullptr;
     s->nrec = 0;
+    dev_free(s->res_list);
+    dev_free(s->res_start);
+    dev_free(s->res_stage);
+    s->res_list = nullptr;
+    s->res_start = nullptr;
+    s->res_stage = nullptr;
     if (nrec > 0) {
         CK(dev_malloc((void**)&s->rtaps, taps.size() * sizeof(Tap)));
         CK(cudaMemcpyAsync(s->rtaps, taps.data(), taps.size() * sizeof(Tap),
                            cudaMemcpyHostToDevice, s->stream));
+        std::vector<int2> list;
+        std::vector<int> start;
+        if (s->res) {
+            resident_taps(*s->res, s->g, taps.data(), (int)taps.size(), &list, &start);
+            const size_t row = taps.size() * sizeof(float);
+            s->res_chunk = (int)std::min<size_t>(kResidentSteps, std::max<size_t>(16, kResidentStage / row));
+            CK(dev_malloc((void**)&s->res_list, list.size() * sizeof(int2)));
+            CK(dev_malloc((void**)&s->res_start, start.size() * sizeof(int)));
+            CK(dev_malloc((void**)&s->res_stage, s->res_chunk * row));
+            CK(cudaMemcpyAsync(s->res_list, list.data(), list.size() * sizeof(int2),
+                               cudaMemcpyHostToDevice, s->stream));
+            CK(cudaMemcpyAsync(s->res_start, start.data(), start.size() * sizeof(int),
+                               cudaMemcpyHostToDevice, s->stream));
+        }
         CK(cudaStreamSynchronize(s->stream));
     }
     s->nrec = nrec;

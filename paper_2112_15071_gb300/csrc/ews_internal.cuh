@@ -21,6 +21,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
 #include "../../include/ews.h"
 
 namespace ews {
@@ -150,9 +152,11 @@ __device__ __forceinline__ float zdiff(const DevGrid& g, const ZW& zw, const ZT&
                     : zt.iA * a + zt.iB * b + zt.iC * c + zt.iD * d;
     } else if constexpr (FS == ZS_FWD) {
         // Eq. 4, or its inner pair alone on the switched planes
-        return (HALF ? zw.h2 : zw.i2) ? g.c1z2 * (c - b) : g.c1z * (c - b) + g.c2z * (d - a);
+        const float in = __fsub_rn(c, b);
+        return (HALF ? zw.h2 : zw.i2) ? __fmul_rn(g.c1z2, in)
+                                      : __fmaf_rn(g.c2z, __fsub_rn(d, a), __fmul_rn(g.c1z, in));
     } else {
-        return g.c1z * (c - b) + g.c2z * (d - a);
+        return __fmaf_rn(g.c2z, __fsub_rn(d, a), __fmul_rn(g.c1z, __fsub_rn(c, b)));
     }
 }
 
@@ -446,6 +450,45 @@ cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const De
                          const DevBoundary& B, float dt, const DevSource& S, const float* wavelet,
                          int n, int* err, cudaStream_t st);
 }  // namespace fused
+
+// The time loop of a small grid in one cooperative launch with the fields
+// resident in shared memory (ews_resident.cu; FP32 storage, every boundary,
+// with a free surface or a coarse medium grid too): one CTA per block of the
+// grid, nbx x nby x nbz blocks of at most lz planes.
+struct ResidentPlan {
+    int nbx = 0, nby = 0, nbz = 0, lz = 0;
+    int lines[3] = {0, 0, 0};     // halo lines of a block's face per axis, at most
+};
+struct ResidentRun {
+    const ResidentPlan* plan;
+    DevGrid g;
+    DevFields F;
+    DevMedium M;
+    DevBoundary B;
+    const DevSource* S;
+    const float* wavelet;
+    float dt;
+    int n0, nsteps;
+    unsigned long long* inbox;    // resident_inbox_bytes(), zero before the first launch
+    unsigned epoch;               // steps of all launches with this inbox before
+    int* err;
+    int nrec;
+    const Tap* taps;              // receiver taps [3 nrec][8]
+    const int2* tlist;            // taps by CTA (resident_taps)
+    const int* tstart;
+    float* stage;                 // [nsteps][24 nrec]
+    float* seis;                  // null: no recording
+    int ld;
+    float* vcap;                  // history slot of v^{n0+1/2}, or null
+    long long fstride;
+};
+// False where the grid does not fit `sms` CTAs.
+bool resident_plan(const DevGrid& g, int bnd, int sms, ResidentPlan* out);
+size_t resident_inbox_bytes(const ResidentPlan& p);
+cudaError_t resident_prepare(const ResidentPlan& p, int bnd);
+void resident_taps(const ResidentPlan& p, const DevGrid& g, const Tap* taps, int ntap,
+                   std::vector<int2>* list, std::vector<int>* start);
+cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st);
 
 // History buffer of the reverse pass: nslot slots of 3 fields, slot s field c
 // at hist + (3 s + c) * fstride, pitched like the wavefields; and its 8 FP32

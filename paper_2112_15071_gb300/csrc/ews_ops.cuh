@@ -64,7 +64,7 @@ __device__ __forceinline__ void inject_tap(const DevGrid& g, const DevFields& F,
                                            const float* __restrict__ wavelet, int n, int t,
                                            int* err) {
     const Tap tp = S.tap[t];
-    float amp = tp.w * __ldg(wavelet + n);
+    float amp = __fmul_rn(tp.w, __ldg(wavelet + n));
     if (S.kind == 1) {
         if (g.cm[2]) {           // coarse medium: 1 / rho sampled at the v point
             const int c = tp.q - VX;
@@ -94,7 +94,7 @@ __device__ __forceinline__ float record_one(const DevGrid& g, const DevFields& F
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
         const Tap q = tp[m];
-        acc += q.w * Io<T>::get(reinterpret_cast<const T*>(F.f[q.q]) + cidx(g, q.i, q.j, q.k));
+        acc = __fmaf_rn(q.w, Io<T>::get(reinterpret_cast<const T*>(F.f[q.q]) + cidx(g, q.i, q.j, q.k)), acc);
     }
     return acc;
 }

@@ -84,6 +84,16 @@ struct ews_sim {
     // second set of wavefields of the fused step (9 * fstride floats, laid
     // out like `fields`), held with its plan
     float* fields2 = nullptr;
+    // time loop of a small grid in one launch (null where it does not fit):
+    // its CTAs' halo inboxes with the steps they have served, the receiver
+    // taps by CTA, and the staged tap values of up to res_chunk steps
+    ResidentPlan* res = nullptr;
+    unsigned long long* res_inbox = nullptr;
+    unsigned res_epoch = 0;
+    int2* res_list = nullptr;
+    int* res_start = nullptr;
+    float* res_stage = nullptr;
+    int res_chunk = 0;
     cudaStream_t stream = nullptr;
     // launch accounting and optional per-launch event timing
     long long launches[EWS_NKERNEL] = {};

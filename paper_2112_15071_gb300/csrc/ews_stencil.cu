@@ -44,6 +44,7 @@
 #include <new>
 #include <type_traits>
 
+#include "ews_arith.cuh"
 #include "ews_internal.cuh"
 #include "ews_ops.cuh"
 #ifndef EWS_L2PROMO
@@ -482,9 +483,9 @@ __device__ __forceinline__ void aux_refill(const Maps& maps, const Geo<BND, T>& 
 // psi = b psi + a d; d += psi for the three terms of one damped direction.
 __device__ __forceinline__ void pml_upd(float& p0, float& p1, float& p2, float a, float b,
                                         float& d0, float& d1, float& d2) {
-    p0 = b * p0 + a * d0; d0 += p0;
-    p1 = b * p1 + a * d1; d1 += p1;
-    p2 = b * p2 + a * d2; d2 += p2;
+    ar::pml(p0, a, b, d0);
+    ar::pml(p1, a, b, d1);
+    ar::pml(p2, a, b, d2);
 }
 
 // Field tile element as FP32.
@@ -608,16 +609,16 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
             const float* qyz = Q.yz[rr];
             const float* qzz = Q.zz[rr];
             // vx at (i+1/2, j, k)
-            float dxx = g.c1x * (F(hxx, R + 1) - F(hxx, R)) + g.c2x * (F(hxx, R + 2) - F(hxx, R - 1));
-            float dxy = g.c1y * (F(hxy, R) - F(hxy, R - HX)) + g.c2y * (F(hxy, R + HX) - F(hxy, R - 2 * HX));
+            float dxx = ar::d4(g.c1x, g.c2x, F(hxx, R - 1), F(hxx, R), F(hxx, R + 1), F(hxx, R + 2));
+            float dxy = ar::d4(g.c1y, g.c2y, F(hxy, R - 2 * HX), F(hxy, R - HX), F(hxy, R), F(hxy, R + HX));
             float dxz = zdiff<ZF, false>(g, zw, zt, qxz[A], qxz[B], qxz[C], qxz[D]);
             // vy at (i, j+1/2, k)
-            float dyx = g.c1x * (F(hxy, R) - F(hxy, R - 1)) + g.c2x * (F(hxy, R + 1) - F(hxy, R - 2));
-            float dyy = g.c1y * (F(hyy, RY + TX) - F(hyy, RY)) + g.c2y * (F(hyy, RY + 2 * TX) - F(hyy, RY - TX));
+            float dyx = ar::d4(g.c1x, g.c2x, F(hxy, R - 2), F(hxy, R - 1), F(hxy, R), F(hxy, R + 1));
+            float dyy = ar::d4(g.c1y, g.c2y, F(hyy, RY - TX), F(hyy, RY), F(hyy, RY + TX), F(hyy, RY + 2 * TX));
             float dyz = zdiff<ZF, false>(g, zw, zt, qyz[A], qyz[B], qyz[C], qyz[D]);
             // vz at (i, j, k+1/2)
-            float dzx = g.c1x * (F(hxz, R) - F(hxz, R - 1)) + g.c2x * (F(hxz, R + 1) - F(hxz, R - 2));
-            float dzy = g.c1y * (F(hyz, RY) - F(hyz, RY - TX)) + g.c2y * (F(hyz, RY + TX) - F(hyz, RY - 2 * TX));
+            float dzx = ar::d4(g.c1x, g.c2x, F(hxz, R - 2), F(hxz, R - 1), F(hxz, R), F(hxz, R + 1));
+            float dzy = ar::d4(g.c1y, g.c2y, F(hyz, RY - 2 * TX), F(hyz, RY - TX), F(hyz, RY), F(hyz, RY + TX));
             float dzz = zdiff<ZF, true>(g, zw, zt, qzz[A], qzz[B], qzz[C], qzz[D]);
             if constexpr (kScaled<T>) {     // stored -> physical units
                 dxx *= P.inv[SXX]; dxy *= P.inv[SXY]; dxz *= P.inv[SXZ];
@@ -656,8 +657,8 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 const float* qhx = Q.hx[rr];
                 const float* qhy = Q.hy[rr];
                 const float* qhz = Q.hz[rr];
-                const float exx = g.c1x * (F(vhx, R) - F(vhx, R - 1)) + g.c2x * (F(vhx, R + 1) - F(vhx, R - 2));
-                const float eyy = g.c1y * (F(vhy, R) - F(vhy, R - HX)) + g.c2y * (F(vhy, R + HX) - F(vhy, R - 2 * HX));
+                const float exx = ar::d4(g.c1x, g.c2x, F(vhx, R - 2), F(vhx, R - 1), F(vhx, R), F(vhx, R + 1));
+                const float eyy = ar::d4(g.c1y, g.c2y, F(vhy, R - 2 * HX), F(vhy, R - HX), F(vhy, R), F(vhy, R + HX));
                 constexpr int FW = ZF == ZS_NONE ? ZS_NONE : ZS_FWD;   // forward strain rates
                 const float ezz = zdiff<FW, false>(g, zw, zt, qhz[A], qhz[B], qhz[C], qhz[D]);
                 const float gxy = g.c1y * (F(vhx, R + HX) - F(vhx, R)) + g.c2y * (F(vhx, R + 2 * HX) - F(vhx, R - HX)) +
@@ -709,13 +710,13 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 bz = __fdividef(1.0f, lerp1(Q.ch.lo[rr][0], Q.ch.hi[rr][0], zh.f));
             } else {
                 const float r0 = hr[RF];
-                bx = __fdividef(2.0f, r0 + hr[RF + G.cx]);
-                by = __fdividef(2.0f, r0 + hr[RF + G.cy[rr]]);
-                bz = __fdividef(2.0f, r0 + (ktop ? hr1[RF] : r0));
+                bx = ar::buoyancy(r0, hr[RF + G.cx]);
+                by = ar::buoyancy(r0, hr[RF + G.cy[rr]]);
+                bz = ar::buoyancy(r0, ktop ? hr1[RF] : r0);
             }
-            float vx = F(vc, VC_VX * CORE + rr * TX) + P.dto[VX] * bx * (dxx + dxy + dxz);
-            float vy = F(vc, VC_VY * CORE + rr * TX) + P.dto[VY] * by * (dyx + dyy + dyz);
-            float vz = F(vc, VC_VZ * CORE + rr * TX) + P.dto[VZ] * bz * (dzx + dzy + dzz);
+            float vx = ar::vnew(F(vc, VC_VX * CORE + rr * TX), P.dto[VX], bx, dxx, dxy, dxz);
+            float vy = ar::vnew(F(vc, VC_VY * CORE + rr * TX), P.dto[VY], by, dyx, dyy, dyz);
+            float vz = ar::vnew(F(vc, VC_VZ * CORE + rr * TX), P.dto[VZ], bz, dzx, dzy, dzz);
             if (BND == BND_SPONGE) {
                 const float Gs = G3 * G.gy[rr];
                 vx *= Gs; vy *= Gs; vz *= Gs;
@@ -881,16 +882,16 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
             const float* qvy = Q.vy[rr];
             const float* qvz = Q.vz[rr];
             // normal strain rates at (i, j, k)
-            float exx = g.c1x * (F(hvx, R) - F(hvx, R - 1)) + g.c2x * (F(hvx, R + 1) - F(hvx, R - 2));
-            float eyy = g.c1y * (F(hvy, R) - F(hvy, R - HX)) + g.c2y * (F(hvy, R + HX) - F(hvy, R - 2 * HX));
+            float exx = ar::d4(g.c1x, g.c2x, F(hvx, R - 2), F(hvx, R - 1), F(hvx, R), F(hvx, R + 1));
+            float eyy = ar::d4(g.c1y, g.c2y, F(hvy, R - 2 * HX), F(hvy, R - HX), F(hvy, R), F(hvy, R + HX));
             float ezz = zdiff<ZF, false>(g, zw, zt, qvz[A], qvz[B], qvz[C], qvz[D]);
             // shear terms at the shear points
-            float vxy = g.c1y * (F(hvx, R + HX) - F(hvx, R)) + g.c2y * (F(hvx, R + 2 * HX) - F(hvx, R - HX));
-            float vyx = g.c1x * (F(hvy, R + 1) - F(hvy, R)) + g.c2x * (F(hvy, R + 2) - F(hvy, R - 1));
+            float vxy = ar::d4(g.c1y, g.c2y, F(hvx, R - HX), F(hvx, R), F(hvx, R + HX), F(hvx, R + 2 * HX));
+            float vyx = ar::d4(g.c1x, g.c2x, F(hvy, R - 1), F(hvy, R), F(hvy, R + 1), F(hvy, R + 2));
             float vxz = zdiff<ZF, true>(g, zw, zt, qvx[A], qvx[B], qvx[C], qvx[D]);
-            float vzx = g.c1x * (F(hvz, R + 1) - F(hvz, R)) + g.c2x * (F(hvz, R + 2) - F(hvz, R - 1));
+            float vzx = ar::d4(g.c1x, g.c2x, F(hvz, R - 1), F(hvz, R), F(hvz, R + 1), F(hvz, R + 2));
             float vyz = zdiff<ZF, true>(g, zw, zt, qvy[A], qvy[B], qvy[C], qvy[D]);
-            float vzy = g.c1y * (F(hvz, R + HX) - F(hvz, R)) + g.c2y * (F(hvz, R + 2 * HX) - F(hvz, R - HX));
+            float vzy = ar::d4(g.c1y, g.c2y, F(hvz, R - HX), F(hvz, R), F(hvz, R + HX), F(hvz, R + 2 * HX));
             if constexpr (kScaled<T>) {     // stored -> physical units
                 exx *= P.inv[VX]; vxy *= P.inv[VX]; vxz *= P.inv[VX];
                 eyy *= P.inv[VY]; vyx *= P.inv[VY]; vyz *= P.inv[VY];
@@ -951,25 +952,25 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
                 mu0 = hmu[RF];
                 const float mxp = hmu[RF + G.cx], myp = hmu[RF + cyr];
                 const float mzp = hmu1[RF];
-                mxy = 0.25f * (mu0 + mxp + myp + hmu[RF + G.cx + cyr]);
-                mxz = 0.25f * (mu0 + mxp + mzp + hmu1[RF + G.cx]);
-                myz = 0.25f * (mu0 + myp + mzp + hmu1[RF + cyr]);
+                mxy = ar::mean4(mu0, mxp, myp, hmu[RF + G.cx + cyr]);
+                mxz = ar::mean4(mu0, mxp, mzp, hmu1[RF + G.cx]);
+                myz = ar::mean4(mu0, myp, mzp, hmu1[RF + cyr]);
                 if constexpr (ZF != ZS_NONE) {
                     // xz / yz shear points on the free-surface plane z = ks - 1/2:
                     // harmonic mean of the 4 cells (vacuum-formulation reading)
                     if (k == g.fs - 1) {
-                        mxz = 4.0f / (1.0f / mu0 + 1.0f / mxp + 1.0f / mzp + 1.0f / hmu1[RF + G.cx]);
-                        myz = 4.0f / (1.0f / mu0 + 1.0f / myp + 1.0f / mzp + 1.0f / hmu1[RF + cyr]);
+                        mxz = ar::harm4(mu0, mxp, mzp, hmu1[RF + G.cx]);
+                        myz = ar::harm4(mu0, myp, mzp, hmu1[RF + cyr]);
                     }
                 }
             }
-            const float l2m = lam + 2.0f * mu0;
-            float s0 = F(cr, SC_SXX * CORE + rr * TX) + P.dto[SXX] * (l2m * exx + lam * (eyy + ezz));
-            float s1 = F(cr, SC_SYY * CORE + rr * TX) + P.dto[SYY] * (l2m * eyy + lam * (exx + ezz));
-            float s2 = F(cr, SC_SZZ * CORE + rr * TX) + P.dto[SZZ] * (l2m * ezz + lam * (exx + eyy));
-            float s3 = F(cr, SC_SXY * CORE + rr * TX) + P.dto[SXY] * mxy * (vxy + vyx);
-            float s4 = F(cr, SC_SXZ * CORE + rr * TX) + P.dto[SXZ] * mxz * (vxz + vzx);
-            float s5 = F(cr, SC_SYZ * CORE + rr * TX) + P.dto[SYZ] * myz * (vyz + vzy);
+            const float l2m = ar::l2m(lam, mu0);
+            float s0 = ar::snormal(F(cr, SC_SXX * CORE + rr * TX), P.dto[SXX], l2m, lam, exx, eyy, ezz);
+            float s1 = ar::snormal(F(cr, SC_SYY * CORE + rr * TX), P.dto[SYY], l2m, lam, eyy, exx, ezz);
+            float s2 = ar::snormal(F(cr, SC_SZZ * CORE + rr * TX), P.dto[SZZ], l2m, lam, ezz, exx, eyy);
+            float s3 = ar::sshear(F(cr, SC_SXY * CORE + rr * TX), P.dto[SXY], mxy, vxy, vyx);
+            float s4 = ar::sshear(F(cr, SC_SXZ * CORE + rr * TX), P.dto[SXZ], mxz, vxz, vzx);
+            float s5 = ar::sshear(F(cr, SC_SYZ * CORE + rr * TX), P.dto[SYZ], myz, vyz, vzy);
             if (BND == BND_SPONGE) {
                 const float Gs = G3 * G.gy[rr];
                 s0 *= Gs; s1 *= Gs; s2 *= Gs; s3 *= Gs; s4 *= Gs; s5 *= Gs;

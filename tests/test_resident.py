@@ -1,0 +1,88 @@
+"""The time loop of small grids in one launch with the fields resident on the
+SMs: blocks of at most 16 x 16 x 12 cells exchange halos step by step.  Its
+arithmetic is that of the passes, rounding by rounding, so seismograms and
+wavefields must equal those of the passes (which runs with per-launch
+profiling take) bit for bit -- at block edges and remainders on every axis,
+with one block and with the most, for every boundary and source kind, with a
+free surface, with a coarse medium grid, over several launches, in chunks,
+and with more receivers than one launch stages."""
+import numpy as np
+import pytest
+
+from paper_2112_15071_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ews():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2112_15071_gb300 import ews as E
+    E.load()
+    yield E
+
+
+def both(ews, p):
+    """(seismograms, state) of a run in one launch and of the passes."""
+    sim = ews.simulation_for(p)
+    got, state = sim.run(p.nt, p.dt), sim.get_state()
+    sim.set_tile_shape("32x8")
+    sim.set_profiling(True)
+    want = sim.run(p.nt, p.dt)
+    return (got, state), (want, sim.get_state())
+
+
+def same(a, b):
+    assert np.abs(b[0]).max() > 0
+    assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+# one block; 16 + 1 and 2 x 16 + 1 cells; 4, 5, 8 and 9..12 planes a block
+# (the thread shapes); many small blocks; the largest grids that fit
+SIZES = [(12, 11, 10), (17, 16, 9), (33, 18, 5), (16, 47, 33), (64, 60, 61), (31, 14, 150),
+         (80, 75, 71)]
+
+
+@pytest.mark.parametrize("n", SIZES)
+@pytest.mark.parametrize("boundary", ["none", "sponge", "cpml"])
+def test_equals_the_passes(ews, n, boundary):
+    kind = "force" if n[0] % 2 else "moment"
+    p = synth.small_problem(*n, nt=24, boundary=boundary, kind=kind, width=2, seed=301)
+    same(*both(ews, p))
+
+
+@pytest.mark.parametrize("at", [(15.6, 15.6, 7.6), (16.4, 15.4, 8.4), (1.2, 30.6, 22.6)])
+@pytest.mark.parametrize("kind", ["moment", "force"])
+def test_source_across_blocks(ews, at, kind):
+    """Taps of the source and of receivers in several blocks, or at the edge."""
+    p = synth.small_problem(33, 33, 25, nt=30, boundary="none", kind=kind, width=4, seed=303)
+    p.src_pos = np.array(at) * np.array(p.spacing)
+    p.rec_pos = np.array([[16.5, 16.5, 8.5], [15.5, 10.0, 7.5], [31.0, 31.0, 23.0]]) * np.array(p.spacing)
+    same(*both(ews, p))
+
+
+@pytest.mark.parametrize("boundary", ["sponge", "cpml"])
+def test_surface_and_coarse_medium(ews, boundary):
+    p = synth.small_problem(40, 36, 30, nt=30, boundary=boundary, kind="moment", width=5, seed=304)
+    p.free_surface = (8, 1e-3)
+    same(*both(ews, p))
+    q = synth.small_problem(40, 36, 30, nt=30, boundary=boundary, kind="force", width=5, seed=305,
+                            layered=False)
+    synth.with_coarse_medium(q, (9, 7, 5), seed=305, layer_vp=(2400.0, 2700.0, 2950.0))
+    same(*both(ews, q))
+
+
+def test_chunks_and_staged_receivers(ews):
+    """1500 receivers stage fewer steps than the run has (several launches);
+    a run in uneven chunks continues the same state."""
+    p = synth.small_problem(40, 36, 28, nt=70, boundary="sponge", kind="moment", width=5, seed=306,
+                            nrec=1500)
+    a, b = both(ews, p)
+    same(a, b)
+    sim = ews.simulation_for(p)
+    seis = np.zeros_like(a[0])
+    for n0, k in ((0, 1), (1, 32), (33, 37)):
+        sim.advance(n0, k, p.dt, seis, p.nt)
+    assert np.array_equal(seis, a[0]) and np.array_equal(sim.get_state(), a[1])
