@@ -493,7 +493,11 @@ ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, do
     DevMedium M = s->M();
     const DevSource S = source_taps(s, src, dt);
     const DevFields set[2] = {s->F(), s->F2()};
-    const float inv[NFIELD] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
+    float dto[NFIELD], inv[NFIELD];
+    for (int q = 0; q < NFIELD; ++q) {
+        dto[q] = (float)(dt * s->scale[q]);
+        inv[q] = 1.0f / s->scale[q];
+    }
     const int stor = s->opt.storage;
     s->fresh = false;
     ews_status st;
@@ -501,8 +505,7 @@ ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, do
     for (int n = n0; n < n0 + nsteps; ++n) {
         const int dir = (n - n0) & 1;
         const DevFields& out = set[dir ^ 1];
-        CK(fused::launch_fused(fp, dir, s->g, M, s->B, (float)dt, S, s->wavelet, n, s->err,
-                               s->stream));
+        CK(fused::launch_fused(fp, dir, s->g, M, s->B, dto, inv, S, s->wavelet, n, s->err, s->stream));
         if ((st = mark(s, EWS_KERNEL_STEP)) != EWS_OK) return st;
         const bool rec = s->nrec > 0 && dseis;
         if (S.kind == EWS_SOURCE_MOMENT && rec) {
@@ -1260,8 +1263,25 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
         ews_destroy(s);
         return st;
     };
-    e = dev_malloc((void**)&s->fields, NFIELD * s->fstride * s->es);
+    // the wavefields; on small grids the halo inboxes of the resident time loop
+    // follow them in the same allocation (zero before the first launch, too)
+    int sms = 0, coop = 0;
+    ResidentPlan rp;
+    size_t inbox = 0;
+    const size_t fbytes = (NFIELD * s->fstride * s->es + 255) / 256 * 256;
+    if (s->wide() && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+        resident_plan(s->g, o.boundary, sms, &rp)) {
+        e = resident_prepare(rp, o.boundary);
+        if (e != cudaSuccess)
+            return cleanup(fail(EWS_ECUDA, "resident time loop: %s", cudaGetErrorString(e)));
+        s->res = new (std::nothrow) ResidentPlan(rp);
+        if (!s->res) return cleanup(fail(EWS_ENOMEM, "host allocation failed"));
+        inbox = resident_inbox_bytes(rp);
+    }
+    e = dev_malloc((void**)&s->fields, fbytes + inbox);
     if (e != cudaSuccess) return cleanup(fail(EWS_ENOMEM, "wavefields: %s", cudaGetErrorString(e)));
+    if (inbox) s->res_inbox = reinterpret_cast<unsigned long long*>((char*)s->fields + fbytes);
     e = dev_malloc((void**)&s->medium, 3 * s->fstride * sizeof(float));
     if (e != cudaSuccess) return cleanup(fail(EWS_ENOMEM, "medium: %s", cudaGetErrorString(e)));
     const int nmax = std::max(g.nx, std::max(g.ny, g.nz));
@@ -1278,7 +1298,7 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
             return cleanup(fail(EWS_ENOMEM, "C-PML memory: %s", cudaGetErrorString(e)));
         for (int t = 0; t < 18; ++t) s->B.psi[t] = s->psi + t * s->fstride;
     }
-    e = cudaMemset(s->fields, 0, NFIELD * s->fstride * s->es);
+    e = cudaMemset(s->fields, 0, fbytes + inbox);
     if (e == cudaSuccess) e = cudaMemset(s->medium, 0, 3 * s->fstride * sizeof(float));
     if (e == cudaSuccess && s->psi) e = cudaMemset(s->psi, 0, s->psi_floats * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(s->err, 0, sizeof(int));
@@ -1287,22 +1307,6 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
     e = stencil_plan_create(s->g, s->F(), s->M(), s->B, o.storage, &s->plan);
     if (e != cudaSuccess)
         return cleanup(fail(EWS_ECUDA, "stencil plan (TMA descriptors): %s", cudaGetErrorString(e)));
-    int sms = 0, coop = 0;
-    ResidentPlan rp;
-    if (s->wide() && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        resident_plan(s->g, o.boundary, sms, &rp)) {
-        e = resident_prepare(rp, o.boundary);
-        if (e != cudaSuccess)
-            return cleanup(fail(EWS_ECUDA, "resident time loop: %s", cudaGetErrorString(e)));
-        e = dev_malloc((void**)&s->res_inbox, resident_inbox_bytes(rp));
-        if (e != cudaSuccess) return cleanup(fail(EWS_ENOMEM, "halo inboxes: %s", cudaGetErrorString(e)));
-        e = cudaMemset(s->res_inbox, 0, resident_inbox_bytes(rp));
-        if (e == cudaSuccess) e = cudaDeviceSynchronize();
-        if (e != cudaSuccess) return cleanup(fail(EWS_ECUDA, "halo inboxes: %s", cudaGetErrorString(e)));
-        s->res = new (std::nothrow) ResidentPlan(rp);
-        if (!s->res) return cleanup(fail(EWS_ENOMEM, "host allocation failed"));
-    }
     *out = s;
     return EWS_OK;
 }
@@ -1324,10 +1328,6 @@ void ews_destroy(ews_sim* s) {
     dev_free(s->wavelet);
     dev_free(s->rtaps);
     delete s->res;
-    dev_free(s->res_inbox);
-    dev_free(s->res_list);
-    dev_free(s->res_start);
-    dev_free(s->res_stage);
     dev_free(s->seis_buf);
     dev_free(s->adj);
     dev_free(s->acc64);
@@ -1504,25 +1504,33 @@ ews_status ews_set_receivers(ews_sim* s, int nrec, const double* pos) {
     dev_free(s->rtaps);
     s->rtaps = nullptr;
     s->nrec = 0;
-    dev_free(s->res_list);
-    dev_free(s->res_start);
-    dev_free(s->res_stage);
     s->res_list = nullptr;
     s->res_start = nullptr;
     s->res_stage = nullptr;
     if (nrec > 0) {
-        CK(dev_malloc((void**)&s->rtaps, taps.size() * sizeof(Tap)));
-        CK(cudaMemcpyAsync(s->rtaps, taps.data(), taps.size() * sizeof(Tap),
-                           cudaMemcpyHostToDevice, s->stream));
+        // the taps; for the resident time loop, in the same allocation, the
+        // taps by CTA and the staging rows
         std::vector<int2> list;
         std::vector<int> start;
+        const size_t tb = (taps.size() * sizeof(Tap) + 255) / 256 * 256;
+        size_t lb = 0, sb = 0, gb = 0;
         if (s->res) {
             resident_taps(*s->res, s->g, taps.data(), (int)taps.size(), &list, &start);
             const size_t row = taps.size() * sizeof(float);
             s->res_chunk = (int)std::min<size_t>(kResidentSteps, std::max<size_t>(16, kResidentStage / row));
-            CK(dev_malloc((void**)&s->res_list, list.size() * sizeof(int2)));
-            CK(dev_malloc((void**)&s->res_start, start.size() * sizeof(int)));
-            CK(dev_malloc((void**)&s->res_stage, s->res_chunk * row));
+            lb = (list.size() * sizeof(int2) + 255) / 256 * 256;
+            sb = (start.size() * sizeof(int) + 255) / 256 * 256;
+            gb = s->res_chunk * row;
+        }
+        char* base = nullptr;
+        CK(dev_malloc((void**)&base, tb + lb + sb + gb));
+        s->rtaps = reinterpret_cast<Tap*>(base);
+        CK(cudaMemcpyAsync(s->rtaps, taps.data(), taps.size() * sizeof(Tap),
+                           cudaMemcpyHostToDevice, s->stream));
+        if (s->res) {
+            s->res_list = reinterpret_cast<int2*>(base + tb);
+            s->res_start = reinterpret_cast<int*>(base + tb + lb);
+            s->res_stage = reinterpret_cast<float*>(base + tb + lb + sb);
             CK(cudaMemcpyAsync(s->res_list, list.data(), list.size() * sizeof(int2),
                                cudaMemcpyHostToDevice, s->stream));
             CK(cudaMemcpyAsync(s->res_start, start.data(), start.size() * sizeof(int),

@@ -1,73 +1,188 @@
 // ews_fused.cu -- one launch per time step: the velocity pass (Eq. 1) and the
-// stress pass (Eq. 2/3) of Sec. 2.3 fused, for FP32 wavefields with a sponge
-// or no absorbing boundary.
+// stress pass (Eq. 2/3) of Sec. 2.3 fused, for a sponge or no absorbing
+// boundary.
 //
 // The two-pass step moves 120 bytes per cell (velocity: 10 reads, 3 writes;
-// stress: 11 reads, 6 writes).  This step reads sigma^n, v^{n-1/2} and the
-// medium once and writes v^{n+1/2} and sigma^{n+1} once: 84 bytes.  To need
-// no exchange between CTAs it reads from one set of wavefields (A) and
-// writes to a second set (B), so nothing a neighbour still reads is ever
-// overwritten, and each CTA computes the new velocity on its 32 x 8 tile
-// plus the 2-cell ring its stress differences reach (36 x 12 cells, the ring
-// computed redundantly by the neighbours too) and on 2 planes above and below
-// its z-chunk.  The ring's velocity stays in shared memory; the CTA writes
-// only its own cells and planes.
+// stress: 11 reads, 6 writes) and runs at the DRAM rate on large FP32 grids.
+// This step reads sigma^n, v^{n-1/2} and the medium once and writes
+// v^{n+1/2} and sigma^{n+1} once: 84 bytes.  To need no exchange between CTAs
+// it reads from one set of wavefields (A) and writes to a second set (B), so
+// nothing a neighbour still reads is ever overwritten, and each CTA computes
+// the new velocity on its 32 x TY tile plus the 2-cell ring its stress
+// differences reach (36 x (TY + 4) cells, the ring computed redundantly by
+// the neighbours too) and on 2 planes above and below its z-chunk.
 //
-// Pipeline per CTA (tile x0, y0; z-chunk z0 .. z1): plane p of sigma^n,
-// v^{n-1/2} and rho arrives in a 4-slot TMA ring (boxes over the 36 x 12
-// velocity region and its halo).  Thread (tx, ty) owns tile cell (x0 + tx,
-// y0 + ty); threads below 176 also own one cell of the ring.  At arrival p
-// each thread computes the new velocity of plane kv = p - 2 at its cells
-// (z-derivatives from per-thread register queues) into a 4-plane shared
-// ring; after one barrier, the stress of plane ks = kv - 2 at its tile cell
-// (x / y differences of the new velocity from the shared ring, z-differences
-// and sigma^n of the cell from register queues, lambda and mu from a
-// 3-entry TMA buffer).  One barrier per plane: the 4-plane ring keeps a
-// plane until every thread has passed the next barrier after its last
-// reader, and the TMA refills of a slot or an entry go out after the barrier
-// that follows its last use.  Every mbarrier wait is bounded.  A point force
-// (Sec. 2.4 source term of Eq. 1) is added to the new velocity of its tap
-// cells before the stress uses them; a moment source and the receivers run
-// after the step, on B, as in the two-pass loop.  The arithmetic per cell is
-// that of the two passes.
-#define EWS_TILE_Y 8
-#define EWS_ROWS 1
-#define EWS_SHAPE_NS fused
-#include "ews_stencil.cu"
+// What bounds it is instruction issue and latency before DRAM, so a thread
+// owns a pair of x-neighbours: shared memory is read in pairs, y- and
+// z-differences and the updates are packed two-wide operations (f32x2), and
+// x-differences subtract lane by lane and go on packed.  One CTA per SM, 32 x
+// 24 cells: its 504 threads (16 warps) may use 128 registers, which the
+// columns need, and the ring adds 31 % velocity work (32 x 8 tiles: 69 %).
+// Taller tiles leave 96 or 80 registers a thread and spill (32 x 28: 35
+// Gcell/s at 1024 x 1024 x 512), lower ones have fewer warps (32 x 20: 59.7,
+// 32 x 16: 56.0, with 3 slots 63.1).  Row-wise thread order keeps the
+// half-warps on 16 neighbouring pairs of one row (no bank conflicts) and the
+// stress threads in full warps; the ring's outer columns have threads of
+// their own.  Edge masks are selects, not branches: a branch around them for
+// interior tiles cut the schedule apart (55.0 against 61.3).
+//
+// Measured (GB300, FP32, sponge, Gcell/s, against the two passes): 1024 x
+// 1024 x 512 62.7 (50.5), 256^3 61.0 (51.3); 0.78 and 0.76 of the copy peak
+// on 84 bytes a cell.  291 warp instructions per 32 cells at 1.8 per cycle
+// and SM; stalls: shared-memory and barrier latency at 4 warps per scheduler.
+//
+// Pipeline per CTA (tile x0, y0; z-chunk z0 .. z1), step m for velocity plane
+// k = z0 - 5 + m.  The copies of step m bring each field at the plane at which
+// plane k completes its stencil: sxx, syy, sxy, v at k; sxz, syz, rho at k + 1;
+// szz at k + 2 -- so only z-columns are held in registers, and a slot is read
+// in one step only (two slots: one in use, one in flight).  The new
+// velocity goes to a 5-plane shared ring; after one barrier the stress of
+// plane k - 2 is computed from it, with sigma^n of the cell from the register
+// columns and lambda, mu from a two-entry TMA buffer.  The first three steps
+// only fill the columns.
+//
+// Every mbarrier wait is bounded.  A point force (Sec. 2.4 source term of Eq.
+// 1) is added to the new velocity of its tap cells before the stress uses
+// them; a moment source and the receivers run after the step, on B, as in the
+// two-pass loop.  The arithmetic per cell is that of the two passes, rounding
+// by rounding (ews_arith.cuh).
+#include <cuda_bf16.h>
+#include <cuda_fp16.h>
+
+#include <algorithm>
+
+#include "ews_arith.cuh"
+#include "ews_internal.cuh"
+#include "ews_ops.cuh"
+#include "ews_tma.cuh"
 
 namespace ews {
 namespace fused {
 namespace {
 
-constexpr int EX = TX + 4, EY = TY + 4;          // velocity region: x0-2 .. x0+33, y0-2 .. y0+9
-constexpr int NE = EX * EY;                      // 432 cells
-constexpr int NRING = NE - CORE;                 // 176 ring cells
-constexpr int BW = TX + 8;                       // box width (x from x0-4: 16-byte aligned)
-// slot: sxx sxz (x halos, rows y0-2..y0+9), syy syz (y halos, rows y0-4..y0+11),
-// sxy (both), szz vx vy vz (the region), rho (the region + 1 row / column)
-constexpr int XB = BW * EY * 4, YB = BW * (EY + 4) * 4, ZB = BW * EY * 4, RB = BW * (EY + 1) * 4;
-constexpr int O_XP = 0, O_YP = O_XP + 2 * XB, O_XY = O_YP + 2 * YB, O_ZV = O_XY + YB;
-constexpr int O_RHO = O_ZV + 4 * ZB, FSLOT = r128(O_RHO + RB);
-constexpr int F_TX = 2 * XB + 3 * YB + 4 * ZB + RB;
-static_assert(O_YP % 128 == 0 && O_XY % 128 == 0 && O_ZV % 128 == 0 && O_RHO % 128 == 0,
-              "TMA destinations 128-byte aligned");
-// stress-side entries: lambda (core tile) and mu (box x0-4.., y0..y0+8)
-constexpr int LB = CORE * 4, MUB = BW * (TY + 1) * 4, SENT = r128(LB + MUB), NSENT = 3;
-constexpr int NVN = 4;                           // planes of the new-velocity ring
-constexpr int VNEW = 3 * NE * 4;                 // new velocity of one plane over the region
-constexpr int F_SMEM = NSLOT * FSLOT + NSENT * SENT + NVN * VNEW + 8 * (NSLOT + NSENT);
-static_assert(2 * (F_SMEM + 1024) <= 227 * 1024, "two CTAs per SM");
+constexpr int TX = 32;                           // tile width
+constexpr int EXP = TX / 2 + 2;                  // pairs of a region row (x0-2 .. x0+33)
+constexpr int VS = TX + 4;                       // row stride of the new-velocity ring
+constexpr int MBW = TX + 8;                      // FP32 medium boxes: x from x0-4
+constexpr int NV = 5;                            // planes of the new-velocity ring
+constexpr int NS = 2;                            // slots (one in use, the next in flight)
+constexpr int NE = NS + 1;                       // entries of the medium buffer (read a phase later)
+
+// ---- pairs of floats (x-neighbours) ----
+using f2 = unsigned long long;
+__device__ __forceinline__ f2 pk(float a, float b) {
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float lo(f2 a) { return __uint_as_float((unsigned)a); }
+__device__ __forceinline__ float hi(f2 a) { return __uint_as_float((unsigned)(a >> 32)); }
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ f2 sub2(f2 a, f2 b) {
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f2 dup(float a) { return pk(a, a); }
+// ar::d4 on pairs
+__device__ __forceinline__ f2 d4p(f2 c1, f2 c2, f2 a, f2 b, f2 c, f2 d) {
+    return fma2(c1, sub2(c, b), mul2(c2, sub2(d, a)));
+}
+// ar::d4 along x for the pair (i, i+1) from the pairs at i-2, i, i+2: to the
+// half points (DP: samples i-1 .. i+2) or to the integer points (i-2 .. i+1).
+template <bool DP>
+__device__ __forceinline__ f2 d4x(f2 c1, f2 c2, f2 l, f2 c, f2 r) {
+    f2 in, out;
+    if (DP) {
+        in = pk(__fsub_rn(hi(c), lo(c)), __fsub_rn(lo(r), hi(c)));
+        out = pk(__fsub_rn(lo(r), hi(l)), __fsub_rn(hi(r), lo(c)));
+    } else {
+        in = pk(__fsub_rn(lo(c), hi(l)), __fsub_rn(hi(c), lo(c)));
+        out = pk(__fsub_rn(hi(c), lo(l)), __fsub_rn(lo(r), hi(l)));
+    }
+    return fma2(c1, in, mul2(c2, out));
+}
+
+// ---- storage types ----
+template <typename T> struct S2;
+template <> struct S2<float> {
+    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    __device__ static f2 ld(const float* p) { return *reinterpret_cast<const f2*>(p); }
+    __device__ static f2 round(f2 x) { return x; }
+    __device__ static void st(float* p, f2 x) { *reinterpret_cast<f2*>(p) = x; }
+};
+template <> struct S2<__nv_bfloat16> {
+    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
+    __device__ static f2 ld(const __nv_bfloat16* p) {
+        const unsigned u = *reinterpret_cast<const unsigned*>(p);
+        return pk(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
+    }
+    __device__ static f2 round(f2 x) {
+        return pk(__bfloat162float(__float2bfloat16_rn(lo(x))), __bfloat162float(__float2bfloat16_rn(hi(x))));
+    }
+    __device__ static void st(__nv_bfloat16* p, f2 x) {
+        *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(lo(x), hi(x));
+    }
+};
+template <> struct S2<__half> {
+    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
+    __device__ static f2 ld(const __half* p) {
+        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(p));
+        return pk(v.x, v.y);
+    }
+    __device__ static f2 round(f2 x) {
+        return pk(__half2float(__float2half_rn(lo(x))), __half2float(__float2half_rn(hi(x))));
+    }
+    __device__ static void st(__half* p, f2 x) {
+        *reinterpret_cast<__half2*>(p) = __floats2half2_rn(lo(x), hi(x));
+    }
+};
+
+// ---- shared-memory layout ----
+// Slot of one step (boxes BW wide from x0 - HO): sxx, sxz rows y0-2 ..; syy
+// rows y0-3 ..; syz, sxy rows y0-4 ..; szz, vx vy vz rows y0-2 ..; rho FP32.
+template <typename T, int TY>
+struct FL {
+    static constexpr int ES = (int)sizeof(T), HO = 16 / ES, BW = TX + 2 * HO;
+    static constexpr int EY = TY + 4, NR = 16 * EY;                  // region rows; row threads
+    static constexpr int NT = (EXP * EY + 31) / 32 * 32;             // threads
+    static constexpr int RB = EY * BW * ES, RB3 = (EY + 3) * BW * ES, MRB = (EY + 1) * MBW * 4;
+    static constexpr int SXX_ = 0, SXZ_ = r128(SXX_ + RB), SYY_ = r128(SXZ_ + RB), SYZ_ = r128(SYY_ + RB3),
+                         SXY_ = r128(SYZ_ + RB3), SZZ_ = r128(SXY_ + RB3), V_ = r128(SZZ_ + RB),
+                         RHO_ = r128(V_ + 3 * RB), SLOT = r128(RHO_ + MRB);
+    static constexpr int FULL_TX = 3 * RB + 3 * RB3 + 3 * RB + MRB;  // all fields
+    static constexpr int PRE_TX = 2 * RB + RB3 + MRB;                // sxz, syz, szz, rho
+    static constexpr int LB = TX * TY * 4, MUB = (TY + 1) * MBW * 4, ENT = r128(r128(LB) + MUB);
+    static constexpr int VPL = 3 * EY * VS;                          // floats of one ring plane
+    static constexpr int O_V = NS * SLOT, O_E = r128(O_V + NV * VPL * 4), O_BAR = O_E + NE * ENT;
+    static constexpr int SMEM = O_BAR + (NS + 2) * 8;
+};
 
 struct FusedMaps {
-    CUtensorMap xp, yp, xy, zv, rho, lam, mu;
+    CUtensorMap x1, y1, xy, zz, v, rho, lam, mu; // x1: sxx / sxz boxes, y1: syy / syz boxes
 };
 
 struct FusedParams {
     DevGrid g;
-    DevFields fin, fout;        // sigma^n, v^{n-1/2} from fin; v^{n+1/2}, sigma^{n+1} to fout
+    DevFields fout;             // v^{n+1/2}, sigma^{n+1}
     DevMedium M;
     DevBoundary B;
-    float dt;
+    float dt1[3], dt2[3], dt4[3];   // dt x scale: sxx syy szz; twice it: v; a quarter: sxy sxz syz
+    float inv[NFIELD];
     int ntx, nty, zchunk;
     int* err;
     DevSource S;                // force taps (kind 1) of this step; else ntap 0
@@ -76,381 +191,434 @@ struct FusedParams {
     int sk0, sk1;               // planes of the force taps
 };
 
-__device__ __forceinline__ void issue_v(const FusedMaps& m, unsigned char* slot, uint64_t* bar,
-                                        int x0, int y0, int z) {
-    mbar_expect_tx(bar, (uint32_t)F_TX);
-    tma_load_4d(slot + O_XP, &m.xp, bar, x0 - 4, y0 - 2, z, fslot(SXX));      // sxx sxz
-    tma_load_4d(slot + O_YP, &m.yp, bar, x0 - 4, y0 - 4, z, fslot(SYY));      // syy syz
-    tma_load_3d(slot + O_XY, &m.xy, bar, x0 - 4, y0 - 4, z);                  // sxy
-    tma_load_4d(slot + O_ZV, &m.zv, bar, x0 - 4, y0 - 2, z, fslot(SZZ));      // szz vx vy vz
-    tma_load_3d(slot + O_RHO, &m.rho, bar, x0 - 4, y0 - 2, z);
-}
-__device__ __forceinline__ void issue_s(const FusedMaps& m, unsigned char* ent, uint64_t* bar,
-                                        int x0, int y0, int z) {
-    mbar_expect_tx(bar, (uint32_t)(LB + MUB));
-    tma_load_3d(ent, &m.lam, bar, x0, y0, z);
-    tma_load_3d(ent + LB, &m.mu, bar, x0 - 4, y0, z);
+// First step with velocity, first that brings the medium of the stress (mu of
+// plane z0), first with stress.
+constexpr int M_VEL = 3, M_MED = 6, M_STR = 7;
+
+// Issue the copies of step m (velocity plane k = z0 - 5 + m): sxz, syz, rho
+// of plane k + 1 and szz of k + 2; from M_VEL on sxx, syy, sxy, v of plane k;
+// from M_MED on lambda of plane k - 2 and mu of k - 1.  Medium planes clamp
+// at the top.
+template <typename T, int TY>
+__device__ __forceinline__ void issue_step(const FusedMaps& mp, unsigned char* sm, uint64_t* bar, int x0,
+                                           int y0, int z0, int m, int nz) {
+    using L = FL<T, TY>;
+    const int k = z0 - 5 + m;
+    unsigned char* slot = sm + (m % NS) * L::SLOT;
+    mbar_expect_tx(bar, (uint32_t)(m < M_VEL ? L::PRE_TX : m < M_MED ? L::FULL_TX : L::FULL_TX + L::LB + L::MUB));
+    tma_load_4d(slot + L::SXZ_, &mp.x1, bar, x0 - L::HO, y0 - 2, k + 1, fslot(SXZ));
+    tma_load_4d(slot + L::SYZ_, &mp.y1, bar, x0 - L::HO, y0 - 4, k + 1, fslot(SYZ));
+    tma_load_3d(slot + L::SZZ_, &mp.zz, bar, x0 - L::HO, y0 - 2, k + 2);
+    tma_load_3d(slot + L::RHO_, &mp.rho, bar, x0 - 4, y0 - 2, min(k + 1, nz - 1));
+    if (m < M_VEL) return;
+    tma_load_4d(slot + L::SXX_, &mp.x1, bar, x0 - L::HO, y0 - 2, k, fslot(SXX));
+    tma_load_4d(slot + L::SYY_, &mp.y1, bar, x0 - L::HO, y0 - 3, k, fslot(SYY));
+    tma_load_3d(slot + L::SXY_, &mp.xy, bar, x0 - L::HO, y0 - 4, k);
+    tma_load_4d(slot + L::V_, &mp.v, bar, x0 - L::HO, y0 - 2, k, fslot(VX));
+    if (m < M_MED) return;
+    unsigned char* ent = sm + L::O_E + (m % NE) * L::ENT;
+    tma_load_3d(ent, &mp.lam, bar, x0, y0, k - 2);
+    tma_load_3d(ent + r128(L::LB), &mp.mu, bar, x0 - 4, y0, min(k - 1, nz - 1));
 }
 
-// Per-thread queues.  Cell 0 is the thread's tile cell, cell 1 its ring cell.
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Per-thread state across steps.
 struct FQ {
-    float zz[2][4], xz[2][4], yz[2][4];          // sigma z-queues of the two cells
-    float vx[4], vy[4], vz[4];                   // new-velocity z-queues of the tile cell
-    float sg[2][6];                              // sigma^n of the tile cell, planes by parity
-    float vzp;                                   // new vz of the tile cell, previous plane
-    bool bad;                                    // a stress-side wait gave up
+    f2 zz[4], xz[4], yz[4];     // columns: szz k-1 .. k+2, sxz / syz k-2 .. k+1
+    f2 xx[2], yy[2], xy[2];     // sigma^n of planes k-2, k-1 by parity (tile threads)
+    f2 dz;                      // d sxz/dx + d syz/dy at plane k
+    f2 bx, by, r0;              // half buoyancies and density at plane k
+    f2 vzc;                     // new vz at plane k - 4 (tile threads)
+    f2 mu2, mxy, ma, mb;        // 2 mu, its xy sum, mu + mu(x+1), mu + mu(y+1) at plane k - 2
+    float gz[4];                // sponge gains of planes k + 1 (fetched ahead), k, k - 1, k - 2
+    bool bad, ovf;
 };
 
-template <int BND>
+template <int BND, typename T, int TY>
 struct FGeo {
-    int x0, y0, z0, z1, ke;                      // medium planes z0 .. ke - 1 for the stress
-    int e[2];                                    // region index of the cells
-    int ox[2], oy[2];                            // offsets in the x-row / y-row boxes
-    int cxr[2], cyr[2];                          // rho +x / +y offsets (clamped at the top edges)
-    bool in[2];                                  // the cell lies inside the grid (x, y)
-    bool ring;                                   // the thread has a ring cell
-    float gx[2], gy[2];                          // sponge gains G(i), G(j)
-    int ci[2], cj[2];                            // grid i, j of the cells
-    int mcx, mcy;                                // mu +x / +y offsets of the tile cell (clamped)
+    int x0, y0, z0, z1, M;
+    int row, rp;                // region row, pair in the row
+    int oc;                     // offset of the pair in a box that starts at row y0 - 2
+    bool reg, tile;             // the thread has a region pair / a tile pair
+    bool in0, in1;              // lanes inside the grid (x, y)
+    bool cx0, cx1;              // lane + 1 inside the grid along x
+    bool cy;                    // row + 1 inside the grid
+    f2 gx;
+    float gy;
+    long long o;                // element of the pair in plane 0
+    // values at x + 1 of the pair c with r the pair after it, clamped at the
+    // grid's end
+    __device__ __forceinline__ f2 next_x(f2 c, f2 r) const {
+        return pk(cx0 ? hi(c) : lo(c), cx1 ? lo(r) : hi(c));
+    }
     __device__ __forceinline__ FGeo(const FusedParams& P, int item) {
+        using L = FL<T, TY>;
         const DevGrid& g = P.g;
         const int ntile = P.ntx * P.nty;
-        const int t = item % ntile;
+        const int tl = item % ntile;
         z0 = (item / ntile) * P.zchunk;
         z1 = min(g.nz, z0 + P.zchunk);
-        ke = min(z1 + 1, g.nz);
-        x0 = (t % P.ntx) * TX;
-        y0 = (t / P.ntx) * TY;
-        const int tid = threadIdx.y * TX + threadIdx.x;
-        ring = tid < NRING;
-        // ring cells: rows 0, 1, TY+2, TY+3 of the region, then columns 0, 1,
-        // TX+2, TX+3 of rows 2 .. TY+1
-        int rx, ry;
-        if (tid < 4 * EX) {
-            const int q = tid / EX;
-            rx = tid % EX;
-            ry = q < 2 ? q : q + TY;
+        M = z1 - z0 + 7;
+        x0 = (tl % P.ntx) * TX;
+        y0 = (tl / P.ntx) * TY;
+        const int t = threadIdx.x;
+        if (t < L::NR) {
+            row = t >> 4;
+            rp = 1 + (t & 15);
         } else {
-            const int s = min(tid, NRING - 1) - 4 * EX;
-            ry = 2 + s / 4;
-            rx = (s & 3) < 2 ? (s & 3) : (s & 3) + TX;
+            const int u = t - L::NR;
+            row = u >> 1;
+            rp = (u & 1) ? EXP - 1 : 0;
         }
-        const int exs[2] = {(int)threadIdx.x + 2, rx}, eys[2] = {(int)threadIdx.y + 2, ry};
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const int ex = exs[c], ey = eys[c];
-            e[c] = ey * EX + ex;
-            ci[c] = x0 - 2 + ex;
-            cj[c] = y0 - 2 + ey;
-            in[c] = (c == 0 || ring) && ci[c] >= 0 && ci[c] < g.nx && cj[c] >= 0 && cj[c] < g.ny;
-            ox[c] = ey * BW + ex + 2;
-            oy[c] = (ey + 2) * BW + ex + 2;
-            cxr[c] = (ci[c] + 1 < g.nx) ? 1 : 0;
-            cyr[c] = (cj[c] + 1 < g.ny) ? BW : 0;
-            gx[c] = (BND == BND_SPONGE && in[c]) ? __ldg(P.B.g[0] + ci[c]) : 1.0f;
-            gy[c] = (BND == BND_SPONGE && in[c]) ? __ldg(P.B.g[1] + cj[c]) : 1.0f;
+        reg = t < L::EY * EXP;
+        if (!reg) row = 0;
+        tile = t < L::NR && row >= 2 && row < 2 + TY;
+        const int i = x0 - 2 + 2 * rp, j = y0 - 2 + row;
+        const bool iny = reg && j >= 0 && j < g.ny;
+        in0 = iny && i >= 0 && i < g.nx;
+        in1 = iny && i + 1 >= 0 && i + 1 < g.nx;
+        tile = tile && in0;
+        cx0 = i + 1 < g.nx;
+        cx1 = i + 2 < g.nx;
+        cy = j + 1 < g.ny;
+        oc = row * L::BW + L::HO - 2 + 2 * rp;
+        gx = dup(1.0f);
+        gy = 1.0f;
+        if (BND == BND_SPONGE) {
+            gx = pk(in0 ? __ldg(P.B.g[0] + i) : 1.0f, in1 ? __ldg(P.B.g[0] + i + 1) : 1.0f);
+            gy = iny ? __ldg(P.B.g[1] + j) : 1.0f;
         }
-        mcx = (ci[0] + 1 < g.nx) ? 1 : 0;
-        mcy = (cj[0] + 1 < g.ny) ? BW : 0;
+        o = (long long)j * g.pitch + i;
     }
 };
 
-// Plane k of the stress-side medium buffer: entry k mod 3, filled for the
-// ((k - z0) / 3)-th time.
-__device__ __forceinline__ int sent_of(int k) { return ((k % NSENT) + NSENT) % NSENT; }
+template <typename T> constexpr bool kScaled = sizeof(T) == 2;
+__device__ __forceinline__ bool over2(f2 x) { return fabsf(lo(x)) > 65504.0f || fabsf(hi(x)) > 65504.0f; }
 
-// Bounded-failure exit of thread 0 at the barrier of arrival m (m = number
-// of arrivals after the last one): record, then wait (bounded) for the
-// copies still in flight -- ring arrivals m .. issued - 1, and the last
-// filling of each medium-buffer entry -- so the CTA leaves no copy into its
-// shared memory behind.
-__device__ __noinline__ void fused_fail(int* err, uint64_t* bars, int m, int z0, int z1, int ke) {
-    atomicOr(err, 1);
-    const int P8 = z1 - z0 + 8;
-    const int issued = min(P8, max(NSLOT, m + 2));
-    for (int q = m; q < issued; ++q)
-        if (!mbar_wait(&bars[q & (NSLOT - 1)], (uint32_t)((q >> 2) & 1))) return;
-    // medium planes issued: z0 .. last (after the barrier of arrival m',
-    // plane z0 - 9 + m' is refilled with plane z0 - 6 + m')
-    const int last = min(ke - 1, max(z0 + NSENT - 1, z0 + m - 7));
-    for (int k = max(z0, last - NSENT + 1); k <= last; ++k)
-        if (!mbar_wait(&bars[NSLOT + sent_of(k)], (uint32_t)(((k - z0) / NSENT) & 1))) return;
-}
-
-// New velocity (Eq. 1) of region cell c at plane kv, from the slot of plane
-// kv (sl2), rho of plane kv + 1 (sl1) and the sigma z-queues.
-template <int BND, int PH, int c>
-__device__ __forceinline__ void vel_cell(const FusedParams& P, const FGeo<BND>& G, const FQ& Q,
-                                         const float* sl1, const float* sl2, bool ktop, float gz,
-                                         float& vx, float& vy, float& vz, float* sn) {
-    const DevGrid& g = P.g;
-    constexpr int A = (PH + 1) & 3, B = (PH + 2) & 3, C = (PH + 3) & 3, D = PH;  // oldest..newest
-    const float* hxx = sl2 + O_XP / 4 + G.ox[c];
-    const float* hxz = hxx + XB / 4;
-    const float* hyy = sl2 + O_YP / 4 + G.oy[c];
-    const float* hyz = hyy + YB / 4;
-    const float* hxy = sl2 + O_XY / 4 + G.oy[c];
-    const float* vc = sl2 + O_ZV / 4 + G.ox[c];
-    const float* hr = sl2 + O_RHO / 4 + G.ox[c];
-    const float* hr1 = sl1 + O_RHO / 4 + G.ox[c];                  // plane kv + 1
-    const float* qxz = Q.xz[c];
-    const float* qyz = Q.yz[c];
-    const float* qzz = Q.zz[c];
-    // vx at (i+1/2, j, k)
-    const float dxx = g.c1x * (hxx[1] - hxx[0]) + g.c2x * (hxx[2] - hxx[-1]);
-    const float dxy = g.c1y * (hxy[0] - hxy[-BW]) + g.c2y * (hxy[BW] - hxy[-2 * BW]);
-    const float dxz = g.c1z * (qxz[C] - qxz[B]) + g.c2z * (qxz[D] - qxz[A]);
-    // vy at (i, j+1/2, k)
-    const float dyx = g.c1x * (hxy[0] - hxy[-1]) + g.c2x * (hxy[1] - hxy[-2]);
-    const float dyy = g.c1y * (hyy[BW] - hyy[0]) + g.c2y * (hyy[2 * BW] - hyy[-BW]);
-    const float dyz = g.c1z * (qyz[C] - qyz[B]) + g.c2z * (qyz[D] - qyz[A]);
-    // vz at (i, j, k+1/2)
-    const float dzx = g.c1x * (hxz[0] - hxz[-1]) + g.c2x * (hxz[1] - hxz[-2]);
-    const float dzy = g.c1y * (hyz[0] - hyz[-BW]) + g.c2y * (hyz[BW] - hyz[-2 * BW]);
-    const float dzz = g.c1z * (qzz[C] - qzz[B]) + g.c2z * (qzz[D] - qzz[A]);
-    if (c == 0) {               // sigma^n of the tile cell, for its stress two planes later
-        sn[0] = hxx[0];         // sxx
-        sn[1] = hyy[0];         // syy
-        sn[2] = qzz[B];         // szz (plane kv)
-        sn[3] = hxy[0];         // sxy
-        sn[4] = hxz[0];         // sxz
-        sn[5] = hyz[0];         // syz
-    }
-    // buoyancy at the v points: 1 / mean of the two adjacent densities
-    const float r0 = hr[0];
-    const float bx = __fdividef(2.0f, r0 + hr[G.cxr[c]]);
-    const float by = __fdividef(2.0f, r0 + hr[G.cyr[c]]);
-    const float bz = __fdividef(2.0f, r0 + (ktop ? hr1[0] : r0));
-    vx = vc[1 * (ZB / 4)] + P.dt * bx * (dxx + dxy + dxz);
-    vy = vc[2 * (ZB / 4)] + P.dt * by * (dyx + dyy + dyz);
-    vz = vc[3 * (ZB / 4)] + P.dt * bz * (dzx + dzy + dzz);
-    if (BND == BND_SPONGE) {
-        const float Gs = G.gx[c] * gz * G.gy[c];
-        vx *= Gs; vy *= Gs; vz *= Gs;
-    }
-}
-
-// One arrival of the fused pipeline, ring position PH = m mod 4: plane
-// p = z0 - 4 + m lands; new velocity of plane kv = p - 2; stress of plane
-// ks = kv - 2.  Returns false if the CTA must stop (a wait gave up).
-template <int BND, int PH>
-__device__ __forceinline__ bool fused_step(const FusedMaps& maps, const FusedParams& P,
-                                           const FGeo<BND>& G, FQ& Q, unsigned char* sm,
-                                           uint64_t* bars, int m) {
-    const DevGrid& g = P.g;
-    constexpr int S0 = PH, S1 = (PH + 3) & 3, S2 = (PH + 2) & 3;     // planes p, p-1, p-2
-    constexpr int A = (PH + 1) & 3, B = (PH + 2) & 3, C = (PH + 3) & 3, D = PH;
-    constexpr int SQ = PH & 1;                                       // sigma^n queue entry
-    const int P8 = G.z1 - G.z0 + 8;
-    const int p = G.z0 - 4 + m, kv = p - 2, ks = kv - 2;
-    const bool dov = m >= 4, dos = m >= 8 && ks < G.z1;
-    unsigned char* sent = sm + NSLOT * FSLOT;
-    float* vnew = reinterpret_cast<float*>(sent + NSENT * SENT);
-    uint64_t* sbars = bars + NSLOT;
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    const float gz = (BND == BND_SPONGE && dov && kv >= 0 && kv < g.nz) ? __ldg(P.B.g[2] + kv) : 1.0f;
-    const float gzs = (BND == BND_SPONGE && dos) ? __ldg(P.B.g[2] + ks) : 1.0f;
-    const bool ok = mbar_wait(&bars[S0], (uint32_t)((m >> 2) & 1));
-    const float* sl0 = reinterpret_cast<const float*>(sm + S0 * FSLOT);
-    const float* sl1 = reinterpret_cast<const float*>(sm + S1 * FSLOT);
-    const float* sl2 = reinterpret_cast<const float*>(sm + S2 * FSLOT);
-    // sigma_zz of plane p, sigma_xz / sigma_yz of plane p - 1
-    Q.zz[0][PH] = sl0[O_ZV / 4 + G.ox[0]];
-    if (m > 0) {
-        Q.xz[0][PH] = sl1[O_XP / 4 + XB / 4 + G.ox[0]];
-        Q.yz[0][PH] = sl1[O_YP / 4 + YB / 4 + G.oy[0]];
-    }
-    if (G.ring) {
-        Q.zz[1][PH] = sl0[O_ZV / 4 + G.ox[1]];
-        if (m > 0) {
-            Q.xz[1][PH] = sl1[O_XP / 4 + XB / 4 + G.ox[1]];
-            Q.yz[1][PH] = sl1[O_YP / 4 + YB / 4 + G.oy[1]];
+// Slot (= its barrier) and medium entry of a step, and the phase of the
+// slot's barrier.
+struct Turn {
+    int s = 0, ent = 0;
+    uint32_t par = 0;
+    __device__ __forceinline__ void next(int entry_bytes) {
+        if (++s == NS) {
+            s = 0;
+            par ^= 1u;
         }
+        ent = ent + entry_bytes == NE * entry_bytes ? 0 : ent + entry_bytes;
     }
-    // ---- new velocity of plane kv at the thread's cells ----
-    float* vn = vnew + (kv & (NVN - 1)) * 3 * NE;
-    float vx0 = 0.f, vy0 = 0.f, vz0 = 0.f;
-    float sn[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    if (dov && ok) {
-        const bool kin = kv >= 0 && kv < g.nz;
-        const bool ktop = kv + 1 < g.nz;
-        if (kin && G.in[0]) {
-            vel_cell<BND, PH, 0>(P, G, Q, sl1, sl2, ktop, gz, vx0, vy0, vz0, sn);
-            if (kv >= G.z0 && kv < G.z1) {       // own plane: to the output set
-                const long long o = (long long)kv * g.plane + (long long)G.cj[0] * g.pitch + G.ci[0];
-                P.fout.f[VX][o] = vx0;
-                P.fout.f[VY][o] = vy0;
-                P.fout.f[VZ][o] = vz0;
+};
+
+// One step of the pipeline, m mod 4 == PH; STAGE 0: columns only, 1: velocity,
+// 2: velocity, and the medium of plane z0, 3: velocity and stress.  ring:
+// offsets of the new-velocity planes k, k-1, k-2, k-3 (floats); ent: of the
+// medium entry of this step.
+template <int BND, typename T, int TY, int PH, int STAGE>
+__device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedParams& P,
+                                           const FGeo<BND, T, TY>& G, FQ& Q, unsigned char* sm,
+                                           uint64_t* bars, int m, const int (&ring)[4], const Turn& tn) {
+    using L = FL<T, TY>;
+    using S = S2<T>;
+    constexpr int BW = L::BW;
+    const DevGrid& g = P.g;
+    constexpr int A = (PH + 1) & 3, B = (PH + 2) & 3, C = (PH + 3) & 3, D = PH;   // oldest..newest
+    constexpr int CB = NS + (PH & 1), HQ = PH & 1;                    // barrier of the warps' counts
+    const int k = G.z0 - 5 + m;
+    unsigned char* slot = sm + tn.s * L::SLOT;
+    float* vring = reinterpret_cast<float*>(sm + L::O_V);
+    const f2 c1x = dup(g.c1x), c2x = dup(g.c2x), c1y = dup(g.c1y), c2y = dup(g.c2y), c1z = dup(g.c1z), c2z = dup(g.c2z);
+    if (BND == BND_SPONGE) {
+        Q.gz[3] = Q.gz[2];
+        Q.gz[2] = Q.gz[1];
+        Q.gz[1] = Q.gz[0];
+        Q.gz[0] = __ldg(P.B.g[2] + min(max(k + 1, 0), g.nz - 1));
+    }
+    // this step's copies; and every warp past its velocity phase of step m - 2
+    // (so past stress m - 3): the ring plane written below is free, the one
+    // read by the stress is complete
+    Q.bad |= !mbar_wait(&bars[tn.s], tn.par);
+    if (STAGE > 0 || PH >= 2) Q.bad |= !mbar_wait(&bars[CB], (uint32_t)(((m - 2) >> 1) & 1));
+    // sigma^n of plane k - 2, about to leave the columns
+    f2 s0, s1, s2, s3, s4, s5;
+    s2 = Q.zz[D];
+    s0 = Q.xx[HQ];
+    s1 = Q.yy[HQ];
+    s3 = Q.xy[HQ];
+    {
+        const T* fxz = reinterpret_cast<const T*>(slot + L::SXZ_) + G.oc;              // plane k + 1
+        const T* fyz = reinterpret_cast<const T*>(slot + L::SYZ_) + G.oc + 2 * BW;
+        const float* fr = reinterpret_cast<const float*>(slot + L::RHO_) + G.row * MBW + 2 + 2 * G.rp;
+        const f2 cxz = S::ld(fxz), cyz = S::ld(fyz);
+        Q.zz[D] = S::ld(reinterpret_cast<const T*>(slot + L::SZZ_) + G.oc);            // plane k + 2
+        Q.xz[D] = cxz;
+        Q.yz[D] = cyz;
+        // density and buoyancies of plane k + 1
+        const f2 r1 = S2<float>::ld(fr), rx = S2<float>::ld(fr + 2), ry = S2<float>::ld(fr + (G.cy ? MBW : 0));
+        if constexpr (STAGE > 0) {
+            const f2 sz = add2(Q.r0, r1);
+            const T* fxx = reinterpret_cast<const T*>(slot + L::SXX_) + G.oc;
+            const T* fyy = reinterpret_cast<const T*>(slot + L::SYY_) + G.oc + BW;
+            const T* fxy = reinterpret_cast<const T*>(slot + L::SXY_) + G.oc + 2 * BW;
+            const T* fv = reinterpret_cast<const T*>(slot + L::V_) + G.oc;
+            const f2 cxx = S::ld(fxx), cyy = S::ld(fyy), cxy = S::ld(fxy);
+            Q.xx[HQ] = cxx;
+            Q.yy[HQ] = cyy;
+            Q.xy[HQ] = cxy;
+            f2 dxx = d4x<true>(c1x, c2x, S::ld(fxx - 2), cxx, S::ld(fxx + 2));
+            f2 dxy = d4p(c1y, c2y, S::ld(fxy - 2 * BW), S::ld(fxy - BW), cxy, S::ld(fxy + BW));
+            f2 dxz = d4p(c1z, c2z, Q.xz[A], Q.xz[B], Q.xz[C], Q.xz[D]);
+            f2 dyx = d4x<false>(c1x, c2x, S::ld(fxy - 2), cxy, S::ld(fxy + 2));
+            f2 dyy = d4p(c1y, c2y, S::ld(fyy - BW), cyy, S::ld(fyy + BW), S::ld(fyy + 2 * BW));
+            f2 dyz = d4p(c1z, c2z, Q.yz[A], Q.yz[B], Q.yz[C], Q.yz[D]);
+            f2 dzz = d4p(c1z, c2z, Q.zz[A], Q.zz[B], Q.zz[C], Q.zz[D]);
+            if (kScaled<T>) {
+                dxx = mul2(dxx, dup(P.inv[SXX])); dxy = mul2(dxy, dup(P.inv[SXY])); dxz = mul2(dxz, dup(P.inv[SXZ]));
+                dyx = mul2(dyx, dup(P.inv[SXY])); dyy = mul2(dyy, dup(P.inv[SYY])); dyz = mul2(dyz, dup(P.inv[SYZ]));
+                dzz = mul2(dzz, dup(P.inv[SZZ]));
+            }
+            // (2 dt) r with r = 1 / (r0 + r1) has the bits of dt (2 r)
+            const f2 bz = pk(ar::rcp(lo(sz)), ar::rcp(hi(sz)));
+            f2 vx = fma2(mul2(dup(P.dt2[0]), Q.bx), add2(add2(dxx, dxy), dxz), S::ld(fv));
+            f2 vy = fma2(mul2(dup(P.dt2[kScaled<T> ? 1 : 0]), Q.by), add2(add2(dyx, dyy), dyz), S::ld(fv + L::RB / L::ES));
+            f2 vz = fma2(mul2(dup(P.dt2[kScaled<T> ? 2 : 0]), bz), add2(Q.dz, dzz), S::ld(fv + 2 * (L::RB / L::ES)));
+            if (BND == BND_SPONGE) {
+                const f2 gs = mul2(mul2(G.gx, dup(Q.gz[1])), dup(G.gy));
+                vx = mul2(vx, gs); vy = mul2(vy, gs); vz = mul2(vz, gs);
+            }
+            const bool kin = k >= 0 && k < g.nz;         // zero outside the grid
+            const bool i0 = kin && G.in0, i1 = kin && G.in1;
+            vx = pk(i0 ? lo(vx) : 0.0f, i1 ? hi(vx) : 0.0f);
+            vy = pk(i0 ? lo(vy) : 0.0f, i1 ? hi(vy) : 0.0f);
+            vz = pk(i0 ? lo(vz) : 0.0f, i1 ? hi(vz) : 0.0f);
+            if (std::is_same<T, __half>::value) Q.ovf |= over2(vx) | over2(vy) | over2(vz);
+            if (G.tile && k >= G.z0 && k < G.z1) {
+                const long long o = (long long)k * g.plane + G.o;
+                S::st((T*)P.fout.f[VX] + o, vx);
+                S::st((T*)P.fout.f[VY] + o, vy);
+                S::st((T*)P.fout.f[VZ] + o, vz);
+            }
+            if (G.reg) {
+                float* vn = vring + ring[0] + G.row * VS + 2 * G.rp;
+                *reinterpret_cast<f2*>(vn) = S::round(vx);
+                *reinterpret_cast<f2*>(vn + L::EY * VS) = S::round(vy);
+                *reinterpret_cast<f2*>(vn + 2 * L::EY * VS) = S::round(vz);
             }
         }
-        vn[G.e[0]] = vx0;
-        vn[NE + G.e[0]] = vy0;
-        vn[2 * NE + G.e[0]] = vz0;
-        if (G.ring) {
-            float vx1 = 0.f, vy1 = 0.f, vz1 = 0.f;
-            if (kin && G.in[1]) vel_cell<BND, PH, 1>(P, G, Q, sl1, sl2, ktop, gz, vx1, vy1, vz1, sn);
-            vn[G.e[1]] = vx1;
-            vn[NE + G.e[1]] = vy1;
-            vn[2 * NE + G.e[1]] = vz1;
+        Q.r0 = r1;
+        const f2 sx = add2(r1, G.next_x(r1, rx)), sy = add2(r1, ry);
+        Q.bx = pk(ar::rcp(lo(sx)), ar::rcp(hi(sx)));
+        Q.by = pk(ar::rcp(lo(sy)), ar::rcp(hi(sy)));
+        f2 dzx = d4x<false>(c1x, c2x, S::ld(fxz - 2), cxz, S::ld(fxz + 2));
+        f2 dzy = d4p(c1y, c2y, S::ld(fyz - 2 * BW), S::ld(fyz - BW), cyz, S::ld(fyz + BW));
+        if (kScaled<T>) {
+            dzx = mul2(dzx, dup(P.inv[SXZ]));
+            dzy = mul2(dzy, dup(P.inv[SYZ]));
         }
+        Q.dz = add2(dzx, dzy);
     }
-    if (__syncthreads_or(!ok || Q.bad)) {
-        if (tid == 0) fused_fail(P.err, bars, m, G.z0, G.z1, G.ke);
-        return false;
+    s4 = Q.xz[A];                                    // sxz, syz of plane k - 2
+    s5 = Q.yz[A];
+    // the warp is done with this step's slot and its part of the ring plane
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) mbar_arrive(&bars[CB]);
+    // the last warp, which has no stress to compute, refills the slot for step
+    // m + NS once every warp is
+    if (threadIdx.x == L::NT - 32 && m + NS < G.M) {
+        Q.bad |= !mbar_wait(&bars[CB], (uint32_t)((m >> 1) & 1));
+        issue_step<T, TY>(maps, sm, &bars[tn.s], G.x0, G.y0, G.z0, m + NS, g.nz);
     }
-    if (tid == 0) {
-        // the slot of plane p - 2 is free: refill it with plane p + 2
-        if (m >= 2 && m + 2 < P8) issue_v(maps, sm + S2 * FSLOT, &bars[S2], G.x0, G.y0, p + 2);
-        // the medium entry of plane ks - 1 (stress of the previous arrival) is
-        // free: refill it with plane ks + 2
-        const int kd = ks - 1;
-        if (m >= 9 && kd < G.z1 && kd + NSENT < G.ke)
-            issue_s(maps, sent + sent_of(kd) * SENT, &sbars[sent_of(kd)], G.x0, G.y0, kd + NSENT);
-    }
-    // point force of step n (Sec. 2.4 source term of Eq. 1) on its tap cells
-    // inside the region, before the stress reads them
-    if (dov && kv >= P.sk0 && kv <= P.sk1) {               // uniform across the CTA
-        if (tid < P.S.ntap) {
-            const Tap tp = P.S.tap[tid];
+    // point force of step n on its tap cells inside the region
+    if (STAGE > 0 && k >= P.sk0 && k <= P.sk1) {     // uniform across the CTA
+        __syncthreads();
+        if ((int)threadIdx.x < P.S.ntap) {
+            const Tap tp = P.S.tap[threadIdx.x];
             const int ex = tp.i - (G.x0 - 2), ey = tp.j - (G.y0 - 2);
-            if (tp.k == kv && ex >= 0 && ex < EX && ey >= 0 && ey < EY) {
-                float amp = tp.w * __ldg(P.wavelet + P.n);
+            if (tp.k == k && ex >= 0 && ex < TX + 4 && ey >= 0 && ey < L::EY) {
+                float amp = __fmul_rn(tp.w, __ldg(P.wavelet + P.n));
                 amp *= ops::buoy(P.M, g, tp.q - VX, tp.i, tp.j, tp.k);
                 amp *= ops::gain(P.B, tp.i, tp.j, tp.k);
-                atomicAdd(vn + (tp.q - VX) * NE + ey * EX + ex, amp);
-                if (kv >= G.z0 && kv < G.z1 && ex >= 2 && ex < 2 + TX && ey >= 2 && ey < 2 + TY)
-                    atomicAdd((tp.q == VX ? P.fout.f[VX] : tp.q == VY ? P.fout.f[VY] : P.fout.f[VZ]) +
-                                  ops::cidx(g, tp.i, tp.j, tp.k), amp);
+                float* v = vring + ring[0] + (tp.q - VX) * L::EY * VS + ey * VS + ex;
+                float x;
+                if constexpr (sizeof(T) == 4) {
+                    x = __fadd_rn(*v, amp);
+                } else {                             // the passes add the rounded amount
+                    x = __fadd_rn(*v, ops::Io<T>::get_value(amp));
+                    if (std::is_same<T, __half>::value && fabsf(x) > 65504.0f) Q.ovf = true;
+                    x = ops::Io<T>::get_value(x);
+                }
+                *v = x;
+                if (k >= G.z0 && k < G.z1 && ex >= 2 && ex < 2 + TX && ey >= 2 && ey < 2 + TY) {
+                    T* f = (T*)(tp.q == VX ? P.fout.f[VX] : tp.q == VY ? P.fout.f[VY] : P.fout.f[VZ]);
+                    f[ops::cidx(g, tp.i, tp.j, tp.k)] = ops::Io<T>::put(x);
+                }
             }
         }
         __syncthreads();
-        vx0 = vn[G.e[0]];
-        vy0 = vn[NE + G.e[0]];
-        vz0 = vn[2 * NE + G.e[0]];
     }
-    // new-velocity queues of the tile cell: vx, vy of plane kv, vz of kv - 1
-    if (dov) {
-        Q.vx[PH] = vx0;
-        Q.vy[PH] = vy0;
-        Q.vz[PH] = Q.vzp;
-        Q.vzp = vz0;
-    }
-    // ---- stress of plane ks at the tile cell (Eq. 2/3) ----
-    if (dos) {
-        const int sb = sent_of(ks), sb1 = sent_of(ks + 1);
-        bool okS = mbar_wait(&sbars[sb], (uint32_t)(((ks - G.z0) / NSENT) & 1));
-        if (ks + 1 < G.ke)
-            okS = mbar_wait(&sbars[sb1], (uint32_t)(((ks + 1 - G.z0) / NSENT) & 1)) && okS;
-        Q.bad |= !okS;
-        if (okS && G.in[0]) {
-            const float* hvx = vnew + (ks & (NVN - 1)) * 3 * NE + G.e[0];   // plane ks
-            const float* hvy = hvx + NE;
-            const float* hvz = hvx + 2 * NE;
-            // normal strain rates at (i, j, k)
-            const float exx = g.c1x * (hvx[0] - hvx[-1]) + g.c2x * (hvx[1] - hvx[-2]);
-            const float eyy = g.c1y * (hvy[0] - hvy[-EX]) + g.c2y * (hvy[EX] - hvy[-2 * EX]);
-            const float ezz = g.c1z * (Q.vz[C] - Q.vz[B]) + g.c2z * (Q.vz[D] - Q.vz[A]);
-            // shear terms at the shear points
-            const float vxy = g.c1y * (hvx[EX] - hvx[0]) + g.c2y * (hvx[2 * EX] - hvx[-EX]);
-            const float vyx = g.c1x * (hvy[1] - hvy[0]) + g.c2x * (hvy[2] - hvy[-1]);
-            const float vxz = g.c1z * (Q.vx[C] - Q.vx[B]) + g.c2z * (Q.vx[D] - Q.vx[A]);
-            const float vzx = g.c1x * (hvz[1] - hvz[0]) + g.c2x * (hvz[2] - hvz[-1]);
-            const float vyz = g.c1z * (Q.vy[C] - Q.vy[B]) + g.c2z * (Q.vy[D] - Q.vy[A]);
-            const float vzy = g.c1y * (hvz[EX] - hvz[0]) + g.c2y * (hvz[2 * EX] - hvz[-EX]);
-            // medium: lambda, mu at the cell; mu means at the shear points
-            const unsigned char* e0 = sent + sb * SENT;
-            const unsigned char* e1 = sent + (ks + 1 < g.nz ? sb1 : sb) * SENT;   // plane ks + 1
-            const int tc = threadIdx.y * TX + threadIdx.x;
-            const float lam = reinterpret_cast<const float*>(e0)[tc];
-            const int mo = threadIdx.y * BW + threadIdx.x + 4;
-            const float* hmu = reinterpret_cast<const float*>(e0 + LB) + mo;
-            const float* hmu1 = reinterpret_cast<const float*>(e1 + LB) + mo;
-            const float mu0 = hmu[0], mxp = hmu[G.mcx], myp = hmu[G.mcy], mzp = hmu1[0];
-            const float mxy = 0.25f * (mu0 + mxp + myp + hmu[G.mcx + G.mcy]);
-            const float mxz = 0.25f * (mu0 + mxp + mzp + hmu1[G.mcx]);
-            const float myz = 0.25f * (mu0 + myp + mzp + hmu1[G.mcy]);
-            const float l2m = lam + 2.0f * mu0;
-            const float* sg = Q.sg[SQ];
-            float s0 = sg[0] + P.dt * (l2m * exx + lam * (eyy + ezz));
-            float s1 = sg[1] + P.dt * (l2m * eyy + lam * (exx + ezz));
-            float s2 = sg[2] + P.dt * (l2m * ezz + lam * (exx + eyy));
-            float s3 = sg[3] + P.dt * mxy * (vxy + vyx);
-            float s4 = sg[4] + P.dt * mxz * (vxz + vzx);
-            float s5 = sg[5] + P.dt * myz * (vyz + vzy);
-            if (BND == BND_SPONGE) {
-                const float Gs = G.gx[0] * gzs * G.gy[0];
-                s0 *= Gs; s1 *= Gs; s2 *= Gs; s3 *= Gs; s4 *= Gs; s5 *= Gs;
+    // ---- stress of plane k - 2 at the tile pair (Eq. 2/3) ----
+    if constexpr (STAGE >= 2) {
+        if (G.tile) {
+            const unsigned char* ent = sm + L::O_E + tn.ent;
+            const float* hm = reinterpret_cast<const float*>(ent + r128(L::LB)) + (G.row - 2) * MBW + 2 + 2 * G.rp;
+            const float* hy = hm + (G.cy ? MBW : 0);
+            // mu of plane k - 1 and its x, y and xy neighbours
+            const f2 m1 = S2<float>::ld(hm), m1r = S2<float>::ld(hm + 2), my = S2<float>::ld(hy), myr = S2<float>::ld(hy + 2);
+            const f2 mx = G.next_x(m1, m1r), mxy4 = G.next_x(my, myr);
+            const f2 na = add2(m1, mx), nb = add2(m1, my);
+            const int e = G.row * VS + 2 * G.rp;
+            const float* v2 = vring + ring[2] + e;                                   // plane k - 2
+            const float* v3 = vring + ring[3] + e;
+            const float* v1 = vring + ring[1] + e;
+            const float* v0 = vring + ring[0] + e;
+            constexpr int FS = L::EY * VS;
+            auto ld = [](const float* p) { return S2<float>::ld(p); };
+            const f2 vz3 = ld(v3 + 2 * FS), czv = ld(v2 + 2 * FS);
+            if constexpr (STAGE == 3) {
+                const f2 cvx = ld(v2), cvy = ld(v2 + FS);
+                f2 exx = d4x<false>(c1x, c2x, ld(v2 - 2), cvx, ld(v2 + 2));
+                f2 vxy = d4p(c1y, c2y, ld(v2 - VS), cvx, ld(v2 + VS), ld(v2 + 2 * VS));
+                f2 vxz = d4p(c1z, c2z, ld(v3), cvx, ld(v1), ld(v0));
+                f2 eyy = d4p(c1y, c2y, ld(v2 + FS - 2 * VS), ld(v2 + FS - VS), cvy, ld(v2 + FS + VS));
+                f2 vyx = d4x<true>(c1x, c2x, ld(v2 + FS - 2), cvy, ld(v2 + FS + 2));
+                f2 vyz = d4p(c1z, c2z, ld(v3 + FS), cvy, ld(v1 + FS), ld(v0 + FS));
+                f2 ezz = d4p(c1z, c2z, Q.vzc, vz3, czv, ld(v1 + 2 * FS));
+                f2 vzx = d4x<true>(c1x, c2x, ld(v2 + 2 * FS - 2), czv, ld(v2 + 2 * FS + 2));
+                f2 vzy = d4p(c1y, c2y, ld(v2 + 2 * FS - VS), czv, ld(v2 + 2 * FS + VS), ld(v2 + 2 * FS + 2 * VS));
+                if (kScaled<T>) {
+                    const f2 ix = dup(P.inv[VX]), iy = dup(P.inv[VY]), iz = dup(P.inv[VZ]);
+                    exx = mul2(exx, ix); vxy = mul2(vxy, ix); vxz = mul2(vxz, ix);
+                    eyy = mul2(eyy, iy); vyx = mul2(vyx, iy); vyz = mul2(vyz, iy);
+                    ezz = mul2(ezz, iz); vzx = mul2(vzx, iz); vzy = mul2(vzy, iz);
+                }
+                const f2 lam = S2<float>::ld(reinterpret_cast<const float*>(ent) + (G.row - 2) * TX + 2 * (G.rp - 1));
+                const f2 l2m = add2(Q.mu2, lam);
+                // sums of four: (dt / 4) times the sum has the bits of dt times the mean
+                const f2 mxz = add2(add2(Q.ma, m1), mx), myz = add2(add2(Q.mb, m1), my);
+                s0 = fma2(dup(P.dt1[0]), fma2(l2m, exx, mul2(lam, add2(eyy, ezz))), s0);
+                s1 = fma2(dup(P.dt1[kScaled<T> ? 1 : 0]), fma2(l2m, eyy, mul2(lam, add2(exx, ezz))), s1);
+                s2 = fma2(dup(P.dt1[kScaled<T> ? 2 : 0]), fma2(l2m, ezz, mul2(lam, add2(exx, eyy))), s2);
+                s3 = fma2(mul2(dup(P.dt4[0]), Q.mxy), add2(vxy, vyx), s3);
+                s4 = fma2(mul2(dup(P.dt4[kScaled<T> ? 1 : 0]), mxz), add2(vxz, vzx), s4);
+                s5 = fma2(mul2(dup(P.dt4[kScaled<T> ? 2 : 0]), myz), add2(vyz, vzy), s5);
+                if (BND == BND_SPONGE) {
+                    const f2 gs = mul2(mul2(G.gx, dup(Q.gz[3])), dup(G.gy));
+                    s0 = mul2(s0, gs); s1 = mul2(s1, gs); s2 = mul2(s2, gs);
+                    s3 = mul2(s3, gs); s4 = mul2(s4, gs); s5 = mul2(s5, gs);
+                }
+                if (!G.in1) {              // the padding stays zero
+                    s0 = pk(lo(s0), 0.f); s1 = pk(lo(s1), 0.f); s2 = pk(lo(s2), 0.f);
+                    s3 = pk(lo(s3), 0.f); s4 = pk(lo(s4), 0.f); s5 = pk(lo(s5), 0.f);
+                }
+                if (std::is_same<T, __half>::value)
+                    Q.ovf |= over2(s0) | over2(s1) | over2(s2) | over2(s3) | over2(s4) | over2(s5);
+                const long long o = (long long)(k - 2) * g.plane + G.o;
+                S::st((T*)P.fout.f[SXX] + o, s0);
+                S::st((T*)P.fout.f[SYY] + o, s1);
+                S::st((T*)P.fout.f[SZZ] + o, s2);
+                S::st((T*)P.fout.f[SXY] + o, s3);
+                S::st((T*)P.fout.f[SXZ] + o, s4);
+                S::st((T*)P.fout.f[SYZ] + o, s5);
             }
-            const long long o = (long long)ks * g.plane + (long long)G.cj[0] * g.pitch + G.ci[0];
-            P.fout.f[SXX][o] = s0;
-            P.fout.f[SYY][o] = s1;
-            P.fout.f[SZZ][o] = s2;
-            P.fout.f[SXY][o] = s3;
-            P.fout.f[SXZ][o] = s4;
-            P.fout.f[SYZ][o] = s5;
+            Q.vzc = vz3;
+            Q.mu2 = add2(m1, m1);
+            Q.ma = na;
+            Q.mb = nb;
+            Q.mxy = add2(add2(na, my), mxy4);
         }
     }
-    // sigma^n of plane kv waits in the entry of plane ks for two arrivals
-#pragma unroll
-    for (int q = 0; q < 6; ++q) Q.sg[SQ][q] = sn[q];
-    return true;
 }
 
-template <int BND>
-__global__ void __launch_bounds__(NTH, 2) k_fused(const __grid_constant__ FusedMaps maps,
-                                                  const FusedParams P) {
+template <int BND, typename T, int TY>
+__global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constant__ FusedMaps maps,
+                                                           const __grid_constant__ FusedParams P) {
+    using L = FL<T, TY>;
     extern __shared__ __align__(128) unsigned char sm[];
-    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + NSLOT * FSLOT + NSENT * SENT + NVN * VNEW);
-    const int tid = threadIdx.y * TX + threadIdx.x;
-    if (tid == 0) {
-        for (int s = 0; s < NSLOT + NSENT; ++s) mbar_init(&bars[s], 1);
+    // bars[0..NS-1]: copies of a step arrived; the last two: warps past its velocity phase
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::O_BAR);
+    const FGeo<BND, T, TY> G(P, (int)blockIdx.x);
+    if (threadIdx.x == L::NT - 32) {
+        for (int s = 0; s < NS + 2; ++s) mbar_init(&bars[s], s < NS ? 1 : L::NT / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int s = 0; s < NS; ++s) issue_step<T, TY>(maps, sm, &bars[s], G.x0, G.y0, G.z0, s, P.g.nz);
     }
     __syncthreads();
-    const FGeo<BND> G(P, (int)blockIdx.x);
-    const int P8 = G.z1 - G.z0 + 8;               // arrivals: planes z0-4 .. z1+3
-    if (tid == 0) {
-        for (int s = 0; s < NSLOT && s < P8; ++s)
-            issue_v(maps, sm + s * FSLOT, &bars[s], G.x0, G.y0, G.z0 - 4 + s);
-        unsigned char* sent = sm + NSLOT * FSLOT;
-        for (int k = G.z0; k < G.z0 + NSENT && k < G.ke; ++k)
-            issue_s(maps, sent + sent_of(k) * SENT, &bars[NSLOT + sent_of(k)], G.x0, G.y0, k);
-    }
     FQ Q;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        Q.zz[0][q] = Q.zz[1][q] = Q.xz[0][q] = Q.xz[1][q] = Q.yz[0][q] = Q.yz[1][q] = 0.f;
-        Q.vx[q] = Q.vy[q] = Q.vz[q] = 0.f;
+    for (int q = 0; q < 4; ++q) Q.zz[q] = Q.xz[q] = Q.yz[q] = 0;
+    Q.xx[0] = Q.xx[1] = Q.yy[0] = Q.yy[1] = Q.xy[0] = Q.xy[1] = 0;
+    Q.dz = Q.bx = Q.by = Q.r0 = Q.vzc = Q.mu2 = Q.mxy = Q.ma = Q.mb = 0;
+    Q.gz[0] = Q.gz[1] = Q.gz[2] = Q.gz[3] = 1.0f;
+    Q.bad = Q.ovf = false;
+    int ring[4] = {0, 4 * L::VPL, 3 * L::VPL, 2 * L::VPL};            // planes k .. k - 3
+    Turn tn;
+    auto next = [&]() {
+        const int nw = ring[0] + L::VPL == NV * L::VPL ? 0 : ring[0] + L::VPL;
+        ring[3] = ring[2];
+        ring[2] = ring[1];
+        ring[1] = ring[0];
+        ring[0] = nw;
+        tn.next(L::ENT);
+    };
+    fused_step<BND, T, TY, 0, 0>(maps, P, G, Q, sm, bars, 0, ring, tn); next();
+    fused_step<BND, T, TY, 1, 0>(maps, P, G, Q, sm, bars, 1, ring, tn); next();
+    fused_step<BND, T, TY, 2, 0>(maps, P, G, Q, sm, bars, 2, ring, tn); next();
+    fused_step<BND, T, TY, 3, 1>(maps, P, G, Q, sm, bars, 3, ring, tn); next();
+    fused_step<BND, T, TY, 0, 1>(maps, P, G, Q, sm, bars, 4, ring, tn); next();
+    fused_step<BND, T, TY, 1, 1>(maps, P, G, Q, sm, bars, 5, ring, tn); next();
+    fused_step<BND, T, TY, 2, 2>(maps, P, G, Q, sm, bars, 6, ring, tn); next();
+    fused_step<BND, T, TY, 3, 3>(maps, P, G, Q, sm, bars, 7, ring, tn); next();
+    int m = M_STR + 1;
+    bool stop = __syncthreads_or(Q.bad);
+    while (m < G.M && !stop) {
+        fused_step<BND, T, TY, 0, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+        next();
+        if (++m < G.M) {
+            fused_step<BND, T, TY, 1, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+            next();
+            if (++m < G.M) {
+                fused_step<BND, T, TY, 2, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                next();
+                if (++m < G.M) {
+                    fused_step<BND, T, TY, 3, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                    next();
+                    ++m;
+                }
+            }
+        }
+        // a wait that gave up ends the CTA here; the check costs one barrier in
+        // four steps
+        stop = __syncthreads_or(Q.bad);
     }
-#pragma unroll
-    for (int q = 0; q < 6; ++q) Q.sg[0][q] = Q.sg[1][q] = 0.f;
-    Q.vzp = 0.f;
-    Q.bad = false;
-    for (int m = 0; m < P8; m += 4) {
-        if (!fused_step<BND, 0>(maps, P, G, Q, sm, bars, m)) return;
-        if (m + 1 < P8 && !fused_step<BND, 1>(maps, P, G, Q, sm, bars, m + 1)) return;
-        if (m + 2 < P8 && !fused_step<BND, 2>(maps, P, G, Q, sm, bars, m + 2)) return;
-        if (m + 3 < P8 && !fused_step<BND, 3>(maps, P, G, Q, sm, bars, m + 3)) return;
+    if (stop && threadIdx.x == 0) {          // record, and let the copies in flight land (bounded)
+        atomicOr(P.err, 1);
+        for (int q = m; q < m + NS && q < G.M; ++q)
+            if (!mbar_wait(&bars[q % NS], (uint32_t)((q / NS) & 1))) break;
     }
-    // a medium wait of the last stress planes that gave up
-    if (__syncthreads_or(Q.bad) && tid == 0) fused_fail(P.err, bars, P8, G.z0, G.z1, G.ke);
+    if constexpr (std::is_same<T, __half>::value)
+        if (__syncthreads_or(Q.ovf) && threadIdx.x == 0) atomicOr(P.err, 4);
 }
 
+template <typename T, int TY>
 bool encode_fused(FusedMaps* fm, const DevGrid& g, const DevFields& F, const DevMedium& M) {
-    const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
+    using L = FL<T, TY>;
+    const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32, dt = S2<T>::dtype;
     const char* f0 = (const char*)F.f[SXX];                                    // slot 0
     const long long fsb = (const char*)F.f[SXZ] - (const char*)F.f[SXX];
     for (int q = 0; q < NFIELD; ++q)
         if ((const char*)F.f[q] - f0 != fslot(q) * fsb) return false;
     bool ok = true;
-    ok &= encode4(&fm->xp, g, f0, f32, 4, fsb, NFIELD, BW, EY, 2);
-    ok &= encode4(&fm->yp, g, f0, f32, 4, fsb, NFIELD, BW, EY + 4, 2);
-    ok &= encode(&fm->xy, g, F.f[SXY], f32, 4, BW, EY + 4);
-    ok &= encode4(&fm->zv, g, f0, f32, 4, fsb, NFIELD, BW, EY, 4);
-    ok &= encode(&fm->rho, g, M.rho, f32, 4, BW, EY + 1);
+    ok &= encode4(&fm->x1, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY, 1);
+    ok &= encode4(&fm->y1, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY + 3, 1);
+    ok &= encode(&fm->xy, g, F.f[SXY], dt, L::ES, L::BW, L::EY + 3);
+    ok &= encode(&fm->zz, g, F.f[SZZ], dt, L::ES, L::BW, L::EY);
+    ok &= encode4(&fm->v, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY, 3);
+    ok &= encode(&fm->rho, g, M.rho, f32, 4, MBW, L::EY + 1);
     ok &= encode(&fm->lam, g, M.lam, f32, 4, TX, TY);
-    ok &= encode(&fm->mu, g, M.mu, f32, 4, BW, TY + 1);
+    ok &= encode(&fm->mu, g, M.mu, f32, 4, MBW, TY + 1);
     return ok;
 }
 
@@ -460,8 +628,26 @@ struct FusedPlan {
     FusedMaps dir[2];             // reading A (dir 0) or B (dir 1)
     DevFields f[2];
     int kind = 0;
+    int ty = 0, nt = 0, smem = 0;
+    void (*kern)(FusedMaps, FusedParams) = nullptr;
     int ntx = 0, nty = 0, zchunk = 0, grid = 0;
 };
+
+namespace {
+template <typename T, int TY>
+cudaError_t plan_for(FusedPlan* p, const DevGrid& g, const DevFields& A, const DevFields& Bf, const DevMedium& M,
+                     const DevBoundary& B) {
+    using L = FL<T, TY>;
+    static_assert(L::SMEM <= 227 * 1024, "one CTA's shared memory");
+    p->kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY> : k_fused<BND_NONE, T, TY>;
+    p->ty = TY;
+    p->nt = L::NT;
+    p->smem = L::SMEM;
+    if (!encode_fused<T, TY>(&p->dir[0], g, A, M) || !encode_fused<T, TY>(&p->dir[1], g, Bf, M))
+        return cudaErrorInvalidValue;
+    return cudaSuccess;
+}
+}  // namespace
 
 bool fused_supported(const DevGrid& g, const DevBoundary& B, int storage) {
     return storage == EWS_STORAGE_F32 && (B.kind == BND_SPONGE || B.kind == BND_NONE) &&
@@ -474,25 +660,22 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
     p->kind = B.kind;
     p->f[0] = A;
     p->f[1] = Bf;
-    if (!encode_fused(&p->dir[0], g, A, M) || !encode_fused(&p->dir[1], g, Bf, M)) {
-        delete p;
-        return cudaErrorInvalidValue;
-    }
     int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    cudaError_t e = plan_for<float, 24>(p, g, A, Bf, M, B);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    auto kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE> : k_fused<BND_NONE>;
-    if (e == cudaSuccess) e = prepare(kern, F_SMEM, &occ);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(p->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, p->kern, p->nt, p->smem);
     if (e == cudaSuccess && occ < 1) e = cudaErrorInvalidConfiguration;
     if (e != cudaSuccess) {
         delete p;
         return e;
     }
     p->ntx = (g.nx + TX - 1) / TX;
-    p->nty = (g.ny + TY - 1) / TY;
+    p->nty = (g.ny + p->ty - 1) / p->ty;
     const long long ntile = (long long)p->ntx * p->nty;
-    // a chunk loads 4 planes beyond its own on each side
-    p->zchunk = chunk_planes(ntile, (long long)sms * occ, g.nz, 16, 4);
+    // a chunk runs 4 more velocity planes than it has planes and 3 light steps
+    p->zchunk = chunk_planes(ntile, (long long)sms * occ, g.nz, 8, 6);
     p->grid = (int)(ntile * ((g.nz + p->zchunk - 1) / p->zchunk));
     *out = p;
     return cudaSuccess;
@@ -501,15 +684,19 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
 void fused_plan_destroy(FusedPlan* p) { delete p; }
 
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
-                         const DevBoundary& B, float dt, const DevSource& S, const float* wavelet,
-                         int n, int* err, cudaStream_t st) {
+                         const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
+                         const float* wavelet, int n, int* err, cudaStream_t st) {
     FusedParams P{};
     P.g = g;
-    P.fin = p->f[dir];
     P.fout = p->f[dir ^ 1];
     P.M = M;
     P.B = B;
-    P.dt = dt;
+    for (int q = 0; q < NFIELD; ++q) P.inv[q] = inv[q];
+    for (int c = 0; c < 3; ++c) {
+        P.dt1[c] = dto[SXX + c];
+        P.dt2[c] = 2.0f * dto[VX + c];
+        P.dt4[c] = 0.25f * dto[SXY + c];
+    }
     P.ntx = p->ntx;
     P.nty = p->nty;
     P.zchunk = p->zchunk;
@@ -523,15 +710,11 @@ cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const De
         P.wavelet = wavelet;
         P.n = n;
         for (int t = 0; t < S.ntap; ++t) {
-            P.sk0 = S.tap[t].k < P.sk0 ? S.tap[t].k : P.sk0;
-            P.sk1 = S.tap[t].k > P.sk1 ? S.tap[t].k : P.sk1;
+            P.sk0 = std::min(P.sk0, S.tap[t].k);
+            P.sk1 = std::max(P.sk1, S.tap[t].k);
         }
     }
-    const dim3 blk(TX, RY);
-    if (p->kind == BND_SPONGE)
-        k_fused<BND_SPONGE><<<p->grid, blk, F_SMEM, st>>>(p->dir[dir], P);
-    else
-        k_fused<BND_NONE><<<p->grid, blk, F_SMEM, st>>>(p->dir[dir], P);
+    p->kern<<<p->grid, p->nt, p->smem, st>>>(p->dir[dir], P);
     return cudaGetLastError();
 }
 

@@ -144,7 +144,8 @@ __host__ __device__ __forceinline__ ZT ztransposed(const DevGrid& g, int k) {
 
 // One z-difference from the four samples a..d (lowest plane first) of an
 // integer-z (HALF false) or half-integer-z (HALF true) output.
-template <int FS, bool HALF>
+// WIDE: every rounding written out, as in ews_arith.cuh (FP32 wavefields).
+template <int FS, bool HALF, bool WIDE = true>
 __device__ __forceinline__ float zdiff(const DevGrid& g, const ZW& zw, const ZT& zt, float a,
                                        float b, float c, float d) {
     if constexpr (FS == ZS_ADJ) {
@@ -152,11 +153,14 @@ __device__ __forceinline__ float zdiff(const DevGrid& g, const ZW& zw, const ZT&
                     : zt.iA * a + zt.iB * b + zt.iC * c + zt.iD * d;
     } else if constexpr (FS == ZS_FWD) {
         // Eq. 4, or its inner pair alone on the switched planes
+        if constexpr (!WIDE)
+            return (HALF ? zw.h2 : zw.i2) ? g.c1z2 * (c - b) : g.c1z * (c - b) + g.c2z * (d - a);
         const float in = __fsub_rn(c, b);
         return (HALF ? zw.h2 : zw.i2) ? __fmul_rn(g.c1z2, in)
-                                      : __fmaf_rn(g.c2z, __fsub_rn(d, a), __fmul_rn(g.c1z, in));
+                                      : __fmaf_rn(g.c1z, in, __fmul_rn(g.c2z, __fsub_rn(d, a)));
     } else {
-        return __fmaf_rn(g.c2z, __fsub_rn(d, a), __fmul_rn(g.c1z, __fsub_rn(c, b)));
+        if constexpr (!WIDE) return g.c1z * (c - b) + g.c2z * (d - a);
+        return __fmaf_rn(g.c1z, __fsub_rn(c, b), __fmul_rn(g.c2z, __fsub_rn(d, a)));
     }
 }
 
@@ -447,8 +451,8 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
                               const DevMedium& M, const DevBoundary& B, FusedPlan** out);
 void fused_plan_destroy(FusedPlan* p);
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
-                         const DevBoundary& B, float dt, const DevSource& S, const float* wavelet,
-                         int n, int* err, cudaStream_t st);
+                         const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
+                         const float* wavelet, int n, int* err, cudaStream_t st);
 }  // namespace fused
 
 // The time loop of a small grid in one cooperative launch with the fields

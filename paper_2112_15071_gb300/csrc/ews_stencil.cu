@@ -38,7 +38,6 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
-#include <cudaTypedefs.h>
 
 #include <algorithm>
 #include <new>
@@ -47,9 +46,7 @@
 #include "ews_arith.cuh"
 #include "ews_internal.cuh"
 #include "ews_ops.cuh"
-#ifndef EWS_L2PROMO
-#define EWS_L2PROMO CU_TENSOR_MAP_L2_PROMOTION_L2_256B
-#endif
+#include "ews_tma.cuh"
 
 // This file is compiled once per tile shape.  The default build (32 x 8
 // tiles) has every pass form, the batched executor and the entry points of
@@ -86,7 +83,6 @@ constexpr int ROWS = EWS_ROWS;                    // cells per thread (adjacent 
 constexpr int RY = TY / ROWS;                     // thread rows
 constexpr int NTH = TX * RY;                      // threads per CTA
 static_assert(TY % ROWS == 0, "rows per thread must divide the tile height");
-constexpr unsigned long long kWaitNs = 2000000000ull;  // 2 s per wait
 
 // Storage of the 9 wavefields: FP32, BF16 or FP16 (arithmetic is FP32).  A
 // TMA tile must start on a 16-byte boundary, so a halo box of 16-bit fields
@@ -110,8 +106,6 @@ template <> struct St<__half> {
     __device__ static float ld(const __half* p) { return __half2float(*p); }
     __device__ static __half put(float x) { return __float2half_rn(x); }
 };
-
-constexpr int r128(int b) { return (b + 127) / 128 * 128; }
 
 // Slot layout of one plane, in bytes, following the copies that fill it
 // (fields in their physical slot order, fslot):
@@ -208,73 +202,6 @@ constexpr int blocks_for(size_t smem) {
            : (227 * 1024) / (int)(smem + 1024) > (sizeof(T) == 4 ? 3 : 4)
                ? (sizeof(T) == 4 ? 3 : 4)
                : (227 * 1024) / (int)(smem + 1024);
-}
-
-// --- PTX wrappers -------------------------------------------------------------
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-    return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
-                 : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
-                 "r"(bytes)
-                 : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
-
-__device__ __forceinline__ unsigned long long now_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Bounded wait on the phase `parity` of an mbarrier.
-__device__ __noinline__ bool mbar_wait_slow(uint64_t* bar, uint32_t parity) {
-    const unsigned long long t0 = now_ns();
-    while (true) {
-        if (mbar_try(bar, parity)) return true;
-        if (now_ns() - t0 > kWaitNs) return false;
-        __nanosleep(64);
-    }
-}
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-    return mbar_try(bar, parity) || mbar_wait_slow(bar, parity);
-}
-
-__device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar,
-                                            int x, int y, int z) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5}], [%2];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z)
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, uint64_t* bar,
-                                            int x, int y, int z, int w) {
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes"
-        " [%0], [%1, {%3, %4, %5, %6}], [%2];" ::"r"(smem_u32(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(smem_u32(bar)), "r"(x), "r"(y), "r"(z),
-        "r"(w)
-        : "memory");
 }
 
 // Tensor maps of one pass, in slot order: halo[] then core[] as listed in
@@ -481,11 +408,12 @@ __device__ __forceinline__ void aux_refill(const Maps& maps, const Geo<BND, T>& 
 }
 
 // psi = b psi + a d; d += psi for the three terms of one damped direction.
+template <bool WIDE>
 __device__ __forceinline__ void pml_upd(float& p0, float& p1, float& p2, float a, float b,
                                         float& d0, float& d1, float& d2) {
-    ar::pml(p0, a, b, d0);
-    ar::pml(p1, a, b, d1);
-    ar::pml(p2, a, b, d2);
+    ar::Form<WIDE>::pml(p0, a, b, d0);
+    ar::Form<WIDE>::pml(p1, a, b, d1);
+    ar::Form<WIDE>::pml(p2, a, b, d2);
 }
 
 // Field tile element as FP32.
@@ -541,6 +469,7 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                                          unsigned& psi_par, bool& ovf) {
     float* psib = psi_base(sm);
     using L = Lay<T>;
+    using AR = ar::Form<sizeof(T) == 4>;
     constexpr int HX = L::HX;
     constexpr int SB = RS ? RS : vslot_bytes<T, MODE>();
     constexpr int PB = PH & 1;                                     // psi entry of plane k
@@ -609,17 +538,17 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
             const float* qyz = Q.yz[rr];
             const float* qzz = Q.zz[rr];
             // vx at (i+1/2, j, k)
-            float dxx = ar::d4(g.c1x, g.c2x, F(hxx, R - 1), F(hxx, R), F(hxx, R + 1), F(hxx, R + 2));
-            float dxy = ar::d4(g.c1y, g.c2y, F(hxy, R - 2 * HX), F(hxy, R - HX), F(hxy, R), F(hxy, R + HX));
-            float dxz = zdiff<ZF, false>(g, zw, zt, qxz[A], qxz[B], qxz[C], qxz[D]);
+            float dxx = AR::d4(g.c1x, g.c2x, F(hxx, R - 1), F(hxx, R), F(hxx, R + 1), F(hxx, R + 2));
+            float dxy = AR::d4(g.c1y, g.c2y, F(hxy, R - 2 * HX), F(hxy, R - HX), F(hxy, R), F(hxy, R + HX));
+            float dxz = zdiff<ZF, false, sizeof(T) == 4>(g, zw, zt, qxz[A], qxz[B], qxz[C], qxz[D]);
             // vy at (i, j+1/2, k)
-            float dyx = ar::d4(g.c1x, g.c2x, F(hxy, R - 2), F(hxy, R - 1), F(hxy, R), F(hxy, R + 1));
-            float dyy = ar::d4(g.c1y, g.c2y, F(hyy, RY - TX), F(hyy, RY), F(hyy, RY + TX), F(hyy, RY + 2 * TX));
-            float dyz = zdiff<ZF, false>(g, zw, zt, qyz[A], qyz[B], qyz[C], qyz[D]);
+            float dyx = AR::d4(g.c1x, g.c2x, F(hxy, R - 2), F(hxy, R - 1), F(hxy, R), F(hxy, R + 1));
+            float dyy = AR::d4(g.c1y, g.c2y, F(hyy, RY - TX), F(hyy, RY), F(hyy, RY + TX), F(hyy, RY + 2 * TX));
+            float dyz = zdiff<ZF, false, sizeof(T) == 4>(g, zw, zt, qyz[A], qyz[B], qyz[C], qyz[D]);
             // vz at (i, j, k+1/2)
-            float dzx = ar::d4(g.c1x, g.c2x, F(hxz, R - 2), F(hxz, R - 1), F(hxz, R), F(hxz, R + 1));
-            float dzy = ar::d4(g.c1y, g.c2y, F(hyz, RY - 2 * TX), F(hyz, RY - TX), F(hyz, RY), F(hyz, RY + TX));
-            float dzz = zdiff<ZF, true>(g, zw, zt, qzz[A], qzz[B], qzz[C], qzz[D]);
+            float dzx = AR::d4(g.c1x, g.c2x, F(hxz, R - 2), F(hxz, R - 1), F(hxz, R), F(hxz, R + 1));
+            float dzy = AR::d4(g.c1y, g.c2y, F(hyz, RY - 2 * TX), F(hyz, RY - TX), F(hyz, RY), F(hyz, RY + TX));
+            float dzz = zdiff<ZF, true, sizeof(T) == 4>(g, zw, zt, qzz[A], qzz[B], qzz[C], qzz[D]);
             if constexpr (kScaled<T>) {     // stored -> physical units
                 dxx *= P.inv[SXX]; dxy *= P.inv[SXY]; dxz *= P.inv[SXZ];
                 dyx *= P.inv[SXY]; dyy *= P.inv[SYY]; dyz *= P.inv[SYZ];
@@ -631,17 +560,17 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 const long long oo = o + rr * g.pitch;
                 if (G.sx) {
                     float p0 = ps[0 * CORE], p1 = ps[1 * CORE], p2 = ps[2 * CORE];
-                    pml_upd(p0, p1, p2, G.pax, G.pbx, dxx, dyx, dzx);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, G.pax, G.pbx, dxx, dyx, dzx);
                     P.B.psi[0][oo] = p0; P.B.psi[1][oo] = p1; P.B.psi[2][oo] = p2;
                 }
                 if (G.sy[rr]) {
                     float p0 = ps[3 * CORE], p1 = ps[4 * CORE], p2 = ps[5 * CORE];
-                    pml_upd(p0, p1, p2, G.pay[rr], G.pby[rr], dxy, dyy, dzy);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, G.pay[rr], G.pby[rr], dxy, dyy, dzy);
                     P.B.psi[6][oo] = p0; P.B.psi[7][oo] = p1; P.B.psi[8][oo] = p2;
                 }
                 if (sz) {
                     float p0 = ps[6 * CORE], p1 = ps[7 * CORE], p2 = ps[8 * CORE];
-                    pml_upd(p0, p1, p2, paz, pbz, dxz, dyz, dzz);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, paz, pbz, dxz, dyz, dzz);
                     P.B.psi[12][oo] = p0; P.B.psi[13][oo] = p1; P.B.psi[14][oo] = p2;
                 }
             }
@@ -657,15 +586,15 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 const float* qhx = Q.hx[rr];
                 const float* qhy = Q.hy[rr];
                 const float* qhz = Q.hz[rr];
-                const float exx = ar::d4(g.c1x, g.c2x, F(vhx, R - 2), F(vhx, R - 1), F(vhx, R), F(vhx, R + 1));
-                const float eyy = ar::d4(g.c1y, g.c2y, F(vhy, R - 2 * HX), F(vhy, R - HX), F(vhy, R), F(vhy, R + HX));
+                const float exx = AR::d4(g.c1x, g.c2x, F(vhx, R - 2), F(vhx, R - 1), F(vhx, R), F(vhx, R + 1));
+                const float eyy = AR::d4(g.c1y, g.c2y, F(vhy, R - 2 * HX), F(vhy, R - HX), F(vhy, R), F(vhy, R + HX));
                 constexpr int FW = ZF == ZS_NONE ? ZS_NONE : ZS_FWD;   // forward strain rates
-                const float ezz = zdiff<FW, false>(g, zw, zt, qhz[A], qhz[B], qhz[C], qhz[D]);
+                const float ezz = zdiff<FW, false, sizeof(T) == 4>(g, zw, zt, qhz[A], qhz[B], qhz[C], qhz[D]);
                 const float gxy = g.c1y * (F(vhx, R + HX) - F(vhx, R)) + g.c2y * (F(vhx, R + 2 * HX) - F(vhx, R - HX)) +
                                   g.c1x * (F(vhy, R + 1) - F(vhy, R)) + g.c2x * (F(vhy, R + 2) - F(vhy, R - 1));
-                const float gxz = zdiff<FW, true>(g, zw, zt, qhx[A], qhx[B], qhx[C], qhx[D]) +
+                const float gxz = zdiff<FW, true, sizeof(T) == 4>(g, zw, zt, qhx[A], qhx[B], qhx[C], qhx[D]) +
                                   g.c1x * (F(vhz, R + 1) - F(vhz, R)) + g.c2x * (F(vhz, R + 2) - F(vhz, R - 1));
-                const float gyz = zdiff<FW, true>(g, zw, zt, qhy[A], qhy[B], qhy[C], qhy[D]) +
+                const float gyz = zdiff<FW, true, sizeof(T) == 4>(g, zw, zt, qhy[A], qhy[B], qhy[C], qhy[D]) +
                                   g.c1y * (F(vhz, R + HX) - F(vhz, R)) + g.c2y * (F(vhz, R + 2 * HX) - F(vhz, R - HX));
                 const float uxx = F(hxx, R), uyy = F(hyy, RY), uzz = F(vc, VC_SZZ * CORE + rr * TX);
                 const float gdt = P.X.gdt;
@@ -710,13 +639,13 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 bz = __fdividef(1.0f, lerp1(Q.ch.lo[rr][0], Q.ch.hi[rr][0], zh.f));
             } else {
                 const float r0 = hr[RF];
-                bx = ar::buoyancy(r0, hr[RF + G.cx]);
-                by = ar::buoyancy(r0, hr[RF + G.cy[rr]]);
-                bz = ar::buoyancy(r0, ktop ? hr1[RF] : r0);
+                bx = AR::buoyancy(r0, hr[RF + G.cx]);
+                by = AR::buoyancy(r0, hr[RF + G.cy[rr]]);
+                bz = AR::buoyancy(r0, ktop ? hr1[RF] : r0);
             }
-            float vx = ar::vnew(F(vc, VC_VX * CORE + rr * TX), P.dto[VX], bx, dxx, dxy, dxz);
-            float vy = ar::vnew(F(vc, VC_VY * CORE + rr * TX), P.dto[VY], by, dyx, dyy, dyz);
-            float vz = ar::vnew(F(vc, VC_VZ * CORE + rr * TX), P.dto[VZ], bz, dzx, dzy, dzz);
+            float vx = AR::vnew(F(vc, VC_VX * CORE + rr * TX), P.dto[VX], bx, dxx, dxy, dxz);
+            float vy = AR::vnew(F(vc, VC_VY * CORE + rr * TX), P.dto[VY], by, dyx, dyy, dyz);
+            float vz = AR::vnew(F(vc, VC_VZ * CORE + rr * TX), P.dto[VZ], bz, dzx, dzy, dzz);
             if (BND == BND_SPONGE) {
                 const float Gs = G3 * G.gy[rr];
                 vx *= Gs; vy *= Gs; vz *= Gs;
@@ -837,6 +766,7 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
                                          unsigned& psi_par, bool& ovf) {
     float* psib = psi_base(sm);
     using L = Lay<T>;
+    using AR = ar::Form<sizeof(T) == 4>;
     constexpr int HX = L::HX;
     constexpr int SB = RS ? RS : L::SSLOT;
     constexpr int HS = L::HB;                                      // halo tile stride
@@ -882,16 +812,16 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
             const float* qvy = Q.vy[rr];
             const float* qvz = Q.vz[rr];
             // normal strain rates at (i, j, k)
-            float exx = ar::d4(g.c1x, g.c2x, F(hvx, R - 2), F(hvx, R - 1), F(hvx, R), F(hvx, R + 1));
-            float eyy = ar::d4(g.c1y, g.c2y, F(hvy, R - 2 * HX), F(hvy, R - HX), F(hvy, R), F(hvy, R + HX));
-            float ezz = zdiff<ZF, false>(g, zw, zt, qvz[A], qvz[B], qvz[C], qvz[D]);
+            float exx = AR::d4(g.c1x, g.c2x, F(hvx, R - 2), F(hvx, R - 1), F(hvx, R), F(hvx, R + 1));
+            float eyy = AR::d4(g.c1y, g.c2y, F(hvy, R - 2 * HX), F(hvy, R - HX), F(hvy, R), F(hvy, R + HX));
+            float ezz = zdiff<ZF, false, sizeof(T) == 4>(g, zw, zt, qvz[A], qvz[B], qvz[C], qvz[D]);
             // shear terms at the shear points
-            float vxy = ar::d4(g.c1y, g.c2y, F(hvx, R - HX), F(hvx, R), F(hvx, R + HX), F(hvx, R + 2 * HX));
-            float vyx = ar::d4(g.c1x, g.c2x, F(hvy, R - 1), F(hvy, R), F(hvy, R + 1), F(hvy, R + 2));
-            float vxz = zdiff<ZF, true>(g, zw, zt, qvx[A], qvx[B], qvx[C], qvx[D]);
-            float vzx = ar::d4(g.c1x, g.c2x, F(hvz, R - 1), F(hvz, R), F(hvz, R + 1), F(hvz, R + 2));
-            float vyz = zdiff<ZF, true>(g, zw, zt, qvy[A], qvy[B], qvy[C], qvy[D]);
-            float vzy = ar::d4(g.c1y, g.c2y, F(hvz, R - HX), F(hvz, R), F(hvz, R + HX), F(hvz, R + 2 * HX));
+            float vxy = AR::d4(g.c1y, g.c2y, F(hvx, R - HX), F(hvx, R), F(hvx, R + HX), F(hvx, R + 2 * HX));
+            float vyx = AR::d4(g.c1x, g.c2x, F(hvy, R - 1), F(hvy, R), F(hvy, R + 1), F(hvy, R + 2));
+            float vxz = zdiff<ZF, true, sizeof(T) == 4>(g, zw, zt, qvx[A], qvx[B], qvx[C], qvx[D]);
+            float vzx = AR::d4(g.c1x, g.c2x, F(hvz, R - 1), F(hvz, R), F(hvz, R + 1), F(hvz, R + 2));
+            float vyz = zdiff<ZF, true, sizeof(T) == 4>(g, zw, zt, qvy[A], qvy[B], qvy[C], qvy[D]);
+            float vzy = AR::d4(g.c1y, g.c2y, F(hvz, R - HX), F(hvz, R), F(hvz, R + HX), F(hvz, R + 2 * HX));
             if constexpr (kScaled<T>) {     // stored -> physical units
                 exx *= P.inv[VX]; vxy *= P.inv[VX]; vxz *= P.inv[VX];
                 eyy *= P.inv[VY]; vyx *= P.inv[VY]; vyz *= P.inv[VY];
@@ -902,17 +832,17 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
                 const long long oo = o + rr * g.pitch;
                 if (G.sx) {
                     float p0 = ps[0 * CORE], p1 = ps[1 * CORE], p2 = ps[2 * CORE];
-                    pml_upd(p0, p1, p2, G.pax, G.pbx, exx, vyx, vzx);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, G.pax, G.pbx, exx, vyx, vzx);
                     P.B.psi[3][oo] = p0; P.B.psi[4][oo] = p1; P.B.psi[5][oo] = p2;
                 }
                 if (G.sy[rr]) {
                     float p0 = ps[3 * CORE], p1 = ps[4 * CORE], p2 = ps[5 * CORE];
-                    pml_upd(p0, p1, p2, G.pay[rr], G.pby[rr], eyy, vxy, vzy);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, G.pay[rr], G.pby[rr], eyy, vxy, vzy);
                     P.B.psi[9][oo] = p0; P.B.psi[10][oo] = p1; P.B.psi[11][oo] = p2;
                 }
                 if (sz) {
                     float p0 = ps[6 * CORE], p1 = ps[7 * CORE], p2 = ps[8 * CORE];
-                    pml_upd(p0, p1, p2, paz, pbz, ezz, vxz, vyz);
+                    pml_upd<sizeof(T) == 4>(p0, p1, p2, paz, pbz, ezz, vxz, vyz);
                     P.B.psi[15][oo] = p0; P.B.psi[16][oo] = p1; P.B.psi[17][oo] = p2;
                 }
             }
@@ -952,25 +882,25 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
                 mu0 = hmu[RF];
                 const float mxp = hmu[RF + G.cx], myp = hmu[RF + cyr];
                 const float mzp = hmu1[RF];
-                mxy = ar::mean4(mu0, mxp, myp, hmu[RF + G.cx + cyr]);
-                mxz = ar::mean4(mu0, mxp, mzp, hmu1[RF + G.cx]);
-                myz = ar::mean4(mu0, myp, mzp, hmu1[RF + cyr]);
+                mxy = AR::mean4(mu0, mxp, myp, hmu[RF + G.cx + cyr]);
+                mxz = AR::mean4(mu0, mxp, mzp, hmu1[RF + G.cx]);
+                myz = AR::mean4(mu0, myp, mzp, hmu1[RF + cyr]);
                 if constexpr (ZF != ZS_NONE) {
                     // xz / yz shear points on the free-surface plane z = ks - 1/2:
                     // harmonic mean of the 4 cells (vacuum-formulation reading)
                     if (k == g.fs - 1) {
-                        mxz = ar::harm4(mu0, mxp, mzp, hmu1[RF + G.cx]);
-                        myz = ar::harm4(mu0, myp, mzp, hmu1[RF + cyr]);
+                        mxz = AR::harm4(mu0, mxp, mzp, hmu1[RF + G.cx]);
+                        myz = AR::harm4(mu0, myp, mzp, hmu1[RF + cyr]);
                     }
                 }
             }
-            const float l2m = ar::l2m(lam, mu0);
-            float s0 = ar::snormal(F(cr, SC_SXX * CORE + rr * TX), P.dto[SXX], l2m, lam, exx, eyy, ezz);
-            float s1 = ar::snormal(F(cr, SC_SYY * CORE + rr * TX), P.dto[SYY], l2m, lam, eyy, exx, ezz);
-            float s2 = ar::snormal(F(cr, SC_SZZ * CORE + rr * TX), P.dto[SZZ], l2m, lam, ezz, exx, eyy);
-            float s3 = ar::sshear(F(cr, SC_SXY * CORE + rr * TX), P.dto[SXY], mxy, vxy, vyx);
-            float s4 = ar::sshear(F(cr, SC_SXZ * CORE + rr * TX), P.dto[SXZ], mxz, vxz, vzx);
-            float s5 = ar::sshear(F(cr, SC_SYZ * CORE + rr * TX), P.dto[SYZ], myz, vyz, vzy);
+            const float l2m = AR::l2m(lam, mu0);
+            float s0 = AR::snormal(F(cr, SC_SXX * CORE + rr * TX), P.dto[SXX], l2m, lam, exx, eyy, ezz);
+            float s1 = AR::snormal(F(cr, SC_SYY * CORE + rr * TX), P.dto[SYY], l2m, lam, eyy, exx, ezz);
+            float s2 = AR::snormal(F(cr, SC_SZZ * CORE + rr * TX), P.dto[SZZ], l2m, lam, ezz, exx, eyy);
+            float s3 = AR::sshear(F(cr, SC_SXY * CORE + rr * TX), P.dto[SXY], mxy, vxy, vyx);
+            float s4 = AR::sshear(F(cr, SC_SXZ * CORE + rr * TX), P.dto[SXZ], mxz, vxz, vzx);
+            float s5 = AR::sshear(F(cr, SC_SYZ * CORE + rr * TX), P.dto[SYZ], myz, vyz, vzy);
             if (BND == BND_SPONGE) {
                 const float Gs = G3 * G.gy[rr];
                 s0 *= Gs; s1 *= Gs; s2 *= Gs; s3 *= Gs; s4 *= Gs; s5 *= Gs;
@@ -1349,51 +1279,6 @@ __global__ void __launch_bounds__(NTH, GRAD ? 2 : 3)
 }
 #endif  // EWS_FULL
 
-PFN_cuTensorMapEncodeTiled_v12000 encoder() {
-    static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000,
-                                             cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(p);
-    }
-    return fn;
-}
-
-// Tensor map of nt pitched [nz][ny][pitch] arrays lying tstride bytes apart,
-// as a 4D tensor [array][nz][ny][pitch], with a box of bw x bh x 1 x bt.
-bool encode4(CUtensorMap* map, const DevGrid& g, const void* base, CUtensorMapDataType dt,
-             int esize, long long tstride, int nt, int bw, int bh, int bt) {
-    auto fn = encoder();
-    if (!fn) return false;
-    cuuint64_t dims[4] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz, (cuuint64_t)nt};
-    cuuint64_t strides[3] = {(cuuint64_t)g.pitch * esize, (cuuint64_t)g.plane * esize,
-                             (cuuint64_t)tstride};
-    cuuint32_t box[4] = {(cuuint32_t)bw, (cuuint32_t)bh, 1, (cuuint32_t)bt};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    CUresult r = fn(map, dt, 4, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, EWS_L2PROMO,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
-// Tensor map of one pitched [nz][ny][pitch] array with a box of bw x bh x 1.
-bool encode(CUtensorMap* map, const DevGrid& g, const void* base, CUtensorMapDataType dt,
-            int esize, int bw, int bh) {
-    auto fn = encoder();
-    if (!fn) return false;
-    cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz};
-    cuuint64_t strides[2] = {(cuuint64_t)g.pitch * esize, (cuuint64_t)g.plane * esize};
-    cuuint32_t box[3] = {(cuuint32_t)bw, (cuuint32_t)bh, 1};
-    cuuint32_t es[3] = {1, 1, 1};
-    CUresult r = fn(map, dt, 3, const_cast<void*>(base), dims, strides, box, es,
-                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, EWS_L2PROMO,
-                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS;
-}
-
 template <typename K>
 cudaError_t prepare(K kern, size_t smem, int* blocks_per_sm) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1518,32 +1403,6 @@ struct StencilPlan {
 };
 
 namespace {
-
-// Planes per z-chunk of a pass over ntile tile columns with `slots` CTAs
-// resident at once: the chunk count n (chunks of at least min_planes
-// planes) that minimises the modelled pass time, the waves of (tile, chunk)
-// CTAs times the planes each CTA marches through, ceil(ntile n / slots) x
-// (nz / n + halo) with `halo` the planes a chunk loads beyond its own on
-// each side; ties go to more chunks.  Measured against the earlier rule of
-// about four waves (GB300, Gcell/s): 192^3 sponge 48.4 vs 44.5, 192^3 C-PML
-// 35.4 vs 33.8, 128^3 sponge 50.5 vs 39.4, 1024 x 1024 x 512 BF16 (32 x 16
-// tiles) 78.9 vs 75.9, 256^3 C-PML unchanged (7 chunks either way).  Chunks
-// of at least 4 planes: small grids, whose few columns leave most SMs idle,
-// get more CTAs (64 x 64 x 32 sponge: 11.3 Gcell/s with 4-plane chunks, 9.1
-// with at least 8 planes; 64^3 19.9 vs 17.5).
-int chunk_planes(long long ntile, long long slots, int nz, int min_planes, int halo) {
-    long long best_n = 1, best_cost = -1;
-    for (long long n = 1; n <= std::max(1, nz / min_planes); ++n) {
-        const long long zc = (nz + n - 1) / n;
-        const long long nn = (nz + zc - 1) / zc;               // chunks of zc planes
-        const long long cost = ((ntile * nn + slots - 1) / slots) * (zc + halo);
-        if (best_cost < 0 || cost <= best_cost) {
-            best_cost = cost;
-            best_n = n;
-        }
-    }
-    return (int)((nz + best_n - 1) / best_n);
-}
 
 cudaError_t plan_build(StencilPlan* p, const DevGrid& g, const DevFields& F, const DevMedium& M,
                        const DevBoundary& B, int storage) {
