@@ -597,40 +597,50 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
 bool resident_eligible(const ews_sim* s) {
     return s->res && s->tile_req == EWS_TILE_AUTO && !s->profiling;
 }
-ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
-                          float* dseis, int ld, float* vcap) {
-    const DevSource S = source_taps(s, src, dt);
-    const bool rec = s->nrec > 0 && dseis;
+ResidentRun resident_run(const ews_sim* s, const DevFields& F, double dt, int nrec, int ld) {
     ResidentRun r{};
     r.plan = s->res;
     r.g = s->g;
-    r.F = s->F();
+    r.F = F;
     r.M = s->M();
     r.B = s->B;
-    r.S = &S;
-    r.wavelet = s->wavelet;
     r.dt = (float)dt;
     r.inbox = s->res_inbox;
     r.err = s->err;
-    r.nrec = rec ? s->nrec : 0;
+    r.nrec = nrec;
     r.taps = s->rtaps;
     r.tlist = s->res_list;
     r.tstart = s->res_start;
     r.stage = s->res_stage;
-    r.seis = rec ? dseis : nullptr;
     r.ld = ld;
     r.fstride = (long long)s->fstride;
+    return r;
+}
+// Tags of the next launch of `nsteps` steps.
+ews_status resident_epoch(ews_sim* s, ResidentRun* r, int nsteps) {
+    if (s->res_epoch > 0xF0000000u) {                  // before the tags wrap around
+        CK(cudaMemsetAsync(s->res_inbox, 0, resident_inbox_bytes(*s->res), s->stream));
+        s->res_epoch = 0;
+    }
+    r->nsteps = nsteps;
+    r->epoch = s->res_epoch;
+    s->res_epoch += (unsigned)nsteps;
+    return EWS_OK;
+}
+ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
+                          float* dseis, int ld, float* vcap) {
+    const DevSource S = source_taps(s, src, dt);
+    const bool rec = s->nrec > 0 && dseis;
+    ResidentRun r = resident_run(s, s->F(), dt, rec ? s->nrec : 0, ld);
+    r.S = &S;
+    r.wavelet = s->wavelet;
+    r.seis = rec ? dseis : nullptr;
     s->fresh = false;
     const int chunk = rec ? s->res_chunk : kResidentSteps;
     for (int m = 0; m < nsteps; m += chunk) {
         r.n0 = n0 + m;
-        r.nsteps = std::min(chunk, nsteps - m);
-        if (s->res_epoch > 0xF0000000u) {              // before the tags wrap around
-            CK(cudaMemsetAsync(s->res_inbox, 0, resident_inbox_bytes(*s->res), s->stream));
-            s->res_epoch = 0;
-        }
-        r.epoch = s->res_epoch;
-        s->res_epoch += (unsigned)r.nsteps;
+        const ews_status st = resident_epoch(s, &r, std::min(chunk, nsteps - m));
+        if (st != EWS_OK) return st;
         // v^{n+1/2} of step n0 + m goes to slot m + 1 of the history
         r.vcap = vcap ? vcap + (size_t)(m + 1) * 3 * s->fstride : nullptr;
         CK(launch_resident(r, s->stream));
@@ -963,7 +973,16 @@ ews_status adjoint_core(ews_sim* s, int nt, double dt, int ckpt_every, const flo
                 if ((st = steps(s, s->src, n0, n1 - n0, dt, nullptr, nt, s->vhist)) != EWS_OK)
                     return st;
             }
-            for (int m = n1 - 1; m >= n0; --m) {
+            // small grids: the range in one launch (per kResidentSteps)
+            const bool resident = resident_eligible(s) &&
+                                  resident_adjoint_supported(*s->res, s->g, s->opt.boundary);
+            for (int e = n1; resident && e > n0; e -= kResidentSteps) {
+                ResidentRun r = resident_run(s, AF, -dt, s->nrec > 0 && sadj ? s->nrec : 0, nt);
+                r.n0 = std::max(n0, e - kResidentSteps);
+                if ((st = resident_epoch(s, &r, e - r.n0)) != EWS_OK) return st;
+                CK(launch_resident_adjoint(r, ResidentAdjoint{s->vhist, n0, e < n1, K, A, fdt, sadj}, s->stream));
+            }
+            for (int m = resident ? n0 - 1 : n1 - 1; m >= n0; --m) {
                 VelExtra X{};
                 for (int q = 0; q < 8; ++q) X.acc[q] = A.acc[q];
                 X.fstride = (long long)fs;

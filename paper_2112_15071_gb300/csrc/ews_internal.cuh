@@ -493,6 +493,20 @@ cudaError_t resident_prepare(const ResidentPlan& p, int bnd);
 void resident_taps(const ResidentPlan& p, const DevGrid& g, const Tap* taps, int ntap,
                    std::vector<int2>* list, std::vector<int>* start);
 cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st);
+// The reverse sweep (transformed variables; sponge or no boundary, no free
+// surface) of steps r.n0 + r.nsteps - 1 .. r.n0 on the adjoint fields r.F with
+// r.dt negative; slot n - h0 + 1 of the history holds v^{n+1/2}.
+struct ResidentAdjoint {
+    const float* vhist;
+    int h0;                       // first step of the history range
+    int vnext;                    // steps after the last one of this launch were done before
+    int flush;                    // FP32 accumulators go to FP64 every `flush` steps
+    AdjFields A;
+    float gdt;                    // forward dt
+    const float* sadj;            // residual [3 nrec][r.ld]
+};
+bool resident_adjoint_supported(const ResidentPlan& p, const DevGrid& g, int bnd);
+cudaError_t launch_resident_adjoint(const ResidentRun& r, const ResidentAdjoint& a, cudaStream_t st);
 
 // History buffer of the reverse pass: nslot slots of 3 fields, slot s field c
 // at hist + (3 s + c) * fstride, pitched like the wavefields; and its 8 FP32

@@ -41,9 +41,12 @@ namespace {
 constexpr int MX = 16, MY = 16;                  // largest block in x and y
 constexpr int SX = MX + 4, SP = SX * (MY + 4);   // shared-memory strides (row, plane)
 constexpr int MAXZ = 12;                         // largest block in z
-constexpr int FCAP = SP * (MAXZ + 4);           // elements of one field
+// Elements of one field in shared memory, by the planes of a block (the
+// 768-thread kernels serve blocks of 9 to 12 planes).
+constexpr int fcap(int lz) { return SP * (lz <= 8 ? 12 : MAXZ + 4); }
 constexpr int COLS = MX * MY;                    // threads of one z-group
-static_assert(NFIELD * FCAP * 4 + 1024 <= 227 * 1024, "fields fit one CTA's shared memory");
+static_assert(NFIELD * fcap(MAXZ) * 4 + 1024 <= 227 * 1024 && (NFIELD + 3) * fcap(8) * 4 + 1024 <= 227 * 1024,
+              "fields (and the history's, reverse) fit one CTA's shared memory");
 
 struct ResParams {
     DevGrid g;
@@ -63,6 +66,17 @@ struct ResParams {
     float* stage;                                // [nsteps][ntap] v at the taps, or null
     int ntap;
     float* vcap;                                 // history slot of step n0 (3 fields), or null
+    // reverse sweep (n0 + nsteps - 1 down to n0): the history, slot n - h0 + 1
+    // holding v^{n+1/2}; whether slot n0 + nsteps - h0 + 1 exists; the
+    // accumulators, added to FP64 every `flush` steps; the residual
+    const float* vhist;
+    int h0, vnext, flush;
+    AdjFields A;
+    float gdt;
+    const float* sadj;
+    int ld;
+    const Tap* taps;
+    float* coef;                                 // [ntap] scratch, by place in tlist
     long long fstride;                           // elements between fields
     unsigned long long wait_ns;
 };
@@ -123,7 +137,7 @@ template <bool DP>
 __device__ __forceinline__ bool from_hi(int v) { return v == 2 || (DP && v == 1); }
 
 // Halo layers of the first step, from the global fields.
-template <bool VEL>
+template <bool VEL, int FCAP>
 __device__ __forceinline__ void halo_first(const HaloLine& h, const ResParams& P, float* sm) {
     if (h.axis < 0) return;
     int q[3];
@@ -138,7 +152,7 @@ __device__ __forceinline__ void halo_first(const HaloLine& h, const ResParams& P
         }
 }
 // Receive the layers of one exchange (VEL: sigma, for the velocity phase).
-template <bool VEL>
+template <bool VEL, int FCAP>
 __device__ __forceinline__ bool halo_recv(const HaloLine& h, const ResParams& P, float* sm, unsigned tag) {
     if (h.axis < 0) return true;
     const unsigned long long* in = P.inbox + h.in + (VEL ? 0 : 9 * P.lines);
@@ -186,7 +200,7 @@ __device__ __forceinline__ bool halo_recv(const HaloLine& h, const ResParams& P,
 // Send this CTA's face layers of one exchange: to the neighbour below, whose
 // layers L and L + 1 are this CTA's cells 0 and 1, and to the one above,
 // whose layers -1 and -2 are the last two.
-template <bool VEL>
+template <bool VEL, int FCAP>
 __device__ __forceinline__ void halo_send(const HaloLine& h, const ResParams& P, const float* sm, unsigned tag) {
     if (h.axis < 0) return;
     int q[3];
@@ -205,8 +219,14 @@ __device__ __forceinline__ void halo_send(const HaloLine& h, const ResParams& P,
     }
 }
 
-template <int BND, int FS, int CPT, int MAXT>
+// ADJ: the reverse sweep in transformed variables (F are the adjoint fields,
+// dt is negative): the velocity phase also accumulates the gradient products
+// of the pass k_velocity<M_GRAD>, with the forward velocity's history staged
+// as three more shared fields, and the residual is injected after it.
+template <int BND, int FS, int CPT, int MAXT, bool ADJ = false>
 __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ ResParams P) {
+    constexpr int FCAP = fcap(MAXT == 768 ? MAXZ : 8);
+    constexpr int H0 = NFIELD;                   // first history field
     extern __shared__ __align__(16) float sm[];
     __shared__ float s_amp[kMaxSrcTaps][2];      // buoyancy, gain of the block's source taps
     __shared__ int s_off[kMaxSrcTaps];           // their shared offset, -1: not in this block
@@ -229,7 +249,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
     const int plane = (int)g.plane;
     const int go = gk * plane + gj * g.pitch + gi;
 
-    for (int x = t; x < NFIELD * FCAP; x += NT) sm[x] = 0.0f;
+    for (int x = t; x < (NFIELD + (ADJ ? 3 : 0)) * FCAP; x += NT) sm[x] = 0.0f;
     if (t == 0) s_src = 0;
     __syncthreads();
     // medium of the thread's cells at their staggered points; sponge gains
@@ -333,7 +353,25 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
             s_amp[t][1] = ops::gain(P.B, q.i, q.j, q.k);
         }
     }
-    const int tl0 = P.stage ? __ldg(P.tstart + cta) : 0, tl1 = P.stage ? __ldg(P.tstart + cta + 1) : 0;
+    const bool listed = ADJ ? P.sadj != nullptr : P.stage != nullptr;
+    const int tl0 = listed ? __ldg(P.tstart + cta) : 0, tl1 = listed ? __ldg(P.tstart + cta + 1) : 0;
+    // reverse sweep: accumulators, v^{n+3/2} and the residual's factors
+    float acc[ADJ ? CPT : 1][8], vnx[ADJ ? CPT : 1][3];
+    if constexpr (ADJ) {
+#pragma unroll
+        for (int c = 0; c < CPT; ++c)
+            if (c < nc) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) acc[c][q] = P.A.acc[q][go + c * plane];
+                const long long hs = (long long)(P.n0 + P.nsteps - P.h0 + 1) * 3 * P.fstride + go + c * plane;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) vnx[c][q] = P.vnext ? __ldg(P.vhist + hs + q * P.fstride) : 0.0f;
+            }
+        for (int x = tl0 + t; x < tl1; x += NT) {
+            const Tap q = P.taps[__ldg(P.tlist + x).y];
+            P.coef[x] = ops::gain(P.B, q.i, q.j, q.k) * ops::buoy(P.M, g, q.q - VX, q.i, q.j, q.k) * q.w;
+        }
+    }
     __syncthreads();
     const bool src = s_src != 0;
 
@@ -352,7 +390,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
 
     float* vcap = P.vcap;
     for (int m = 0; m < P.nsteps; ++m) {
-        const int n = P.n0 + m;
+        const int n = ADJ ? P.n0 + P.nsteps - 1 - m : P.n0 + m;
         // opaque to the compiler, so that addresses derived from these are
         // formed where they are used and not kept (spilled) across steps
         asm volatile("" : "+r"(h.in), "+r"(h.lo), "+r"(h.hi), "+r"(h.so), "+r"(h.axis));
@@ -370,9 +408,47 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
                     }
                 }
         }
+        // reverse sweep: the history of this step, read before the wait (own
+        // cells, and the layers its strain rates reach across the faces)
+        float hv[ADJ ? CPT : 1][3], hl[ADJ ? 9 : 1];
+        if constexpr (ADJ) {
+            const float* hist = P.vhist + (long long)(n - P.h0 + 1) * 3 * P.fstride;
+#pragma unroll
+            for (int c = 0; c < CPT; ++c)
+                if (c < nc)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) hv[c][q] = __ldg(hist + q * P.fstride + go + c * plane);
+            if (h.axis >= 0) {
+                int q[3];
+                line_fields<false>(h.axis, q);
+#pragma unroll
+                for (int e = 0; e < 9; ++e) {
+                    const bool dp = e >= 3, hi = dp ? from_hi<true>(e % 3) : from_hi<false>(e % 3);
+                    const int at = dp ? layer_at<true>(h, e % 3) : layer_at<false>(h, e % 3);
+                    if ((hi ? h.hi : h.lo) >= 0) hl[e] = __ldg(hist + q[e / 3] * P.fstride + h.go + at * h.gs);
+                }
+            }
+        }
         bool ok = true;
-        if (m > 0) ok = halo_recv<true>(h, P, sm, P.epoch + m);
-        else halo_first<true>(h, P, sm);
+        if (m > 0) ok = halo_recv<true, FCAP>(h, P, sm, P.epoch + m);
+        else halo_first<true, FCAP>(h, P, sm);
+        if constexpr (ADJ) {
+#pragma unroll
+            for (int c = 0; c < CPT; ++c)
+                if (c < nc)
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) sm[(H0 + q) * FCAP + so + c * SP] = hv[c][q];
+            if (h.axis >= 0) {
+                int q[3];
+                line_fields<false>(h.axis, q);
+#pragma unroll
+                for (int e = 0; e < 9; ++e) {
+                    const bool dp = e >= 3, hi = dp ? from_hi<true>(e % 3) : from_hi<false>(e % 3);
+                    const int at = dp ? layer_at<true>(h, e % 3) : layer_at<false>(h, e % 3);
+                    if ((hi ? h.hi : h.lo) >= 0) sm[(H0 + q[e / 3]) * FCAP + h.so + at * h.ss] = hl[e];
+                }
+            }
+        }
         if (__syncthreads_or(!ok)) return;
         if (nc > 0) {
             const float* s = sm + so;
@@ -419,6 +495,36 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
                         P.B.psi[12][o] = pz[c][0]; P.B.psi[13][o] = pz[c][1]; P.B.psi[14][o] = pz[c][2];
                     }
                 }
+                if constexpr (ADJ) {
+                    // gradient products of this reverse step (see k_velocity, M_GRAD)
+                    const float* hx = s + H0 * FCAP + c * SP;
+                    const float* hy = hx + FCAP;
+                    const float* hz = hy + FCAP;
+                    const float ex = ar::d4(g.c1x, g.c2x, hx[-2], hx[-1], hx[0], hx[1]);
+                    const float ey = ar::d4(g.c1y, g.c2y, hy[-2 * SX], hy[-SX], hy[0], hy[SX]);
+                    const float ez = ar::d4(g.c1z, g.c2z, hz[-2 * SP], hz[-SP], hz[0], hz[SP]);
+                    const float gxy = ar::d4(g.c1y, g.c2y, hx[-SX], hx[0], hx[SX], hx[2 * SX]) +
+                                      ar::d4(g.c1x, g.c2x, hy[-1], hy[0], hy[1], hy[2]);
+                    const float gxz = ar::d4(g.c1z, g.c2z, hx[-SP], hx[0], hx[SP], hx[2 * SP]) +
+                                      ar::d4(g.c1x, g.c2x, hz[-1], hz[0], hz[1], hz[2]);
+                    const float gyz = ar::d4(g.c1z, g.c2z, hy[-SP], hy[0], hy[SP], hy[2 * SP]) +
+                                      ar::d4(g.c1y, g.c2y, hz[-SX], hz[0], hz[SX], hz[2 * SX]);
+                    const float ux = s[SXX * FCAP + c * SP], uy = s[SYY * FCAP + c * SP], uz = s[SZZ * FCAP + c * SP];
+                    acc[c][0] += P.gdt * (ex + ey + ez) * (ux + uy + uz);
+                    acc[c][1] += P.gdt * (ex * ux + ey * uy + ez * uz);
+                    acc[c][2] += P.gdt * gxy * s[SXY * FCAP + c * SP];
+                    acc[c][3] += P.gdt * gxz * s[SXZ * FCAP + c * SP];
+                    acc[c][4] += P.gdt * gyz * s[SYZ * FCAP + c * SP];
+                    if (m > 0 || P.vnext) {
+                        const float iG = 1.0f / mg[c];
+                        acc[c][5] += (vnx[c][0] * iG - hx[0]) * s[VX * FCAP + c * SP];
+                        acc[c][6] += (vnx[c][1] * iG - hy[0]) * s[VY * FCAP + c * SP];
+                        acc[c][7] += (vnx[c][2] * iG - hz[0]) * s[VZ * FCAP + c * SP];
+                    }
+                    vnx[c][0] = hx[0];
+                    vnx[c][1] = hy[0];
+                    vnx[c][2] = hz[0];
+                }
                 v[c][0] = ar::vnew(s[VX * FCAP + c * SP], P.dt, mb[c][0], dxx, dxy, dxz);
                 v[c][1] = ar::vnew(s[VY * FCAP + c * SP], P.dt, mb[c][1], dyx, dyy, dyz);
                 v[c][2] = ar::vnew(s[VZ * FCAP + c * SP], P.dt, mb[c][2], dzx, dzy, dzz);
@@ -439,14 +545,22 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
             __syncthreads();
             inject(n, vcap);
         }
+        if (ADJ && tl1 > tl0) {                  // residual of step n (taps may share a cell)
+            __syncthreads();
+            for (int x = tl0 + t; x < tl1; x += NT) {
+                const int2 e = __ldg(P.tlist + x);
+                atomicAdd(sm + e.x, P.coef[x] * __ldg(P.sadj + (long long)(e.y >> 3) * P.ld + n));
+            }
+        }
         __syncthreads();
-        halo_send<false>(h, P, sm, P.epoch + m + 1);
+        halo_send<false, FCAP>(h, P, sm, P.epoch + m + 1);
         if (vcap) vcap += 3 * P.fstride;
         // v^{n+1/2} at the receiver taps of this block
-        for (int x = tl0 + t; x < tl1; x += NT) {
-            const int2 e = __ldg(P.tlist + x);
-            P.stage[(size_t)m * P.ntap + e.y] = sm[e.x];
-        }
+        if (!ADJ)
+            for (int x = tl0 + t; x < tl1; x += NT) {
+                const int2 e = __ldg(P.tlist + x);
+                P.stage[(size_t)m * P.ntap + e.y] = sm[e.x];
+            }
         // ---- stress phase ----
         asm volatile("" : "+r"(h.in), "+r"(h.lo), "+r"(h.hi), "+r"(h.so), "+r"(h.axis));
         if (BND == BND_CPML) {
@@ -461,7 +575,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
                     }
                 }
         }
-        ok = halo_recv<false>(h, P, sm, P.epoch + m + 1);
+        ok = halo_recv<false, FCAP>(h, P, sm, P.epoch + m + 1);
         if (__syncthreads_or(!ok)) return;
         if (nc > 0) {
             const float* s = sm + so;
@@ -529,8 +643,25 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
             inject(n, nullptr);
         }
         __syncthreads();
-        if (m + 1 < P.nsteps) halo_send<true>(h, P, sm, P.epoch + m + 1);
+        if (m + 1 < P.nsteps) halo_send<true, FCAP>(h, P, sm, P.epoch + m + 1);
+        if constexpr (ADJ)
+            if (n > P.h0 && (n - P.h0) % P.flush == 0) {
+#pragma unroll
+                for (int c = 0; c < CPT; ++c)
+                    if (c < nc)
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            P.A.acc64[q][go + c * plane] += (double)acc[c][q];
+                            acc[c][q] = 0.0f;
+                        }
+            }
     }
+    if constexpr (ADJ)
+#pragma unroll
+        for (int c = 0; c < CPT; ++c)
+            if (c < nc)
+#pragma unroll
+                for (int q = 0; q < 8; ++q) P.A.acc[q][go + c * plane] = acc[c][q];
 #pragma unroll
     for (int c = 0; c < CPT; ++c)
         if (c < nc)
@@ -581,7 +712,14 @@ int block_threads(int lz) {
 Kern kernel_for(int bnd, bool fs, int lz) {
     return lz <= 4 ? pick<1, 1024>(bnd, fs) : lz <= 8 ? pick<4, 512>(bnd, fs) : pick<4, 768>(bnd, fs);
 }
-constexpr size_t kSmem = (size_t)NFIELD * FCAP * sizeof(float);
+constexpr size_t smem_bytes(int lz, bool adj) { return (size_t)(NFIELD + (adj ? 3 : 0)) * fcap(lz) * sizeof(float); }
+// Reverse sweep: blocks of at most 8 planes, no C-PML, no free surface.
+Kern adjoint_kernel(int bnd, int lz) {
+    if (lz > 8 || bnd == BND_CPML) return nullptr;
+    if (lz <= 4)
+        return bnd == BND_SPONGE ? k_resident<BND_SPONGE, 0, 1, 1024, true> : k_resident<BND_NONE, 0, 1, 1024, true>;
+    return bnd == BND_SPONGE ? k_resident<BND_SPONGE, 0, 4, 512, true> : k_resident<BND_NONE, 0, 4, 512, true>;
+}
 
 }  // namespace
 
@@ -645,30 +783,31 @@ void resident_taps(const ResidentPlan& p, const DevGrid& g, const Tap* taps, int
         const int c = cta[t];
         const int x = q.i - block_lo(g.nx, p.nbx, c % p.nbx), y = q.j - block_lo(g.ny, p.nby, (c / p.nbx) % p.nby),
                   z = q.k - block_lo(g.nz, p.nbz, c / (p.nbx * p.nby));
-        (*list)[at[c]++] = make_int2(q.q * FCAP + (z + 2) * SP + (y + 2) * SX + x + 2, t);
+        (*list)[at[c]++] = make_int2(q.q * fcap(p.lz) + (z + 2) * SP + (y + 2) * SX + x + 2, t);
     }
 }
 
 cudaError_t resident_prepare(const ResidentPlan& p, int bnd) {
-    int occ = 0;
-    for (int fs = 0; fs < 2; ++fs) {
-        const Kern k = kernel_for(bnd, fs != 0, p.lz);
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
-        const int nt = block_threads(p.lz);
-        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, nt, kSmem);
+    const Kern ks[3] = {kernel_for(bnd, false, p.lz), kernel_for(bnd, true, p.lz), adjoint_kernel(bnd, p.lz)};
+    for (int v = 0; v < 3; ++v) {
+        if (!ks[v]) continue;
+        const size_t smem = smem_bytes(p.lz, v == 2);
+        int occ = 0;
+        cudaError_t e = cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e == cudaSuccess)
+            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, ks[v], block_threads(p.lz), smem);
         if (e != cudaSuccess) return e;
         if (occ < 1) return cudaErrorInvalidConfiguration;
     }
     return cudaSuccess;
 }
 
-// Measured (GB300, us per step, without / with C-PML), against the replayed
-// graph of the passes: 32^3 4.6 / 5.8 (10.0 / 15.4), 70 x 45 x 37 4.8 / 10.7
-// (11.9 / 18.3), 64^3 5.9 / 10.8 (11.9 / 17.8), 80 x 80 x 70 7.9 (17.9).  Of
-// the 2 us a phase takes at 32^3, most is the exchange (store to another SM's
-// poll) and the two barriers around it; at 64^3 the shared-memory loads of the
-// update (29 to 38 words a cell) take half.
-cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st) {
+bool resident_adjoint_supported(const ResidentPlan& p, const DevGrid& g, int bnd) {
+    return adjoint_kernel(bnd, p.lz) != nullptr && g.fs == kNoSurface && !g.cm[0];
+}
+
+namespace {
+ResParams res_params(const ResidentRun& r) {
     const ResidentPlan& p = *r.plan;
     ResParams P{};
     P.g = r.g;
@@ -676,8 +815,7 @@ cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st) {
     P.M = r.M;
     P.B = r.B;
     P.dt = r.dt;
-    P.S = *r.S;
-    P.wavelet = r.wavelet;
+    P.S.kind = -1;
     P.n0 = r.n0;
     P.nsteps = r.nsteps;
     P.inbox = r.inbox;
@@ -691,15 +829,49 @@ cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st) {
     P.nbz = p.nbz;
     P.tlist = r.tlist;
     P.tstart = r.tstart;
-    P.stage = r.seis ? r.stage : nullptr;
     P.ntap = 24 * r.nrec;
-    P.vcap = r.vcap;
     P.fstride = r.fstride;
     P.wait_ns = 2000000000ull;                       // 2 s per wait
+    return P;
+}
+}  // namespace
+
+// Reverse steps n0 + nsteps - 1 .. n0 of one resident history range.
+cudaError_t launch_resident_adjoint(const ResidentRun& r, const ResidentAdjoint& a, cudaStream_t st) {
+    const ResidentPlan& p = *r.plan;
+    ResParams P = res_params(r);
+    P.vhist = a.vhist;
+    P.h0 = a.h0;
+    P.vnext = a.vnext;
+    P.flush = a.flush;
+    P.A = a.A;
+    P.gdt = a.gdt;
+    P.sadj = r.nrec > 0 ? a.sadj : nullptr;
+    P.ld = r.ld;
+    P.taps = r.taps;
+    P.coef = r.stage;
+    void* args[] = {&P};
+    return cudaLaunchCooperativeKernel((const void*)adjoint_kernel(r.B.kind, p.lz), dim3(p.nbx * p.nby * p.nbz),
+                                       dim3(block_threads(p.lz)), args, smem_bytes(p.lz, true), st);
+}
+
+// Measured (GB300, us per step, without / with C-PML), against the replayed
+// graph of the passes: 32^3 4.6 / 5.8 (10.0 / 15.4), 70 x 45 x 37 4.8 / 10.7
+// (11.9 / 18.3), 64^3 5.9 / 10.8 (11.9 / 17.8), 80 x 80 x 70 7.9 (17.9).  Of
+// the 2 us a phase takes at 32^3, most is the exchange (store to another SM's
+// poll) and the two barriers around it; at 64^3 the shared-memory loads of the
+// update (29 to 38 words a cell) take half.
+cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st) {
+    const ResidentPlan& p = *r.plan;
+    ResParams P = res_params(r);
+    P.S = *r.S;
+    P.wavelet = r.wavelet;
+    P.stage = r.seis ? r.stage : nullptr;
+    P.vcap = r.vcap;
     const Kern k = kernel_for(r.B.kind, r.g.fs != kNoSurface, p.lz);
     const dim3 grid(p.nbx * p.nby * p.nbz), blk(block_threads(p.lz));
     void* args[] = {&P};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k, grid, blk, args, kSmem, st);
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k, grid, blk, args, smem_bytes(p.lz, false), st);
     if (e != cudaSuccess || !P.stage) return e;
     const int rows = 3 * r.nrec;
     const long long n = (long long)rows * r.nsteps;

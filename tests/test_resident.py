@@ -86,3 +86,28 @@ def test_chunks_and_staged_receivers(ews):
     for n0, k in ((0, 1), (1, 32), (33, 37)):
         sim.advance(n0, k, p.dt, seis, p.nt)
     assert np.array_equal(seis, a[0]) and np.array_equal(sim.get_state(), a[1])
+
+
+# blocks of at most 4 planes (a thread per cell), of 5 to 8 (4 cells per thread)
+@pytest.mark.parametrize("n", [(12, 11, 10), (33, 18, 17), (16, 47, 33), (64, 60, 61)])
+@pytest.mark.parametrize("boundary", ["none", "sponge"])
+@pytest.mark.parametrize("budget", [-1, 0])
+def test_gradient_equals_the_passes(ews, n, boundary, budget):
+    """The reverse sweep in one launch against the reverse passes: the same
+    products, summed by kernels compiled apart (a few roundings of 6e-8 per
+    step over 45 steps), and residual taps that share cells in either order:
+    1e-5.  History resident (one launch, flushed every 20 steps) and
+    recomputed (one launch per segment)."""
+    p = synth.small_problem(*n, nt=45, boundary=boundary, kind="moment", width=2, seed=307, nrec=40)
+    obs = np.random.default_rng(5).standard_normal((3, 40, p.nt)).astype(np.float32) * 1e-9
+    got = []
+    for shape in ("auto", "32x8"):
+        sim = ews.simulation_for(p)
+        sim.set_tile_shape(shape)
+        sim.set_history_budget(budget)
+        got.append(sim.gradient(p.nt, p.dt, obs, ckpt_every=20))
+    assert got[0][0] == pytest.approx(got[1][0], rel=1e-6)
+    for q in range(3):
+        a, b = got[0][1][q].astype(np.float64), got[1][1][q].astype(np.float64)
+        assert np.linalg.norm(b) > 0
+        assert np.linalg.norm(a - b) <= 1e-5 * np.linalg.norm(b), q
