@@ -436,21 +436,45 @@ static_assert(fslot(SZZ) == 5 && fslot(VX) == 6 && fslot(VY) == 7 &&
 
 // Coarse medium grid: bilinear samples of the medium grid (at the thread's
 // x-y positions) on the two medium planes around the current output plane,
-// for the quantities sampled at integer z (zi) and at half-integer z (zh);
-// refreshed when the output plane crosses a medium plane, so each plane
-// costs one z-interpolation per quantity.
+// for the quantities sampled at integer z (ci) and at half-integer z (ch).
+// Each set is refreshed on its own, when the output plane's sample point
+// crosses a medium plane; its upper samples then become the lower ones, so a
+// crossing samples one medium plane.
 template <int NQ>
 struct CoarseZ {
     float lo[ROWS][NQ], hi[ROWS][NQ];
-    int lvl;
+    int lvl[ROWS];
+    // f(dst, z): the NQ samples on medium plane z; up: 1, or 0 on a one-plane grid
+    template <typename Fn>
+    __device__ __forceinline__ void refresh(int rr, int z, Fn f, int up) {
+        if (lvl[rr] >= 0 && z == lvl[rr] + 1) {
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) lo[rr][q] = hi[rr][q];
+        } else {
+            f(lo[rr], z);
+        }
+        f(hi[rr], z + up);
+        lvl[rr] = z;
+    }
 };
-// Bilinear sample of medium array q on medium plane lvl.
-__device__ __forceinline__ float coarse_bilin(const DevGrid& g, int q, Ax x, Ax y, int lvl) {
-    const int ox = g.mx > 1 ? 1 : 0, oy = g.my > 1 ? g.mx : 0;
-    const float* p = g.cm[q] + ((long long)lvl * g.my + y.i0) * g.mx + x.i0;
-    return lerp1(lerp1(__ldg(p), __ldg(p + ox), x.f), lerp1(__ldg(p + oy), __ldg(p + oy + ox), x.f),
-                 y.f);
-}
+// Bilinear sampling at one x-y position.
+struct CoarseXY {
+    int o, ox, oy;
+    float fx, fy;
+    __device__ __forceinline__ CoarseXY(const DevGrid& g, float x, float y) {
+        const Ax ax = axis_at(x, g.rx, g.mx), ay = axis_at(y, g.ry, g.my);
+        ox = g.mx > 1 ? 1 : 0;
+        oy = g.my > 1 ? g.mx : 0;
+        o = ay.i0 * g.mx + ax.i0;
+        fx = ax.f;
+        fy = ay.f;
+    }
+    // medium array q on medium plane z
+    __device__ __forceinline__ float at(const DevGrid& g, int q, int z) const {
+        const float* p = g.cm[q] + ((long long)z * g.my * g.mx + o);
+        return lerp1(lerp1(__ldg(p), __ldg(p + ox), fx), lerp1(__ldg(p + oy), __ldg(p + oy + ox), fx), fy);
+    }
+};
 
 struct VelQ {
     float zz[ROWS][4], xz[ROWS][4], yz[ROWS][4];   // sigma_zz k-1..k+2, sigma_xz/yz k-2..k+1
@@ -619,20 +643,17 @@ __device__ __forceinline__ bool vel_step(const Maps& maps, const PassParams& P,
                 // coarse medium: 1 / rho sampled at each v point
                 const Ax zk = axis_at((float)k, g.rz, g.mz), zh = axis_at(k + 0.5f, g.rz, g.mz);
                 const int up = g.mz > 1 ? 1 : 0;
-                if (zk.i0 != Q.ci.lvl || zh.i0 != Q.ch.lvl) {   // uniform across the CTA
+                if (zk.i0 != Q.ci.lvl[rr]) {     // uniform across the CTA
                     const float fi = (float)G.i, fj = (float)(G.j0 + rr);
-                    const Ax xi = axis_at(fi, g.rx, g.mx), xh = axis_at(fi + 0.5f, g.rx, g.mx);
-                    const Ax yj = axis_at(fj, g.ry, g.my), yh = axis_at(fj + 0.5f, g.ry, g.my);
-                    Q.ci.lo[rr][0] = coarse_bilin(g, 2, xh, yj, zk.i0);
-                    Q.ci.hi[rr][0] = coarse_bilin(g, 2, xh, yj, zk.i0 + up);
-                    Q.ci.lo[rr][1] = coarse_bilin(g, 2, xi, yh, zk.i0);
-                    Q.ci.hi[rr][1] = coarse_bilin(g, 2, xi, yh, zk.i0 + up);
-                    Q.ch.lo[rr][0] = coarse_bilin(g, 2, xi, yj, zh.i0);
-                    Q.ch.hi[rr][0] = coarse_bilin(g, 2, xi, yj, zh.i0 + up);
-                    if (rr == ROWS - 1) {
-                        Q.ci.lvl = zk.i0;
-                        Q.ch.lvl = zh.i0;
-                    }
+                    const CoarseXY p(g, fi + 0.5f, fj), q(g, fi, fj + 0.5f);
+                    Q.ci.refresh(rr, zk.i0, [&](float* f, int z) {
+                        f[0] = p.at(g, 2, z);
+                        f[1] = q.at(g, 2, z);
+                    }, up);
+                }
+                if (zh.i0 != Q.ch.lvl[rr]) {
+                    const CoarseXY p(g, (float)G.i, (float)(G.j0 + rr));
+                    Q.ch.refresh(rr, zh.i0, [&](float* f, int z) { f[0] = p.at(g, 2, z); }, up);
                 }
                 bx = __fdividef(1.0f, lerp1(Q.ci.lo[rr][0], Q.ci.hi[rr][0], zk.f));
                 by = __fdividef(1.0f, lerp1(Q.ci.lo[rr][1], Q.ci.hi[rr][1], zk.f));
@@ -695,9 +716,9 @@ __device__ __forceinline__ bool vel_tile(const Maps& maps, const PassParams& P, 
         for (int q = 0; q < 4; ++q) {
             Q.zz[rr][q] = 0.f; Q.xz[rr][q] = 0.f; Q.yz[rr][q] = 0.f;
             Q.hx[rr][q] = 0.f; Q.hy[rr][q] = 0.f; Q.hz[rr][q] = 0.f;
-    Q.ci.lvl = -1;
-    Q.ch.lvl = -1;
         }
+#pragma unroll
+    for (int rr = 0; rr < ROWS; ++rr) Q.ci.lvl[rr] = Q.ch.lvl[rr] = -1;
     bool ovf = false;                              // an FP16 value out of range
     for (int m = 0; m < G.P4; m += 4) {
         if (!vel_step<BND, T, MODE, 0, FS, RS>(maps, P, G, Q, sm, bars, m, psi_pend, psi_par, ovf)) return false;
@@ -852,24 +873,22 @@ __device__ __forceinline__ bool str_step(const Maps& maps, const PassParams& P,
                 // coarse medium: lambda, mu at the cell, mu at each shear point
                 const Ax zk = axis_at((float)k, g.rz, g.mz), zh = axis_at(k + 0.5f, g.rz, g.mz);
                 const int up = g.mz > 1 ? 1 : 0;
-                if (zk.i0 != Q.ci.lvl || zh.i0 != Q.ch.lvl) {   // uniform across the CTA
+                if (zk.i0 != Q.ci.lvl[rr]) {     // uniform across the CTA
                     const float fi = (float)G.i, fj = (float)(G.j0 + rr);
-                    const Ax xi = axis_at(fi, g.rx, g.mx), xh = axis_at(fi + 0.5f, g.rx, g.mx);
-                    const Ax yj = axis_at(fj, g.ry, g.my), yh = axis_at(fj + 0.5f, g.ry, g.my);
-                    Q.ci.lo[rr][0] = coarse_bilin(g, 0, xi, yj, zk.i0);
-                    Q.ci.hi[rr][0] = coarse_bilin(g, 0, xi, yj, zk.i0 + up);
-                    Q.ci.lo[rr][1] = coarse_bilin(g, 1, xi, yj, zk.i0);
-                    Q.ci.hi[rr][1] = coarse_bilin(g, 1, xi, yj, zk.i0 + up);
-                    Q.ci.lo[rr][2] = coarse_bilin(g, 1, xh, yh, zk.i0);
-                    Q.ci.hi[rr][2] = coarse_bilin(g, 1, xh, yh, zk.i0 + up);
-                    Q.ch.lo[rr][0] = coarse_bilin(g, 1, xh, yj, zh.i0);
-                    Q.ch.hi[rr][0] = coarse_bilin(g, 1, xh, yj, zh.i0 + up);
-                    Q.ch.lo[rr][1] = coarse_bilin(g, 1, xi, yh, zh.i0);
-                    Q.ch.hi[rr][1] = coarse_bilin(g, 1, xi, yh, zh.i0 + up);
-                    if (rr == ROWS - 1) {
-                        Q.ci.lvl = zk.i0;
-                        Q.ch.lvl = zh.i0;
-                    }
+                    const CoarseXY p(g, fi, fj), q(g, fi + 0.5f, fj + 0.5f);
+                    Q.ci.refresh(rr, zk.i0, [&](float* f, int z) {
+                        f[0] = p.at(g, 0, z);
+                        f[1] = p.at(g, 1, z);
+                        f[2] = q.at(g, 1, z);
+                    }, up);
+                }
+                if (zh.i0 != Q.ch.lvl[rr]) {
+                    const float fi = (float)G.i, fj = (float)(G.j0 + rr);
+                    const CoarseXY p(g, fi + 0.5f, fj), q(g, fi, fj + 0.5f);
+                    Q.ch.refresh(rr, zh.i0, [&](float* f, int z) {
+                        f[0] = p.at(g, 1, z);
+                        f[1] = q.at(g, 1, z);
+                    }, up);
                 }
                 lam = lerp1(Q.ci.lo[rr][0], Q.ci.hi[rr][0], zk.f);
                 mu0 = lerp1(Q.ci.lo[rr][1], Q.ci.hi[rr][1], zk.f);
@@ -941,8 +960,8 @@ __device__ __forceinline__ bool str_tile(const Maps& maps, const PassParams& P, 
     for (int rr = 0; rr < ROWS; ++rr)
 #pragma unroll
         for (int q = 0; q < 4; ++q) { Q.vx[rr][q] = 0.f; Q.vy[rr][q] = 0.f; Q.vz[rr][q] = 0.f; }
-    Q.ci.lvl = -1;
-    Q.ch.lvl = -1;
+#pragma unroll
+    for (int rr = 0; rr < ROWS; ++rr) Q.ci.lvl[rr] = Q.ch.lvl[rr] = -1;
     bool ovf = false;                              // an FP16 value out of range
     for (int m = 0; m < G.P4; m += 4) {
         if (!str_step<BND, T, 0, FS, RS>(maps, P, G, Q, sm, bars, m, psi_pend, psi_par, ovf)) return false;
