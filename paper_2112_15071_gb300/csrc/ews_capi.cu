@@ -83,10 +83,13 @@ bool fused_eligible(const ews_sim* s) {
     return true;
 }
 
-// Shape of the forward passes of a plain (vcap null) or capturing step.
+// Shape of the forward passes of a plain (vcap null) or capturing step.  A
+// capturing step takes the fused step where the simulation already holds its
+// second wavefield set (a gradient allocates none for it).
 int fwd_shape(const ews_sim* s, bool capture) {
-    if (capture || !tile_eligible(s)) return EWS_TILE_32X8;
+    if (!tile_eligible(s)) return EWS_TILE_32X8;
     if (s->tile_used == EWS_TILE_FUSED && !fused_eligible(s)) return EWS_TILE_32X8;
+    if (capture && !(s->tile_used == EWS_TILE_FUSED && s->tplan[EWS_TILE_FUSED])) return EWS_TILE_32X8;
     return s->tile_used;
 }
 
@@ -488,7 +491,7 @@ cudaError_t str_launch(ews_sim* s, int shape, const DevFields& F, const float dt
 // just written, as after the two passes.  An odd step count ends with the
 // state copied back into the simulation's own set.
 ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
-                       float* dseis, int ld) {
+                       float* dseis, int ld, float* vcap) {
     const fused::FusedPlan* fp = static_cast<const fused::FusedPlan*>(s->tplan[EWS_TILE_FUSED]);
     DevMedium M = s->M();
     const DevSource S = source_taps(s, src, dt);
@@ -505,7 +508,9 @@ ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, do
     for (int n = n0; n < n0 + nsteps; ++n) {
         const int dir = (n - n0) & 1;
         const DevFields& out = set[dir ^ 1];
-        CK(fused::launch_fused(fp, dir, s->g, M, s->B, dto, inv, S, s->wavelet, n, s->err, s->stream));
+        float* slot = vcap ? vcap + (size_t)(n - n0 + 1) * 3 * s->fstride : nullptr;
+        CK(fused::launch_fused(fp, dir, s->g, M, s->B, dto, inv, S, s->wavelet, n, slot,
+                               (long long)s->fstride, s->err, s->stream));
         if ((st = mark(s, EWS_KERNEL_STEP)) != EWS_OK) return st;
         const bool rec = s->nrec > 0 && dseis;
         if (S.kind == EWS_SOURCE_MOMENT && rec) {
@@ -535,7 +540,7 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
     const int shape = fwd_shape(s, vcap != nullptr);
     ews_status st0 = tile_plan(s, shape);
     if (st0 != EWS_OK) return st0;
-    if (shape == EWS_TILE_FUSED) return steps_fused(s, src, n0, nsteps, dt, dseis, ld);
+    if (shape == EWS_TILE_FUSED) return steps_fused(s, src, n0, nsteps, dt, dseis, ld, vcap);
     DevFields F = s->F();
     DevMedium M = s->M();
     const DevSource S = source_taps(s, src, dt);

@@ -189,6 +189,8 @@ struct FusedParams {
     const float* wavelet;
     int n;
     int sk0, sk1;               // planes of the force taps
+    float* vcap;                // history slot of v^{n+1/2} (3 fields, hstride apart), FP32
+    long long hstride;
 };
 
 // First step with velocity, first that brings the medium of the stress (mu of
@@ -316,7 +318,8 @@ struct Turn {
 // 2: velocity, and the medium of plane z0, 3: velocity and stress.  ring:
 // offsets of the new-velocity planes k, k-1, k-2, k-3 (floats); ent: of the
 // medium entry of this step.
-template <int BND, typename T, int TY, int PH, int STAGE>
+// CAP: v^{n+1/2} also goes to its history slot.
+template <int BND, typename T, int TY, bool CAP, int PH, int STAGE>
 __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedParams& P,
                                            const FGeo<BND, T, TY>& G, FQ& Q, unsigned char* sm,
                                            uint64_t* bars, int m, const int (&ring)[4], const Turn& tn) {
@@ -399,6 +402,11 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
                 S::st((T*)P.fout.f[VX] + o, vx);
                 S::st((T*)P.fout.f[VY] + o, vy);
                 S::st((T*)P.fout.f[VZ] + o, vz);
+                if constexpr (CAP) {
+                    S2<float>::st(P.vcap + o, vx);
+                    S2<float>::st(P.vcap + P.hstride + o, vy);
+                    S2<float>::st(P.vcap + 2 * P.hstride + o, vz);
+                }
             }
             if (G.reg) {
                 float* vn = vring + ring[0] + G.row * VS + 2 * G.rp;
@@ -453,6 +461,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
                 if (k >= G.z0 && k < G.z1 && ex >= 2 && ex < 2 + TX && ey >= 2 && ey < 2 + TY) {
                     T* f = (T*)(tp.q == VX ? P.fout.f[VX] : tp.q == VY ? P.fout.f[VY] : P.fout.f[VZ]);
                     f[ops::cidx(g, tp.i, tp.j, tp.k)] = ops::Io<T>::put(x);
+                    if constexpr (CAP) P.vcap[(tp.q - VX) * P.hstride + ops::cidx(g, tp.i, tp.j, tp.k)] = x;
                 }
             }
         }
@@ -531,7 +540,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     }
 }
 
-template <int BND, typename T, int TY>
+template <int BND, typename T, int TY, bool CAP>
 __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constant__ FusedMaps maps,
                                                            const __grid_constant__ FusedParams P) {
     using L = FL<T, TY>;
@@ -563,27 +572,27 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
         ring[0] = nw;
         tn.next(L::ENT);
     };
-    fused_step<BND, T, TY, 0, 0>(maps, P, G, Q, sm, bars, 0, ring, tn); next();
-    fused_step<BND, T, TY, 1, 0>(maps, P, G, Q, sm, bars, 1, ring, tn); next();
-    fused_step<BND, T, TY, 2, 0>(maps, P, G, Q, sm, bars, 2, ring, tn); next();
-    fused_step<BND, T, TY, 3, 1>(maps, P, G, Q, sm, bars, 3, ring, tn); next();
-    fused_step<BND, T, TY, 0, 1>(maps, P, G, Q, sm, bars, 4, ring, tn); next();
-    fused_step<BND, T, TY, 1, 1>(maps, P, G, Q, sm, bars, 5, ring, tn); next();
-    fused_step<BND, T, TY, 2, 2>(maps, P, G, Q, sm, bars, 6, ring, tn); next();
-    fused_step<BND, T, TY, 3, 3>(maps, P, G, Q, sm, bars, 7, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 0, 0>(maps, P, G, Q, sm, bars, 0, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 1, 0>(maps, P, G, Q, sm, bars, 1, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 2, 0>(maps, P, G, Q, sm, bars, 2, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 3, 1>(maps, P, G, Q, sm, bars, 3, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 0, 1>(maps, P, G, Q, sm, bars, 4, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 1, 1>(maps, P, G, Q, sm, bars, 5, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 2, 2>(maps, P, G, Q, sm, bars, 6, ring, tn); next();
+    fused_step<BND, T, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, 7, ring, tn); next();
     int m = M_STR + 1;
     bool stop = __syncthreads_or(Q.bad);
     while (m < G.M && !stop) {
-        fused_step<BND, T, TY, 0, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+        fused_step<BND, T, TY, CAP, 0, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
         next();
         if (++m < G.M) {
-            fused_step<BND, T, TY, 1, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+            fused_step<BND, T, TY, CAP, 1, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
             next();
             if (++m < G.M) {
-                fused_step<BND, T, TY, 2, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                fused_step<BND, T, TY, CAP, 2, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
                 next();
                 if (++m < G.M) {
-                    fused_step<BND, T, TY, 3, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                    fused_step<BND, T, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
                     next();
                     ++m;
                 }
@@ -630,6 +639,7 @@ struct FusedPlan {
     int kind = 0;
     int ty = 0, nt = 0, smem = 0;
     void (*kern)(FusedMaps, FusedParams) = nullptr;
+    void (*kern_cap)(FusedMaps, FusedParams) = nullptr;   // also capturing the history
     int ntx = 0, nty = 0, zchunk = 0, grid = 0;
 };
 
@@ -639,7 +649,8 @@ cudaError_t plan_for(FusedPlan* p, const DevGrid& g, const DevFields& A, const D
                      const DevBoundary& B) {
     using L = FL<T, TY>;
     static_assert(L::SMEM <= 227 * 1024, "one CTA's shared memory");
-    p->kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY> : k_fused<BND_NONE, T, TY>;
+    p->kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY, false> : k_fused<BND_NONE, T, TY, false>;
+    p->kern_cap = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY, true> : k_fused<BND_NONE, T, TY, true>;
     p->ty = TY;
     p->nt = L::NT;
     p->smem = L::SMEM;
@@ -665,6 +676,7 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(p->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(p->kern_cap, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem);
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, p->kern, p->nt, p->smem);
     if (e == cudaSuccess && occ < 1) e = cudaErrorInvalidConfiguration;
     if (e != cudaSuccess) {
@@ -685,7 +697,7 @@ void fused_plan_destroy(FusedPlan* p) { delete p; }
 
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
                          const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
-                         const float* wavelet, int n, int* err, cudaStream_t st) {
+                         const float* wavelet, int n, float* vcap, long long hstride, int* err, cudaStream_t st) {
     FusedParams P{};
     P.g = g;
     P.fout = p->f[dir ^ 1];
@@ -714,7 +726,9 @@ cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const De
             P.sk1 = std::max(P.sk1, S.tap[t].k);
         }
     }
-    p->kern<<<p->grid, p->nt, p->smem, st>>>(p->dir[dir], P);
+    P.vcap = vcap;
+    P.hstride = hstride;
+    (vcap ? p->kern_cap : p->kern)<<<p->grid, p->nt, p->smem, st>>>(p->dir[dir], P);
     return cudaGetLastError();
 }
 

@@ -441,7 +441,8 @@ EWS_SHAPE_DECLS(t32x16)
 // One launch per time step (ews_fused.cu): the velocity and stress passes of
 // step n fused, reading sigma^n, v^{n-1/2} from one set of wavefields and
 // writing v^{n+1/2}, sigma^{n+1} to a second set (dir 0: A -> B, dir 1:
-// B -> A), with a point force of step n (S.kind 1) added inside.  FP32
+// B -> A), with a point force of step n (S.kind 1) added inside; with vcap,
+// v^{n+1/2} also into that history slot (3 fields hstride apart).  FP32
 // storage with unit scales, sponge or no absorbing boundary, no free surface
 // or coarse medium grid.
 namespace fused {
@@ -452,7 +453,8 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
 void fused_plan_destroy(FusedPlan* p);
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
                          const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
-                         const float* wavelet, int n, int* err, cudaStream_t st);
+                         const float* wavelet, int n, float* vcap, long long hstride, int* err,
+                         cudaStream_t st);
 }  // namespace fused
 
 // The time loop of a small grid in one cooperative launch with the fields

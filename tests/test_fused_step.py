@@ -201,3 +201,26 @@ def test_tuner_keeps_the_second_set_only_when_it_picks_fused(ews):
     sim = ews.simulation_for(p)
     assert rel(sim.run(p.nt, p.dt), want) <= TOL_SHAPE
     assert sim.tile_shape == "fused"
+
+
+@pytest.mark.parametrize("boundary", ["none", "sponge"])
+@pytest.mark.parametrize("kind", ["moment", "force"])
+@pytest.mark.parametrize("budget", [-1, 0])
+def test_fused_step_captures_the_history(ews, boundary, kind, budget):
+    """A simulation that holds the second wavefield set captures the velocity
+    history with the fused step: its gradient equals that of the two passes
+    (equal bits in the history; residual taps that share cells add in either
+    order: 1e-6), with the history resident and recomputed in segments of an
+    odd length."""
+    p = synth.small_problem(70, 45, 37, nt=45, boundary=boundary, kind=kind, width=6, seed=210)
+    obs = np.random.default_rng(7).standard_normal((3, p.rec_pos.shape[0], p.nt)).astype(np.float32) * 1e-9
+    got = []
+    for shape in ("fused", "32x8"):
+        sim = ews.simulation_for(p)
+        sim.set_tile_shape(shape)
+        sim.set_history_budget(budget)
+        sim.run(p.nt, p.dt)
+        got.append(sim.gradient(p.nt, p.dt, obs, ckpt_every=15))
+    assert got[0][0] == pytest.approx(got[1][0], rel=1e-6)
+    for q in range(3):
+        assert rel(got[0][1][q], got[1][1][q]) <= TOL_SHAPE, q
