@@ -42,10 +42,11 @@ constexpr int MX = 16, MY = 16;                  // largest block in x and y
 constexpr int SX = MX + 4, SP = SX * (MY + 4);   // shared-memory strides (row, plane)
 constexpr int MAXZ = 12;                         // largest block in z
 // Elements of one field in shared memory, by the planes of a block (the
-// 768-thread kernels serve blocks of 9 to 12 planes).
-constexpr int fcap(int lz) { return SP * (lz <= 8 ? 12 : MAXZ + 4); }
+// 1024-thread kernels serve blocks of at most 4, the 512-thread ones of 5 to 8
+// and the 768-thread ones of 9 to 12 planes).
+constexpr int fcap(int lz) { return SP * (lz <= 4 ? 8 : lz <= 8 ? 12 : MAXZ + 4); }
 constexpr int COLS = MX * MY;                    // threads of one z-group
-static_assert(NFIELD * fcap(MAXZ) * 4 + 1024 <= 227 * 1024 && (NFIELD + 3) * fcap(8) * 4 + 1024 <= 227 * 1024,
+static_assert(NFIELD * fcap(MAXZ) * 4 + 1024 <= 227 * 1024 && (NFIELD * fcap(4) + 18 * 1024) * 4 + 1024 <= 227 * 1024 && (NFIELD + 3) * fcap(8) * 4 + 1024 <= 227 * 1024,
               "fields (and the history's, reverse) fit one CTA's shared memory");
 
 struct ResParams {
@@ -225,7 +226,10 @@ __device__ __forceinline__ void halo_send(const HaloLine& h, const ResParams& P,
 // as three more shared fields, and the residual is injected after it.
 template <int BND, int FS, int CPT, int MAXT, bool ADJ = false>
 __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ ResParams P) {
-    constexpr int FCAP = fcap(MAXT == 768 ? MAXZ : 8);
+    constexpr int FCAP = fcap(MAXT == 768 ? MAXZ : MAXT == 512 ? 8 : 4);
+    // With a cell per thread the C-PML memory variables of the block fit shared
+    // memory too (18 rows of MAXT); larger blocks keep them in global memory.
+    constexpr bool PSM = BND == BND_CPML && CPT == 1;
     constexpr int H0 = NFIELD;                   // first history field
     extern __shared__ __align__(16) float sm[];
     __shared__ float s_amp[kMaxSrcTaps][2];      // buoyancy, gain of the block's source taps
@@ -297,6 +301,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
     const float* paz = P.B.pa[2] + gk;
     const float* pbz = P.B.pb[2] + gk;
     auto psz = [&](int c) { return BND == BND_CPML && (gk + c < W || gk + c >= g.nz - W); };
+    float* const ps = sm + NFIELD * FCAP + t;    // PSM: variable q of the thread's cell at ps[q * MAXT]
+    if (PSM && nc > 0) {
+#pragma unroll
+        for (int q = 0; q < 18; ++q)
+            if (q < 6 ? psx : q < 12 ? psy : psz(0)) ps[q * MAXT] = P.B.psi[q][go];
+    }
     // the thread's halo line
     HaloLine h;
     h.axis = -1;
@@ -388,6 +398,20 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
         }
     };
 
+    // memory variables q0 .. q0 + 2 of one cell: from and to shared memory, or
+    // (already fetched) to global memory
+    auto psi_get = [&](float* p, int q0) {
+        if (PSM)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) p[q] = ps[(q0 + q) * MAXT];
+    };
+    auto psi_put = [&](const float* p, int q0, int o) {
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            if (PSM) ps[(q0 + q) * MAXT] = p[q];
+            else P.B.psi[q0 + q][o] = p[q];
+    };
+
     float* vcap = P.vcap;
     for (int m = 0; m < P.nsteps; ++m) {
         const int n = ADJ ? P.n0 + P.nsteps - 1 - m : P.n0 + m;
@@ -396,7 +420,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
         asm volatile("" : "+r"(h.in), "+r"(h.lo), "+r"(h.hi), "+r"(h.so), "+r"(h.axis));
         // ---- velocity phase ----
         float px[CPT][3], py[CPT][3], pz[CPT][3];
-        if (BND == BND_CPML) {                   // memory variables, fetched before the wait
+        if (BND == BND_CPML && !PSM) {           // memory variables, fetched before the wait
 #pragma unroll
             for (int c = 0; c < CPT; ++c)
                 if (c < nc) {
@@ -482,17 +506,20 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
                 if (BND == BND_CPML && c < nc) {
                     const int o = go + c * plane;
                     if (psx) {
+                        psi_get(px[c], 0);
                         ar::pml(px[c][0], pax, pbx, dxx); ar::pml(px[c][1], pax, pbx, dyx); ar::pml(px[c][2], pax, pbx, dzx);
-                        P.B.psi[0][o] = px[c][0]; P.B.psi[1][o] = px[c][1]; P.B.psi[2][o] = px[c][2];
+                        psi_put(px[c], 0, o);
                     }
                     if (psy) {
+                        psi_get(py[c], 6);
                         ar::pml(py[c][0], pay, pby, dxy); ar::pml(py[c][1], pay, pby, dyy); ar::pml(py[c][2], pay, pby, dzy);
-                        P.B.psi[6][o] = py[c][0]; P.B.psi[7][o] = py[c][1]; P.B.psi[8][o] = py[c][2];
+                        psi_put(py[c], 6, o);
                     }
                     if (psz(c)) {
+                        psi_get(pz[c], 12);
                         const float a = __ldg(paz + c), b = __ldg(pbz + c);
                         ar::pml(pz[c][0], a, b, dxz); ar::pml(pz[c][1], a, b, dyz); ar::pml(pz[c][2], a, b, dzz);
-                        P.B.psi[12][o] = pz[c][0]; P.B.psi[13][o] = pz[c][1]; P.B.psi[14][o] = pz[c][2];
+                        psi_put(pz[c], 12, o);
                     }
                 }
                 if constexpr (ADJ) {
@@ -563,7 +590,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
             }
         // ---- stress phase ----
         asm volatile("" : "+r"(h.in), "+r"(h.lo), "+r"(h.hi), "+r"(h.so), "+r"(h.axis));
-        if (BND == BND_CPML) {
+        if (BND == BND_CPML && !PSM) {
 #pragma unroll
             for (int c = 0; c < CPT; ++c)
                 if (c < nc) {
@@ -607,17 +634,20 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
                 if (BND == BND_CPML && c < nc) {
                     const int o = go + c * plane;
                     if (psx) {
+                        psi_get(px[c], 3);
                         ar::pml(px[c][0], pax, pbx, exx); ar::pml(px[c][1], pax, pbx, vyx); ar::pml(px[c][2], pax, pbx, vzx);
-                        P.B.psi[3][o] = px[c][0]; P.B.psi[4][o] = px[c][1]; P.B.psi[5][o] = px[c][2];
+                        psi_put(px[c], 3, o);
                     }
                     if (psy) {
+                        psi_get(py[c], 9);
                         ar::pml(py[c][0], pay, pby, eyy); ar::pml(py[c][1], pay, pby, vxy); ar::pml(py[c][2], pay, pby, vzy);
-                        P.B.psi[9][o] = py[c][0]; P.B.psi[10][o] = py[c][1]; P.B.psi[11][o] = py[c][2];
+                        psi_put(py[c], 9, o);
                     }
                     if (psz(c)) {
+                        psi_get(pz[c], 15);
                         const float a = __ldg(paz + c), b = __ldg(pbz + c);
                         ar::pml(pz[c][0], a, b, ezz); ar::pml(pz[c][1], a, b, vxz); ar::pml(pz[c][2], a, b, vyz);
-                        P.B.psi[15][o] = pz[c][0]; P.B.psi[16][o] = pz[c][1]; P.B.psi[17][o] = pz[c][2];
+                        psi_put(pz[c], 15, o);
                     }
                 }
                 const float l2m = ar::l2m(ml[c], mm[c]);
@@ -667,6 +697,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
         if (c < nc)
 #pragma unroll
             for (int q = 0; q < NFIELD; ++q) P.F.f[q][go + c * plane] = sm[q * FCAP + so + c * SP];
+    if (PSM && nc > 0) {
+#pragma unroll
+        for (int q = 0; q < 18; ++q)
+            if (q < 6 ? psx : q < 12 ? psy : psz(0)) P.B.psi[q][go] = ps[q * MAXT];
+    }
 }
 
 // Receiver samples of the steps of a resident launch from the staged tap
@@ -712,7 +747,10 @@ int block_threads(int lz) {
 Kern kernel_for(int bnd, bool fs, int lz) {
     return lz <= 4 ? pick<1, 1024>(bnd, fs) : lz <= 8 ? pick<4, 512>(bnd, fs) : pick<4, 768>(bnd, fs);
 }
-constexpr size_t smem_bytes(int lz, bool adj) { return (size_t)(NFIELD + (adj ? 3 : 0)) * fcap(lz) * sizeof(float); }
+size_t smem_bytes(int bnd, int lz, bool adj) {
+    const size_t f = (size_t)(NFIELD + (adj ? 3 : 0)) * fcap(lz);
+    return (f + (bnd == BND_CPML && lz <= 4 ? 18 * 1024 : 0)) * sizeof(float);
+}
 // Reverse sweep: blocks of at most 8 planes, no C-PML, no free surface.
 Kern adjoint_kernel(int bnd, int lz) {
     if (lz > 8 || bnd == BND_CPML) return nullptr;
@@ -728,7 +766,9 @@ Kern adjoint_kernel(int bnd, int lz) {
 // half-warp covers one row of up to 16 cells whatever its length, a thread of
 // a block of more than 4 planes 4 of them; blocks of more than 8 planes need
 // 768 threads, whose 80 registers spill: 64^3 in blocks of 8 planes 5.9 us a
-// step, in blocks of 11 planes 7.7).
+// step, in blocks of 11 planes 7.7; with C-PML, blocks of more than 4 planes
+// leave the memory variables in global memory: 70 x 45 x 37 in blocks of 8
+// planes 9.9 us).
 bool resident_plan(const DevGrid& g, int bnd, int sms, ResidentPlan* out) {
     if ((long long)g.nx * g.ny * g.nz > (long long)sms * MX * MY * MAXZ) return false;
     const int maxz = bnd == BND_CPML ? 8 : MAXZ;     // registers of the memory variables
@@ -737,7 +777,7 @@ bool resident_plan(const DevGrid& g, int bnd, int sms, ResidentPlan* out) {
         for (int by = (g.ny + MY - 1) / MY; by <= std::max(1, g.ny / 2) && bx * by <= sms; ++by)
             for (int bz = (g.nz + maxz - 1) / maxz; bz <= std::max(1, g.nz / 2) && bx * by * bz <= sms; ++bz) {
                 const long long lx = (g.nx + bx - 1) / bx, ly = (g.ny + by - 1) / by, lz = (g.nz + bz - 1) / bz;
-                const long long cells = MX * ly * (lz <= 4 ? lz : lz <= 8 ? 8 : 16);
+                const long long cells = MX * ly * (lz <= 4 ? lz : lz <= 8 ? (bnd == BND_CPML ? 16 : 8) : 16);
                 const long long cost = cells + 3 * (ly * lz + lx * lz + lx * ly);
                 if (best < 0 || cost < best) {
                     best = cost;
@@ -791,7 +831,7 @@ cudaError_t resident_prepare(const ResidentPlan& p, int bnd) {
     const Kern ks[3] = {kernel_for(bnd, false, p.lz), kernel_for(bnd, true, p.lz), adjoint_kernel(bnd, p.lz)};
     for (int v = 0; v < 3; ++v) {
         if (!ks[v]) continue;
-        const size_t smem = smem_bytes(p.lz, v == 2);
+        const size_t smem = smem_bytes(bnd, p.lz, v == 2);
         int occ = 0;
         cudaError_t e = cudaFuncSetAttribute(ks[v], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e == cudaSuccess)
@@ -852,12 +892,12 @@ cudaError_t launch_resident_adjoint(const ResidentRun& r, const ResidentAdjoint&
     P.coef = r.stage;
     void* args[] = {&P};
     return cudaLaunchCooperativeKernel((const void*)adjoint_kernel(r.B.kind, p.lz), dim3(p.nbx * p.nby * p.nbz),
-                                       dim3(block_threads(p.lz)), args, smem_bytes(p.lz, true), st);
+                                       dim3(block_threads(p.lz)), args, smem_bytes(r.B.kind, p.lz, true), st);
 }
 
 // Measured (GB300, us per step, without / with C-PML), against the replayed
-// graph of the passes: 32^3 4.6 / 5.8 (10.0 / 15.4), 70 x 45 x 37 4.8 / 10.7
-// (11.9 / 18.3), 64^3 5.9 / 10.8 (11.9 / 17.8), 80 x 80 x 70 7.9 (17.9).  Of
+// graph of the passes: 32^3 4.6 / 4.7 (10.0 / 15.4), 70 x 45 x 37 4.8 / 6.1
+// (11.9 / 18.3), 64^3 5.8 / 10.0 (11.9 / 17.8), 80 x 80 x 70 7.8 (17.9).  Of
 // the 2 us a phase takes at 32^3, most is the exchange (store to another SM's
 // poll) and the two barriers around it; at 64^3 the shared-memory loads of the
 // update (29 to 38 words a cell) take half.
@@ -871,7 +911,7 @@ cudaError_t launch_resident(const ResidentRun& r, cudaStream_t st) {
     const Kern k = kernel_for(r.B.kind, r.g.fs != kNoSurface, p.lz);
     const dim3 grid(p.nbx * p.nby * p.nbz), blk(block_threads(p.lz));
     void* args[] = {&P};
-    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k, grid, blk, args, smem_bytes(p.lz, false), st);
+    cudaError_t e = cudaLaunchCooperativeKernel((const void*)k, grid, blk, args, smem_bytes(r.B.kind, p.lz, false), st);
     if (e != cudaSuccess || !P.stage) return e;
     const int rows = 3 * r.nrec;
     const long long n = (long long)rows * r.nsteps;
