@@ -19,17 +19,19 @@
 // 24 cells: its 504 threads (16 warps) may use 128 registers, which the
 // columns need, and the ring adds 31 % velocity work (32 x 8 tiles: 69 %).
 // Taller tiles leave 96 or 80 registers a thread and spill (32 x 28: 35
-// Gcell/s at 1024 x 1024 x 512), lower ones have fewer warps (32 x 20: 59.7,
-// 32 x 16: 56.0, with 3 slots 63.1).  Row-wise thread order keeps the
+// Gcell/s at 1024 x 1024 x 512), lower ones have fewer warps and more ring (32
+// x 20 with 3 slots 60.3, 32 x 16 with 3 slots 63.9 but 58.7 at 256^3).  Row-wise thread order keeps the
 // half-warps on 16 neighbouring pairs of one row (no bank conflicts) and the
 // stress threads in full warps; the ring's outer columns have threads of
 // their own.  Edge masks are selects, not branches: a branch around them for
 // interior tiles cut the schedule apart (55.0 against 61.3).
 //
 // Measured (GB300, FP32, sponge, Gcell/s, against the two passes): 1024 x
-// 1024 x 512 62.7 (50.5), 256^3 61.0 (51.3); 0.78 and 0.76 of the copy peak
-// on 84 bytes a cell.  291 warp instructions per 32 cells at 1.8 per cycle
-// and SM; stalls: shared-memory and barrier latency at 4 warps per scheduler.
+// 1024 x 512 63.4 (50.5), 256^3 61.7 (51.4), 224^3 58.4 (48.5), 192^3 60.2
+// (50.0 with 32 x 4 tiles); 0.79 and 0.76 of the copy peak on 84 bytes a cell
+// for the first two.  291 warp instructions per 32 cells at 1.8 per cycle and
+// SM; stalls: shared-memory, copy and arithmetic latency at 4 warps per
+// scheduler.
 //
 // Pipeline per CTA (tile x0, y0; z-chunk z0 .. z1), step m for velocity plane
 // k = z0 - 5 + m.  The copies of step m bring each field at the plane at which
@@ -65,6 +67,7 @@ constexpr int EXP = TX / 2 + 2;                  // pairs of a region row (x0-2 
 constexpr int VS = TX + 4;                       // row stride of the new-velocity ring
 constexpr int MBW = TX + 8;                      // FP32 medium boxes: x from x0-4
 constexpr int NV = 5;                            // planes of the new-velocity ring
+constexpr int kMaxChunk = 1024;                  // planes of a z-chunk (its sponge gains sit in shared memory)
 constexpr int NS = 2;                            // slots (one in use, the next in flight)
 constexpr int NE = NS + 1;                       // entries of the medium buffer (read a phase later)
 
@@ -169,7 +172,7 @@ struct FL {
     static constexpr int LB = TX * TY * 4, MUB = (TY + 1) * MBW * 4, ENT = r128(r128(LB) + MUB);
     static constexpr int VPL = 3 * EY * VS;                          // floats of one ring plane
     static constexpr int O_V = NS * SLOT, O_E = r128(O_V + NV * VPL * 4), O_BAR = O_E + NE * ENT;
-    static constexpr int SMEM = O_BAR + (NS + 2) * 8;
+    static constexpr int O_GZ = O_BAR + r128((NS + 2) * 8), SMEM = O_GZ + (kMaxChunk + 8) * 4;
 };
 
 struct FusedMaps {
@@ -235,7 +238,6 @@ struct FQ {
     f2 bx, by, r0;              // half buoyancies and density at plane k
     f2 vzc;                     // new vz at plane k - 4 (tile threads)
     f2 mu2, mxy, ma, mb;        // 2 mu, its xy sum, mu + mu(x+1), mu + mu(y+1) at plane k - 2
-    float gz[4];                // sponge gains of planes k + 1 (fetched ahead), k, k - 1, k - 2
     bool bad, ovf;
 };
 
@@ -333,17 +335,13 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     unsigned char* slot = sm + tn.s * L::SLOT;
     float* vring = reinterpret_cast<float*>(sm + L::O_V);
     const f2 c1x = dup(g.c1x), c2x = dup(g.c2x), c1y = dup(g.c1y), c2y = dup(g.c2y), c1z = dup(g.c1z), c2z = dup(g.c2z);
-    if (BND == BND_SPONGE) {
-        Q.gz[3] = Q.gz[2];
-        Q.gz[2] = Q.gz[1];
-        Q.gz[1] = Q.gz[0];
-        Q.gz[0] = __ldg(P.B.g[2] + min(max(k + 1, 0), g.nz - 1));
-    }
+    const float* gz = reinterpret_cast<const float*>(sm + L::O_GZ) + m;   // gains of planes z0 - 5 + m
     // this step's copies; and every warp past its velocity phase of step m - 2
     // (so past stress m - 3): the ring plane written below is free, the one
     // read by the stress is complete
-    Q.bad |= !mbar_wait(&bars[tn.s], tn.par);
-    if (STAGE > 0 || PH >= 2) Q.bad |= !mbar_wait(&bars[CB], (uint32_t)(((m - 2) >> 1) & 1));
+    // (after a wait that gave up the others are skipped, until the CTA leaves)
+    Q.bad = Q.bad || !mbar_wait(&bars[tn.s], tn.par);
+    if (STAGE > 0 || PH >= 2) Q.bad = Q.bad || !mbar_wait(&bars[CB], (uint32_t)(((m - 2) >> 1) & 1));
     // sigma^n of plane k - 2, about to leave the columns
     f2 s0, s1, s2, s3, s4, s5;
     s2 = Q.zz[D];
@@ -388,7 +386,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
             f2 vy = fma2(mul2(dup(P.dt2[kScaled<T> ? 1 : 0]), Q.by), add2(add2(dyx, dyy), dyz), S::ld(fv + L::RB / L::ES));
             f2 vz = fma2(mul2(dup(P.dt2[kScaled<T> ? 2 : 0]), bz), add2(Q.dz, dzz), S::ld(fv + 2 * (L::RB / L::ES)));
             if (BND == BND_SPONGE) {
-                const f2 gs = mul2(mul2(G.gx, dup(Q.gz[1])), dup(G.gy));
+                const f2 gs = mul2(mul2(G.gx, dup(gz[0])), dup(G.gy));
                 vx = mul2(vx, gs); vy = mul2(vy, gs); vz = mul2(vz, gs);
             }
             const bool kin = k >= 0 && k < g.nz;         // zero outside the grid
@@ -435,7 +433,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     // the last warp, which has no stress to compute, refills the slot for step
     // m + NS once every warp is
     if (threadIdx.x == L::NT - 32 && m + NS < G.M) {
-        Q.bad |= !mbar_wait(&bars[CB], (uint32_t)((m >> 1) & 1));
+        Q.bad = Q.bad || !mbar_wait(&bars[CB], (uint32_t)((m >> 1) & 1));
         issue_step<T, TY>(maps, sm, &bars[tn.s], G.x0, G.y0, G.z0, m + NS, g.nz);
     }
     // point force of step n on its tap cells inside the region
@@ -513,7 +511,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
                 s4 = fma2(mul2(dup(P.dt4[kScaled<T> ? 1 : 0]), mxz), add2(vxz, vzx), s4);
                 s5 = fma2(mul2(dup(P.dt4[kScaled<T> ? 2 : 0]), myz), add2(vyz, vzy), s5);
                 if (BND == BND_SPONGE) {
-                    const f2 gs = mul2(mul2(G.gx, dup(Q.gz[3])), dup(G.gy));
+                    const f2 gs = mul2(mul2(G.gx, dup(gz[-2])), dup(G.gy));
                     s0 = mul2(s0, gs); s1 = mul2(s1, gs); s2 = mul2(s2, gs);
                     s3 = mul2(s3, gs); s4 = mul2(s4, gs); s5 = mul2(s5, gs);
                 }
@@ -554,13 +552,15 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         for (int s = 0; s < NS; ++s) issue_step<T, TY>(maps, sm, &bars[s], G.x0, G.y0, G.z0, s, P.g.nz);
     }
+    if (BND == BND_SPONGE)
+        for (int q = threadIdx.x; q < G.M; q += L::NT)
+            reinterpret_cast<float*>(sm + L::O_GZ)[q] = __ldg(P.B.g[2] + min(max(G.z0 - 5 + q, 0), P.g.nz - 1));
     __syncthreads();
     FQ Q;
 #pragma unroll
     for (int q = 0; q < 4; ++q) Q.zz[q] = Q.xz[q] = Q.yz[q] = 0;
     Q.xx[0] = Q.xx[1] = Q.yy[0] = Q.yy[1] = Q.xy[0] = Q.xy[1] = 0;
     Q.dz = Q.bx = Q.by = Q.r0 = Q.vzc = Q.mu2 = Q.mxy = Q.ma = Q.mb = 0;
-    Q.gz[0] = Q.gz[1] = Q.gz[2] = Q.gz[3] = 1.0f;
     Q.bad = Q.ovf = false;
     int ring[4] = {0, 4 * L::VPL, 3 * L::VPL, 2 * L::VPL};            // planes k .. k - 3
     Turn tn;
@@ -598,9 +598,8 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
                 }
             }
         }
-        // a wait that gave up ends the CTA here; the check costs one barrier in
-        // four steps
-        stop = __syncthreads_or(Q.bad);
+        // a wait that gave up ends the CTA here; one barrier in 64 steps
+        if ((m & 63) < 4 || m >= G.M) stop = __syncthreads_or(Q.bad);
     }
     if (stop && threadIdx.x == 0) {          // record, and let the copies in flight land (bounded)
         atomicOr(P.err, 1);
@@ -687,7 +686,7 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
     p->nty = (g.ny + p->ty - 1) / p->ty;
     const long long ntile = (long long)p->ntx * p->nty;
     // a chunk runs 4 more velocity planes than it has planes and 3 light steps
-    p->zchunk = chunk_planes(ntile, (long long)sms * occ, g.nz, 8, 6);
+    p->zchunk = std::min(kMaxChunk, chunk_planes(ntile, (long long)sms * occ, g.nz, 8, 6));
     p->grid = (int)(ntile * ((g.nz + p->zchunk - 1) / p->zchunk));
     *out = p;
     return cudaSuccess;
