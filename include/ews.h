@@ -402,7 +402,9 @@ ews_status ews_forward_noalloc(const ews_grid* grid, const ews_options* opt,
  * a source/receiver step) of all shots from a device queue; an item waits
  * (bounded, EWS_ETIMEOUT) until its shot's earlier stages are done, so
  * shots of uneven size and step count share the GPU without a grid-wide
- * barrier.  Results equal those of ews_run / ews_gradient on each
+ * barrier.  With every option but ckpt_every at 0 a batch times its first
+ * forward steps both ways, once per composition, and runs its shots one
+ * after the other where that is faster.  Results equal those of ews_run / ews_gradient on each
  * simulation alone (bitwise for the forward, to accumulation order for the
  * gradient). */
 typedef struct {

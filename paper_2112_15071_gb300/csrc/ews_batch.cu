@@ -464,6 +464,146 @@ ews_status choose_batch_chunks(const ews_batch_shot* shots, int nshots, const st
     return EWS_OK;
 }
 
+// ---- the executor or one shot after the other ----
+// The executor runs the 32 x 8 passes of all shots together; one by one, each
+// shot takes its tuned shape, the fused step or the resident loop.  Which is
+// faster depends on the sizes (GB300, forward, Gcell/s, executor / one by
+// one: 12 cubes 96..224 47.9 / 50.1, 12 cubes 96..160 46.8 / 44.5, 8 cubes
+// 64..128 43.3 / 38.4; 4 shots of 96^3: 8.25 / 6.88 ms, with gradients 25.5 /
+// 22.0), so a batch times its first forward steps both ways once per
+// composition and goes one by one where that is at least 3 % faster.
+std::map<std::vector<std::tuple<int, int, int, int, int>>, bool> g_one_by_one;   // under g_tune_mu
+
+// Runs the simulations of a batch on its stream; their own come back after.
+struct StreamSwap {
+    std::vector<std::pair<ews_sim*, cudaStream_t>> own;
+    StreamSwap(const ews_batch_shot* shots, int n, cudaStream_t st) {
+        for (int i = 0; i < n; ++i) {
+            own.emplace_back(shots[i].sim, shots[i].sim->stream);
+            shots[i].sim->stream = st;
+        }
+    }
+    ~StreamSwap() {
+        for (auto& o : own) o.first->stream = o.second;
+    }
+};
+
+ews_status prefer_one_by_one(const ews_batch_shot* shots, int nshots, int bnd, bool any_fs,
+                             cudaStream_t st, bool* out) {
+    *out = false;
+    const int exec = any_fs ? BX_LEAN_FS : BX_LEAN;
+    std::vector<std::tuple<int, int, int, int, int>> key;
+    for (int i = 0; i < nshots; ++i) {
+        const ews_sim* s = shots[i].sim;
+        key.emplace_back(s->g.nx, s->g.ny, s->g.nz, bnd, exec);
+    }
+    std::sort(key.begin(), key.end());
+    {
+        std::lock_guard<std::mutex> lk(g_tune_mu);
+        auto it = g_one_by_one.find(key);
+        if (it != g_one_by_one.end()) {
+            *out = it->second;
+            return EWS_OK;
+        }
+    }
+    int T = 6;
+    for (int i = 0; i < nshots; ++i) T = std::min(T, shots[i].nt);
+    int* d_err = shots[0].sim->err;
+    std::vector<int> zc(nshots);
+    ews_status r;
+    for (int i = 0; i < nshots; ++i)
+        if ((r = tune_zchunk(shots[i].sim, shots[i], bnd,
+                             shots[i].sim->g.fs != kNoSurface ? BX_LEAN_FS : BX_LEAN, 0, d_err, st, &zc[i])) != EWS_OK)
+            return r;
+    int choice = 0;
+    if (nshots > 1 && (r = choose_batch_chunks(shots, nshots, zc, bnd, exec, 0, d_err, st, &choice)) != EWS_OK)
+        return r;
+    std::vector<BatchShot> bs(nshots);
+    std::vector<std::vector<Stage>> progs(nshots);
+    for (int i = 0; i < nshots; ++i) {
+        ews_batch_shot probe = shots[i];
+        probe.seis = nullptr;
+        probe.nt = T;
+        if ((r = fill_shot(bs[i], probe.sim, probe, chunk_for(choice, zc[i], probe.sim->g.nz), d_err, false)) != EWS_OK)
+            return r;
+        for (int n = 0; n < T; ++n) push_step(progs[i], bs[i], n, -1, false);
+    }
+    float together = 1e30f, ms = 0;
+    for (int rep = 0; rep < 2; ++rep) {
+        if ((r = run_persistent(bs, progs, bnd, exec, 0, d_err, st, &ms)) != EWS_OK) return r;
+        together = std::min(together, ms);
+    }
+    // one by one, the loops captured in the first repetition
+    StreamSwap swap(shots, nshots, st);
+    for (int i = 0; i < nshots; ++i)
+        if ((r = sim_choose_tile(shots[i].sim, shots[i].nt, shots[i].dt)) != EWS_OK) return r;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    cudaError_t e = cudaEventCreate(&e0);
+    if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    float alone = 1e30f;
+    r = EWS_OK;
+    for (int rep = 0; rep < 3 && e == cudaSuccess && r == EWS_OK; ++rep) {
+        e = cudaEventRecord(e0, st);
+        for (int i = 0; i < nshots && r == EWS_OK; ++i)
+            r = sim_steps(shots[i].sim, 0, T, shots[i].dt, nullptr, T);
+        if (e == cudaSuccess) e = cudaEventRecord(e1, st);
+        if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+        if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+        if (rep > 0) alone = std::min(alone, ms);
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    if (r != EWS_OK) return r;
+    if (e != cudaSuccess) return report(EWS_ECUDA, "batch trial: %s", cudaGetErrorString(e));
+    for (int i = 0; i < nshots; ++i) BCK(cudaMemsetAsync(shots[i].sim->err, 0, sizeof(int), st));
+    *out = alone < 0.97f * together;
+    std::lock_guard<std::mutex> lk(g_tune_mu);
+    g_one_by_one[key] = *out;
+    return EWS_OK;
+}
+
+ews_status batch_one_by_one(int nshots, ews_batch_shot* shots, int K, cudaStream_t st) {
+    StreamSwap swap(shots, nshots, st);
+    for (int i = 0; i < nshots; ++i) {
+        ews_batch_shot& b = shots[i];
+        ews_sim* s = b.sim;
+        ews_status r;
+        if (b.observed) {
+            // the executor's share of the automatic history budget
+            const double budget = s->hist_budget;
+            if (budget < 0) s->hist_budget = sim_history_budget(s, 0.5 / nshots);
+            r = ews_gradient(s, b.nt, b.dt, b.observed, 1, &b.misfit, b.g_lam, b.g_mu, b.g_rho, 1, K);
+            for (int j = 0; j < i && r == EWS_ENOMEM; ++j)         // earlier shots' gradient state
+                if (shots[j].observed) {
+                    if ((r = ews_release_workspace(shots[j].sim)) != EWS_OK) break;
+                    r = ews_gradient(s, b.nt, b.dt, b.observed, 1, &b.misfit, b.g_lam, b.g_mu, b.g_rho, 1, K);
+                }
+            s->hist_budget = budget;
+            if (r != EWS_OK) return r;
+            if (b.seis && s->nrec > 0)
+                BCK(cudaMemcpyAsync(b.seis, s->aux, (size_t)3 * s->nrec * b.nt * sizeof(float),
+                                    cudaMemcpyDeviceToDevice, st));
+        } else {
+            if ((r = sim_choose_tile(s, b.nt, b.dt)) != EWS_OK || (r = ews_reset(s)) != EWS_OK ||
+                (r = sim_steps(s, 0, b.nt, b.dt, b.seis, b.nt)) != EWS_OK)
+                return r;
+        }
+    }
+    std::vector<int> herr(nshots, 0);
+    for (int i = 0; i < nshots; ++i)
+        BCK(cudaMemcpyAsync(&herr[i], shots[i].sim->err, sizeof(int), cudaMemcpyDeviceToHost, st));
+    BCK(cudaStreamSynchronize(st));
+    int all = 0;
+    for (int i = 0; i < nshots; ++i)
+        if (herr[i]) {
+            all |= herr[i];
+            BCK(cudaMemsetAsync(shots[i].sim->err, 0, sizeof(int), st));
+        }
+    if (all & 3) return report(EWS_ETIMEOUT, "batched shots: a pipeline wait gave up (flags %d)", all);
+    if (all & 16) return report(EWS_ENONFINITE, "batched shots: a receiver recorded NaN or Inf");
+    return EWS_OK;
+}
+
 // The persistent executor over all the given shots in one captured graph.
 ews_status batch_persistent(int nshots, ews_batch_shot* shots, const ews_batch_options& o, int bnd,
                             bool grad, bool any_fs, cudaStream_t st) {
@@ -693,6 +833,7 @@ ews_status ews_batch_tuning_import(const ews_tuned_zchunk* in, int n) {
     }
     std::lock_guard<std::mutex> lk(ews::g_tune_mu);
     ews::g_choice.clear();                      // batch-level choices were made against the old entries
+    ews::g_one_by_one.clear();
     for (int k = 0; k < n; ++k) {
         const ews_tuned_zchunk& e = in[k];
         ews::g_tuned[std::make_tuple(e.nx, e.ny, e.nz, e.boundary,
@@ -706,6 +847,7 @@ void ews_batch_tuning_clear(void) {
     std::lock_guard<std::mutex> lk(ews::g_tune_mu);
     ews::g_tuned.clear();
     ews::g_choice.clear();
+    ews::g_one_by_one.clear();
 }
 
 ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options* opt,
@@ -776,6 +918,19 @@ ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options*
         return EWS_OK;
     }
 
+    // explicit executor options ask for the executor; so do profiled
+    // simulations (their launches would be counted) and FP16 checkpoints,
+    // which it keeps in FP32
+    bool plain = o.zchunk == 0 && o.ctas_per_sm == 0 && o.dep_wait_ms == 0 && !o.test_unsatisfiable;
+    for (int i = 0; i < nshots; ++i)
+        plain = plain && !shots[i].sim->profiling &&
+                !(shots[i].observed && shots[i].sim->ckpt_pref == EWS_STORAGE_F16);
+    if (plain) {
+        bool alone = false;
+        ews_status r = prefer_one_by_one(shots, nshots, bnd, any_fs, st, &alone);
+        if (r != EWS_OK) return r;
+        if (alone) return batch_one_by_one(nshots, shots, K0, st);
+    }
     if (!grad) return batch_persistent(nshots, shots, o, bnd, false, any_fs, st);
     std::vector<int> all(nshots);
     for (int i = 0; i < nshots; ++i) all[i] = i;

@@ -1066,6 +1066,12 @@ ews_status sim_ready(ews_sim* s, int n_end, double dt) { return ensure_ready(s, 
 
 DevSource sim_source(const ews_sim* s, double dt) { return source_taps(s, s->src, dt); }
 
+ews_status sim_choose_tile(ews_sim* s, int nt, double dt) { return choose_tile(s, nt, dt); }
+
+ews_status sim_steps(ews_sim* s, int n0, int nsteps, double dt, float* dseis, int ld) {
+    return steps(s, s->src, n0, nsteps, dt, dseis, ld);
+}
+
 ews_status sim_adjoint_buffers(ews_sim* s, int nt, int nckpt, int hslots, bool with_obs,
                                int ckpt_storage) {
     const size_t fs = s->fstride;

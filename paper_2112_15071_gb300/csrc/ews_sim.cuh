@@ -162,6 +162,10 @@ ews_status sim_adjoint_buffers(ews_sim* s, int nt, int nckpt, int hslots, bool w
                                int ckpt_storage = EWS_STORAGE_F32);
 // Stencil plan of the adjoint fields with its history map on s->vhist.
 ews_status sim_adjoint_plan(ews_sim* s);
+// Tile shape of a run from rest (timed trials for a new grid, which leave the
+// wavefields to be reset), and steps of the time loop.
+ews_status sim_choose_tile(ews_sim* s, int nt, double dt);
+ews_status sim_steps(ews_sim* s, int n0, int nsteps, double dt, float* dseis, int ld);
 // History budget in bytes: the set value, or (automatic) `share` of the
 // device memory free now plus what the history buffer already holds.
 double sim_history_budget(const ews_sim* s, double share);
