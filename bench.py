@@ -225,6 +225,7 @@ def kernel_source_sha() -> str:
     pkg = os.path.join(ROOT, "paper_2112_15071_gb300")
     for f in (os.path.join(pkg, "csrc", "ews_stencil.cu"), os.path.join(pkg, "csrc", "ews_fused.cu"),
               os.path.join(pkg, "csrc", "ews_internal.cuh"),
+              os.path.join(pkg, "csrc", "ews_arith.cuh"), os.path.join(pkg, "csrc", "ews_tma.cuh"),
               os.path.join(pkg, "csrc", "ews_ops.cuh"), os.path.join(ROOT, "include", "ews.h"),
               os.path.join(pkg, "_build.py")):
         h.update(open(f, "rb").read())

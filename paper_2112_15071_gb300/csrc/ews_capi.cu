@@ -766,7 +766,14 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         set_tile_used(s, EWS_TILE_32X8);
         return EWS_OK;
     }
-    const int T = std::min(nt, 6);
+    if (resident_eligible(s)) {                 // the passes do not run: no trial
+        std::lock_guard<std::mutex> lk(g_tile_mu);
+        g_tile[key] = EWS_TILE_32X8;
+        set_tile_used(s, EWS_TILE_32X8);
+        return EWS_OK;
+    }
+    int T = std::min(nt, 6);
+    bool grown = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     cudaError_t ce = cudaEventCreate(&e1);
@@ -788,19 +795,29 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
             tile_plan(s, EWS_TILE_FUSED) == EWS_OK)
             cand.push_back(EWS_TILE_FUSED);
     }
+    // trials replay a captured loop, as runs do (direct launches favour the
+    // shapes with fewer of them)
     for (int shape : cand) {
         s->tile_used = shape;
+        s->gen++;
         float ms = 1e30f;
-        for (int rep = 0; rep < 3 && st == EWS_OK; ++rep) {   // the first is a warm-up
+        for (int rep = 0; rep < 3 && st == EWS_OK; ++rep) {   // the first captures and warms up
             ce = cudaEventRecord(e0, s->stream);
-            if (ce == cudaSuccess && (st = steps_direct(s, s->src, 0, T, dt, nullptr, T, nullptr)) != EWS_OK)
-                break;
+            if (ce == cudaSuccess && (st = steps(s, s->src, 0, T, dt, nullptr, T)) != EWS_OK) break;
             if (ce == cudaSuccess) ce = cudaEventRecord(e1, s->stream);
             if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
             float t = 0.0f;
             if (ce == cudaSuccess) ce = cudaEventElapsedTime(&t, e0, e1);
             if (ce != cudaSuccess) break;
             if (rep > 0) ms = std::min(ms, t);
+            // six steps of a small grid are too short to tell shapes 5 % apart
+            // (128 x 128 x 64: 0.15 ms): trials of half a millisecond
+            if (rep == 1 && !grown && t < 0.5f && T < nt) {
+                grown = true;
+                T = std::min(nt, std::min(64, (int)(T * 0.5f / std::max(t, 1e-3f)) + 1));
+                ms = 1e30f;
+                rep = -1;
+            }
         }
         if (st != EWS_OK || ce != cudaSuccess) break;
         // another shape replaces 32 x 8 (timed first) only if it is 2 %
@@ -814,10 +831,13 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     s->tile_used = EWS_TILE_32X8;
-    if (best != EWS_TILE_FUSED || st != EWS_OK || ce != cudaSuccess) {
+    s->gen++;                                   // the trials' loops are not run again
+    const cudaError_t se = cudaStreamSynchronize(s->stream);
+    if (se == cudaSuccess) {
+        for (GraphEntry& ge : s->graphs) cudaGraphExecDestroy(ge.exec);
+        s->graphs.clear();
         // the second wavefield set is only kept for the shape that uses it
-        const cudaError_t se = cudaStreamSynchronize(s->stream);
-        if (se == cudaSuccess) drop_fused(s);
+        if (best != EWS_TILE_FUSED || st != EWS_OK || ce != cudaSuccess) drop_fused(s);
     }
     if (st != EWS_OK) return st;
     if (ce != cudaSuccess) return fail(EWS_ECUDA, "tile tuner: %s", cudaGetErrorString(ce));

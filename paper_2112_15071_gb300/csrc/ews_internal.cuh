@@ -153,11 +153,7 @@ __device__ __forceinline__ float zdiff(const DevGrid& g, const ZW& zw, const ZT&
                     : zt.iA * a + zt.iB * b + zt.iC * c + zt.iD * d;
     } else if constexpr (FS == ZS_FWD) {
         // Eq. 4, or its inner pair alone on the switched planes
-        if constexpr (!WIDE)
-            return (HALF ? zw.h2 : zw.i2) ? g.c1z2 * (c - b) : g.c1z * (c - b) + g.c2z * (d - a);
-        const float in = __fsub_rn(c, b);
-        return (HALF ? zw.h2 : zw.i2) ? __fmul_rn(g.c1z2, in)
-                                      : __fmaf_rn(g.c1z, in, __fmul_rn(g.c2z, __fsub_rn(d, a)));
+        return (HALF ? zw.h2 : zw.i2) ? g.c1z2 * (c - b) : g.c1z * (c - b) + g.c2z * (d - a);
     } else {
         if constexpr (!WIDE) return g.c1z * (c - b) + g.c2z * (d - a);
         return __fmaf_rn(g.c1z, __fsub_rn(c, b), __fmul_rn(g.c2z, __fsub_rn(d, a)));
