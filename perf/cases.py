@@ -216,7 +216,7 @@ def prepare(case, seed):
         if case["call"] == "gradient":
             shot["grad"] = torch.zeros((3,) + p["shape"], device=DEV)
         if case["snapshots"]:
-            shot["snaps"] = torch.zeros((p["nt"] // case["snapshots"],) + p["n"][::-1], device=DEV)
+            shot["snaps"] = torch.zeros((p["nt"] // case["snapshots"],) + p["shape"], device=DEV)
         state["shots"].append(shot)
     if case["call"] == "autograd":            # the cotangent that a misfit would send back
         gen = torch.Generator(device=DEV).manual_seed(seed)
