@@ -179,6 +179,37 @@ def _ptr(a, dtype=np.float32):
     return arr.ctypes.data_as(C.c_void_p), 0
 
 
+# What the calls on each live simulation read and write, by handle: cells,
+# receivers, snapshot interval and fields.  The C ABI takes bare pointers, so a
+# buffer that a call would run past the end of is refused here.
+_sizes = {}
+
+
+def _sized(sim):
+    return _sizes.get(getattr(sim, "value", sim))
+
+
+def _need(a, n, what):
+    """Refuse a buffer of fewer than n elements."""
+    if a is None:
+        return
+    have = a.numel() if hasattr(a, "data_ptr") else np.asarray(a).size
+    if have < n:
+        raise EwsError(EWS_EINVAL, f"{what} holds {have} elements, the call needs {n}")
+
+
+def _need_cells(sim, arrays, what, fields=1):
+    z = _sized(sim)
+    for a in arrays if z else ():
+        _need(a, fields * z["cells"], what)
+
+
+def _need_traces(sim, a, nt, what):
+    z = _sized(sim)
+    if z:
+        _need(a, 3 * z["nrec"] * int(nt), what)
+
+
 # --- entry points (same names as include/ews.h) ----------------------------
 
 def ews_version() -> int:
@@ -214,11 +245,16 @@ def ews_create(grid: ews_grid, opt: ews_options | None):
     h = C.c_void_p()
     _check(load().ews_create(C.byref(grid), C.byref(opt) if opt is not None else None,
                              C.byref(h)))
+    every = opt.snapshot_every if opt is not None else 0
+    fields = bin(opt.snapshot_mask).count("1") if opt is not None else 0
+    _sizes[h.value] = {"cells": grid.nx * grid.ny * grid.nz, "nrec": 0, "every": every,
+                       "fields": fields}
     return h
 
 
 def ews_destroy(sim):
     if sim:
+        _sizes.pop(getattr(sim, "value", sim), None)
         load().ews_destroy(sim)
 
 
@@ -229,12 +265,14 @@ def ews_set_stream(sim, stream_handle: int):
 def ews_set_model_lame(sim, lam, mu, rho):
     (pl, d0), (pm, d1), (pr, d2) = _ptr(lam), _ptr(mu), _ptr(rho)
     assert d0 == d1 == d2, "model arrays must share residency"
+    _need_cells(sim, (lam, mu, rho), "model array")
     _check(load().ews_set_model_lame(sim, pl, pm, pr, d0))
 
 
 def ews_set_model_vel(sim, vp, vs, rho):
     (pa, d0), (pb, d1), (pr, d2) = _ptr(vp), _ptr(vs), _ptr(rho)
     assert d0 == d1 == d2, "model arrays must share residency"
+    _need_cells(sim, (vp, vs, rho), "model array")
     _check(load().ews_set_model_vel(sim, pa, pb, pr, d0))
 
 
@@ -253,6 +291,8 @@ def ews_set_receivers(sim, pos):
     r = np.ascontiguousarray(pos, np.float64).reshape(-1, 3)
     _check(load().ews_set_receivers(sim, int(r.shape[0]),
                                     r.ctypes.data_as(C.c_void_p) if r.size else None))
+    if _sized(sim):
+        _sized(sim)["nrec"] = int(r.shape[0])
 
 
 def ews_set_model_coarse(sim, a, b, rho, from_velocities: bool = False):
@@ -275,11 +315,16 @@ def ews_run(sim, nt: int, dt: float, seis, snapshots=None):
     pn, devn = _ptr(snapshots)
     if snapshots is not None:
         assert devn == dev, "seis and snapshots must share residency"
+    _need_traces(sim, seis, nt, "seis")
+    z = _sized(sim)
+    if z and z["every"] > 0:
+        _need(snapshots, int(nt) // z["every"] * z["fields"] * z["cells"], "snapshots")
     _check(load().ews_run(sim, int(nt), float(dt), ps, dev, pn))
 
 
 def ews_advance(sim, n0: int, nsteps: int, dt: float, seis, ld: int):
     ps, dev = _ptr(seis)
+    _need_traces(sim, seis, ld, "seis")
     _check(load().ews_advance(sim, int(n0), int(nsteps), float(dt), ps, int(ld), dev))
 
 
@@ -289,11 +334,13 @@ def ews_reset(sim):
 
 def ews_get_state(sim, out):
     p, dev = _ptr(out)
+    _need_cells(sim, (out,), "state", 9)
     _check(load().ews_get_state(sim, p, dev))
 
 
 def ews_set_state(sim, state):
     p, dev = _ptr(state)
+    _need_cells(sim, (state,), "state", 9)
     _check(load().ews_set_state(sim, p, dev))
 
 
@@ -329,6 +376,8 @@ def ews_adjoint(sim, nt: int, dt: float, seis_adj, g_lam, g_mu, g_rho, ckpt_ever
     pa, da = _ptr(seis_adj)
     (pl, d0), (pm, d1), (pr, d2) = _ptr(g_lam), _ptr(g_mu), _ptr(g_rho)
     assert d0 == d1 == d2, "gradient outputs must share residency"
+    _need_traces(sim, seis_adj, nt, "seis_adj")
+    _need_cells(sim, (g_lam, g_mu, g_rho), "gradient output")
     _check(load().ews_adjoint(sim, int(nt), float(dt), pa, da, pl, pm, pr, d0, int(ckpt_every)))
 
 
@@ -337,6 +386,8 @@ def ews_gradient(sim, nt: int, dt: float, observed, g_lam, g_mu, g_rho, ckpt_eve
     po, do = _ptr(observed)
     (pl, d0), (pm, d1), (pr, d2) = _ptr(g_lam), _ptr(g_mu), _ptr(g_rho)
     assert d0 == d1 == d2, "gradient outputs must share residency"
+    _need_traces(sim, observed, nt, "observed")
+    _need_cells(sim, (g_lam, g_mu, g_rho), "gradient output")
     mis = C.c_double(0.0)
     _check(load().ews_gradient(sim, int(nt), float(dt), po, do, C.byref(mis), pl, pm, pr, d0,
                                int(ckpt_every)))
@@ -360,6 +411,10 @@ def ews_batch(shots, mode: int = EWS_BATCH_PERSISTENT, ckpt_every: int = 0, zchu
             if t is not None:
                 p, dev = _ptr(t)
                 assert dev == 1, f"{key} must be a CUDA tensor"
+                if key in ("seis", "observed"):
+                    _need_traces(b.sim, t, b.nt, key)
+                else:
+                    _need_cells(b.sim, (t,), key)
                 setattr(b, key, p.value)
     opt = ews_batch_options(int(mode), int(ckpt_every), int(zchunk), int(ctas_per_sm),
                             int(dep_wait_ms), int(bool(test_unsatisfiable)))
@@ -379,6 +434,8 @@ def ews_fwi_iteration(shots, lam, mu, rho, max_rel_step: float = 0.02, ckpt_ever
         arr[i].dt = float(d["dt"])
         p, dev = _ptr(d["observed"])
         assert dev == 1, "observed must be a CUDA tensor"
+        _need_traces(arr[i].sim, d["observed"], d["nt"], "observed")
+        _need_cells(arr[i].sim, (lam, mu, rho), "model array")
         arr[i].observed = p.value
     ptrs = []
     for t in (lam, mu, rho):
@@ -542,6 +599,10 @@ def ews_forward_noalloc(grid: ews_grid, opt: ews_options | None, lam, mu, rho, k
     cc = np.asarray(comp, np.float64).ravel()
     c[:cc.size] = cc
     r = np.ascontiguousarray(rec_pos, np.float64).reshape(-1, 3)
+    for a in (lam, mu, rho):
+        _need(a, grid.nx * grid.ny * grid.nz, "model array")
+    _need(wavelet, int(nt), "wavelet")
+    _need(seis, 3 * r.shape[0] * int(nt), "seis")
     _check(load().ews_forward_noalloc(
         C.byref(grid), C.byref(opt) if opt is not None else None, ptrs[0], ptrs[1], ptrs[2],
         int(kind), p.ctypes.data_as(C.c_void_p), c.ctypes.data_as(C.c_void_p), ptrs[3],

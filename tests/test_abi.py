@@ -203,3 +203,67 @@ def test_memory_limit_calls_are_host_only():
         assert e.value.status == ews.EWS_EINVAL
     finally:
         ews.ews_set_memory_limit(-1.0)
+
+
+@pytest.mark.parametrize("call", ["run", "snapshots", "advance", "get_state", "set_state", "model",
+                                  "gradient", "observed", "adjoint", "batch", "fwi", "noalloc"])
+def test_short_buffers_are_refused(monkeypatch, call):
+    """A buffer of fewer elements than a call reads or writes is refused by
+    the binding (the C ABI takes bare pointers and would run past its end);
+    one of exactly that size, or larger, reaches the library."""
+    class Lib:
+        calls = 0
+
+        def __getattr__(self, name):
+            def f(*a):
+                if name == "ews_create":
+                    a[2]._obj.value = 77
+                elif name != "ews_set_receivers":
+                    Lib.calls += 1
+                return ews.EWS_OK
+            return f
+
+    class Cuda(np.ndarray):                          # what _ptr takes for a CUDA tensor
+        is_cuda, data_ptr, numel = True, lambda s: s.ctypes.data, lambda s: s.size
+        is_contiguous = lambda s: s.flags.c_contiguous
+
+    def dev(n):
+        import torch
+        a = np.zeros(n, np.float32).view(Cuda)
+        monkeypatch.setattr(Cuda, "dtype", torch.float32, raising=False)
+        return a
+
+    monkeypatch.setattr(ews, "load", lambda *a: Lib())
+    grid, opt = ews.ews_grid(7, 5, 4, 1.0, 1.0, 1.0), ews.ews_options(0, 0, 0, 3, 0b101, 0.0, 0.0, 0.0)
+    cells, nrec, nt = 140, 2, 10
+    sim = ews.ews_create(grid, opt)
+    ews.ews_set_receivers(sim, np.ones((nrec, 3)))
+    f32 = lambda n: np.zeros(n, np.float32)
+    shot = lambda **k: dict(dict(sim=sim, nt=nt, dt=1.0), **k)
+    full, go = {
+        "run": (3 * nrec * nt, lambda a: ews.ews_run(sim, nt, 1.0, a)),
+        "snapshots": (3 * 2 * cells, lambda a: ews.ews_run(sim, nt, 1.0, f32(3 * nrec * nt), a)),
+        "advance": (3 * nrec * 20, lambda a: ews.ews_advance(sim, 5, 5, 1.0, a, 20)),
+        "get_state": (9 * cells, lambda a: ews.ews_get_state(sim, a)),
+        "set_state": (9 * cells, lambda a: ews.ews_set_state(sim, a)),
+        "model": (cells, lambda a: ews.ews_set_model_vel(sim, f32(cells), a, f32(cells))),
+        "gradient": (cells, lambda a: ews.ews_gradient(sim, nt, 1.0, f32(3 * nrec * nt), f32(cells),
+                                                       f32(cells), a)),
+        "observed": (3 * nrec * nt, lambda a: ews.ews_gradient(sim, nt, 1.0, a, *[f32(cells)] * 3)),
+        "adjoint": (3 * nrec * nt, lambda a: ews.ews_adjoint(sim, nt, 1.0, a, *[f32(cells)] * 3)),
+        "batch": (cells, lambda a: ews.ews_batch([shot(g_mu=a)])),
+        "fwi": (3 * nrec * nt, lambda a: ews.ews_fwi_iteration([shot(observed=a)], *[dev(cells)] * 3)),
+        "noalloc": (nt, lambda a: ews.ews_forward_noalloc(
+            grid, opt, dev(cells), dev(cells), dev(cells), 0, np.ones(3), np.zeros(6), a,
+            np.ones((nrec, 3)), nt, 1.0, dev(3 * nrec * nt))),
+    }[call]
+    make = dev if call in ("batch", "fwi", "noalloc") else f32
+    try:
+        with pytest.raises(ews.EwsError) as e:
+            go(make(full - 1))
+        assert e.value.status == ews.EWS_EINVAL and Lib.calls == 0
+        go(make(full))
+        go(make(full + 3))
+        assert Lib.calls == 2
+    finally:
+        ews.ews_destroy(sim)
