@@ -18,6 +18,7 @@
 #include "../../include/ews.h"
 #include "ews_internal.cuh"
 #include "ews_sim.cuh"
+#include "ews_tuner.cuh"
 
 using namespace ews;
 
@@ -772,8 +773,6 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         set_tile_used(s, EWS_TILE_32X8);
         return EWS_OK;
     }
-    int T = std::min(nt, 6);
-    bool grown = false;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     CK(cudaEventCreate(&e0));
     cudaError_t ce = cudaEventCreate(&e1);
@@ -781,8 +780,6 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         cudaEventDestroy(e0);
         return fail(EWS_ECUDA, "tile tuner: %s", cudaGetErrorString(ce));
     }
-    int best = EWS_TILE_32X8;
-    float best_ms = 1e30f;
     ews_status st = EWS_OK;
     std::vector<int> cand = {EWS_TILE_32X8, EWS_TILE_32X4, EWS_TILE_32X16};
     // the fused step, if it applies and its second wavefield set takes at
@@ -796,38 +793,23 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
             cand.push_back(EWS_TILE_FUSED);
     }
     // trials replay a captured loop, as runs do (direct launches favour the
-    // shapes with fewer of them)
-    for (int shape : cand) {
+    // shapes with fewer of them); the first of three captures and warms up
+    const int best = fastest_shape(cand, nt, [&](int shape, int T, float* ms) {
         s->tile_used = shape;
         s->gen++;
-        float ms = 1e30f;
-        for (int rep = 0; rep < 3 && st == EWS_OK; ++rep) {   // the first captures and warms up
+        *ms = 1e30f;
+        for (int rep = 0; rep < 3; ++rep) {
             ce = cudaEventRecord(e0, s->stream);
-            if (ce == cudaSuccess && (st = steps(s, s->src, 0, T, dt, nullptr, T)) != EWS_OK) break;
+            if (ce == cudaSuccess && (st = steps(s, s->src, 0, T, dt, nullptr, T)) != EWS_OK) return false;
             if (ce == cudaSuccess) ce = cudaEventRecord(e1, s->stream);
             if (ce == cudaSuccess) ce = cudaEventSynchronize(e1);
             float t = 0.0f;
             if (ce == cudaSuccess) ce = cudaEventElapsedTime(&t, e0, e1);
-            if (ce != cudaSuccess) break;
-            if (rep > 0) ms = std::min(ms, t);
-            // six steps of a small grid are too short to tell shapes 5 % apart
-            // (128 x 128 x 64: 0.15 ms): trials of half a millisecond
-            if (rep == 1 && !grown && t < 0.5f && T < nt) {
-                grown = true;
-                T = std::min(nt, std::min(64, (int)(T * 0.5f / std::max(t, 1e-3f)) + 1));
-                ms = 1e30f;
-                rep = -1;
-            }
+            if (ce != cudaSuccess) return false;
+            if (rep > 0) *ms = std::min(*ms, t);
         }
-        if (st != EWS_OK || ce != cudaSuccess) break;
-        // another shape replaces 32 x 8 (timed first) only if it is 2 %
-        // faster, so shapes within timing noise of each other do not
-        // change from run to run
-        if (shape == EWS_TILE_32X8 ? ms < best_ms : ms < 0.98f * best_ms) {
-            best_ms = ms;
-            best = shape;
-        }
-    }
+        return true;
+    });
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     s->tile_used = EWS_TILE_32X8;
