@@ -1334,7 +1334,8 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
     if (e == cudaSuccess) e = cudaMemset(s->medium, 0, 3 * s->fstride * sizeof(float));
     if (e == cudaSuccess && s->psi) e = cudaMemset(s->psi, 0, s->psi_floats * sizeof(float));
     if (e == cudaSuccess) e = cudaMemset(s->err, 0, sizeof(int));
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    // (not the whole device, which fails while another thread captures its loop)
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) return cleanup(fail(EWS_ECUDA, "memset: %s", cudaGetErrorString(e)));
     e = stencil_plan_create(s->g, s->F(), s->M(), s->B, o.storage, &s->plan);
     if (e != cudaSuccess)
@@ -1345,8 +1346,7 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
 
 void ews_destroy(ews_sim* s) {
     if (!s) return;
-    if (s->stream) cudaStreamSynchronize(s->stream);
-    else cudaDeviceSynchronize();
+    cudaStreamSynchronize(s->stream);
     dev_free(s->fields);
     dev_free(s->medium);
     dev_free(s->cmed);
@@ -1718,8 +1718,7 @@ ews_status ews_set_state(ews_sim* s, const float* in, int on_device) {
 
 ews_status ews_release_workspace(ews_sim* s) {
     if (!s) return fail(EWS_EINVAL, "null simulation");
-    if (s->stream) CK(cudaStreamSynchronize(s->stream));
-    else CK(cudaDeviceSynchronize());
+    CK(cudaStreamSynchronize(s->stream));
     for (GraphEntry& ge : s->graphs) cudaGraphExecDestroy(ge.exec);
     s->graphs.clear();
     stencil_plan_destroy(s->adj_plan);
