@@ -247,7 +247,8 @@ ews_status ews_gradient(ews_sim* sim, int nt, double dt, const float* observed,
 
 /* Free the working memory the simulation keeps between calls: adjoint
  * state and accumulators, checkpoints, velocity history, seismogram and
- * state staging, the adjoint stencil plan and captured time-loop graphs
+ * state staging, the second wavefield set of the fused step, the adjoint
+ * stencil plan and captured time-loop graphs
  * (the wavefields, medium, source and receivers stay).  Later calls
  * allocate again as needed.  Synchronises the simulation's stream. */
 ews_status ews_release_workspace(ews_sim* sim);
@@ -280,21 +281,25 @@ ews_status ews_get_field_scales(ews_sim* sim, float* scale);
  * sponge, 32 x 16 for BF16 with a sponge).  Every shape runs the same
  * arithmetic per cell in the same order (separately compiled, so results
  * agree to FP32 rounding).  EWS_TILE_FUSED runs both passes of a step in one
- * launch (32 x 8 tiles, the velocity of a 2-cell ring around each tile
+ * launch (32 x 24 tiles, the velocity of a 2-cell ring around each tile
  * recomputed by its neighbours), reading one set of wavefields and writing a
  * second one that the library allocates (9 more wavefields of device
- * memory, released when the tuner picks another shape); it serves FP32
- * storage at unit field scales with a sponge or no absorbing boundary, and
- * other runs fall back to 32 x 8.  It moves 84 bytes per cell instead of
- * 120 but recomputes the ring, so on a GB300 it is bound by instruction
- * issue and runs slower than the two passes (0.78x at 256^3, 0.89x at
- * 1024 x 1024 x 512); the tuner times it where the second set takes at
- * most a quarter of the free device memory.  With EWS_TILE_AUTO (the default),
- * ews_run picks the shape for its grid size, boundary and storage type from
- * a per-process table, filling a missing entry by timing a few steps with
- * each shape before the run (the wavefields are reset afterwards); plain
- * forward steps use it (runs with a free surface or a coarse medium grid,
- * the adjoint's forward part and batched shots keep 32 x 8). */
+ * memory, 36 bytes per cell); it serves FP32 storage at unit field scales
+ * with a sponge or no absorbing boundary, and other runs fall back to 32 x 8.
+ * It moves 84 bytes per cell instead of 120 (on a GB300 1.20x the two passes
+ * at 256^3, 1.26x at 1024 x 1024 x 512).
+ * With EWS_TILE_AUTO (the default), ews_run picks the shape for its grid
+ * size, boundary and storage type from a per-process table, filling a missing
+ * entry by timing a few steps with each shape before the run (the wavefields
+ * are reset afterwards).  Plain forward steps use it; runs with a free surface
+ * or a coarse medium grid keep 32 x 8, and so do the steps of an adjoint or
+ * gradient that write the velocity history, unless the simulation holds the
+ * fused step's second set from an earlier run.
+ * The second set, of the automatic shape, takes at most a quarter of the
+ * device memory free when it is allocated; without that room the run takes
+ * 32 x 8.  The simulation keeps the set for its next run;
+ * ews_release_workspace frees it, and so does any allocation of the library,
+ * for whatever simulation, that does not fit otherwise. */
 enum {
     EWS_TILE_AUTO = 0,
     EWS_TILE_32X8 = 1,

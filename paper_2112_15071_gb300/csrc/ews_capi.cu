@@ -12,6 +12,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <thread>
 #include <tuple>
 #include <vector>
 
@@ -94,11 +95,52 @@ int fwd_shape(const ews_sim* s, bool capture) {
     return s->tile_used;
 }
 
-void drop_fused(ews_sim* s) {
+// ---- second wavefield sets ----
+// Simulations that hold a set, so that another allocation can have it
+// (give_back_set).  Host threads: the owner's calls look at and use their set
+// only inside a SetInUse scope; give_back_set takes only sets outside one and
+// never waits for a scope, so neither can block the other for long.
+std::mutex g_sets_mu;
+std::vector<ews_sim*> g_sets;
+
+struct SetInUse {
+    ews_sim* s;
+    explicit SetInUse(ews_sim* sim) : s(sim) {
+        if (s->set_depth++ > 0) return;
+        for (int idle = 0; !s->set_use.compare_exchange_weak(idle, 1); idle = 0) std::this_thread::yield();
+    }
+    ~SetInUse() {
+        if (--s->set_depth == 0) s->set_use.store(0);
+    }
+    SetInUse(const SetInUse&) = delete;
+};
+
+// Frees the set and its plan once the steps that used it are done; loops
+// captured with it are not run again.
+void free_set(ews_sim* s) {
+    if (s->set_done) cudaEventSynchronize(s->set_done);
     fused::fused_plan_destroy(static_cast<fused::FusedPlan*>(s->tplan[EWS_TILE_FUSED]));
     s->tplan[EWS_TILE_FUSED] = nullptr;
     dev_free(s->fields2);
     s->fields2 = nullptr;
+    s->set_gen++;
+}
+
+void drop_fused(ews_sim* s) {
+    SetInUse use(s);
+    if (!s->fields2) return;
+    {
+        std::lock_guard<std::mutex> lk(g_sets_mu);
+        g_sets.erase(std::remove(g_sets.begin(), g_sets.end(), s), g_sets.end());
+    }
+    free_set(s);
+}
+
+// The fused step's set takes at most a quarter of the device memory still free.
+bool set_fits(const ews_sim* s) {
+    size_t fr = 0, tot = 0;
+    const double set = (double)NFIELD * s->fstride * sizeof(float);
+    return cudaMemGetInfo(&fr, &tot) == cudaSuccess && set <= 0.25 * std::min((double)fr, dev_headroom());
 }
 
 void drop_tile_plans(ews_sim* s) {
@@ -112,7 +154,7 @@ ews_status tile_plan(ews_sim* s, int shape) {
     if (shape == EWS_TILE_32X8 || s->tplan[shape]) return EWS_OK;
     if (shape == EWS_TILE_FUSED) {
         const size_t bytes = (size_t)NFIELD * s->fstride * sizeof(float);
-        cudaError_t e = dev_malloc((void**)&s->fields2, bytes);
+        cudaError_t e = dev_malloc((void**)&s->fields2, bytes, false);
         if (e != cudaSuccess) {
             s->fields2 = nullptr;
             return fail(EWS_ENOMEM, "second wavefield set of the fused step (%zu bytes): %s", bytes,
@@ -120,6 +162,8 @@ ews_status tile_plan(ews_sim* s, int shape) {
         }
         fused::FusedPlan* p = nullptr;
         e = cudaMemsetAsync(s->fields2, 0, bytes, s->stream);
+        if (e == cudaSuccess && !s->set_done) e = cudaEventCreateWithFlags(&s->set_done, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(s->set_done, s->stream);
         if (e == cudaSuccess) e = fused::fused_plan_create(s->g, s->F(), s->F2(), s->M(), s->B, &p);
         if (e != cudaSuccess) {
             dev_free(s->fields2);
@@ -127,6 +171,8 @@ ews_status tile_plan(ews_sim* s, int shape) {
             return fail(EWS_ECUDA, "fused step plan: %s", cudaGetErrorString(e));
         }
         s->tplan[shape] = p;
+        std::lock_guard<std::mutex> lk(g_sets_mu);
+        g_sets.push_back(s);
         return EWS_OK;
     }
     if (shape == EWS_TILE_32X4) {
@@ -153,6 +199,20 @@ ews_status report(ews_status s, const char* fmt, ...) {
     va_end(ap);
     enomem_tail(s);                                    // as in fail()
     return s;
+}
+// Frees one second wavefield set that no call is using; false: there is none.
+bool give_back_set() {
+    std::lock_guard<std::mutex> lk(g_sets_mu);
+    for (size_t k = 0; k < g_sets.size(); ++k) {
+        ews_sim* s = g_sets[k];
+        int idle = 0;
+        if (!s->set_use.compare_exchange_strong(idle, 2)) continue;
+        g_sets.erase(g_sets.begin() + (long)k);
+        free_set(s);
+        s->set_use.store(0);
+        return true;
+    }
+    return false;
 }
 }  // namespace ews
 
@@ -662,6 +722,35 @@ ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps,
     return EWS_OK;
 }
 
+void set_tile_used(ews_sim* s, int shape) {
+    if (shape != s->tile_used) {
+        s->tile_used = shape;
+        s->gen++;                               // recapture the time loops
+    }
+}
+
+bool set_held_or_fits(ews_sim* s) {
+    SetInUse use(s);
+    return s->fields2 || set_fits(s);
+}
+
+// Makes the plan of the next steps' shape.  With the automatic shape, the
+// fused step gives way to the 32 x 8 passes where its second wavefield set is
+// not to be had.
+ews_status plan_steps(ews_sim* s, bool capture) {
+    const int shape = fwd_shape(s, capture);
+    const bool chosen = shape == EWS_TILE_FUSED && s->tile_req == EWS_TILE_AUTO;
+    if (chosen && !s->tplan[shape] && !set_fits(s)) {
+        set_tile_used(s, EWS_TILE_32X8);
+        return EWS_OK;
+    }
+    const ews_status st = tile_plan(s, shape);
+    if (st != EWS_ENOMEM || !chosen) return st;
+    g_err[0] = 0;
+    set_tile_used(s, EWS_TILE_32X8);
+    return EWS_OK;
+}
+
 // The time loop of steps_direct, captured once into a CUDA graph per
 // (state generation, step range, dt, output buffers) and replayed: one
 // graph launch per call instead of 4-5 kernel launches per step.  With
@@ -671,17 +760,24 @@ ews_status steps(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double d
                  float* dseis, int ld, float* vcap = nullptr) {
     if (resident_eligible(s) && nsteps > 0)
         return steps_resident(s, src, n0, nsteps, dt, dseis, ld, vcap);
+    SetInUse use(s);
+    // the shape's plan exists before a capture starts
+    ews_status sp = plan_steps(s, vcap != nullptr);
+    if (sp != EWS_OK) return sp;
+    struct Done {                              // what was enqueued has the set until then
+        ews_sim* s;
+        ~Done() {
+            if (s->fields2) cudaEventRecord(s->set_done, s->stream);
+        }
+    } done{s};
     if (s->profiling || nsteps <= 0) return steps_direct(s, src, n0, nsteps, dt, dseis, ld, vcap);
     GraphEntry* hit = nullptr;
     for (GraphEntry& ge : s->graphs)
-        if (ge.gen == s->gen && ge.n0 == n0 && ge.nsteps == nsteps && ge.ld == ld && ge.dt == dt &&
+        if (ge.gen == s->gen && ge.set_gen == s->set_gen && ge.n0 == n0 && ge.nsteps == nsteps && ge.ld == ld && ge.dt == dt &&
             ge.dseis == dseis && ge.vcap == vcap)
             hit = &ge;
     if (!hit) {
         if (!s->cap_stream) CK(cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking));
-        // the tile shape's plan exists before the capture starts
-        ews_status sp = tile_plan(s, fwd_shape(s, vcap != nullptr));
-        if (sp != EWS_OK) return sp;
         long long before[EWS_NKERNEL];
         std::memcpy(before, s->launches, sizeof(before));
         cudaStream_t user = s->stream;
@@ -703,6 +799,7 @@ ews_status steps(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double d
         cudaGraphDestroy(graph);
         if (ei != cudaSuccess) return fail(EWS_ECUDA, "graph instantiate: %s", cudaGetErrorString(ei));
         ge.gen = s->gen;
+        ge.set_gen = s->set_gen;
         ge.n0 = n0;
         ge.nsteps = nsteps;
         ge.ld = ld;
@@ -731,13 +828,6 @@ std::tuple<int, int, int, int, int> tile_key(const ews_sim* s) {
     return std::make_tuple(s->grid.nx, s->grid.ny, s->grid.nz, s->opt.boundary, s->opt.storage);
 }
 
-void set_tile_used(ews_sim* s, int shape) {
-    if (shape != s->tile_used) {
-        s->tile_used = shape;
-        s->gen++;                               // recapture the time loops
-    }
-}
-
 // Before a run from rest: the requested shape, else the table's entry for
 // this grid, else the fastest of a few timed steps with each shape (taken
 // from rest and thrown away: the caller resets the wavefields afterwards).
@@ -758,8 +848,8 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         std::lock_guard<std::mutex> lk(g_tile_mu);
         auto it = g_tile.find(key);
         if (it != g_tile.end()) {
-            set_tile_used(s, it->second == EWS_TILE_FUSED && !fused_eligible(s) ? EWS_TILE_32X8
-                                                                                : it->second);
+            const bool fused = it->second == EWS_TILE_FUSED;
+            set_tile_used(s, fused && !(fused_eligible(s) && set_held_or_fits(s)) ? EWS_TILE_32X8 : it->second);
             return EWS_OK;
         }
     }
@@ -780,18 +870,13 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         cudaEventDestroy(e0);
         return fail(EWS_ECUDA, "tile tuner: %s", cudaGetErrorString(ce));
     }
+    SetInUse use(s);                            // no trial loses its set
     ews_status st = EWS_OK;
     std::vector<int> cand = {EWS_TILE_32X8, EWS_TILE_32X4, EWS_TILE_32X16};
-    // the fused step, if it applies and its second wavefield set takes at
-    // most a quarter of the device memory still free
-    if (fused_eligible(s)) {
-        size_t fr = 0, tot = 0;
-        const double set = (double)NFIELD * s->fstride * sizeof(float);
-        if (cudaMemGetInfo(&fr, &tot) == cudaSuccess &&
-            set <= 0.25 * std::min((double)fr, dev_headroom()) &&
-            tile_plan(s, EWS_TILE_FUSED) == EWS_OK)
-            cand.push_back(EWS_TILE_FUSED);
-    }
+    // the fused step, if it applies and there is room for its second
+    // wavefield set
+    if (fused_eligible(s) && set_fits(s) && tile_plan(s, EWS_TILE_FUSED) == EWS_OK)
+        cand.push_back(EWS_TILE_FUSED);
     // trials replay a captured loop, as runs do (direct launches favour the
     // shapes with fewer of them); the first of three captures and warms up
     const int best = fastest_shape(cand, nt, [&](int shape, int T, float* ms) {
@@ -1125,6 +1210,8 @@ ews_status sim_adjoint_buffers(ews_sim* s, int nt, int nckpt, int hslots, bool w
     return EWS_OK;
 }
 
+void sim_drop_set(ews_sim* s) { drop_fused(s); }
+
 double sim_history_budget(const ews_sim* s, double share) {
     if (s->hist_budget >= 0) return s->hist_budget;
     size_t free_b = 0, total_b = 0;
@@ -1374,6 +1461,7 @@ void ews_destroy(ews_sim* s) {
     for (cudaEvent_t e : s->ev_pool) cudaEventDestroy(e);
     for (GraphEntry& ge : s->graphs) cudaGraphExecDestroy(ge.exec);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
+    if (s->set_done) cudaEventDestroy(s->set_done);
     delete s;
 }
 
@@ -1730,6 +1818,7 @@ ews_status ews_release_workspace(ews_sim* s) {
         dev_free(*b);
         *b = nullptr;
     }
+    drop_fused(s);
     dev_free(s->acc64);
     s->acc64 = nullptr;
     dev_free(s->dmisfit);

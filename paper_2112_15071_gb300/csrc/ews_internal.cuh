@@ -245,9 +245,13 @@ ews_status report(ews_status s, const char* fmt, ...);
 // optional process-wide limit of ews_set_memory_limit.  dev_malloc returns
 // cudaErrorMemoryAllocation, without calling CUDA, for a request above the
 // limit; dev_headroom is the room left under it (INFINITY without a limit).
-cudaError_t dev_malloc(void** p, size_t bytes);
+// A request that does not fit frees the second wavefield sets no call is using
+// (give_back_set, ews_capi.cu: one set a call, false if there is none), unless
+// give_back is false.
+cudaError_t dev_malloc(void** p, size_t bytes, bool give_back = true);
 void dev_free(void* p);
 double dev_headroom();
+bool give_back_set();
 
 // Stencil passes (ews_stencil.cu): TMA tensor maps and launch geometry are
 // built once per simulation (the field and medium addresses never change).

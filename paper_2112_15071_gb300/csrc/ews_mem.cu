@@ -9,6 +9,9 @@
 // every caller's out-of-memory path (EWS_ENOMEM, partial set-up released,
 // the simulation still usable) runs the same way in both cases.  A service
 // that shares its GPU with other work can so bound what the solver takes.
+// The second wavefield sets that simulations keep for the fused step only buy
+// speed, so a request that does not fit gets them back first (give_back_set),
+// one by one: they make no call fail that would have had room without them.
 // (ews_forward_noalloc allocates nothing and is not counted.)
 #include <cuda_runtime.h>
 
@@ -26,9 +29,8 @@ std::unordered_map<void*, size_t> g_live;   // pointer -> bytes
 size_t g_in_use = 0;
 double g_limit = -1.0;                      // < 0: no cap
 
-}  // namespace
-
-cudaError_t dev_malloc(void** p, size_t bytes) {
+// One attempt of dev_malloc.
+cudaError_t try_malloc(void** p, size_t bytes) {
     *p = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_mu);
@@ -40,12 +42,23 @@ cudaError_t dev_malloc(void** p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
     std::lock_guard<std::mutex> lk(g_mu);
     if (e != cudaSuccess) {
+        // the caller may go on without: no error of its next call
+        if (cudaPeekAtLastError() == cudaErrorMemoryAllocation) (void)cudaGetLastError();
         g_in_use -= bytes;
         *p = nullptr;
         return e;
     }
     g_live[*p] = bytes;
     return cudaSuccess;
+}
+
+}  // namespace
+
+cudaError_t dev_malloc(void** p, size_t bytes, bool give_back) {
+    cudaError_t e;
+    while ((e = try_malloc(p, bytes)) == cudaErrorMemoryAllocation && give_back && give_back_set()) {
+    }
+    return e;
 }
 
 void dev_free(void* p) {

@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <vector>
 
 #include "../../include/ews.h"
@@ -21,7 +22,7 @@ struct SourceSpec {
 // One captured time loop: a CUDA graph of steps n0 .. n0 + nsteps - 1 with
 // everything its kernel parameters depend on as the key.
 struct GraphEntry {
-    unsigned long long gen;
+    unsigned long long gen, set_gen;
     int n0, nsteps, ld;
     double dt;
     const float* dseis;
@@ -82,8 +83,16 @@ struct ews_sim {
     int tile_used = EWS_TILE_32X8;
     void* tplan[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
     // second set of wavefields of the fused step (9 * fstride floats, laid
-    // out like `fields`), held with its plan
+    // out like `fields`), held with its plan between runs; holds nothing a
+    // later step needs, and may be freed for another allocation while no call
+    // is in a SetInUse scope (set_use 0; 1 in use, 2 being freed; set_depth
+    // counts the owner's nested scopes).  set_gen counts the sets freed,
+    // set_done follows the last steps that used one.
     float* fields2 = nullptr;
+    std::atomic<int> set_use{0};
+    int set_depth = 0;
+    unsigned long long set_gen = 0;
+    cudaEvent_t set_done = nullptr;
     // time loop of a small grid in one launch (null where it does not fit):
     // its CTAs' halo inboxes with the steps they have served, the receiver
     // taps by CTA, and the staged tap values of up to res_chunk steps
@@ -166,6 +175,8 @@ ews_status sim_adjoint_plan(ews_sim* s);
 // wavefields to be reset), and steps of the time loop.
 ews_status sim_choose_tile(ews_sim* s, int nt, double dt);
 ews_status sim_steps(ews_sim* s, int n0, int nsteps, double dt, float* dseis, int ld);
+// Frees the second wavefield set of the fused step, if the simulation holds one.
+void sim_drop_set(ews_sim* s);
 // History budget in bytes: the set value, or (automatic) `share` of the
 // device memory free now plus what the history buffer already holds.
 double sim_history_budget(const ews_sim* s, double share);

@@ -176,3 +176,97 @@ def test_gradient_batch_runs_in_waves_under_the_limit(ews):
             assert ma[i] == pytest.approx(mb[i], rel=1e-6)
             for k in ("g_lam", "g_mu", "g_rho"):
                 assert rel(a[i][k].cpu().numpy(), b[i][k].cpu().numpy()) <= 1e-5, (i, k)
+
+
+def fused_problem(ews, seed):
+    """A grid beyond the one-launch time loop whose tile-table entry is the
+    fused step, and the bytes of one of its fields."""
+    p = synth.small_problem(96, 72, 72, nt=30, boundary="sponge", width=6, seed=seed, kind="moment")
+    ews.ews_tile_tuning_import([{"nx": 96, "ny": 72, "nz": 72, "boundary": "sponge", "storage": "f32",
+                                 "shape": "fused"}])
+    return p, 4 * 96 * 72 * 72
+
+
+def test_second_wavefield_sets_give_way(ews):
+    """The set that a simulation keeps for the fused step makes no call fail:
+    another simulation that does not fit beside it gets its memory, and a run
+    that finds no room for one takes the two passes (to the rounding of the
+    two kernels, 1e-6).  A shape asked for by name still fails."""
+    p, field = fused_problem(ews, 11)
+    a = ews.simulation_for(p)
+    a.set_tile_shape("32x8")
+    a.run(p.nt, p.dt)                                  # the seismogram buffer of host runs
+    a.set_tile_shape("auto")
+    before = ews.ews_memory_in_use()
+    want = a.run(p.nt, p.dt)
+    assert a.tile_shape == "fused" and ews.ews_memory_in_use() == before + 9 * field
+    try:
+        ews.ews_set_memory_limit(ews.ews_memory_in_use() + 4 * field)
+        b = ews.simulation_for(p)                      # 12 fields: the set's 9 and 3 of the 4
+        assert rel(b.run(p.nt, p.dt), want) <= 1e-6 and b.tile_shape == "32x8"
+        assert rel(a.run(p.nt, p.dt), want) <= 1e-6 and a.tile_shape == "32x8"
+        b.set_tile_shape("fused")
+        with pytest.raises(ews.EwsError) as e:
+            b.run(p.nt, p.dt)
+        assert e.value.status == ews.EWS_ENOMEM
+    finally:
+        ews.ews_set_memory_limit(-1)
+    assert np.array_equal(a.run(p.nt, p.dt), want) and a.tile_shape == "fused"
+    a.release_workspace()                              # frees the set
+    b.close()
+    assert ews.ews_memory_in_use() <= before
+    assert np.array_equal(a.run(p.nt, p.dt), want)
+    # the gradient's working memory gets the set as well
+    obs = np.zeros_like(want)
+    try:
+        ews.ews_set_memory_limit(before + 9 * field + (1 << 16))
+        with pytest.raises(ews.EwsError) as e:         # more than the set
+            a.gradient(p.nt, p.dt, obs, ckpt_every=10)
+        assert e.value.status == ews.EWS_ENOMEM
+        assert ews.ews_memory_in_use() < before + 9 * field
+    finally:
+        ews.ews_set_memory_limit(-1)
+    assert np.array_equal(a.run(p.nt, p.dt), want)
+
+
+def test_sets_are_taken_between_the_runs_of_another_thread(ews):
+    """One thread runs the fused step while another creates simulations that
+    take its set back whenever no run is using it: every run gives the same."""
+    import threading
+    p, field = fused_problem(ews, 12)
+    a = ews.simulation_for(p)
+    want = a.run(p.nt, p.dt)
+    stop, bad, shapes = threading.Event(), [], set()
+
+    def runs():
+        while not stop.is_set() and not bad:
+            try:
+                got = a.run(p.nt, p.dt)
+            except ews.EwsError as e:
+                bad.append(e)
+                return
+            shapes.add(a.tile_shape)
+            if rel(got, want) > 1e-6:
+                bad.append(rel(got, want))
+
+    t = threading.Thread(target=runs)
+    try:
+        ews.ews_set_memory_limit(ews.ews_memory_in_use() + 40 * field)   # a quarter holds a set
+        t.start()
+        for _ in range(30):
+            held = []
+            while len(held) < 8:                       # at most three fit
+                try:
+                    held.append(ews.Simulation(96, 72, 72, p.spacing, boundary="sponge", width=6))
+                except ews.EwsError as e:
+                    assert e.status == ews.EWS_ENOMEM
+                    break
+            assert 3 <= len(held) < 8
+            for s in held:
+                s.close()
+    finally:
+        stop.set()
+        t.join()
+        ews.ews_set_memory_limit(-1)
+        ews.ews_tile_tuning_clear()
+    assert not bad and "fused" in shapes
