@@ -424,15 +424,20 @@ typedef struct {
     double misfit;            /* out: J = dt/2 sum (seis - observed)^2                */
 } ews_batch_shot;
 
-enum { EWS_BATCH_PERSISTENT = 0, EWS_BATCH_SEQUENTIAL = 1 };
+enum { EWS_BATCH_PERSISTENT = 0, EWS_BATCH_SEQUENTIAL = 1, EWS_BATCH_ONE_BY_ONE = 2 };
 
 typedef struct {
-    int mode;                 /* EWS_BATCH_PERSISTENT, or EWS_BATCH_SEQUENTIAL: each
+    int mode;                 /* EWS_BATCH_PERSISTENT; EWS_BATCH_SEQUENTIAL: each
                                * shot through ews_run / ews_gradient in turn (the
-                               * one-by-one reference)                                 */
+                               * reference); EWS_BATCH_ONE_BY_ONE: the shots one after
+                               * the other with one synchronisation at the end, what
+                               * EWS_BATCH_PERSISTENT does where that times faster (no
+                               * simulation may have profiling on)                     */
     int ckpt_every;           /* gradient checkpoint interval (0: 50)                 */
     int zchunk;               /* planes per tile in z; 0: picked per grid size by the
-                               * autotuner (timed trial launches; see the table below) */
+                               * autotuner (timed trial launches; see the table below).
+                               * Any option but ckpt_every set: always the launches of
+                               * all shots together                                    */
     int ctas_per_sm;          /* resident CTAs per SM to launch (0: as many as fit)   */
     int dep_wait_ms;          /* give-up time of one dependency wait (0: 4000 ms)     */
     int test_unsatisfiable;   /* testing only: the last item waits for an item that

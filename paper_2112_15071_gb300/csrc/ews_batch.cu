@@ -861,7 +861,7 @@ ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options*
     if (nshots <= 0 || !shots) return report(EWS_EINVAL, "no shots");
     ews_batch_options o{};
     if (opt) o = *opt;
-    if (o.mode != EWS_BATCH_PERSISTENT && o.mode != EWS_BATCH_SEQUENTIAL)
+    if (o.mode != EWS_BATCH_PERSISTENT && o.mode != EWS_BATCH_SEQUENTIAL && o.mode != EWS_BATCH_ONE_BY_ONE)
         return report(EWS_EINVAL, "unknown batch mode %d", o.mode);
     if (o.ckpt_every < 0 || o.zchunk < 0 || o.ctas_per_sm < 0 || o.dep_wait_ms < 0)
         return report(EWS_EINVAL, "negative batch option");
@@ -890,6 +890,8 @@ ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options*
             return report(EWS_EINVAL, "shot %d: fluid cells (mu = 0) are not batched", i);
         if (s->g.fs != kNoSurface) any_fs = true;
         if (s->g.cm[0]) return report(EWS_EINVAL, "shot %d: coarse medium grids are not batched", i);
+        if (s->profiling && o.mode == EWS_BATCH_ONE_BY_ONE)
+            return report(EWS_EINVAL, "shot %d: profiled simulations take the sequential mode", i);
     }
     const int K0 = o.ckpt_every > 0 ? o.ckpt_every : 50;
 
@@ -923,6 +925,7 @@ ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options*
         return EWS_OK;
     }
 
+    if (o.mode == EWS_BATCH_ONE_BY_ONE) return batch_one_by_one(nshots, shots, K0, st);
     // explicit executor options ask for the executor; so do profiled
     // simulations (their launches would be counted) and FP16 checkpoints,
     // which it keeps in FP32

@@ -76,7 +76,7 @@ class ews_tuned_tile(C.Structure):
                 ("storage", C.c_int), ("shape", C.c_int)]
 
 
-EWS_BATCH_PERSISTENT, EWS_BATCH_SEQUENTIAL = 0, 1
+EWS_BATCH_PERSISTENT, EWS_BATCH_SEQUENTIAL, EWS_BATCH_ONE_BY_ONE = 0, 1, 2
 EWS_TILE_AUTO, EWS_TILE_32X8, EWS_TILE_32X4, EWS_TILE_32X16, EWS_TILE_FUSED = 0, 1, 2, 3, 4
 TILE = {"auto": EWS_TILE_AUTO, "32x8": EWS_TILE_32X8, "32x4": EWS_TILE_32X4,
         "32x16": EWS_TILE_32X16, "fused": EWS_TILE_FUSED}

@@ -1,4 +1,6 @@
-"""Batched shots in one persistent launch (ews_batch).
+"""Batched shots (ews_batch): in persistent launches of the executor, or one
+after the other where that times faster; tests meant for one of the two ask
+for it and check, by the simulations' launch counts, that it ran.
 
 The executor runs the same stencil, source, receiver and adjoint work items
 as ews_run / ews_gradient, scheduled by per-shot dependency counters; so
@@ -48,6 +50,19 @@ def shots_for(ews, probs, grad=False, obs=None):
     return out
 
 
+# The two ways through ews_batch: all shots in the executor's launches (any
+# option but ckpt_every asks for them), or one after the other.
+ROUTES = {"executor": lambda ews: {"zchunk": 12}, "one_by_one": lambda ews: {"mode": ews.EWS_BATCH_ONE_BY_ONE}}
+
+
+def took(shots, route):
+    """Each simulation counts the launches of its own time loop, the
+    executor's are no simulation's."""
+    for d in shots:
+        n = d["sim"].profile(reset=True)[1].sum()
+        assert n == 0 if route == "executor" else n > 0
+
+
 def problems(kinds=("moment", "force", "moment"), nts=(70, 45, 90)):
     dims = [(40, 36, 28), (70, 45, 37), (33, 65, 40)]
     return [synth.small_problem(*dims[i], nt=nts[i], boundary="sponge", width=5, kind=kinds[i],
@@ -71,7 +86,8 @@ def test_forward_batch_matches_run(ews, zchunk, ctas):
         assert rel(d["sim"].get_state(), ref.get_state()) <= 1e-6
 
 
-def test_gradient_batch_matches_one_by_one(ews, orc):
+@pytest.mark.parametrize("route", ROUTES)
+def test_gradient_batch_matches_one_by_one(ews, orc, route):
     import torch
     probs = problems(kinds=("moment", "force"), nts=(60, 75))
     rng = np.random.default_rng(2)
@@ -80,7 +96,8 @@ def test_gradient_batch_matches_one_by_one(ews, orc):
     a = shots_for(ews, probs, grad=True, obs=obs)
     b = shots_for(ews, probs, grad=True, obs=obs)
     a[1]["sim"].set_history_budget(0)         # one shot recomputes its segments
-    ma = ews.ews_batch(a, ckpt_every=20)
+    ma = ews.ews_batch(a, ckpt_every=20, **ROUTES[route](ews))
+    took(a, route)
     mb = ews.ews_batch(b, mode=ews.EWS_BATCH_SEQUENTIAL, ckpt_every=20)
     torch.cuda.synchronize()
     for i in range(len(probs)):
@@ -88,20 +105,22 @@ def test_gradient_batch_matches_one_by_one(ews, orc):
         assert rel(a[i]["seis"].cpu().numpy(), b[i]["seis"].cpu().numpy()) <= 1e-6
         for k in ("g_lam", "g_mu", "g_rho"):
             assert rel(a[i][k].cpu().numpy(), b[i][k].cpu().numpy()) <= 1e-5, (i, k)
-    # and against the FP64 adjoint of the oracle for the first shot
-    p = probs[0]
-    seis = orc.run_problem(p)
-    want = orc.gradient(p, p.dt * (seis - obs[0].astype(np.float64)), ckpt_every=20)
-    for q, k in enumerate(("g_lam", "g_mu", "g_rho")):
-        assert rel(a[0][k].cpu().numpy(), want[q]) <= 1e-4
+    # and against the FP64 adjoint of the oracle
+    for i, p in enumerate(probs):
+        seis = orc.run_problem(p)
+        want = orc.gradient(p, p.dt * (seis - obs[i].astype(np.float64)), ckpt_every=20)
+        for q, k in enumerate(("g_lam", "g_mu", "g_rho")):
+            assert rel(a[i][k].cpu().numpy(), want[q]) <= 1e-4, (i, k)
 
 
-def test_mixed_forward_and_gradient_shots(ews, orc):
+@pytest.mark.parametrize("route", ROUTES)
+def test_mixed_forward_and_gradient_shots(ews, orc, route):
     import torch
     probs = problems(kinds=("moment", "force"), nts=(50, 40))
     obs = [orc.run_problem(probs[0]).astype(np.float32) * 1.1]
     shots = shots_for(ews, probs[:1], grad=True, obs=obs) + shots_for(ews, probs[1:])
-    ews.ews_batch(shots, ckpt_every=16)
+    ews.ews_batch(shots, ckpt_every=16, **ROUTES[route](ews))
+    took(shots, route)
     torch.cuda.synchronize()
     want = ews.simulation_for(probs[1]).run(probs[1].nt, probs[1].dt)
     assert rel(shots[1]["seis"].cpu().numpy(), want) <= 1e-6
@@ -109,6 +128,22 @@ def test_mixed_forward_and_gradient_shots(ews, orc):
     mis, g = sim.gradient(probs[0].nt, probs[0].dt, obs[0], ckpt_every=16)
     for q, k in enumerate(("g_lam", "g_mu", "g_rho")):
         assert rel(shots[0][k].cpu().numpy(), g[q]) <= 1e-5
+
+
+@pytest.mark.parametrize("route", ROUTES)
+def test_forward_batch_matches_the_oracle(ews, orc, route):
+    import torch
+    probs = problems()
+    shots = shots_for(ews, probs)
+    own = torch.cuda.Stream()
+    for d in shots:
+        d["sim"].set_stream(own.cuda_stream)
+    ews.ews_batch(shots, **ROUTES[route](ews))
+    took(shots, route)
+    for p, d in zip(probs, shots):
+        assert rel(d["seis"].cpu().numpy(), orc.run_problem(p)) <= 1e-5
+        # the simulation is usable on its own stream again
+        assert rel(d["sim"].run(p.nt, p.dt), d["seis"].cpu().numpy()) <= 1e-6
 
 
 def test_validation(ews):
@@ -163,13 +198,13 @@ def test_batched_gradient_with_bf16_checkpoints(ews):
         for d in shots:
             d["sim"].set_checkpoint_storage("bf16")
             d["sim"].set_history_budget(0)
-        ews.ews_batch(shots, ckpt_every=15, mode=mode)
+        ews.ews_batch(shots, ckpt_every=15, mode=mode, **({} if mode else ROUTES["executor"](ews)))
         torch.cuda.synchronize()
         runs.append(shots)
     f32 = shots_for(ews, probs, grad=True, obs=obs)
     for d in f32:
         d["sim"].set_history_budget(0)
-    ews.ews_batch(f32, ckpt_every=15)
+    ews.ews_batch(f32, ckpt_every=15, **ROUTES["executor"](ews))
     torch.cuda.synchronize()
     a, b = runs
     for i in range(len(probs)):

@@ -162,7 +162,7 @@ def test_gradient_batch_runs_in_waves_under_the_limit(ews):
     per_shot = (17 + 16 + 18 + 63 + 4) * field
     try:
         ews.ews_set_memory_limit(ews.ews_memory_in_use() + 2.5 * per_shot)
-        ma = ews.ews_batch(a, ckpt_every=20)
+        ma = ews.ews_batch(a, ckpt_every=20, zchunk=12)      # the executor's waves
         torch.cuda.synchronize()
         for d in a:                                    # the last wave's state
             d["sim"].release_workspace()
@@ -192,6 +192,8 @@ def test_second_wavefield_sets_give_way(ews):
     another simulation that does not fit beside it gets its memory, and a run
     that finds no room for one takes the two passes (to the rounding of the
     two kernels, 1e-6).  A shape asked for by name still fails."""
+    import gc
+    gc.collect()                                       # simulations of other tests
     p, field = fused_problem(ews, 11)
     a = ews.simulation_for(p)
     a.set_tile_shape("32x8")
@@ -232,7 +234,9 @@ def test_second_wavefield_sets_give_way(ews):
 def test_sets_are_taken_between_the_runs_of_another_thread(ews):
     """One thread runs the fused step while another creates simulations that
     take its set back whenever no run is using it: every run gives the same."""
+    import gc
     import threading
+    gc.collect()                                       # simulations of other tests
     p, field = fused_problem(ews, 12)
     a = ews.simulation_for(p)
     want = a.run(p.nt, p.dt)
@@ -255,13 +259,13 @@ def test_sets_are_taken_between_the_runs_of_another_thread(ews):
         t.start()
         for _ in range(30):
             held = []
-            while len(held) < 8:                       # at most three fit
+            while len(held) < 40:                      # three or four fit
                 try:
                     held.append(ews.Simulation(96, 72, 72, p.spacing, boundary="sponge", width=6))
                 except ews.EwsError as e:
                     assert e.status == ews.EWS_ENOMEM
                     break
-            assert 3 <= len(held) < 8
+            assert 3 <= len(held) <= 4
             for s in held:
                 s.close()
     finally:

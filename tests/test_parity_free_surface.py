@@ -121,7 +121,7 @@ def test_surface_batched_forward(ews, orc):
     for p in probs:
         shots.append({"sim": ews.simulation_for(p), "nt": p.nt, "dt": p.dt,
                       "seis": torch.zeros((3, p.rec_pos.shape[0], p.nt), device="cuda")})
-    ews.ews_batch(shots)
+    ews.ews_batch(shots, zchunk=12)                    # the executor
     torch.cuda.synchronize()
     for p, d in zip(probs, shots):
         want = orc.run_problem(p)
@@ -176,7 +176,7 @@ def test_surface_batched_gradient(ews):
     a = shots()
     rng = np.random.default_rng(5)
     b = shots()
-    ews.ews_batch(a, ckpt_every=20)
+    ews.ews_batch(a, ckpt_every=20, zchunk=12)         # the executor
     ews.ews_batch(b, ckpt_every=20, mode=ews.EWS_BATCH_SEQUENTIAL)
     torch.cuda.synchronize()
     for i in range(len(probs)):

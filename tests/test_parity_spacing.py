@@ -161,7 +161,7 @@ def test_batched_forward_unequal_spacing(ews, orc):
                                  nrec=6, seed=42, spacing=SPACINGS[1])]
     shots = [{"sim": ews.simulation_for(p), "nt": p.nt, "dt": p.dt,
               "seis": torch.zeros((3, p.rec_pos.shape[0], p.nt), device="cuda")} for p in probs]
-    ews.ews_batch(shots)
+    ews.ews_batch(shots, zchunk=12)                    # the executor
     torch.cuda.synchronize()
     for p, d in zip(probs, shots):
         assert rel(d["seis"].cpu().numpy(), orc.run_problem(p)) <= TOL
