@@ -477,16 +477,19 @@ ews_status choose_batch_chunks(const ews_batch_shot* shots, int nshots, const st
 // Time one by one over time together, under g_tune_mu:
 std::map<std::vector<std::tuple<int, int, int, int, int>>, float> g_one_by_one;
 
-// Runs the simulations of a batch on its stream; their own come back after.
+// Runs the simulations of a batch on its stream; their own come back after,
+// once what was enqueued is done (also where a call in between failed).
 struct StreamSwap {
     std::vector<std::pair<ews_sim*, cudaStream_t>> own;
-    StreamSwap(const ews_batch_shot* shots, int n, cudaStream_t st) {
+    cudaStream_t st;
+    StreamSwap(const ews_batch_shot* shots, int n, cudaStream_t stream) : st(stream) {
         for (int i = 0; i < n; ++i) {
             own.emplace_back(shots[i].sim, shots[i].sim->stream);
             shots[i].sim->stream = st;
         }
     }
     ~StreamSwap() {
+        cudaStreamSynchronize(st);
         for (auto& o : own) o.first->stream = o.second;
     }
 };
