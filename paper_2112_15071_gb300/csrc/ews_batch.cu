@@ -937,10 +937,21 @@ ews_status ews_batch(int nshots, ews_batch_shot* shots, const ews_batch_options*
         plain = plain && !shots[i].sim->profiling &&
                 !(shots[i].observed && shots[i].sim->ckpt_pref == EWS_STORAGE_F16);
     if (plain) {
+        std::vector<ews_sim*> bare;            // hold no second wavefield set yet
+        for (int i = 0; i < nshots; ++i)
+            if (!shots[i].sim->fields2) bare.push_back(shots[i].sim);
         bool alone = false;
         ews_status r = prefer_one_by_one(shots, nshots, bnd, any_fs, grad, st, &alone);
-        if (r != EWS_OK) return r;
-        if (alone) return batch_one_by_one(nshots, shots, K0, st);
+        if (r == EWS_OK && alone) {
+            r = batch_one_by_one(nshots, shots, K0, st);
+            if (r != EWS_ENOMEM) return r;
+            for (int i = 0; i < nshots; ++i)
+                if (shots[i].observed && (r = ews_release_workspace(shots[i].sim)) != EWS_OK) return r;
+        }
+        // the executor needs no second sets: those of the trial go, and where
+        // memory was short it may still run
+        for (ews_sim* s : bare) sim_drop_set(s);
+        if (r != EWS_OK && r != EWS_ENOMEM) return r;
     }
     if (!grad) return batch_persistent(nshots, shots, o, bnd, false, any_fs, st);
     std::vector<int> all(nshots);

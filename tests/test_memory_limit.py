@@ -184,6 +184,8 @@ def fused_problem(ews, seed):
     p = synth.small_problem(96, 72, 72, nt=30, boundary="sponge", width=6, seed=seed, kind="moment")
     ews.ews_tile_tuning_import([{"nx": 96, "ny": 72, "nz": 72, "boundary": "sponge", "storage": "f32",
                                  "shape": "fused"}])
+    # receivers that the wave reaches within the run
+    p.rec_pos = np.array([p.src_pos + np.array(o) * p.spacing for o in ([3.2, 1.1, 0.4], [-2.3, 2.6, 3.9])])
     return p, 4 * 96 * 72 * 72
 
 
@@ -274,3 +276,57 @@ def test_sets_are_taken_between_the_runs_of_another_thread(ews):
         ews.ews_set_memory_limit(-1)
         ews.ews_tile_tuning_clear()
     assert not bad and "fused" in shapes
+
+
+def test_batch_without_room_for_second_sets(ews):
+    """Shots that would run one by one with the fused step, where the memory
+    limit leaves no room for its second wavefield sets: the batch runs all the
+    same, and keeps none of the memory of its trial."""
+    import torch
+    import gc
+    gc.collect()
+    p, field = fused_problem(ews, 13)
+    ews.ews_batch_tuning_clear()
+    try:
+        want = ews.simulation_for(p).run(p.nt, p.dt)
+        for shape in ("fused", "auto"):                # by name (ENOMEM alone), from the table
+            shots = [{"sim": ews.simulation_for(p), "nt": p.nt, "dt": p.dt,
+                      "seis": torch.zeros((3, p.rec_pos.shape[0], p.nt), device="cuda")}
+                     for _ in range(2)]
+            for d in shots:
+                d["sim"].set_tile_shape(shape)
+            before = ews.ews_memory_in_use()
+            ews.ews_set_memory_limit(before + 8 * field)
+            ews.ews_batch(shots)
+            ews.ews_set_memory_limit(-1)
+            for d in shots:
+                assert rel(d["seis"].cpu().numpy(), want) <= 1e-6
+            assert ews.ews_memory_in_use() == before
+            ews.ews_batch_tuning_clear()
+    finally:
+        ews.ews_set_memory_limit(-1)
+        ews.ews_batch_tuning_clear()
+        ews.ews_tile_tuning_clear()
+
+
+@pytest.mark.parametrize("mode", ["default", "one_by_one"])
+def test_batch_trial_keeps_no_set_where_the_executor_wins(ews, mode):
+    """A batch leaves its simulations a second wavefield set only where it ran
+    them with the fused step."""
+    import torch
+    p, field = fused_problem(ews, 14)
+    ews.ews_batch_tuning_clear()
+    shots = [{"sim": ews.simulation_for(p), "nt": p.nt, "dt": p.dt,
+              "seis": torch.zeros((3, p.rec_pos.shape[0], p.nt), device="cuda")} for _ in range(3)]
+    before = ews.ews_memory_in_use()
+    try:
+        kw = {} if mode == "default" else {"mode": ews.EWS_BATCH_ONE_BY_ONE}
+        ews.ews_batch(shots, **kw)
+        ran = [d["sim"].profile(reset=True)[1] for d in shots]
+        ews.ews_batch(shots, **kw)                     # the cached choice
+        alone = [d["sim"].profile(reset=True)[1].sum() > 0 for d in shots]
+        assert len(set(alone)) == 1 and (mode == "default" or all(alone)), ran
+        assert ews.ews_memory_in_use() == before + (27 * field if alone[0] else 0)
+    finally:
+        ews.ews_batch_tuning_clear()
+        ews.ews_tile_tuning_clear()
