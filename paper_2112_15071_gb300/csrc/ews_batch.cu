@@ -14,6 +14,7 @@
 #include <vector>
 
 #include "ews_sim.cuh"
+#include "ews_tuner.cuh"
 
 namespace ews {
 namespace {
@@ -475,7 +476,7 @@ ews_status choose_batch_chunks(const ews_batch_shot* shots, int nshots, const st
 // gradient shots 13 %, because their reverse passes gain from running together
 // (8 shots of 128^3: forward 1.06x one by one, gradients 0.65 / 0.74 s).
 // Time one by one over time together, under g_tune_mu:
-std::map<std::vector<std::tuple<int, int, int, int, int>>, float> g_one_by_one;
+std::map<std::vector<int>, float> g_one_by_one;
 
 // Runs the simulations of a batch on its stream; their own come back after,
 // once what was enqueued is done (also where a call in between failed).
@@ -499,12 +500,15 @@ ews_status prefer_one_by_one(const ews_batch_shot* shots, int nshots, int bnd, b
     const float limit = grad ? 0.87f : 0.97f;
     *out = false;
     const int exec = any_fs ? BX_LEAN_FS : BX_LEAN;
-    std::vector<std::tuple<int, int, int, int, int>> key;
+    int T = 6, dev = 0;
+    std::vector<std::array<int, 4>> forms;
     for (int i = 0; i < nshots; ++i) {
         const ews_sim* s = shots[i].sim;
-        key.emplace_back(s->g.nx, s->g.ny, s->g.nz, bnd, exec);
+        T = std::min(T, shots[i].nt);
+        forms.push_back({s->g.nx, s->g.ny, s->g.nz, s->tile_req});
     }
-    std::sort(key.begin(), key.end());
+    BCK(cudaGetDevice(&dev));
+    const std::vector<int> key = batch_key(std::move(forms), bnd, exec, T, dev);
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_one_by_one.find(key);
@@ -513,8 +517,6 @@ ews_status prefer_one_by_one(const ews_batch_shot* shots, int nshots, int bnd, b
             return EWS_OK;
         }
     }
-    int T = 6;
-    for (int i = 0; i < nshots; ++i) T = std::min(T, shots[i].nt);
     int* d_err = shots[0].sim->err;
     std::vector<int> zc(nshots);
     ews_status r;

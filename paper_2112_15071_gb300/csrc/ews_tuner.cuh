@@ -1,6 +1,8 @@
-// ews_tuner.cuh -- the tile tuner's choice among timed trials (host code only).
+// ews_tuner.cuh -- the tile tuner's choice among timed trials, and what the
+// choice of a batch is kept under (host code only).
 #pragma once
 #include <algorithm>
+#include <array>
 #include <cstddef>
 #include <vector>
 
@@ -29,6 +31,18 @@ int fastest_shape(const std::vector<int>& cand, int nt, Time time) {
         }
     }
     return best;
+}
+
+// What the choice between the executor and one shot after the other depends
+// on: the grids with the tile shape asked for each (nx, ny, nz, shape; in any
+// order), the boundary and the executor's form, the steps of the trial and the
+// device it was timed on.
+inline std::vector<int> batch_key(std::vector<std::array<int, 4>> shots, int boundary, int exec, int steps,
+                                  int device) {
+    std::sort(shots.begin(), shots.end());
+    std::vector<int> key = {boundary, exec, steps, device};
+    for (const auto& s : shots) key.insert(key.end(), s.begin(), s.end());
+    return key;
 }
 
 }  // namespace ews

@@ -1,7 +1,8 @@
-"""The tile tuner's choice among timed trials, with made-up timings (host
-code, compiled from the library's own header): every shape is timed over the
-same number of steps, whichever side of the half-millisecond line each one's
-trial falls on."""
+"""The tuner's host code, compiled from the library's own header.  The choice
+of a tile shape among timed trials, with made-up timings: every shape is timed
+over the same number of steps, whichever side of the half-millisecond line each
+one's trial falls on.  And what a batch's choice is kept under: everything it
+was timed with."""
 import ctypes
 import os
 import subprocess
@@ -24,17 +25,29 @@ extern "C" int choose(const float* us, int n, int nt, int stop_at, int* steps) {
         return true;
     });
 }
+extern "C" int same_key(const int* a, int na, const int* b, int nb) {
+    // boundary, exec, steps, device, then 4 numbers a shot
+    auto key = [](const int* p, int n) {
+        std::vector<std::array<int, 4>> s;
+        for (int k = 4; k + 3 < n; k += 4) s.push_back({p[k], p[k + 1], p[k + 2], p[k + 3]});
+        return ews::batch_key(s, p[0], p[1], p[2], p[3]);
+    };
+    return key(a, na) == key(b, nb);
+}
 """
 
 
 @pytest.fixture(scope="module")
-def choose(tmp_path_factory):
+def lib(tmp_path_factory):
     d = tmp_path_factory.mktemp("tuner")
     src, so = str(d / "choose.cc"), str(d / "choose.so")
     open(src, "w").write(SRC)
     subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, src, "-o", so], check=True)
-    lib = ctypes.CDLL(so)
+    return ctypes.CDLL(so)
 
+
+@pytest.fixture
+def choose(lib):
     def f(us, nt=100, stop_at=0):
         steps = (ctypes.c_int * len(us))()
         best = lib.choose((ctypes.c_float * len(us))(*us), len(us), nt, stop_at, steps)
@@ -61,3 +74,16 @@ def test_trials_end_with_the_run(choose):
     assert choose([10, 5], nt=9) == (2, [9, 9])
     # a trial that fails ends the choice
     assert choose([10, 5, 1], stop_at=2)[0] == 1
+
+
+def test_a_batch_choice_is_kept_under_all_it_depends_on(lib):
+    def same(a, b):
+        return bool(lib.same_key((ctypes.c_int * len(a))(*a), len(a), (ctypes.c_int * len(b))(*b), len(b)))
+    base = [1, 0, 6, 0, 96, 80, 64, 0, 48, 48, 48, 0]
+    assert same(base, base)
+    assert same(base, base[:4] + base[8:] + base[4:8])           # the shots in another order
+    for k in range(len(base)):                                   # any number another
+        assert not same(base, base[:k] + [base[k] + 1] + base[k + 1:]), k
+    assert not same(base, base + base[4:8]) and not same(base, base[:8])
+    # the shape asked for belongs to its grid
+    assert not same(base[:7] + [4] + base[8:], base[:11] + [4])
