@@ -577,7 +577,11 @@ ews_status batch_one_by_one(int nshots, ews_batch_shot* shots, int K, cudaStream
     for (int i = 0; i < nshots; ++i) {
         ews_batch_shot& b = shots[i];
         ews_sim* s = b.sim;
-        ews_status r;
+        // the same shape for every shot as in the trial, also from a kept choice
+        // (a gradient captures its history with the fused step only where that
+        // has its second set already)
+        ews_status r = sim_choose_tile(s, b.nt, b.dt);
+        if (r != EWS_OK) return r;
         if (b.observed) {
             // the executor's share of the automatic history budget
             const double budget = s->hist_budget;
@@ -594,7 +598,7 @@ ews_status batch_one_by_one(int nshots, ews_batch_shot* shots, int K, cudaStream
                 BCK(cudaMemcpyAsync(b.seis, s->aux, (size_t)3 * s->nrec * b.nt * sizeof(float),
                                     cudaMemcpyDeviceToDevice, st));
         } else {
-            if ((r = sim_choose_tile(s, b.nt, b.dt)) != EWS_OK || (r = ews_reset(s)) != EWS_OK ||
+            if ((r = ews_reset(s)) != EWS_OK ||
                 (r = sim_steps(s, 0, b.nt, b.dt, b.seis, b.nt)) != EWS_OK)
                 return r;
         }

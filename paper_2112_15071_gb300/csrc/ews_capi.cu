@@ -1153,7 +1153,12 @@ ews_status sim_ready(ews_sim* s, int n_end, double dt) { return ensure_ready(s, 
 
 DevSource sim_source(const ews_sim* s, double dt) { return source_taps(s, s->src, dt); }
 
-ews_status sim_choose_tile(ews_sim* s, int nt, double dt) { return choose_tile(s, nt, dt); }
+ews_status sim_choose_tile(ews_sim* s, int nt, double dt) {
+    const ews_status st = choose_tile(s, nt, dt);
+    if (st != EWS_OK || resident_eligible(s)) return st;
+    SetInUse use(s);
+    return plan_steps(s, false);
+}
 
 ews_status sim_steps(ews_sim* s, int n0, int nsteps, double dt, float* dseis, int ld) {
     return steps(s, s->src, n0, nsteps, dt, dseis, ld);

@@ -172,7 +172,7 @@ ews_status sim_adjoint_buffers(ews_sim* s, int nt, int nckpt, int hslots, bool w
 // Stencil plan of the adjoint fields with its history map on s->vhist.
 ews_status sim_adjoint_plan(ews_sim* s);
 // Tile shape of a run from rest (timed trials for a new grid, which leave the
-// wavefields to be reset), and steps of the time loop.
+// wavefields to be reset) with its plan, and steps of the time loop.
 ews_status sim_choose_tile(ews_sim* s, int nt, double dt);
 ews_status sim_steps(ews_sim* s, int n0, int nsteps, double dt, float* dseis, int ld);
 // Frees the second wavefield set of the fused step, if the simulation holds one.

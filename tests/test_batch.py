@@ -263,3 +263,31 @@ def test_imported_tuning_is_used_without_retuning(ews, tmp_path):
             assert rel(d["seis"].cpu().numpy(), want) <= 1e-6
     finally:
         ews.ews_batch_tuning_clear()
+
+
+def test_gradients_one_by_one_take_the_tuned_shape(ews):
+    """Shots that go one by one run the shape of the table, gradients too and
+    on simulations that have not run before: what the choice was timed with."""
+    import torch
+    p = synth.small_problem(96, 72, 72, nt=60, boundary="sponge", width=6, seed=91, nrec=4)
+    p.rec_pos = np.array([p.src_pos + (k + 1.3) * np.array(p.spacing) for k in range(4)])
+    ews.ews_tile_tuning_import([{"nx": 96, "ny": 72, "nz": 72, "boundary": "sponge", "storage": "f32",
+                                 "shape": "fused"}])
+    try:
+        grads = []
+        for _ in range(2):
+            obs = [np.ones((3, 4, p.nt), np.float32) * 1e-9] * 2
+            shots = shots_for(ews, [p, p], grad=True, obs=obs)
+            ews.ews_batch(shots, ckpt_every=10, mode=ews.EWS_BATCH_ONE_BY_ONE)
+            for d in shots:
+                assert d["sim"].tile_shape == "fused"
+                n = d["sim"].profile()[1]
+                assert n[ews.EWS_KERNEL_STEP] == p.nt and n[ews.EWS_KERNEL_VELOCITY] == 0
+            grads.append(shots[1]["g_mu"].cpu().numpy())
+        assert np.linalg.norm(grads[0]) > 0 and rel(grads[1], grads[0]) <= 1e-6
+        sim = ews.simulation_for(p)
+        sim.set_tile_shape("32x8")
+        want = sim.gradient(p.nt, p.dt, obs[0], ckpt_every=10)[1]
+        assert rel(grads[0], want[1]) <= 1e-6
+    finally:
+        ews.ews_tile_tuning_clear()
