@@ -342,12 +342,15 @@ enum {
     EWS_KERNEL_RECORD = 3,     /* receiver sampling, Sec. 2.4                  */
     EWS_KERNEL_POINTS = 4,     /* moment injection + receivers in one launch   */
     EWS_KERNEL_STEP = 5,       /* velocity + stress passes in one launch       */
+    EWS_KERNEL_LOOP = 6,       /* all steps of a call on a small grid          */
     EWS_NKERNEL = 8
 };
 
-/* When on, every kernel launch of the simulation is bracketed by CUDA
- * events on its stream and its duration accumulated per class.  Launch
- * counts are accumulated whether or not timing is on. */
+/* When on, every kernel launch of the time loop is bracketed by CUDA
+ * events on its stream and its duration accumulated per class; a small grid
+ * then runs the passes, step by step, instead of EWS_KERNEL_LOOP.  Launch
+ * counts are accumulated whether or not timing is on.  The launches of a
+ * reverse sweep and of ews_batch's executor are not counted. */
 ews_status ews_set_profiling(ews_sim* sim, int on);
 
 /* Accumulated milliseconds and launch counts per kernel class since the

@@ -658,8 +658,7 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
 }
 
 // Steps n0 .. n0 + nsteps - 1 of a small grid with the fields resident in
-// shared memory, one launch per res_chunk steps.  Accounted like the passes
-// it runs: per step one velocity pass, one stress pass and the point terms.
+// shared memory, one launch per res_chunk steps (and one of the receivers).
 bool resident_eligible(const ews_sim* s) {
     return s->res && s->tile_req == EWS_TILE_AUTO && !s->profiling;
 }
@@ -710,14 +709,8 @@ ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps,
         // v^{n+1/2} of step n0 + m goes to slot m + 1 of the history
         r.vcap = vcap ? vcap + (size_t)(m + 1) * 3 * s->fstride : nullptr;
         CK(launch_resident(r, s->stream));
-    }
-    s->launches[EWS_KERNEL_VELOCITY] += nsteps;
-    s->launches[EWS_KERNEL_STRESS] += nsteps;
-    if (S.kind == EWS_SOURCE_MOMENT && rec) {
-        s->launches[EWS_KERNEL_POINTS] += nsteps;
-    } else {
-        if (S.kind >= 0) s->launches[EWS_KERNEL_INJECT] += nsteps;
-        if (rec) s->launches[EWS_KERNEL_RECORD] += nsteps;
+        s->launches[EWS_KERNEL_LOOP] += 1;
+        if (rec) s->launches[EWS_KERNEL_RECORD] += 1;
     }
     return EWS_OK;
 }

@@ -259,6 +259,7 @@ def test_graph_replay_equals_direct_launches(ews):
     from paper_2112_15071_gb300 import synth
     p = synth.small_problem(70, 45, 37, nt=80, boundary="cpml", width=6, kind="force", seed=9)
     sim = ews.simulation_for(p)
+    sim.set_tile_shape("32x8")                   # not the one launch that small grids take
     a = sim.run(p.nt, p.dt)
     sa = sim.get_state()
     b = sim.run(p.nt, p.dt)                      # replay of the cached graph

@@ -88,6 +88,26 @@ def test_chunks_and_staged_receivers(ews):
     assert np.array_equal(seis, a[0]) and np.array_equal(sim.get_state(), a[1])
 
 
+def test_launches_are_counted_as_they_are(ews):
+    """One launch, and one of the receivers, for as many steps as the staging
+    holds; none of the passes."""
+    for nrec, calls in ((5, 1), (1500, 3)):            # 4 MiB hold 29 steps of 1500 receivers
+        p = synth.small_problem(40, 36, 28, nt=70, boundary="sponge", kind="moment", width=5, seed=308,
+                                nrec=nrec)
+        sim = ews.simulation_for(p)
+        sim.run(p.nt, p.dt)
+        ms, n = sim.profile(reset=True)
+        assert n[ews.EWS_KERNEL_LOOP] == calls and n[ews.EWS_KERNEL_RECORD] == calls
+        assert n.sum() == 2 * calls
+        sim.advance(0, 10, p.dt, None, 10)             # nothing recorded
+        n = sim.profile(reset=True)[1]
+        assert n[ews.EWS_KERNEL_LOOP] == 1 and n.sum() == 1
+        sim.set_profiling(True)                        # the passes, one by one
+        sim.run(p.nt, p.dt)
+        n = sim.profile()[1]
+        assert n[ews.EWS_KERNEL_VELOCITY] == p.nt and n[ews.EWS_KERNEL_LOOP] == 0
+
+
 # blocks of at most 4 planes (a thread per cell), of 5 to 8 (4 cells per thread)
 @pytest.mark.parametrize("n", [(12, 11, 10), (33, 18, 17), (16, 47, 33), (64, 60, 61)])
 @pytest.mark.parametrize("boundary", ["none", "sponge"])
