@@ -291,7 +291,10 @@ ews_status ews_get_field_scales(ews_sim* sim, float* scale);
  * With EWS_TILE_AUTO (the default), ews_run picks the shape for its grid
  * size, boundary and storage type from a per-process table, filling a missing
  * entry by timing a few steps with each shape before the run (the wavefields
- * are reset afterwards).  Plain forward steps use it; runs with a free surface
+ * are reset afterwards).  FP32 grids of up to about 467 000 cells (fewer with
+ * C-PML) have no use for it: their whole time loop runs in one launch with
+ * the fields resident on the SMs, unless a shape is asked for by name or
+ * per-launch profiling is on.  Plain forward steps use it; runs with a free surface
  * or a coarse medium grid keep 32 x 8, and so do the steps of an adjoint or
  * gradient that write the velocity history, unless the simulation holds the
  * fused step's second set from an earlier run.
@@ -305,13 +308,15 @@ enum {
     EWS_TILE_32X8 = 1,
     EWS_TILE_32X4 = 2,
     EWS_TILE_32X16 = 3,
-    EWS_TILE_FUSED = 4
+    EWS_TILE_FUSED = 4,
+    EWS_TILE_RESIDENT = 5         /* only reported, by ews_get_tile_shape          */
 };
 
 /* Use this shape for later runs (EWS_TILE_AUTO: the tuned one). */
 ews_status ews_set_tile_shape(ews_sim* sim, int shape);
 /* The shape the forward passes of the last run used (EWS_TILE_32X8 ..
- * EWS_TILE_FUSED). */
+ * EWS_TILE_FUSED), or EWS_TILE_RESIDENT: a small grid's time loop in one
+ * launch, which has no tiles. */
 int ews_get_tile_shape(ews_sim* sim);
 
 /* Tile-shape table, one entry per grid size, boundary and storage type;

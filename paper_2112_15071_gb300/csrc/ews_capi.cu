@@ -751,8 +751,8 @@ ews_status plan_steps(ews_sim* s, bool capture) {
 // them).
 ews_status steps(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
                  float* dseis, int ld, float* vcap = nullptr) {
-    if (resident_eligible(s) && nsteps > 0)
-        return steps_resident(s, src, n0, nsteps, dt, dseis, ld, vcap);
+    s->ran_loop = resident_eligible(s) && nsteps > 0;
+    if (s->ran_loop) return steps_resident(s, src, n0, nsteps, dt, dseis, ld, vcap);
     SetInUse use(s);
     // the shape's plan exists before a capture starts
     ews_status sp = plan_steps(s, vcap != nullptr);
@@ -836,6 +836,10 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
                                                                               : s->tile_req);
         return EWS_OK;
     }
+    if (resident_eligible(s)) {                 // no pass runs: nothing to look up or to time
+        set_tile_used(s, EWS_TILE_32X8);
+        return EWS_OK;
+    }
     const auto key = tile_key(s);
     {
         std::lock_guard<std::mutex> lk(g_tile_mu);
@@ -847,12 +851,6 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
         }
     }
     if (s->profiling) {
-        set_tile_used(s, EWS_TILE_32X8);
-        return EWS_OK;
-    }
-    if (resident_eligible(s)) {                 // the passes do not run: no trial
-        std::lock_guard<std::mutex> lk(g_tile_mu);
-        g_tile[key] = EWS_TILE_32X8;
         set_tile_used(s, EWS_TILE_32X8);
         return EWS_OK;
     }
@@ -1249,11 +1247,12 @@ ews_status ews_set_tile_shape(ews_sim* s, int shape) {
     if (shape < EWS_TILE_AUTO || shape > EWS_TILE_FUSED)
         return fail(EWS_EINVAL, "unknown tile shape %d", shape);
     s->tile_req = shape;
+    s->ran_loop = false;
     if (shape != EWS_TILE_AUTO) set_tile_used(s, tile_eligible(s) ? shape : EWS_TILE_32X8);
     return EWS_OK;
 }
 
-int ews_get_tile_shape(ews_sim* s) { return s ? s->tile_used : 0; }
+int ews_get_tile_shape(ews_sim* s) { return !s ? 0 : s->ran_loop ? EWS_TILE_RESIDENT : s->tile_used; }
 
 int ews_tile_tuned(const ews_grid* grid, int boundary, int storage) {
     if (!grid) return 0;

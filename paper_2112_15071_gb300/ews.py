@@ -80,6 +80,7 @@ EWS_BATCH_PERSISTENT, EWS_BATCH_SEQUENTIAL, EWS_BATCH_ONE_BY_ONE = 0, 1, 2
 EWS_TILE_AUTO, EWS_TILE_32X8, EWS_TILE_32X4, EWS_TILE_32X16, EWS_TILE_FUSED = 0, 1, 2, 3, 4
 TILE = {"auto": EWS_TILE_AUTO, "32x8": EWS_TILE_32X8, "32x4": EWS_TILE_32X4,
         "32x16": EWS_TILE_32X16, "fused": EWS_TILE_FUSED}
+EWS_TILE_RESIDENT = 5                  # reported only
 
 _lock = threading.Lock()
 _lib = None
@@ -484,7 +485,7 @@ def ews_batch_tuning_clear() -> None:
     load().ews_batch_tuning_clear()
 
 
-_TILE_NAMES = {v: k for k, v in TILE.items()}
+_TILE_NAMES = {EWS_TILE_RESIDENT: "resident", **{v: k for k, v in TILE.items()}}
 _STORAGE_NAMES = {v: k for k, v in STORAGE.items()}
 
 

@@ -175,8 +175,8 @@ def test_fused_falls_back_where_it_does_not_apply(ews):
 
 
 def test_tuner_keeps_the_second_set_only_when_it_picks_fused(ews):
-    p = synth.small_problem(64, 48, 40, nt=30, boundary="sponge", kind="moment", width=6,
-                            seed=209)
+    p = synth.small_problem(96, 72, 72, nt=30, boundary="sponge", kind="moment", width=6,
+                            seed=209)                    # beyond the one-launch time loop
     field = 4 * ((p.nx + 31) // 32 * 32) * p.ny * p.nz
     base = ews.ews_memory_in_use()
     s8 = ews.simulation_for(p)

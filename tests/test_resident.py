@@ -108,6 +108,34 @@ def test_launches_are_counted_as_they_are(ews):
         assert n[ews.EWS_KERNEL_VELOCITY] == p.nt and n[ews.EWS_KERNEL_LOOP] == 0
 
 
+def test_the_route_is_reported_and_leaves_the_table_alone(ews):
+    """Neither run nor table entry is one of the passes': nothing was timed."""
+    p = synth.small_problem(40, 36, 28, nt=20, boundary="sponge", kind="moment", width=5, seed=309)
+    key = (ews.ews_grid(p.nx, p.ny, p.nz, *p.spacing), "sponge", "f32")
+    ews.ews_tile_tuning_clear()
+    sim = ews.simulation_for(p)
+    sim.run(p.nt, p.dt)
+    assert sim.tile_shape == "resident" and ews.ews_tile_tuned(*key) == 0
+    entry = {"nx": p.nx, "ny": p.ny, "nz": p.nz, "boundary": "sponge", "storage": "f32", "shape": "32x4"}
+    ews.ews_tile_tuning_import([entry])                # of a run that took the passes
+    try:
+        sim.run(p.nt, p.dt)
+        assert sim.tile_shape == "resident" and ews.ews_tile_tuning_export() == [entry]
+        sim.set_profiling(True)
+        sim.run(p.nt, p.dt)
+        assert sim.tile_shape == "32x4"
+        sim.set_profiling(False)
+        sim.set_tile_shape("32x16")
+        assert sim.tile_shape == "32x16"
+        sim.run(p.nt, p.dt)
+        assert sim.tile_shape == "32x16"
+        with pytest.raises(ews.EwsError) as e:         # a report, not a request
+            sim.set_tile_shape(ews.EWS_TILE_RESIDENT)
+        assert e.value.status == ews.EWS_EINVAL
+    finally:
+        ews.ews_tile_tuning_clear()
+
+
 # blocks of at most 4 planes (a thread per cell), of 5 to 8 (4 cells per thread)
 @pytest.mark.parametrize("n", [(12, 11, 10), (33, 18, 17), (16, 47, 33), (64, 60, 61)])
 @pytest.mark.parametrize("boundary", ["none", "sponge"])

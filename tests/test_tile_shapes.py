@@ -73,8 +73,8 @@ def test_every_shape_matches_the_oracle(ews, orc, shape):
 
 def test_tuner_fills_the_table_without_changing_results(ews):
     ews.ews_tile_tuning_clear()
-    p = synth.small_problem(64, 48, 40, nt=50, boundary="sponge", kind="moment", width=6,
-                            seed=103)
+    p = synth.small_problem(96, 72, 72, nt=50, boundary="sponge", kind="moment", width=6,
+                            seed=103)                    # beyond the one-launch time loop
     g = ews.ews_grid(p.nx, p.ny, p.nz, *p.spacing)
     assert ews.ews_tile_tuned(g, "sponge", "f32") == 0
     sim = ews.simulation_for(p)                          # automatic shape
@@ -90,7 +90,7 @@ def test_tuner_fills_the_table_without_changing_results(ews):
 
 
 def test_imported_entry_is_used(ews):
-    p = synth.small_problem(40, 36, 28, nt=30, boundary="cpml", kind="force", width=5, seed=104)
+    p = synth.small_problem(96, 72, 72, nt=30, boundary="cpml", kind="force", width=5, seed=104)
     ews.ews_tile_tuning_import([{"nx": p.nx, "ny": p.ny, "nz": p.nz, "boundary": "cpml",
                                  "storage": "f32", "shape": "32x16"}])
     sim = ews.simulation_for(p)
