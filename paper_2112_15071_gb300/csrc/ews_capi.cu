@@ -660,7 +660,7 @@ ews_status steps_direct(ews_sim* s, const SourceSpec& src, int n0, int nsteps, d
 // Steps n0 .. n0 + nsteps - 1 of a small grid with the fields resident in
 // shared memory, one launch per res_chunk steps (and one of the receivers).
 bool resident_eligible(const ews_sim* s) {
-    return s->res && s->tile_req == EWS_TILE_AUTO && !s->profiling;
+    return s->res && (s->nrec == 0 || s->res_list) && s->tile_req == EWS_TILE_AUTO && !s->profiling;
 }
 ResidentRun resident_run(const ews_sim* s, const DevFields& F, double dt, int nrec, int ld) {
     ResidentRun r{};
@@ -1380,7 +1380,9 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
         return st;
     };
     // the wavefields; on small grids the halo inboxes of the resident time loop
-    // follow them in the same allocation (zero before the first launch, too)
+    // follow them in the same allocation (zero before the first launch, too).
+    // Where the loop's kernels or the inboxes are not to be had, the grid runs
+    // the passes.
     int sms = 0, coop = 0;
     ResidentPlan rp;
     size_t inbox = 0;
@@ -1388,14 +1390,19 @@ ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** ou
     if (s->wide() && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
         resident_plan(s->g, o.boundary, sms, &rp)) {
-        e = resident_prepare(rp, o.boundary);
-        if (e != cudaSuccess)
-            return cleanup(fail(EWS_ECUDA, "resident time loop: %s", cudaGetErrorString(e)));
-        s->res = new (std::nothrow) ResidentPlan(rp);
-        if (!s->res) return cleanup(fail(EWS_ENOMEM, "host allocation failed"));
-        inbox = resident_inbox_bytes(rp);
+        if (resident_prepare(rp, o.boundary) == cudaSuccess)
+            s->res = new (std::nothrow) ResidentPlan(rp);
+        else
+            (void)cudaGetLastError();          // not an error of the passes' launches
     }
+    if (s->res) inbox = resident_inbox_bytes(rp);
     e = dev_malloc((void**)&s->fields, fbytes + inbox);
+    if (e == cudaErrorMemoryAllocation && inbox) {
+        delete s->res;
+        s->res = nullptr;
+        inbox = 0;
+        e = dev_malloc((void**)&s->fields, fbytes);
+    }
     if (e != cudaSuccess) return cleanup(fail(EWS_ENOMEM, "wavefields: %s", cudaGetErrorString(e)));
     if (inbox) s->res_inbox = reinterpret_cast<unsigned long long*>((char*)s->fields + fbytes);
     e = dev_malloc((void**)&s->medium, 3 * s->fstride * sizeof(float));
@@ -1640,11 +1647,14 @@ ews_status ews_set_receivers(ews_sim* s, int nrec, const double* pos) {
             gb = s->res_chunk * row;
         }
         char* base = nullptr;
-        CK(dev_malloc((void**)&base, tb + lb + sb + gb));
+        cudaError_t e = dev_malloc((void**)&base, tb + lb + sb + gb);
+        const bool staged = e == cudaSuccess && s->res;
+        if (e == cudaErrorMemoryAllocation && s->res) e = dev_malloc((void**)&base, tb);   // for the passes
+        CK(e);
         s->rtaps = reinterpret_cast<Tap*>(base);
         CK(cudaMemcpyAsync(s->rtaps, taps.data(), taps.size() * sizeof(Tap),
                            cudaMemcpyHostToDevice, s->stream));
-        if (s->res) {
+        if (staged) {
             s->res_list = reinterpret_cast<int2*>(base + tb);
             s->res_start = reinterpret_cast<int*>(base + tb + lb);
             s->res_stage = reinterpret_cast<float*>(base + tb + lb + sb);

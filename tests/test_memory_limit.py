@@ -330,3 +330,39 @@ def test_batch_trial_keeps_no_set_where_the_executor_wins(ews, mode):
     finally:
         ews.ews_batch_tuning_clear()
         ews.ews_tile_tuning_clear()
+
+
+def test_small_grids_run_the_passes_where_the_loop_lacks_memory(ews):
+    """The one-launch time loop of small grids has inboxes beside the
+    wavefields and staging beside the receivers; what fitted the limit without
+    them still does, and runs the passes (equal bits)."""
+    import gc
+    gc.collect()
+    p = synth.small_problem(40, 36, 28, nt=40, boundary="sponge", width=5, seed=15, nrec=1500)
+    base = ews.ews_memory_in_use()
+    ref = ews.simulation_for(p)
+    took = ews.ews_memory_in_use() - base
+    want = ref.run(p.nt, p.dt)
+    assert np.abs(want).max() > 0 and ref.tile_shape == "resident"
+    ref.close()
+    base = ews.ews_memory_in_use()
+    field = 4 * 64 * 36 * 28                           # pitched rows of 64
+    seis = 4 * want.size
+    try:
+        # wavefields, medium, taps of 20 bytes and a little, but no inbox and no staging
+        ews.ews_set_memory_limit(base + 12 * field + 24 * 1500 * 20 + seis + (1 << 15))
+        assert took + seis > ews.ews_memory_limit() - base
+        sim = ews.simulation_for(p)
+        assert np.array_equal(sim.run(p.nt, p.dt), want) and sim.tile_shape != "resident"
+        sim.close()
+        ews.ews_set_memory_limit(-1)
+        sim = ews.simulation_for(p)                    # inboxes, but no staging
+        sim.set_receivers(p.rec_pos[:1])
+        ews.ews_set_memory_limit(ews.ews_memory_in_use() + 24 * 1500 * 20 + seis + (1 << 12))
+        sim.set_receivers(p.rec_pos)
+        assert np.array_equal(sim.run(p.nt, p.dt), want) and sim.tile_shape != "resident"
+        ews.ews_set_memory_limit(-1)
+        sim.set_receivers(p.rec_pos)
+        assert np.array_equal(sim.run(p.nt, p.dt), want) and sim.tile_shape == "resident"
+    finally:
+        ews.ews_set_memory_limit(-1)
