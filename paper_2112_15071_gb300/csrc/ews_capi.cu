@@ -67,6 +67,16 @@ constexpr double kC2 = -1.0 / 24.0;
 
 int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+// Receiver taps in one block up to which the resident loop serves them: their
+// block's CTA stages them one by one, and adds the residual to them with atomics
+// in the reverse sweep, while the others wait.  Forward, 100 steps, all receivers
+// in one block, loop / passes (GB300, ms, 32^3 and 64^3): 24 000 taps 0.71 / 1.21
+// and 0.97 / 1.39, 72 000 taps 1.30 / 1.21 and 1.64 / 1.39.  Gradient with the
+// reverse sweep in the loop / in the passes after a resident forward: 7200 taps
+// 3.66 / 4.10 (both in the passes), 9000 (one plane) 3.44 / 3.60, 15 000 4.27 /
+// 3.96, 24 000 7.31 / 3.64 (all 64^3), 24 000 6.11 / 3.12 (32^3).
+constexpr int kResidentTaps = 49152, kResidentAdjTaps = 8192;
+
 // Steps of one resident launch without receivers, and the bytes of staged tap
 // values one may fill with them (a launch costs about two steps).
 constexpr int kResidentSteps = 4096;
@@ -692,6 +702,10 @@ ews_status resident_epoch(ews_sim* s, ResidentRun* r, int nsteps) {
     s->res_epoch += (unsigned)nsteps;
     return EWS_OK;
 }
+// Whether steps that record, or not, run in it.
+bool resident_steps(const ews_sim* s, bool record) {
+    return resident_eligible(s) && (!record || s->res_taps <= kResidentTaps);
+}
 ews_status steps_resident(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
                           float* dseis, int ld, float* vcap) {
     const DevSource S = source_taps(s, src, dt);
@@ -751,7 +765,7 @@ ews_status plan_steps(ews_sim* s, bool capture) {
 // them).
 ews_status steps(ews_sim* s, const SourceSpec& src, int n0, int nsteps, double dt,
                  float* dseis, int ld, float* vcap = nullptr) {
-    s->ran_loop = resident_eligible(s) && nsteps > 0;
+    s->ran_loop = resident_steps(s, s->nrec > 0 && dseis) && nsteps > 0;
     if (s->ran_loop) return steps_resident(s, src, n0, nsteps, dt, dseis, ld, vcap);
     SetInUse use(s);
     // the shape's plan exists before a capture starts
@@ -836,7 +850,7 @@ ews_status choose_tile(ews_sim* s, int nt, double dt) {
                                                                               : s->tile_req);
         return EWS_OK;
     }
-    if (resident_eligible(s)) {                 // no pass runs: nothing to look up or to time
+    if (resident_steps(s, true)) {              // no pass runs: nothing to look up or to time
         set_tile_used(s, EWS_TILE_32X8);
         return EWS_OK;
     }
@@ -1057,7 +1071,7 @@ ews_status adjoint_core(ews_sim* s, int nt, double dt, int ckpt_every, const flo
                     return st;
             }
             // small grids: the range in one launch (per kResidentSteps)
-            const bool resident = resident_eligible(s) &&
+            const bool resident = resident_eligible(s) && s->res_taps <= kResidentAdjTaps &&
                                   resident_adjoint_supported(*s->res, s->g, s->opt.boundary);
             for (int e = n1; resident && e > n0; e -= kResidentSteps) {
                 ResidentRun r = resident_run(s, AF, -dt, s->nrec > 0 && sadj ? s->nrec : 0, nt);
@@ -1146,7 +1160,7 @@ DevSource sim_source(const ews_sim* s, double dt) { return source_taps(s, s->src
 
 ews_status sim_choose_tile(ews_sim* s, int nt, double dt) {
     const ews_status st = choose_tile(s, nt, dt);
-    if (st != EWS_OK || resident_eligible(s)) return st;
+    if (st != EWS_OK || resident_steps(s, true)) return st;
     SetInUse use(s);
     return plan_steps(s, false);
 }
@@ -1631,6 +1645,7 @@ ews_status ews_set_receivers(ews_sim* s, int nrec, const double* pos) {
     s->res_list = nullptr;
     s->res_start = nullptr;
     s->res_stage = nullptr;
+    s->res_taps = 0;
     if (nrec > 0) {
         // the taps; for the resident time loop, in the same allocation, the
         // taps by CTA and the staging rows
@@ -1642,6 +1657,7 @@ ews_status ews_set_receivers(ews_sim* s, int nrec, const double* pos) {
             resident_taps(*s->res, s->g, taps.data(), (int)taps.size(), &list, &start);
             const size_t row = taps.size() * sizeof(float);
             s->res_chunk = (int)std::min<size_t>(kResidentSteps, std::max<size_t>(16, kResidentStage / row));
+            for (size_t c = 0; c + 1 < start.size(); ++c) s->res_taps = std::max(s->res_taps, start[c + 1] - start[c]);
             lb = (list.size() * sizeof(int2) + 255) / 256 * 256;
             sb = (start.size() * sizeof(int) + 255) / 256 * 256;
             gb = s->res_chunk * row;

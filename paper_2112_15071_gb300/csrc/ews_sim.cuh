@@ -103,6 +103,7 @@ struct ews_sim {
     int* res_start = nullptr;
     float* res_stage = nullptr;
     int res_chunk = 0;
+    int res_taps = 0;             // receiver taps of the block with most
     bool ran_loop = false;        // the last steps ran in it
     cudaStream_t stream = nullptr;
     // launch accounting and optional per-launch event timing

@@ -88,6 +88,33 @@ def test_chunks_and_staged_receivers(ews):
     assert np.array_equal(seis, a[0]) and np.array_equal(sim.get_state(), a[1])
 
 
+# 24 taps a receiver, all in one block (16 x 16 x 8 cells of a 64^3 grid): up
+# to and beyond the lines of the reverse sweep (8192) and the forward loop (49152)
+@pytest.mark.parametrize("nrec", [341, 342, 2048, 2049])
+def test_crowded_receivers(ews, nrec):
+    """Receivers that share a block beyond what its CTA serves faster: the
+    passes take them, with equal bits forward; the gradient to the order in
+    which the residuals of one cell add up (2049 terms of like sign: about
+    sqrt(2049) roundings of 6e-8 either way) and the separately compiled
+    products: 1e-5."""
+    p = synth.small_problem(64, 64, 64, nt=45, boundary="sponge", kind="moment", width=4, seed=310)
+    p.src_pos = np.array([24.6, 24.2, 29.7]) * np.array(p.spacing)
+    rng = np.random.default_rng(8)
+    p.rec_pos = (np.array([23.0, 23.0, 27.0]) + rng.uniform(0.2, 0.4, (nrec, 3))) * np.array(p.spacing)
+    same(*both(ews, p))
+    sim = ews.simulation_for(p)
+    seis = sim.run(p.nt, p.dt)
+    assert sim.tile_shape == ("resident" if nrec <= 2048 else "32x8")
+    obs = (0.9 * seis).astype(np.float32)
+    a = sim.gradient(p.nt, p.dt, obs, ckpt_every=20)
+    sim.set_tile_shape("32x8")
+    b = sim.gradient(p.nt, p.dt, obs, ckpt_every=20)
+    assert a[0] == pytest.approx(b[0], rel=1e-6)
+    for q in range(3):
+        x, y = a[1][q].astype(np.float64), b[1][q].astype(np.float64)
+        assert 0 < np.linalg.norm(y) and np.linalg.norm(x - y) <= 1e-5 * np.linalg.norm(y), q
+
+
 def test_launches_are_counted_as_they_are(ews):
     """One launch, and one of the receivers, for as many steps as the staging
     holds; none of the passes."""
