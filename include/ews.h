@@ -291,13 +291,20 @@ ews_status ews_get_field_scales(ews_sim* sim, float* scale);
  * With EWS_TILE_AUTO (the default), ews_run picks the shape for its grid
  * size, boundary and storage type from a per-process table, filling a missing
  * entry by timing a few steps with each shape before the run (the wavefields
- * are reset afterwards).  FP32 grids of up to about 467 000 cells (fewer with
- * C-PML) have no use for it: their whole time loop runs in one launch with
- * the fields resident on the SMs, unless a shape is asked for by name or
- * per-launch profiling is on.  Plain forward steps use it; runs with a free surface
+ * are reset afterwards).  Plain forward steps use it; runs with a free surface
  * or a coarse medium grid keep 32 x 8, and so do the steps of an adjoint or
  * gradient that write the velocity history, unless the simulation holds the
  * fused step's second set from an earlier run.
+ * FP32 grids of up to about 467 000 cells (fewer with C-PML) have no use for
+ * the table: their whole time loop runs in one launch with the fields resident
+ * on the SMs, unless a shape is asked for by name, per-launch profiling is on,
+ * or one block of the grid (at most 16 x 16 x 12 cells) has more than about
+ * 2000 receivers; the passes give equal bits.  Such loops fill the GPU: those
+ * of several host threads run one after the other.  Alone they take less than
+ * half the passes' time; from six threads, on 24^3 to 56^3 cells, the passes
+ * take 0.56 to 0.90 of theirs (with 64^3 cells and more the loop stays
+ * ahead).  A program with many small runs at a time asks for EWS_TILE_32X8, or
+ * gives them to ews_batch.
  * The second set, of the automatic shape, takes at most a quarter of the
  * device memory free when it is allocated; without that room the run takes
  * 32 x 8.  The simulation keeps the set for its next run;

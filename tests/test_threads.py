@@ -60,3 +60,39 @@ def test_loops_are_captured_while_others_come_and_go(ews):
     assert not failed
     for k, g in enumerate(got):
         assert np.array_equal(g, want[k % len(dts)]), k
+
+
+@pytest.mark.parametrize("n,threads", [((24, 22, 20), 8), ((64, 60, 61), 3)])
+def test_small_grids_in_several_threads(ews, n, threads):
+    """One-launch loops, each with a CTA on most SMs, asked for on several
+    streams at once: every run and gradient as alone."""
+    import torch
+    p = synth.small_problem(*n, nt=40, boundary="sponge", width=4, seed=402)
+    ref = ews.simulation_for(p)
+    want = ref.run(p.nt, p.dt)
+    obs = (0.9 * want).astype(np.float32)
+    gwant = ref.gradient(p.nt, p.dt, obs, ckpt_every=15)[1]
+    sims = [ews.simulation_for(p) for _ in range(threads)]
+    streams = [torch.cuda.Stream() for _ in sims]
+    for s, st in zip(sims, streams):
+        s.set_stream(st.cuda_stream)
+    bad = []
+
+    def work(s):
+        try:
+            for _ in range(12):
+                if not np.array_equal(s.run(p.nt, p.dt), want):
+                    bad.append("run")
+                g = s.gradient(p.nt, p.dt, obs, ckpt_every=15)[1]
+                # products and residuals in either order: 1e-5 as elsewhere
+                bad.extend(q for q in range(3) if rel(g[q], gwant[q]) > 1e-5)
+        except ews.EwsError as e:
+            bad.append(e)
+
+    pool = [threading.Thread(target=work, args=(s,)) for s in sims]
+    for t in pool:
+        t.start()
+    for t in pool:
+        t.join()
+    assert not bad, bad
+    assert all(s.tile_shape == "resident" for s in sims)
