@@ -567,11 +567,7 @@ ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, do
     DevMedium M = s->M();
     const DevSource S = source_taps(s, src, dt);
     const DevFields set[2] = {s->F(), s->F2()};
-    float dto[NFIELD], inv[NFIELD];
-    for (int q = 0; q < NFIELD; ++q) {
-        dto[q] = (float)(dt * s->scale[q]);
-        inv[q] = 1.0f / s->scale[q];
-    }
+    const float inv[NFIELD] = {1, 1, 1, 1, 1, 1, 1, 1, 1};
     const int stor = s->opt.storage;
     s->fresh = false;
     ews_status st;
@@ -580,7 +576,7 @@ ews_status steps_fused(ews_sim* s, const SourceSpec& src, int n0, int nsteps, do
         const int dir = (n - n0) & 1;
         const DevFields& out = set[dir ^ 1];
         float* slot = vcap ? vcap + (size_t)(n - n0 + 1) * 3 * s->fstride : nullptr;
-        CK(fused::launch_fused(fp, dir, s->g, M, s->B, dto, inv, S, s->wavelet, n, slot,
+        CK(fused::launch_fused(fp, dir, s->g, M, s->B, (float)dt, S, s->wavelet, n, slot,
                                (long long)s->fstride, s->err, s->stream));
         if ((st = mark(s, EWS_KERNEL_STEP)) != EWS_OK) return st;
         const bool rec = s->nrec > 0 && dseis;

@@ -48,9 +48,6 @@
 // them; a moment source and the receivers run after the step, on B, as in the
 // two-pass loop.  The arithmetic per cell is that of the two passes, rounding
 // by rounding (ews_arith.cuh).
-#include <cuda_bf16.h>
-#include <cuda_fp16.h>
-
 #include <algorithm>
 
 #include "ews_arith.cuh"
@@ -120,47 +117,15 @@ __device__ __forceinline__ f2 d4x(f2 c1, f2 c2, f2 l, f2 c, f2 r) {
     return fma2(c1, in, mul2(c2, out));
 }
 
-// ---- storage types ----
-template <typename T> struct S2;
-template <> struct S2<float> {
-    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
-    __device__ static f2 ld(const float* p) { return *reinterpret_cast<const f2*>(p); }
-    __device__ static f2 round(f2 x) { return x; }
-    __device__ static void st(float* p, f2 x) { *reinterpret_cast<f2*>(p) = x; }
-};
-template <> struct S2<__nv_bfloat16> {
-    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_BFLOAT16;
-    __device__ static f2 ld(const __nv_bfloat16* p) {
-        const unsigned u = *reinterpret_cast<const unsigned*>(p);
-        return pk(__uint_as_float(u << 16), __uint_as_float(u & 0xFFFF0000u));
-    }
-    __device__ static f2 round(f2 x) {
-        return pk(__bfloat162float(__float2bfloat16_rn(lo(x))), __bfloat162float(__float2bfloat16_rn(hi(x))));
-    }
-    __device__ static void st(__nv_bfloat16* p, f2 x) {
-        *reinterpret_cast<__nv_bfloat162*>(p) = __floats2bfloat162_rn(lo(x), hi(x));
-    }
-};
-template <> struct S2<__half> {
-    static constexpr CUtensorMapDataType dtype = CU_TENSOR_MAP_DATA_TYPE_FLOAT16;
-    __device__ static f2 ld(const __half* p) {
-        const float2 v = __half22float2(*reinterpret_cast<const __half2*>(p));
-        return pk(v.x, v.y);
-    }
-    __device__ static f2 round(f2 x) {
-        return pk(__half2float(__float2half_rn(lo(x))), __half2float(__float2half_rn(hi(x))));
-    }
-    __device__ static void st(__half* p, f2 x) {
-        *reinterpret_cast<__half2*>(p) = __floats2half2_rn(lo(x), hi(x));
-    }
-};
+__device__ __forceinline__ f2 ld2(const float* p) { return *reinterpret_cast<const f2*>(p); }
+__device__ __forceinline__ void st2(float* p, f2 x) { *reinterpret_cast<f2*>(p) = x; }
 
 // ---- shared-memory layout ----
 // Slot of one step (boxes BW wide from x0 - HO): sxx, sxz rows y0-2 ..; syy
-// rows y0-3 ..; syz, sxy rows y0-4 ..; szz, vx vy vz rows y0-2 ..; rho FP32.
-template <typename T, int TY>
+// rows y0-3 ..; syz, sxy rows y0-4 ..; szz, vx vy vz, rho rows y0-2 ...
+template <int TY>
 struct FL {
-    static constexpr int ES = (int)sizeof(T), HO = 16 / ES, BW = TX + 2 * HO;
+    static constexpr int ES = 4, HO = 4, BW = TX + 2 * HO;
     static constexpr int EY = TY + 4, NR = 16 * EY;                  // region rows; row threads
     static constexpr int NT = (EXP * EY + 31) / 32 * 32;             // threads
     static constexpr int RB = EY * BW * ES, RB3 = (EY + 3) * BW * ES, MRB = (EY + 1) * MBW * 4;
@@ -184,15 +149,14 @@ struct FusedParams {
     DevFields fout;             // v^{n+1/2}, sigma^{n+1}
     DevMedium M;
     DevBoundary B;
-    float dt1[3], dt2[3], dt4[3];   // dt x scale: sxx syy szz; twice it: v; a quarter: sxy sxz syz
-    float inv[NFIELD];
+    float dt, dt2, dt4;         // dt, twice it, a quarter of it
     int ntx, nty, zchunk;
     int* err;
     DevSource S;                // force taps (kind 1) of this step; else ntap 0
     const float* wavelet;
     int n;
     int sk0, sk1;               // planes of the force taps
-    float* vcap;                // history slot of v^{n+1/2} (3 fields, hstride apart), FP32
+    float* vcap;                // history slot of v^{n+1/2} (3 fields, hstride apart)
     long long hstride;
 };
 
@@ -204,10 +168,10 @@ constexpr int M_VEL = 3, M_MED = 6, M_STR = 7;
 // of plane k + 1 and szz of k + 2; from M_VEL on sxx, syy, sxy, v of plane k;
 // from M_MED on lambda of plane k - 2 and mu of k - 1.  Medium planes clamp
 // at the top.
-template <typename T, int TY>
+template <int TY>
 __device__ __forceinline__ void issue_step(const FusedMaps& mp, unsigned char* sm, uint64_t* bar, int x0,
                                            int y0, int z0, int m, int nz) {
-    using L = FL<T, TY>;
+    using L = FL<TY>;
     const int k = z0 - 5 + m;
     unsigned char* slot = sm + (m % NS) * L::SLOT;
     mbar_expect_tx(bar, (uint32_t)(m < M_VEL ? L::PRE_TX : m < M_MED ? L::FULL_TX : L::FULL_TX + L::LB + L::MUB));
@@ -238,10 +202,10 @@ struct FQ {
     f2 bx, by, r0;              // half buoyancies and density at plane k
     f2 vzc;                     // new vz at plane k - 4 (tile threads)
     f2 mu2, mxy, ma, mb;        // 2 mu, its xy sum, mu + mu(x+1), mu + mu(y+1) at plane k - 2
-    bool bad, ovf;
+    bool bad;
 };
 
-template <int BND, typename T, int TY>
+template <int BND, int TY>
 struct FGeo {
     int x0, y0, z0, z1, M;
     int row, rp;                // region row, pair in the row
@@ -259,7 +223,7 @@ struct FGeo {
         return pk(cx0 ? hi(c) : lo(c), cx1 ? lo(r) : hi(c));
     }
     __device__ __forceinline__ FGeo(const FusedParams& P, int item) {
-        using L = FL<T, TY>;
+        using L = FL<TY>;
         const DevGrid& g = P.g;
         const int ntile = P.ntx * P.nty;
         const int tl = item % ntile;
@@ -299,9 +263,6 @@ struct FGeo {
     }
 };
 
-template <typename T> constexpr bool kScaled = sizeof(T) == 2;
-__device__ __forceinline__ bool over2(f2 x) { return fabsf(lo(x)) > 65504.0f || fabsf(hi(x)) > 65504.0f; }
-
 // Slot (= its barrier) and medium entry of a step, and the phase of the
 // slot's barrier.
 struct Turn {
@@ -321,12 +282,11 @@ struct Turn {
 // offsets of the new-velocity planes k, k-1, k-2, k-3 (floats); ent: of the
 // medium entry of this step.
 // CAP: v^{n+1/2} also goes to its history slot.
-template <int BND, typename T, int TY, bool CAP, int PH, int STAGE>
+template <int BND, int TY, bool CAP, int PH, int STAGE>
 __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedParams& P,
-                                           const FGeo<BND, T, TY>& G, FQ& Q, unsigned char* sm,
+                                           const FGeo<BND, TY>& G, FQ& Q, unsigned char* sm,
                                            uint64_t* bars, int m, const int (&ring)[4], const Turn& tn) {
-    using L = FL<T, TY>;
-    using S = S2<T>;
+    using L = FL<TY>;
     constexpr int BW = L::BW;
     const DevGrid& g = P.g;
     constexpr int A = (PH + 1) & 3, B = (PH + 2) & 3, C = (PH + 3) & 3, D = PH;   // oldest..newest
@@ -349,42 +309,37 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     s1 = Q.yy[HQ];
     s3 = Q.xy[HQ];
     {
-        const T* fxz = reinterpret_cast<const T*>(slot + L::SXZ_) + G.oc;              // plane k + 1
-        const T* fyz = reinterpret_cast<const T*>(slot + L::SYZ_) + G.oc + 2 * BW;
+        const float* fxz = reinterpret_cast<const float*>(slot + L::SXZ_) + G.oc;          // plane k + 1
+        const float* fyz = reinterpret_cast<const float*>(slot + L::SYZ_) + G.oc + 2 * BW;
         const float* fr = reinterpret_cast<const float*>(slot + L::RHO_) + G.row * MBW + 2 + 2 * G.rp;
-        const f2 cxz = S::ld(fxz), cyz = S::ld(fyz);
-        Q.zz[D] = S::ld(reinterpret_cast<const T*>(slot + L::SZZ_) + G.oc);            // plane k + 2
+        const f2 cxz = ld2(fxz), cyz = ld2(fyz);
+        Q.zz[D] = ld2(reinterpret_cast<const float*>(slot + L::SZZ_) + G.oc);        // plane k + 2
         Q.xz[D] = cxz;
         Q.yz[D] = cyz;
         // density and buoyancies of plane k + 1
-        const f2 r1 = S2<float>::ld(fr), rx = S2<float>::ld(fr + 2), ry = S2<float>::ld(fr + (G.cy ? MBW : 0));
+        const f2 r1 = ld2(fr), rx = ld2(fr + 2), ry = ld2(fr + (G.cy ? MBW : 0));
         if constexpr (STAGE > 0) {
             const f2 sz = add2(Q.r0, r1);
-            const T* fxx = reinterpret_cast<const T*>(slot + L::SXX_) + G.oc;
-            const T* fyy = reinterpret_cast<const T*>(slot + L::SYY_) + G.oc + BW;
-            const T* fxy = reinterpret_cast<const T*>(slot + L::SXY_) + G.oc + 2 * BW;
-            const T* fv = reinterpret_cast<const T*>(slot + L::V_) + G.oc;
-            const f2 cxx = S::ld(fxx), cyy = S::ld(fyy), cxy = S::ld(fxy);
+            const float* fxx = reinterpret_cast<const float*>(slot + L::SXX_) + G.oc;
+            const float* fyy = reinterpret_cast<const float*>(slot + L::SYY_) + G.oc + BW;
+            const float* fxy = reinterpret_cast<const float*>(slot + L::SXY_) + G.oc + 2 * BW;
+            const float* fv = reinterpret_cast<const float*>(slot + L::V_) + G.oc;
+            const f2 cxx = ld2(fxx), cyy = ld2(fyy), cxy = ld2(fxy);
             Q.xx[HQ] = cxx;
             Q.yy[HQ] = cyy;
             Q.xy[HQ] = cxy;
-            f2 dxx = d4x<true>(c1x, c2x, S::ld(fxx - 2), cxx, S::ld(fxx + 2));
-            f2 dxy = d4p(c1y, c2y, S::ld(fxy - 2 * BW), S::ld(fxy - BW), cxy, S::ld(fxy + BW));
+            f2 dxx = d4x<true>(c1x, c2x, ld2(fxx - 2), cxx, ld2(fxx + 2));
+            f2 dxy = d4p(c1y, c2y, ld2(fxy - 2 * BW), ld2(fxy - BW), cxy, ld2(fxy + BW));
             f2 dxz = d4p(c1z, c2z, Q.xz[A], Q.xz[B], Q.xz[C], Q.xz[D]);
-            f2 dyx = d4x<false>(c1x, c2x, S::ld(fxy - 2), cxy, S::ld(fxy + 2));
-            f2 dyy = d4p(c1y, c2y, S::ld(fyy - BW), cyy, S::ld(fyy + BW), S::ld(fyy + 2 * BW));
+            f2 dyx = d4x<false>(c1x, c2x, ld2(fxy - 2), cxy, ld2(fxy + 2));
+            f2 dyy = d4p(c1y, c2y, ld2(fyy - BW), cyy, ld2(fyy + BW), ld2(fyy + 2 * BW));
             f2 dyz = d4p(c1z, c2z, Q.yz[A], Q.yz[B], Q.yz[C], Q.yz[D]);
             f2 dzz = d4p(c1z, c2z, Q.zz[A], Q.zz[B], Q.zz[C], Q.zz[D]);
-            if (kScaled<T>) {
-                dxx = mul2(dxx, dup(P.inv[SXX])); dxy = mul2(dxy, dup(P.inv[SXY])); dxz = mul2(dxz, dup(P.inv[SXZ]));
-                dyx = mul2(dyx, dup(P.inv[SXY])); dyy = mul2(dyy, dup(P.inv[SYY])); dyz = mul2(dyz, dup(P.inv[SYZ]));
-                dzz = mul2(dzz, dup(P.inv[SZZ]));
-            }
             // (2 dt) r with r = 1 / (r0 + r1) has the bits of dt (2 r)
             const f2 bz = pk(ar::rcp(lo(sz)), ar::rcp(hi(sz)));
-            f2 vx = fma2(mul2(dup(P.dt2[0]), Q.bx), add2(add2(dxx, dxy), dxz), S::ld(fv));
-            f2 vy = fma2(mul2(dup(P.dt2[kScaled<T> ? 1 : 0]), Q.by), add2(add2(dyx, dyy), dyz), S::ld(fv + L::RB / L::ES));
-            f2 vz = fma2(mul2(dup(P.dt2[kScaled<T> ? 2 : 0]), bz), add2(Q.dz, dzz), S::ld(fv + 2 * (L::RB / L::ES)));
+            f2 vx = fma2(mul2(dup(P.dt2), Q.bx), add2(add2(dxx, dxy), dxz), ld2(fv));
+            f2 vy = fma2(mul2(dup(P.dt2), Q.by), add2(add2(dyx, dyy), dyz), ld2(fv + L::RB / L::ES));
+            f2 vz = fma2(mul2(dup(P.dt2), bz), add2(Q.dz, dzz), ld2(fv + 2 * (L::RB / L::ES)));
             if (BND == BND_SPONGE) {
                 const f2 gs = mul2(mul2(G.gx, dup(gz[0])), dup(G.gy));
                 vx = mul2(vx, gs); vy = mul2(vy, gs); vz = mul2(vz, gs);
@@ -394,35 +349,30 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
             vx = pk(i0 ? lo(vx) : 0.0f, i1 ? hi(vx) : 0.0f);
             vy = pk(i0 ? lo(vy) : 0.0f, i1 ? hi(vy) : 0.0f);
             vz = pk(i0 ? lo(vz) : 0.0f, i1 ? hi(vz) : 0.0f);
-            if (std::is_same<T, __half>::value) Q.ovf |= over2(vx) | over2(vy) | over2(vz);
             if (G.tile && k >= G.z0 && k < G.z1) {
                 const long long o = (long long)k * g.plane + G.o;
-                S::st((T*)P.fout.f[VX] + o, vx);
-                S::st((T*)P.fout.f[VY] + o, vy);
-                S::st((T*)P.fout.f[VZ] + o, vz);
+                st2(P.fout.f[VX] + o, vx);
+                st2(P.fout.f[VY] + o, vy);
+                st2(P.fout.f[VZ] + o, vz);
                 if constexpr (CAP) {
-                    S2<float>::st(P.vcap + o, vx);
-                    S2<float>::st(P.vcap + P.hstride + o, vy);
-                    S2<float>::st(P.vcap + 2 * P.hstride + o, vz);
+                    st2(P.vcap + o, vx);
+                    st2(P.vcap + P.hstride + o, vy);
+                    st2(P.vcap + 2 * P.hstride + o, vz);
                 }
             }
             if (G.reg) {
                 float* vn = vring + ring[0] + G.row * VS + 2 * G.rp;
-                *reinterpret_cast<f2*>(vn) = S::round(vx);
-                *reinterpret_cast<f2*>(vn + L::EY * VS) = S::round(vy);
-                *reinterpret_cast<f2*>(vn + 2 * L::EY * VS) = S::round(vz);
+                *reinterpret_cast<f2*>(vn) = vx;
+                *reinterpret_cast<f2*>(vn + L::EY * VS) = vy;
+                *reinterpret_cast<f2*>(vn + 2 * L::EY * VS) = vz;
             }
         }
         Q.r0 = r1;
         const f2 sx = add2(r1, G.next_x(r1, rx)), sy = add2(r1, ry);
         Q.bx = pk(ar::rcp(lo(sx)), ar::rcp(hi(sx)));
         Q.by = pk(ar::rcp(lo(sy)), ar::rcp(hi(sy)));
-        f2 dzx = d4x<false>(c1x, c2x, S::ld(fxz - 2), cxz, S::ld(fxz + 2));
-        f2 dzy = d4p(c1y, c2y, S::ld(fyz - 2 * BW), S::ld(fyz - BW), cyz, S::ld(fyz + BW));
-        if (kScaled<T>) {
-            dzx = mul2(dzx, dup(P.inv[SXZ]));
-            dzy = mul2(dzy, dup(P.inv[SYZ]));
-        }
+        f2 dzx = d4x<false>(c1x, c2x, ld2(fxz - 2), cxz, ld2(fxz + 2));
+        f2 dzy = d4p(c1y, c2y, ld2(fyz - 2 * BW), ld2(fyz - BW), cyz, ld2(fyz + BW));
         Q.dz = add2(dzx, dzy);
     }
     s4 = Q.xz[A];                                    // sxz, syz of plane k - 2
@@ -434,7 +384,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     // m + NS once every warp is
     if (threadIdx.x == L::NT - 32 && m + NS < G.M) {
         Q.bad = Q.bad || !mbar_wait(&bars[CB], (uint32_t)((m >> 1) & 1));
-        issue_step<T, TY>(maps, sm, &bars[tn.s], G.x0, G.y0, G.z0, m + NS, g.nz);
+        issue_step<TY>(maps, sm, &bars[tn.s], G.x0, G.y0, G.z0, m + NS, g.nz);
     }
     // point force of step n on its tap cells inside the region
     if (STAGE > 0 && k >= P.sk0 && k <= P.sk1) {     // uniform across the CTA
@@ -447,18 +397,11 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
                 amp *= ops::buoy(P.M, g, tp.q - VX, tp.i, tp.j, tp.k);
                 amp *= ops::gain(P.B, tp.i, tp.j, tp.k);
                 float* v = vring + ring[0] + (tp.q - VX) * L::EY * VS + ey * VS + ex;
-                float x;
-                if constexpr (sizeof(T) == 4) {
-                    x = __fadd_rn(*v, amp);
-                } else {                             // the passes add the rounded amount
-                    x = __fadd_rn(*v, ops::Io<T>::get_value(amp));
-                    if (std::is_same<T, __half>::value && fabsf(x) > 65504.0f) Q.ovf = true;
-                    x = ops::Io<T>::get_value(x);
-                }
+                const float x = __fadd_rn(*v, amp);
                 *v = x;
                 if (k >= G.z0 && k < G.z1 && ex >= 2 && ex < 2 + TX && ey >= 2 && ey < 2 + TY) {
-                    T* f = (T*)(tp.q == VX ? P.fout.f[VX] : tp.q == VY ? P.fout.f[VY] : P.fout.f[VZ]);
-                    f[ops::cidx(g, tp.i, tp.j, tp.k)] = ops::Io<T>::put(x);
+                    float* f = tp.q == VX ? P.fout.f[VX] : tp.q == VY ? P.fout.f[VY] : P.fout.f[VZ];
+                    f[ops::cidx(g, tp.i, tp.j, tp.k)] = x;
                     if constexpr (CAP) P.vcap[(tp.q - VX) * P.hstride + ops::cidx(g, tp.i, tp.j, tp.k)] = x;
                 }
             }
@@ -472,7 +415,7 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
             const float* hm = reinterpret_cast<const float*>(ent + r128(L::LB)) + (G.row - 2) * MBW + 2 + 2 * G.rp;
             const float* hy = hm + (G.cy ? MBW : 0);
             // mu of plane k - 1 and its x, y and xy neighbours
-            const f2 m1 = S2<float>::ld(hm), m1r = S2<float>::ld(hm + 2), my = S2<float>::ld(hy), myr = S2<float>::ld(hy + 2);
+            const f2 m1 = ld2(hm), m1r = ld2(hm + 2), my = ld2(hy), myr = ld2(hy + 2);
             const f2 mx = G.next_x(m1, m1r), mxy4 = G.next_x(my, myr);
             const f2 na = add2(m1, mx), nb = add2(m1, my);
             const int e = G.row * VS + 2 * G.rp;
@@ -481,35 +424,28 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
             const float* v1 = vring + ring[1] + e;
             const float* v0 = vring + ring[0] + e;
             constexpr int FS = L::EY * VS;
-            auto ld = [](const float* p) { return S2<float>::ld(p); };
-            const f2 vz3 = ld(v3 + 2 * FS), czv = ld(v2 + 2 * FS);
+            const f2 vz3 = ld2(v3 + 2 * FS), czv = ld2(v2 + 2 * FS);
             if constexpr (STAGE == 3) {
-                const f2 cvx = ld(v2), cvy = ld(v2 + FS);
-                f2 exx = d4x<false>(c1x, c2x, ld(v2 - 2), cvx, ld(v2 + 2));
-                f2 vxy = d4p(c1y, c2y, ld(v2 - VS), cvx, ld(v2 + VS), ld(v2 + 2 * VS));
-                f2 vxz = d4p(c1z, c2z, ld(v3), cvx, ld(v1), ld(v0));
-                f2 eyy = d4p(c1y, c2y, ld(v2 + FS - 2 * VS), ld(v2 + FS - VS), cvy, ld(v2 + FS + VS));
-                f2 vyx = d4x<true>(c1x, c2x, ld(v2 + FS - 2), cvy, ld(v2 + FS + 2));
-                f2 vyz = d4p(c1z, c2z, ld(v3 + FS), cvy, ld(v1 + FS), ld(v0 + FS));
-                f2 ezz = d4p(c1z, c2z, Q.vzc, vz3, czv, ld(v1 + 2 * FS));
-                f2 vzx = d4x<true>(c1x, c2x, ld(v2 + 2 * FS - 2), czv, ld(v2 + 2 * FS + 2));
-                f2 vzy = d4p(c1y, c2y, ld(v2 + 2 * FS - VS), czv, ld(v2 + 2 * FS + VS), ld(v2 + 2 * FS + 2 * VS));
-                if (kScaled<T>) {
-                    const f2 ix = dup(P.inv[VX]), iy = dup(P.inv[VY]), iz = dup(P.inv[VZ]);
-                    exx = mul2(exx, ix); vxy = mul2(vxy, ix); vxz = mul2(vxz, ix);
-                    eyy = mul2(eyy, iy); vyx = mul2(vyx, iy); vyz = mul2(vyz, iy);
-                    ezz = mul2(ezz, iz); vzx = mul2(vzx, iz); vzy = mul2(vzy, iz);
-                }
-                const f2 lam = S2<float>::ld(reinterpret_cast<const float*>(ent) + (G.row - 2) * TX + 2 * (G.rp - 1));
+                const f2 cvx = ld2(v2), cvy = ld2(v2 + FS);
+                f2 exx = d4x<false>(c1x, c2x, ld2(v2 - 2), cvx, ld2(v2 + 2));
+                f2 vxy = d4p(c1y, c2y, ld2(v2 - VS), cvx, ld2(v2 + VS), ld2(v2 + 2 * VS));
+                f2 vxz = d4p(c1z, c2z, ld2(v3), cvx, ld2(v1), ld2(v0));
+                f2 eyy = d4p(c1y, c2y, ld2(v2 + FS - 2 * VS), ld2(v2 + FS - VS), cvy, ld2(v2 + FS + VS));
+                f2 vyx = d4x<true>(c1x, c2x, ld2(v2 + FS - 2), cvy, ld2(v2 + FS + 2));
+                f2 vyz = d4p(c1z, c2z, ld2(v3 + FS), cvy, ld2(v1 + FS), ld2(v0 + FS));
+                f2 ezz = d4p(c1z, c2z, Q.vzc, vz3, czv, ld2(v1 + 2 * FS));
+                f2 vzx = d4x<true>(c1x, c2x, ld2(v2 + 2 * FS - 2), czv, ld2(v2 + 2 * FS + 2));
+                f2 vzy = d4p(c1y, c2y, ld2(v2 + 2 * FS - VS), czv, ld2(v2 + 2 * FS + VS), ld2(v2 + 2 * FS + 2 * VS));
+                const f2 lam = ld2(reinterpret_cast<const float*>(ent) + (G.row - 2) * TX + 2 * (G.rp - 1));
                 const f2 l2m = add2(Q.mu2, lam);
                 // sums of four: (dt / 4) times the sum has the bits of dt times the mean
                 const f2 mxz = add2(add2(Q.ma, m1), mx), myz = add2(add2(Q.mb, m1), my);
-                s0 = fma2(dup(P.dt1[0]), fma2(l2m, exx, mul2(lam, add2(eyy, ezz))), s0);
-                s1 = fma2(dup(P.dt1[kScaled<T> ? 1 : 0]), fma2(l2m, eyy, mul2(lam, add2(exx, ezz))), s1);
-                s2 = fma2(dup(P.dt1[kScaled<T> ? 2 : 0]), fma2(l2m, ezz, mul2(lam, add2(exx, eyy))), s2);
-                s3 = fma2(mul2(dup(P.dt4[0]), Q.mxy), add2(vxy, vyx), s3);
-                s4 = fma2(mul2(dup(P.dt4[kScaled<T> ? 1 : 0]), mxz), add2(vxz, vzx), s4);
-                s5 = fma2(mul2(dup(P.dt4[kScaled<T> ? 2 : 0]), myz), add2(vyz, vzy), s5);
+                s0 = fma2(dup(P.dt), fma2(l2m, exx, mul2(lam, add2(eyy, ezz))), s0);
+                s1 = fma2(dup(P.dt), fma2(l2m, eyy, mul2(lam, add2(exx, ezz))), s1);
+                s2 = fma2(dup(P.dt), fma2(l2m, ezz, mul2(lam, add2(exx, eyy))), s2);
+                s3 = fma2(mul2(dup(P.dt4), Q.mxy), add2(vxy, vyx), s3);
+                s4 = fma2(mul2(dup(P.dt4), mxz), add2(vxz, vzx), s4);
+                s5 = fma2(mul2(dup(P.dt4), myz), add2(vyz, vzy), s5);
                 if (BND == BND_SPONGE) {
                     const f2 gs = mul2(mul2(G.gx, dup(gz[-2])), dup(G.gy));
                     s0 = mul2(s0, gs); s1 = mul2(s1, gs); s2 = mul2(s2, gs);
@@ -519,15 +455,13 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
                     s0 = pk(lo(s0), 0.f); s1 = pk(lo(s1), 0.f); s2 = pk(lo(s2), 0.f);
                     s3 = pk(lo(s3), 0.f); s4 = pk(lo(s4), 0.f); s5 = pk(lo(s5), 0.f);
                 }
-                if (std::is_same<T, __half>::value)
-                    Q.ovf |= over2(s0) | over2(s1) | over2(s2) | over2(s3) | over2(s4) | over2(s5);
                 const long long o = (long long)(k - 2) * g.plane + G.o;
-                S::st((T*)P.fout.f[SXX] + o, s0);
-                S::st((T*)P.fout.f[SYY] + o, s1);
-                S::st((T*)P.fout.f[SZZ] + o, s2);
-                S::st((T*)P.fout.f[SXY] + o, s3);
-                S::st((T*)P.fout.f[SXZ] + o, s4);
-                S::st((T*)P.fout.f[SYZ] + o, s5);
+                st2(P.fout.f[SXX] + o, s0);
+                st2(P.fout.f[SYY] + o, s1);
+                st2(P.fout.f[SZZ] + o, s2);
+                st2(P.fout.f[SXY] + o, s3);
+                st2(P.fout.f[SXZ] + o, s4);
+                st2(P.fout.f[SYZ] + o, s5);
             }
             Q.vzc = vz3;
             Q.mu2 = add2(m1, m1);
@@ -538,19 +472,19 @@ __device__ __forceinline__ void fused_step(const FusedMaps& maps, const FusedPar
     }
 }
 
-template <int BND, typename T, int TY, bool CAP>
-__global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constant__ FusedMaps maps,
+template <int BND, int TY, bool CAP>
+__global__ void __launch_bounds__(FL<TY>::NT, 1) k_fused(const __grid_constant__ FusedMaps maps,
                                                            const __grid_constant__ FusedParams P) {
-    using L = FL<T, TY>;
+    using L = FL<TY>;
     extern __shared__ __align__(128) unsigned char sm[];
     // bars[0..NS-1]: copies of a step arrived; the last two: warps past its velocity phase
     uint64_t* bars = reinterpret_cast<uint64_t*>(sm + L::O_BAR);
-    const FGeo<BND, T, TY> G(P, (int)blockIdx.x);
+    const FGeo<BND, TY> G(P, (int)blockIdx.x);
     if (threadIdx.x == L::NT - 32) {
         for (int s = 0; s < NS + 2; ++s) mbar_init(&bars[s], s < NS ? 1 : L::NT / 32);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        for (int s = 0; s < NS; ++s) issue_step<T, TY>(maps, sm, &bars[s], G.x0, G.y0, G.z0, s, P.g.nz);
+        for (int s = 0; s < NS; ++s) issue_step<TY>(maps, sm, &bars[s], G.x0, G.y0, G.z0, s, P.g.nz);
     }
     if (BND == BND_SPONGE)
         for (int q = threadIdx.x; q < G.M; q += L::NT)
@@ -561,7 +495,7 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
     for (int q = 0; q < 4; ++q) Q.zz[q] = Q.xz[q] = Q.yz[q] = 0;
     Q.xx[0] = Q.xx[1] = Q.yy[0] = Q.yy[1] = Q.xy[0] = Q.xy[1] = 0;
     Q.dz = Q.bx = Q.by = Q.r0 = Q.vzc = Q.mu2 = Q.mxy = Q.ma = Q.mb = 0;
-    Q.bad = Q.ovf = false;
+    Q.bad = false;
     int ring[4] = {0, 4 * L::VPL, 3 * L::VPL, 2 * L::VPL};            // planes k .. k - 3
     Turn tn;
     auto next = [&]() {
@@ -572,27 +506,27 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
         ring[0] = nw;
         tn.next(L::ENT);
     };
-    fused_step<BND, T, TY, CAP, 0, 0>(maps, P, G, Q, sm, bars, 0, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 1, 0>(maps, P, G, Q, sm, bars, 1, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 2, 0>(maps, P, G, Q, sm, bars, 2, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 3, 1>(maps, P, G, Q, sm, bars, 3, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 0, 1>(maps, P, G, Q, sm, bars, 4, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 1, 1>(maps, P, G, Q, sm, bars, 5, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 2, 2>(maps, P, G, Q, sm, bars, 6, ring, tn); next();
-    fused_step<BND, T, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, 7, ring, tn); next();
+    fused_step<BND, TY, CAP, 0, 0>(maps, P, G, Q, sm, bars, 0, ring, tn); next();
+    fused_step<BND, TY, CAP, 1, 0>(maps, P, G, Q, sm, bars, 1, ring, tn); next();
+    fused_step<BND, TY, CAP, 2, 0>(maps, P, G, Q, sm, bars, 2, ring, tn); next();
+    fused_step<BND, TY, CAP, 3, 1>(maps, P, G, Q, sm, bars, 3, ring, tn); next();
+    fused_step<BND, TY, CAP, 0, 1>(maps, P, G, Q, sm, bars, 4, ring, tn); next();
+    fused_step<BND, TY, CAP, 1, 1>(maps, P, G, Q, sm, bars, 5, ring, tn); next();
+    fused_step<BND, TY, CAP, 2, 2>(maps, P, G, Q, sm, bars, 6, ring, tn); next();
+    fused_step<BND, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, 7, ring, tn); next();
     int m = M_STR + 1;
     bool stop = __syncthreads_or(Q.bad);
     while (m < G.M && !stop) {
-        fused_step<BND, T, TY, CAP, 0, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+        fused_step<BND, TY, CAP, 0, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
         next();
         if (++m < G.M) {
-            fused_step<BND, T, TY, CAP, 1, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+            fused_step<BND, TY, CAP, 1, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
             next();
             if (++m < G.M) {
-                fused_step<BND, T, TY, CAP, 2, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                fused_step<BND, TY, CAP, 2, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
                 next();
                 if (++m < G.M) {
-                    fused_step<BND, T, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
+                    fused_step<BND, TY, CAP, 3, 3>(maps, P, G, Q, sm, bars, m, ring, tn);
                     next();
                     ++m;
                 }
@@ -606,24 +540,22 @@ __global__ void __launch_bounds__(FL<T, TY>::NT, 1) k_fused(const __grid_constan
         for (int q = m; q < m + NS && q < G.M; ++q)
             if (!mbar_wait(&bars[q % NS], (uint32_t)((q / NS) & 1))) break;
     }
-    if constexpr (std::is_same<T, __half>::value)
-        if (__syncthreads_or(Q.ovf) && threadIdx.x == 0) atomicOr(P.err, 4);
 }
 
-template <typename T, int TY>
+template <int TY>
 bool encode_fused(FusedMaps* fm, const DevGrid& g, const DevFields& F, const DevMedium& M) {
-    using L = FL<T, TY>;
-    const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32, dt = S2<T>::dtype;
+    using L = FL<TY>;
+    const CUtensorMapDataType f32 = CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     const char* f0 = (const char*)F.f[SXX];                                    // slot 0
     const long long fsb = (const char*)F.f[SXZ] - (const char*)F.f[SXX];
     for (int q = 0; q < NFIELD; ++q)
         if ((const char*)F.f[q] - f0 != fslot(q) * fsb) return false;
     bool ok = true;
-    ok &= encode4(&fm->x1, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY, 1);
-    ok &= encode4(&fm->y1, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY + 3, 1);
-    ok &= encode(&fm->xy, g, F.f[SXY], dt, L::ES, L::BW, L::EY + 3);
-    ok &= encode(&fm->zz, g, F.f[SZZ], dt, L::ES, L::BW, L::EY);
-    ok &= encode4(&fm->v, g, f0, dt, L::ES, fsb, NFIELD, L::BW, L::EY, 3);
+    ok &= encode4(&fm->x1, g, f0, f32, L::ES, fsb, NFIELD, L::BW, L::EY, 1);
+    ok &= encode4(&fm->y1, g, f0, f32, L::ES, fsb, NFIELD, L::BW, L::EY + 3, 1);
+    ok &= encode(&fm->xy, g, F.f[SXY], f32, L::ES, L::BW, L::EY + 3);
+    ok &= encode(&fm->zz, g, F.f[SZZ], f32, L::ES, L::BW, L::EY);
+    ok &= encode4(&fm->v, g, f0, f32, L::ES, fsb, NFIELD, L::BW, L::EY, 3);
     ok &= encode(&fm->rho, g, M.rho, f32, 4, MBW, L::EY + 1);
     ok &= encode(&fm->lam, g, M.lam, f32, 4, TX, TY);
     ok &= encode(&fm->mu, g, M.mu, f32, 4, MBW, TY + 1);
@@ -643,17 +575,17 @@ struct FusedPlan {
 };
 
 namespace {
-template <typename T, int TY>
+template <int TY>
 cudaError_t plan_for(FusedPlan* p, const DevGrid& g, const DevFields& A, const DevFields& Bf, const DevMedium& M,
                      const DevBoundary& B) {
-    using L = FL<T, TY>;
+    using L = FL<TY>;
     static_assert(L::SMEM <= 227 * 1024, "one CTA's shared memory");
-    p->kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY, false> : k_fused<BND_NONE, T, TY, false>;
-    p->kern_cap = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, T, TY, true> : k_fused<BND_NONE, T, TY, true>;
+    p->kern = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, TY, false> : k_fused<BND_NONE, TY, false>;
+    p->kern_cap = B.kind == BND_SPONGE ? k_fused<BND_SPONGE, TY, true> : k_fused<BND_NONE, TY, true>;
     p->ty = TY;
     p->nt = L::NT;
     p->smem = L::SMEM;
-    if (!encode_fused<T, TY>(&p->dir[0], g, A, M) || !encode_fused<T, TY>(&p->dir[1], g, Bf, M))
+    if (!encode_fused<TY>(&p->dir[0], g, A, M) || !encode_fused<TY>(&p->dir[1], g, Bf, M))
         return cudaErrorInvalidValue;
     return cudaSuccess;
 }
@@ -671,7 +603,7 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
     p->f[0] = A;
     p->f[1] = Bf;
     int dev = 0, sms = 0, occ = 0;
-    cudaError_t e = plan_for<float, 24>(p, g, A, Bf, M, B);
+    cudaError_t e = plan_for<24>(p, g, A, Bf, M, B);
     if (e == cudaSuccess) e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(p->kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p->smem);
@@ -695,19 +627,16 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
 void fused_plan_destroy(FusedPlan* p) { delete p; }
 
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
-                         const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
-                         const float* wavelet, int n, float* vcap, long long hstride, int* err, cudaStream_t st) {
+                         const DevBoundary& B, float dt, const DevSource& S, const float* wavelet, int n,
+                         float* vcap, long long hstride, int* err, cudaStream_t st) {
     FusedParams P{};
     P.g = g;
     P.fout = p->f[dir ^ 1];
     P.M = M;
     P.B = B;
-    for (int q = 0; q < NFIELD; ++q) P.inv[q] = inv[q];
-    for (int c = 0; c < 3; ++c) {
-        P.dt1[c] = dto[SXX + c];
-        P.dt2[c] = 2.0f * dto[VX + c];
-        P.dt4[c] = 0.25f * dto[SXY + c];
-    }
+    P.dt = dt;
+    P.dt2 = 2.0f * dt;
+    P.dt4 = 0.25f * dt;
     P.ntx = p->ntx;
     P.nty = p->nty;
     P.zchunk = p->zchunk;

@@ -452,9 +452,8 @@ cudaError_t fused_plan_create(const DevGrid& g, const DevFields& A, const DevFie
                               const DevMedium& M, const DevBoundary& B, FusedPlan** out);
 void fused_plan_destroy(FusedPlan* p);
 cudaError_t launch_fused(const FusedPlan* p, int dir, const DevGrid& g, const DevMedium& M,
-                         const DevBoundary& B, const float dto[9], const float inv[9], const DevSource& S,
-                         const float* wavelet, int n, float* vcap, long long hstride, int* err,
-                         cudaStream_t st);
+                         const DevBoundary& B, float dt, const DevSource& S, const float* wavelet, int n,
+                         float* vcap, long long hstride, int* err, cudaStream_t st);
 }  // namespace fused
 
 // The time loop of a small grid in one cooperative launch with the fields

@@ -49,12 +49,10 @@ template <> struct Io<float> {
 template <> struct Io<__nv_bfloat16> {
     __device__ static float get(const __nv_bfloat16* p) { return __bfloat162float(*p); }
     __device__ static __nv_bfloat16 put(float x) { return __float2bfloat16_rn(x); }
-    __device__ static float get_value(float x) { return __bfloat162float(put(x)); }
 };
 template <> struct Io<__half> {
     __device__ static float get(const __half* p) { return __half2float(*p); }
     __device__ static __half put(float x) { return __float2half_rn(x); }
-    __device__ static float get_value(float x) { return __half2float(put(x)); }   // x as stored
 };
 
 // Source tap t at step n (Sec. 2.4 reading): the tap weight holds -dt M / V
