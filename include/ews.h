@@ -326,6 +326,12 @@ ews_status ews_set_tile_shape(ews_sim* sim, int shape);
  * launch, which has no tiles. */
 int ews_get_tile_shape(ews_sim* sim);
 
+/* Testing only: with wait_ms > 0 (at most 1000), in later runs in one launch
+ * (EWS_TILE_RESIDENT) one block of the grid leaves at once, its neighbours'
+ * waits for its halos give up after wait_ms, and the run must end in
+ * EWS_ETIMEOUT.  0: as usual. */
+ews_status ews_test_resident_wait(ews_sim* sim, int wait_ms);
+
 /* Tile-shape table, one entry per grid size, boundary and storage type;
  * can be exported and imported so that a tuning outlives the process (the
  * Python binding stores it with the z-chunk table).  Host memory only. */

@@ -685,6 +685,7 @@ ResidentRun resident_run(const ews_sim* s, const DevFields& F, double dt, int nr
     r.stage = s->res_stage;
     r.ld = ld;
     r.fstride = (long long)s->fstride;
+    r.test_wait_ms = s->res_test_wait;
     return r;
 }
 // Tags of the next launch of `nsteps` steps.
@@ -1259,6 +1260,13 @@ ews_status ews_set_tile_shape(ews_sim* s, int shape) {
     s->tile_req = shape;
     s->ran_loop = false;
     if (shape != EWS_TILE_AUTO) set_tile_used(s, tile_eligible(s) ? shape : EWS_TILE_32X8);
+    return EWS_OK;
+}
+
+ews_status ews_test_resident_wait(ews_sim* s, int wait_ms) {
+    if (!s) return fail(EWS_EINVAL, "null simulation");
+    if (wait_ms < 0 || wait_ms > 1000) return fail(EWS_EINVAL, "wait of %d ms outside [0, 1000]", wait_ms);
+    s->res_test_wait = wait_ms;
     return EWS_OK;
 }
 

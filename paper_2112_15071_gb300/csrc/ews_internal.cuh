@@ -486,6 +486,7 @@ struct ResidentRun {
     int ld;
     float* vcap;                  // history slot of v^{n0+1/2}, or null
     long long fstride;
+    int test_wait_ms;             // > 0: block 0 leaves at once, waits give up after this
 };
 // False where the grid does not fit `sms` CTAs.
 bool resident_plan(const DevGrid& g, int bnd, int sms, ResidentPlan* out);

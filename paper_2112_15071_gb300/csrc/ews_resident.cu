@@ -80,6 +80,7 @@ struct ResParams {
     float* coef;                                 // [ntap] scratch, by place in tlist
     long long fstride;                           // elements between fields
     unsigned long long wait_ns;
+    int mute;                                    // CTA that leaves at once (testing), or -1
 };
 
 __device__ __forceinline__ unsigned long long inbox_load(const unsigned long long* p) {
@@ -237,6 +238,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(const __grid_constant__ Re
     __shared__ int s_src;
     const DevGrid& g = P.g;
     const int t = threadIdx.x, NT = blockDim.x, cta = blockIdx.x;
+    if (cta == P.mute) return;
     const int bi = cta % P.nbx, bj = (cta / P.nbx) % P.nby, bk = cta / (P.nbx * P.nby);
     const int i0 = block_lo(g.nx, P.nbx, bi), j0 = block_lo(g.ny, P.nby, bj), k0 = block_lo(g.nz, P.nbz, bk);
     const int LX = block_lo(g.nx, P.nbx, bi + 1) - i0, LY = block_lo(g.ny, P.nby, bj + 1) - j0,
@@ -871,7 +873,8 @@ ResParams res_params(const ResidentRun& r) {
     P.tstart = r.tstart;
     P.ntap = 24 * r.nrec;
     P.fstride = r.fstride;
-    P.wait_ns = 2000000000ull;                       // 2 s per wait
+    P.wait_ns = r.test_wait_ms > 0 ? r.test_wait_ms * 1000000ull : 2000000000ull;   // 2 s per wait
+    P.mute = r.test_wait_ms > 0 ? 0 : -1;
     return P;
 }
 }  // namespace

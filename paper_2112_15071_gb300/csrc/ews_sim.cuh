@@ -105,6 +105,7 @@ struct ews_sim {
     int res_chunk = 0;
     int res_taps = 0;             // receiver taps of the block with most
     bool ran_loop = false;        // the last steps ran in it
+    int res_test_wait = 0;        // ews_test_resident_wait
     cudaStream_t stream = nullptr;
     // launch accounting and optional per-launch event timing
     long long launches[EWS_NKERNEL] = {};

@@ -122,6 +122,7 @@ SIGNATURES = [
                                _P]),
     ("ews_set_tile_shape", _I, [_P, _I]),
     ("ews_get_tile_shape", _I, [_P]),
+    ("ews_test_resident_wait", _I, [_P, _I]),
     ("ews_tile_tuned", _I, [C.POINTER(ews_grid), _I, _I]),
     ("ews_tile_tuning_export", _I, [C.POINTER(ews_tuned_tile), _I]),
     ("ews_tile_tuning_import", _I, [C.POINTER(ews_tuned_tile), _I]),
@@ -491,6 +492,10 @@ _STORAGE_NAMES = {v: k for k, v in STORAGE.items()}
 
 def ews_set_tile_shape(sim, shape):
     _check(load().ews_set_tile_shape(sim, TILE[shape] if isinstance(shape, str) else int(shape)))
+
+
+def ews_test_resident_wait(sim, wait_ms: int):
+    _check(load().ews_test_resident_wait(sim, int(wait_ms)))
 
 
 def ews_get_tile_shape(sim) -> int:

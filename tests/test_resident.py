@@ -163,6 +163,34 @@ def test_the_route_is_reported_and_leaves_the_table_alone(ews):
         ews.ews_tile_tuning_clear()
 
 
+@pytest.mark.parametrize("n,boundary", [((33, 18, 17), "sponge"), ((64, 64, 64), "sponge"),
+                                        ((80, 75, 71), "none"), ((40, 36, 28), "cpml")])
+def test_a_wait_that_runs_out_ends_the_run(ews, n, boundary):
+    """One block leaves at once: its neighbours' bounded waits give up, all
+    blocks leave, the call returns EWS_ETIMEOUT, and the next run is as usual;
+    the reverse sweep too."""
+    p = synth.small_problem(*n, nt=12, boundary=boundary, kind="moment", width=2, seed=311)
+    sim = ews.simulation_for(p)
+    want = sim.run(p.nt, p.dt)
+    obs = np.ones_like(want) * 1e-9
+    assert sim.tile_shape == "resident"
+    for _ in range(2):
+        ews.ews_test_resident_wait(sim.handle, 50)
+        with pytest.raises(ews.EwsError) as e:
+            sim.run(p.nt, p.dt)
+        assert e.value.status == ews.EWS_ETIMEOUT
+        if boundary != "cpml":
+            with pytest.raises(ews.EwsError) as e:
+                sim.gradient(p.nt, p.dt, obs)
+            assert e.value.status == ews.EWS_ETIMEOUT
+        ews.ews_test_resident_wait(sim.handle, 0)
+        assert np.array_equal(sim.run(p.nt, p.dt), want)
+    for bad in (-1, 2000):
+        with pytest.raises(ews.EwsError) as e:
+            ews.ews_test_resident_wait(sim.handle, bad)
+        assert e.value.status == ews.EWS_EINVAL
+
+
 # blocks of at most 4 planes (a thread per cell), of 5 to 8 (4 cells per thread)
 @pytest.mark.parametrize("n", [(12, 11, 10), (33, 18, 17), (16, 47, 33), (64, 60, 61)])
 @pytest.mark.parametrize("boundary", ["none", "sponge"])
