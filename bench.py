@@ -580,8 +580,8 @@ def storage_report(args, local, with_oracle: bool):
                 "step_launch_ms": round(f_ms, 4),
                 "frac": round(alg["step"] / (f_ms / 1e3) / 1e9 / peak, 4) if f_ms > 0 else None,
                 "note": "frac = 84 B per cell / launch time / peak; the launch is bound by "
-                        "instruction issue (the velocity of a 2-cell ring per tile is "
-                        "recomputed), not by DRAM"}
+                        "latency at 16 warps per SM (the velocity of a 2-cell ring per tile "
+                        "is recomputed) before DRAM"}
         sim.close()
         del seis
     del prob

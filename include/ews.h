@@ -100,7 +100,9 @@ typedef struct ews_sim ews_sim;
 
 /* Create a simulation on the current CUDA device.  Allocates the 9
  * wavefields (of the storage type) and 3 FP32 medium arrays (and C-PML
- * memory variables, FP32).
+ * memory variables, FP32); small FP32 grids, where it can be had, also the
+ * halo buffers of their time loop in one launch (EWS_TILE_RESIDENT), and with
+ * their receivers up to 4 MiB, or 16 steps, of staged samples.
  * opt may be NULL (sponge, W = 16).  *out receives the handle. */
 ews_status ews_create(const ews_grid* grid, const ews_options* opt, ews_sim** out);
 
@@ -428,11 +430,13 @@ ews_status ews_forward_noalloc(const ews_grid* grid, const ews_options* opt,
  * a source/receiver step) of all shots from a device queue; an item waits
  * (bounded, EWS_ETIMEOUT) until its shot's earlier stages are done, so
  * shots of uneven size and step count share the GPU without a grid-wide
- * barrier.  With every option but ckpt_every at 0 a batch times its first
- * forward steps both ways, once per composition, and runs its shots one
- * after the other where that is faster.  Results equal those of ews_run / ews_gradient on each
- * simulation alone (bitwise for the forward, to accumulation order for the
- * gradient). */
+ * barrier.  With every option but ckpt_every at 0 a batch first times its
+ * first forward steps both ways, once per composition (grids, tile shapes
+ * asked for, boundary, steps of the trial, device), and runs its shots one
+ * after the other where that is faster and their memory suffices; batches
+ * with a profiled simulation or FP16 checkpoints always run together.
+ * Results equal those of ews_run / ews_gradient on each simulation alone
+ * (bitwise for the forward, to accumulation order for the gradient). */
 typedef struct {
     ews_sim* sim;             /* configured simulation, used exclusively by this call */
     int nt;                   /* steps (<= the wavelet length)                        */

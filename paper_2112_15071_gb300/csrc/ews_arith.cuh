@@ -34,8 +34,8 @@ __device__ __forceinline__ float sshear(float s, float dto, float mu, float d1, 
     return __fmaf_rn(__fmul_rn(dto, mu), __fadd_rn(d1, d2), s);
 }
 __device__ __forceinline__ float l2m(float lam, float mu) { return __fmaf_rn(2.0f, mu, lam); }
-// 1 / x by the reciprocal instruction (1 ulp), without the range scaling that
-// __fdividef wraps around it: a density needs none.
+// 1 / x by rcp.approx.ftz (at most 1 ulp by the PTX manual; __fdividef is given
+// to 2 ulp): a density is a normal number.
 __device__ __forceinline__ float rcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

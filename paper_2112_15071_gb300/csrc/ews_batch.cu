@@ -468,13 +468,18 @@ ews_status choose_batch_chunks(const ews_batch_shot* shots, int nshots, const st
 // ---- the executor or one shot after the other ----
 // The executor runs the 32 x 8 passes of all shots together; one by one, each
 // shot takes its tuned shape, the fused step or the resident loop.  Which is
-// faster depends on the sizes (GB300, forward, Gcell/s, executor / one by
-// one: 12 cubes 96..224 47.9 / 50.1, 12 cubes 96..160 46.8 / 44.5, 8 cubes
-// 64..128 43.3 / 38.4; 4 shots of 96^3: 8.25 / 6.88 ms, with gradients 25.5 /
-// 22.0), so a batch times its first forward steps both ways once per
-// composition and goes one by one where that is at least 3 % faster -- with
-// gradient shots 13 %, because their reverse passes gain from running together
-// (8 shots of 128^3: forward 1.06x one by one, gradients 0.65 / 0.74 s).
+// faster depends on the sizes, so a batch times its first forward steps both
+// ways once per composition and goes one by one where that is at least 3 %
+// faster -- with gradient shots 13 %, because their reverse passes, which are
+// not timed, gain less from being alone.  One by one over together (GB300, 60
+// steps, sponge), forward, and gradients with checkpoints every 20: 8 x 32^3
+// 1.40, 1.33; 8 x 48^3 1.17, 1.26; 8 x 64^3 0.84, 0.93; 4 x 80^3 1.16, 1.05;
+// 2 x 96^3 0.89, 0.85; 4 x 96^3 0.85, 0.87; 12 x 96^3 1.14, 1.19; 4 x 112^3
+// 0.91, 1.03; 4 x 128^3 0.91, 1.08; 8 x 128^3 0.96, 1.13; 4 x 144^3 0.86, 0.94;
+// 4 x 160^3 0.90, 0.94; 3 x 192^3 0.82, 0.88; 9 cubes 64..128 1.09, 1.17; 9 cubes
+// 96..160 0.99, 1.05; 12 cubes 96..224 0.95 forward.  No choice made at these
+// lines lost; 8 x 64^3 and the gradients of 2 x 96^3 stayed together though one
+// by one is faster (the trial's 6 steps carry a launch each).
 // Time one by one over time together, under g_tune_mu:
 std::map<std::vector<int>, float> g_one_by_one;
 

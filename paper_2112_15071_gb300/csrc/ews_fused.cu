@@ -20,7 +20,8 @@
 // columns need, and the ring adds 31 % velocity work (32 x 8 tiles: 69 %).
 // Taller tiles leave 96 or 80 registers a thread and spill (32 x 28: 35
 // Gcell/s at 1024 x 1024 x 512), lower ones have fewer warps and more ring (32
-// x 20 with 3 slots 60.3, 32 x 16 with 3 slots 63.9 but 58.7 at 256^3).  Row-wise thread order keeps the
+// x 20 with 3 slots 60.3, 32 x 16 with 3 slots 63.9 but 58.7 at 256^3).
+// Row-wise thread order keeps the
 // half-warps on 16 neighbouring pairs of one row (no bank conflicts) and the
 // stress threads in full warps; the ring's outer columns have threads of
 // their own.  Edge masks are selects, not branches: a branch around them for
@@ -29,18 +30,20 @@
 // Measured (GB300, FP32, sponge, Gcell/s, against the two passes): 1024 x
 // 1024 x 512 63.4 (50.5), 256^3 61.7 (51.4), 224^3 58.4 (48.5), 192^3 60.2
 // (50.0 with 32 x 4 tiles); 0.79 and 0.76 of the copy peak on 84 bytes a cell
-// for the first two.  291 warp instructions per 32 cells at 1.8 per cycle and
-// SM; stalls: shared-memory, copy and arithmetic latency at 4 warps per
-// scheduler.
+// for the first two.  282 warp instructions per 32 cells fill 46 % of the issue
+// slots; the warps wait for shared memory, copies and their own arithmetic, at
+// 4 warps per scheduler.
 //
 // Pipeline per CTA (tile x0, y0; z-chunk z0 .. z1), step m for velocity plane
 // k = z0 - 5 + m.  The copies of step m bring each field at the plane at which
 // plane k completes its stencil: sxx, syy, sxy, v at k; sxz, syz, rho at k + 1;
 // szz at k + 2 -- so only z-columns are held in registers, and a slot is read
-// in one step only (two slots: one in use, one in flight).  The new
-// velocity goes to a 5-plane shared ring; after one barrier the stress of
-// plane k - 2 is computed from it, with sigma^n of the cell from the register
-// columns and lambda, mu from a two-entry TMA buffer.  The first three steps
+// in one step only (two slots: one in use, one in flight).  The new velocity
+// goes to a 5-plane shared ring, and the stress of plane k - 2 follows without
+// a barrier: its x and y differences read plane k - 2, complete for two steps
+// (warps count themselves past each step's velocity in an mbarrier), its
+// z-columns are the thread's own; sigma^n of the cell comes from the register
+// columns, lambda and mu from a three-entry TMA buffer.  The first three steps
 // only fill the columns.
 //
 // Every mbarrier wait is bounded.  A point force (Sec. 2.4 source term of Eq.

@@ -736,11 +736,11 @@ Kern pick(int bnd, bool fs) {
     }
 }
 // Cells per thread along z: one z-group of COLS threads per CPT planes.
-// Blocks of at most 4 planes take a thread per cell (32^3: 5.05 us a step),
-// larger ones 4 cells per thread, whose shared columns save loads (70 x 45
-// x 37: 6.3 us, 7.0 with two cells; keeping a thread's own field values in
-// registers as well: 7.0).  Every choice has at least as many threads as
-// halo lines.
+// Blocks of at most 4 planes take a thread per cell (32^3: 4.6 us a step),
+// larger ones 4 cells per thread, whose shared columns save loads (64^3 in
+// blocks of 8 planes: 5.9 us, 6.7 with two cells on 1024 threads; a thread's
+// own field values kept in registers as well gained nothing).  Every choice has
+// at least as many threads as halo lines.
 int cells_per_thread(int lz) { return lz <= 4 ? 1 : 4; }
 int block_threads(int lz) {
     const int cpt = cells_per_thread(lz);

@@ -107,15 +107,18 @@ def test_one_fused_step_from_a_random_state(ews, orc, kind):
     assert rel(seis[:, :, 0], want_seis) <= TOL_ORACLE
 
 
-@pytest.mark.parametrize("corner", [(31.6, 7.6, 18.6), (32.4, 8.4, 19.4), (1.3, 42.6, 34.6)])
+@pytest.mark.parametrize("corner", [(31.6, 23.6, 19.6), (32.4, 24.4, 20.4), (31.6, 7.6, 18.6),
+                                    (32.4, 8.4, 19.4), (1.3, 42.6, 34.6)])
 def test_force_taps_across_tiles_and_z_chunks(ews, orc, corner):
     """A point force whose trilinear taps straddle a tile corner (x = 32,
-    y = 8) and the z-chunk edge (37 planes in two chunks of 19), or sit at
-    the grid's edge: every CTA whose ring holds a tap adds it, the owner
-    alone writes it."""
+    y = 24) and a z-chunk edge (37 planes in four chunks of 10), or one of
+    these alone, or sit at the grid's edge: every CTA whose ring holds a tap
+    adds it, the owner alone writes it."""
     p = synth.small_problem(70, 45, 37, nt=50, boundary="none", kind="force", width=6, seed=204)
     p.src_pos = np.array(corner) * np.array(p.spacing)
-    p.rec_pos = np.array([[31.5, 7.5, 18.5], [32.5, 8.5, 19.5], [10.0, 30.0, 5.0]]) * np.array(p.spacing)
+    near = np.clip(np.array(corner) + np.array([[0.1, 0.1, 0.1], [-1.4, 1.3, -0.9], [3.0, -4.0, 2.0]]),
+                   1.1, np.array([p.nx, p.ny, p.nz]) - 2.1)
+    p.rec_pos = near * np.array(p.spacing)
     ref_seis, ref_state, _ = run(ews, p, "32x8")
     seis, state, _ = run(ews, p, "fused")
     assert rel(seis, ref_seis) <= TOL_SHAPE
