@@ -165,51 +165,50 @@ def _check(status: int):
         raise EwsError(status, msg.decode() if msg else "")
 
 
-def _ptr(a, dtype=np.float32):
-    """(pointer, on_device) of a numpy array or torch tensor."""
+_TORCH_TYPE = {}                                    # numpy type -> torch type, on first use
+
+
+def _ptr(a, dtype=np.float32, need=0, what="buffer"):
+    """(pointer, on_device) of a numpy array or torch tensor; EWS_EINVAL for one
+    of fewer than `need` elements."""
     if a is None:
         return None, 0
     if hasattr(a, "data_ptr"):                      # torch tensor
-        import torch
+        if not _TORCH_TYPE:
+            import torch
+            _TORCH_TYPE.update({np.float32: torch.float32, np.float64: torch.float64})
         assert a.is_contiguous(), "tensor must be contiguous"
-        want = {np.float32: torch.float32, np.float64: torch.float64}[dtype]
+        want = _TORCH_TYPE[dtype]
         assert a.dtype == want, f"tensor dtype must be {want}"
+        if a.numel() < need:
+            _short(what, a.numel(), need)
         return C.c_void_p(a.data_ptr()), int(a.is_cuda)
     arr = np.asarray(a)
     assert arr.dtype == dtype and arr.flags.c_contiguous, \
         f"array must be C-contiguous {np.dtype(dtype).name}"
+    if arr.size < need:
+        _short(what, arr.size, need)
     return arr.ctypes.data_as(C.c_void_p), 0
 
 
-# What the calls on each live simulation read and write, by handle: cells,
-# receivers, snapshot interval and fields.  The C ABI takes bare pointers, so a
-# buffer that a call would run past the end of is refused here.
+def _short(what, have, need):
+    raise EwsError(EWS_EINVAL, f"{what} holds {have} elements, the call needs {need}")
+
+
+# What the calls on each live simulation read and write, by handle.  The C ABI
+# takes bare pointers, so a buffer that a call would run past the end of is
+# refused here.
+class _Sizes:
+    def __init__(self, cells=0, every=0, fields=0):
+        self.cells, self.nrec, self.every, self.fields = cells, 0, every, fields
+
+
 _sizes = {}
+_UNKNOWN = _Sizes()                                 # a handle not made by ews_create here
 
 
 def _sized(sim):
-    return _sizes.get(getattr(sim, "value", sim))
-
-
-def _need(a, n, what):
-    """Refuse a buffer of fewer than n elements."""
-    if a is None:
-        return
-    have = a.numel() if hasattr(a, "data_ptr") else np.asarray(a).size
-    if have < n:
-        raise EwsError(EWS_EINVAL, f"{what} holds {have} elements, the call needs {n}")
-
-
-def _need_cells(sim, arrays, what, fields=1):
-    z = _sized(sim)
-    for a in arrays if z else ():
-        _need(a, fields * z["cells"], what)
-
-
-def _need_traces(sim, a, nt, what):
-    z = _sized(sim)
-    if z:
-        _need(a, 3 * z["nrec"] * int(nt), what)
+    return _sizes.get(getattr(sim, "value", sim), _UNKNOWN)
 
 
 # --- entry points (same names as include/ews.h) ----------------------------
@@ -249,8 +248,7 @@ def ews_create(grid: ews_grid, opt: ews_options | None):
                              C.byref(h)))
     every = opt.snapshot_every if opt is not None else 0
     fields = bin(opt.snapshot_mask).count("1") if opt is not None else 0
-    _sizes[h.value] = {"cells": grid.nx * grid.ny * grid.nz, "nrec": 0, "every": every,
-                       "fields": fields}
+    _sizes[h.value] = _Sizes(grid.nx * grid.ny * grid.nz, every, fields)
     return h
 
 
@@ -265,16 +263,16 @@ def ews_set_stream(sim, stream_handle: int):
 
 
 def ews_set_model_lame(sim, lam, mu, rho):
-    (pl, d0), (pm, d1), (pr, d2) = _ptr(lam), _ptr(mu), _ptr(rho)
+    n = _sized(sim).cells
+    (pl, d0), (pm, d1), (pr, d2) = [_ptr(a, need=n, what="model array") for a in (lam, mu, rho)]
     assert d0 == d1 == d2, "model arrays must share residency"
-    _need_cells(sim, (lam, mu, rho), "model array")
     _check(load().ews_set_model_lame(sim, pl, pm, pr, d0))
 
 
 def ews_set_model_vel(sim, vp, vs, rho):
-    (pa, d0), (pb, d1), (pr, d2) = _ptr(vp), _ptr(vs), _ptr(rho)
+    n = _sized(sim).cells
+    (pa, d0), (pb, d1), (pr, d2) = [_ptr(a, need=n, what="model array") for a in (vp, vs, rho)]
     assert d0 == d1 == d2, "model arrays must share residency"
-    _need_cells(sim, (vp, vs, rho), "model array")
     _check(load().ews_set_model_vel(sim, pa, pb, pr, d0))
 
 
@@ -293,8 +291,8 @@ def ews_set_receivers(sim, pos):
     r = np.ascontiguousarray(pos, np.float64).reshape(-1, 3)
     _check(load().ews_set_receivers(sim, int(r.shape[0]),
                                     r.ctypes.data_as(C.c_void_p) if r.size else None))
-    if _sized(sim):
-        _sized(sim)["nrec"] = int(r.shape[0])
+    if _sized(sim) is not _UNKNOWN:
+        _sized(sim).nrec = int(r.shape[0])
 
 
 def ews_set_model_coarse(sim, a, b, rho, from_velocities: bool = False):
@@ -313,20 +311,19 @@ def ews_set_free_surface(sim, ks: int, eps: float = 1e-3):
 
 
 def ews_run(sim, nt: int, dt: float, seis, snapshots=None):
-    ps, dev = _ptr(seis)
-    pn, devn = _ptr(snapshots)
-    if snapshots is not None:
-        assert devn == dev, "seis and snapshots must share residency"
-    _need_traces(sim, seis, nt, "seis")
     z = _sized(sim)
-    if z and z["every"] > 0:
-        _need(snapshots, int(nt) // z["every"] * z["fields"] * z["cells"], "snapshots")
+    ps, dev = _ptr(seis, need=3 * z.nrec * int(nt), what="seis")
+    if snapshots is None:
+        pn = None
+    else:
+        n = int(nt) // z.every * z.fields * z.cells if z.every > 0 else 0
+        pn, devn = _ptr(snapshots, need=n, what="snapshots")
+        assert devn == dev, "seis and snapshots must share residency"
     _check(load().ews_run(sim, int(nt), float(dt), ps, dev, pn))
 
 
 def ews_advance(sim, n0: int, nsteps: int, dt: float, seis, ld: int):
-    ps, dev = _ptr(seis)
-    _need_traces(sim, seis, ld, "seis")
+    ps, dev = _ptr(seis, need=3 * _sized(sim).nrec * int(ld), what="seis")
     _check(load().ews_advance(sim, int(n0), int(nsteps), float(dt), ps, int(ld), dev))
 
 
@@ -335,14 +332,12 @@ def ews_reset(sim):
 
 
 def ews_get_state(sim, out):
-    p, dev = _ptr(out)
-    _need_cells(sim, (out,), "state", 9)
+    p, dev = _ptr(out, need=9 * _sized(sim).cells, what="state")
     _check(load().ews_get_state(sim, p, dev))
 
 
 def ews_set_state(sim, state):
-    p, dev = _ptr(state)
-    _need_cells(sim, (state,), "state", 9)
+    p, dev = _ptr(state, need=9 * _sized(sim).cells, what="state")
     _check(load().ews_set_state(sim, p, dev))
 
 
@@ -375,21 +370,19 @@ def ews_release_workspace(sim):
 
 
 def ews_adjoint(sim, nt: int, dt: float, seis_adj, g_lam, g_mu, g_rho, ckpt_every: int = 0):
-    pa, da = _ptr(seis_adj)
-    (pl, d0), (pm, d1), (pr, d2) = _ptr(g_lam), _ptr(g_mu), _ptr(g_rho)
+    z = _sized(sim)
+    pa, da = _ptr(seis_adj, need=3 * z.nrec * int(nt), what="seis_adj")
+    (pl, d0), (pm, d1), (pr, d2) = [_ptr(a, need=z.cells, what="gradient output") for a in (g_lam, g_mu, g_rho)]
     assert d0 == d1 == d2, "gradient outputs must share residency"
-    _need_traces(sim, seis_adj, nt, "seis_adj")
-    _need_cells(sim, (g_lam, g_mu, g_rho), "gradient output")
     _check(load().ews_adjoint(sim, int(nt), float(dt), pa, da, pl, pm, pr, d0, int(ckpt_every)))
 
 
 def ews_gradient(sim, nt: int, dt: float, observed, g_lam, g_mu, g_rho, ckpt_every: int = 0):
     """Returns the L2 misfit; gradients are written into g_lam, g_mu, g_rho."""
-    po, do = _ptr(observed)
-    (pl, d0), (pm, d1), (pr, d2) = _ptr(g_lam), _ptr(g_mu), _ptr(g_rho)
+    z = _sized(sim)
+    po, do = _ptr(observed, need=3 * z.nrec * int(nt), what="observed")
+    (pl, d0), (pm, d1), (pr, d2) = [_ptr(a, need=z.cells, what="gradient output") for a in (g_lam, g_mu, g_rho)]
     assert d0 == d1 == d2, "gradient outputs must share residency"
-    _need_traces(sim, observed, nt, "observed")
-    _need_cells(sim, (g_lam, g_mu, g_rho), "gradient output")
     mis = C.c_double(0.0)
     _check(load().ews_gradient(sim, int(nt), float(dt), po, do, C.byref(mis), pl, pm, pr, d0,
                                int(ckpt_every)))
@@ -408,15 +401,12 @@ def ews_batch(shots, mode: int = EWS_BATCH_PERSISTENT, ckpt_every: int = 0, zchu
         b.sim = d["sim"].handle.value if hasattr(d["sim"], "handle") else d["sim"]
         b.nt = int(d["nt"])
         b.dt = float(d["dt"])
+        z = _sized(b.sim)
         for key in ("seis", "observed", "g_lam", "g_mu", "g_rho"):
             t = d.get(key)
             if t is not None:
-                p, dev = _ptr(t)
+                p, dev = _ptr(t, need=z.cells if key[0] == "g" else 3 * z.nrec * b.nt, what=key)
                 assert dev == 1, f"{key} must be a CUDA tensor"
-                if key in ("seis", "observed"):
-                    _need_traces(b.sim, t, b.nt, key)
-                else:
-                    _need_cells(b.sim, (t,), key)
                 setattr(b, key, p.value)
     opt = ews_batch_options(int(mode), int(ckpt_every), int(zchunk), int(ctas_per_sm),
                             int(dep_wait_ms), int(bool(test_unsatisfiable)))
@@ -434,14 +424,13 @@ def ews_fwi_iteration(shots, lam, mu, rho, max_rel_step: float = 0.02, ckpt_ever
         arr[i].sim = d["sim"].handle.value if hasattr(d["sim"], "handle") else d["sim"]
         arr[i].nt = int(d["nt"])
         arr[i].dt = float(d["dt"])
-        p, dev = _ptr(d["observed"])
+        z = _sized(arr[i].sim)
+        p, dev = _ptr(d["observed"], need=3 * z.nrec * arr[i].nt, what="observed")
         assert dev == 1, "observed must be a CUDA tensor"
-        _need_traces(arr[i].sim, d["observed"], d["nt"], "observed")
-        _need_cells(arr[i].sim, (lam, mu, rho), "model array")
         arr[i].observed = p.value
     ptrs = []
     for t in (lam, mu, rho):
-        p, dev = _ptr(t)
+        p, dev = _ptr(t, need=z.cells if shots else 0, what="model array")   # one grid for all shots
         assert dev == 1, "the model must be CUDA tensors"
         ptrs.append(p)
     j0, j1, a = C.c_double(), C.c_double(), C.c_double()
@@ -596,19 +585,17 @@ def ews_forward_noalloc(grid: ews_grid, opt: ews_options | None, lam, mu, rho, k
     """Forward run without any device allocation (see include/ews.h).
     lam, mu, rho, wavelet and seis must be CUDA tensors (device pointers)."""
     ptrs = []
-    for a in (lam, mu, rho, wavelet, seis):
-        p, dev = _ptr(a)
+    r = np.ascontiguousarray(rec_pos, np.float64).reshape(-1, 3)
+    n = grid.nx * grid.ny * grid.nz
+    for a, need, what in ((lam, n, "model array"), (mu, n, "model array"), (rho, n, "model array"),
+                          (wavelet, int(nt), "wavelet"), (seis, 3 * r.shape[0] * int(nt), "seis")):
+        p, dev = _ptr(a, need=need, what=what)
         assert dev == 1, "ews_forward_noalloc takes device buffers"
         ptrs.append(p)
     p = np.ascontiguousarray(pos, np.float64).reshape(3)
     c = np.zeros(6)
     cc = np.asarray(comp, np.float64).ravel()
     c[:cc.size] = cc
-    r = np.ascontiguousarray(rec_pos, np.float64).reshape(-1, 3)
-    for a in (lam, mu, rho):
-        _need(a, grid.nx * grid.ny * grid.nz, "model array")
-    _need(wavelet, int(nt), "wavelet")
-    _need(seis, 3 * r.shape[0] * int(nt), "seis")
     _check(load().ews_forward_noalloc(
         C.byref(grid), C.byref(opt) if opt is not None else None, ptrs[0], ptrs[1], ptrs[2],
         int(kind), p.ctypes.data_as(C.c_void_p), c.ctypes.data_as(C.c_void_p), ptrs[3],
